@@ -121,33 +121,32 @@ typedef struct {
     kmc_alloc_fn alloc; /* optional device allocator; NULL = cudaMalloc */
     kmc_free_fn free;
     void* alloc_ctx;
-    int32_t schedule;   /* 0 = auto: mixed-form replicas whose state fits one SM run in the
-                           replica-resident kernel, the rest one launch per colour phase;
-                           1 = colour-phase launches only; 2 = resident kernel only */
-    int32_t cluster_top; /* resident kernel: how many of the largest replicas of the 1024-thread
-                            class run as 2-CTA thread-block clusters (each CTA holds the replica
-                            and takes half of every phase's fragments; writes are mirrored
-                            through distributed shared memory).  -1 (default) = SMs / 8,
-                            0 = none */
+    int32_t schedule;   /* 0 = auto: replicas whose state fits the shared memory of one SM, or of a
+                           thread-block cluster (cluster_ctas), run in the resident kernels,
+                           the rest one launch per colour phase; 1 = colour-phase launches
+                           only; 2 = resident kernels only (mixed form) */
+    int32_t cluster_top; /* mixed form: how many of the largest replicas of the largest
+                            shared-memory class run as 2-CTA thread-block clusters, a z-slab
+                            each.  -1 (default) = SMs / 8, 0 = none */
     int32_t small_pass; /* colour-phase kernels: sparse fragments run in a pass of their own besides
                            the general one (one warp per fragment); same trajectory.  Mixed form:
                            one thread per fragment (see lane_form); plain form (and mode 2):
                            fragments holding one or two vacancies, 4 or 2 per warp in lock-step.
                            0 (default) = where a phase holds 32768 fragments or more,
                            1 = always, 2 = always and in the grouped form, -1 = never */
-    int32_t test_stuck_wait_us; /* test of the device-side bounded wait (0 = off): the replica-resident
-                                   kernel, after staging its state, waits on a barrier that nothing
+    int32_t test_stuck_wait_us; /* test of the device-side bounded wait (0 = off): the one-CTA
+                                   resident kernel, after staging its state, waits on a barrier that nothing
                                    completes, gives up after this many microseconds (<= 2e6) and
                                    kmc_run returns FKMC_ETIMEOUT with the state untouched */
     int32_t lane_form;  /* mixed form, one-thread-per-fragment pass: 0 (default) = by phase size,
                            1 = registers (up to 4 vacancies, beside the general pass),
                            2 = persistent (up to 8 vacancies in shared memory, a grid that
                            stays resident for the phase; the general pass after it) */
-    int32_t cluster_ctas; /* mixed form: a replica too large for one SM's shared memory runs in the
+    int32_t cluster_ctas; /* a replica too large for one SM's shared memory runs in the
                              cluster-resident kernel (a thread-block cluster of up to 16 CTAs,
                              each holding a z-slab of fragment layers in shared memory, peers'
                              slabs reached through distributed shared memory) where its slabs
-                             fit.  0 (default) = so, with the fewest CTAs that fit; -1 = never
+                             fit.  0 (default) = so, with the most CTAs that fit; -1 = never
                              (the colour-phase kernels); 2..16 = every replica with that many
                              fragment layers or more, with exactly this many CTAs */
     int32_t reserved[2];
@@ -181,14 +180,15 @@ typedef struct {
     int64_t n_Fe;        /* dopants */
     int32_t kernel;      /* how kmc_run advances the replica under the current rates and options:
                             0 = colour-phase kernels (one launch per phase), 1 = replica-resident
-                            kernel (state in one SM's shared memory, or a 2-CTA mirrored pair),
+                            kernel (state in one SM's shared memory, or in two with cluster_top),
                             2 = cluster-resident kernel (z-slabs in a thread-block cluster) */
     int32_t ctas;        /* CTAs holding the replica (kernels 1 and 2), else 0 */
     int32_t draw_phases; /* kernel 1: colour phases whose fragments' first random draws the kernel
                             makes in one batch (8, 4, 2 or 1, as the replica's shared-memory class
                             leaves room), else 0 */
-    int32_t draw_events; /* kernel 1: events per fragment and phase drawn in that batch (4 where
-                            2 or more phases of them fit, else 2), else 0 */
+    int32_t draw_events; /* kernel 1: events per fragment and phase drawn in that batch at most
+                            (mixed form: 4 where 2 or more phases of them fit, else 2; plain
+                            form: 4 or 8), else 0 */
 } kmc_replica_info;
 
 typedef struct kmc_batch kmc_batch;

@@ -150,10 +150,16 @@ struct kmc_batch {
     int32_t* d_reps = nullptr;   // resident replica ids, class by class
     ClusterPlan* d_plans = nullptr;  // cluster-resident replicas' slab plans, grouped by CTA count
     ResCache rcache{};               // fragment totals the resident kernels carry from call to call
-    int64_t* d_nvac = nullptr;   // vacancies per replica
-    // a launch of the replica-resident kernel (one CTA, or a 2-CTA mirrored pair, per
-    // replica; start/count index d_reps) or of the cluster-resident kernel (slabs
-    // == true: one cluster of `cluster` CTAs per replica; start/count index d_plans)
+    uint32_t* vmap = nullptr;        // resident replicas: record index of every vacancy's site
+    VacRec* rec_tmp = nullptr;       // and the stage-out copies of their records
+    Draw* draws = nullptr;           // plain form: first draws of draw_windows windows, two buffers
+    size_t vmap_bytes = 0, tmp_bytes = 0, draws_bytes = 0;
+    int64_t res_frags = 0, res_max_frag = 0;
+    int res_ev = 4, draw_windows = 0;
+    cudaStream_t draw_st = nullptr;
+    cudaEvent_t draw_done[2] = {nullptr, nullptr}, draw_free[2] = {nullptr, nullptr};
+    // a launch of the resident kernel: one CTA per replica (start/count index d_reps)
+    // or, with slabs, one cluster of `cluster` CTAs per replica (index d_plans)
     struct RClass {
         int start, count;
         size_t smem;
@@ -301,6 +307,13 @@ struct kmc_batch {
         if (res_join) cudaEventDestroy(res_join);
         res_st = nullptr;
         res_fork = res_join = nullptr;
+        if (draw_st) cudaStreamDestroy(draw_st);
+        draw_st = nullptr;
+        for (int k = 0; k < 2; ++k) {
+            if (draw_done[k]) cudaEventDestroy(draw_done[k]);
+            if (draw_free[k]) cudaEventDestroy(draw_free[k]);
+            draw_done[k] = draw_free[k] = nullptr;
+        }
         if (null_exec) cudaGraphExecDestroy(null_exec);
         null_exec = nullptr;
         for (auto& g : elec_graphs) cudaGraphExecDestroy(g.exec);
@@ -404,60 +417,74 @@ int plan_residency(kmc_batch* b)
         if (c.done) cudaEventDestroy(c.done);
     }
     b->rclass.clear();
-    const bool allowed = b->opts.precision == FKMC_MIXED && b->opts.schedule != 1 &&
+    const int prec = b->opts.precision == FKMC_MIXED ? 1 : 0;
+    const bool allowed = b->opts.schedule != 1 && (prec == 1 || b->opts.schedule == 0) &&
                          b->cap <= RESIDENT_MAX_SLOTS && !site_path(b) && !b->grains_on;
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 1;
     // launch classes: (shared-memory bound, threads); a replica takes the first
     // class its state fits, so small replicas pack several CTAs per SM and the
-    // largest get the most warps that still fit beside their state.  The
-    // `cluster_top` largest replicas of the 1024-thread class run as 2-CTA
-    // clusters (two SMs each), as long as the GPU has the SMs to spare.
-    const size_t bounds[5] = {24 * 1024, 48 * 1024, 96 * 1024, RESIDENT_MAX_SMEM, RESIDENT_MAX_SMEM};
-    const int threads[5] = {128, 128, 256, 1024, 512};
-    std::vector<std::vector<int>> cls(6);
-    std::vector<size_t> cmax(6, 0), need_of(b->n, 0);
+    // largest get the most warps.
+    const size_t bounds[4] = {24 * 1024, 48 * 1024, 96 * 1024, RESIDENT_MAX_SMEM};
+    const int threads[4] = {128, 128, 256, 512};
+    // events per fragment drawn ahead in the plain form (k_draws): about twice
+    // the expected number of a visit
+    double mean = 0.0;
+    for (int r = 0; r < b->n; ++r)
+        mean = std::max(mean, (double)b->n_vac[r] / ((double)b->desc[r].nf[0] * b->desc[r].nf[1] * b->desc[r].nf[2]));
+    const int plain_ev = mean * b->opts.n_tau <= 0.5 ? 4 : 8;
+    std::vector<std::vector<int>> cls(4);
+    std::vector<size_t> cmax(4, 0), need_of(b->n, 0);
     std::vector<ClusterPlan> plans;
+    std::vector<int> pairs;  // replicas that may run on two CTAs (kmc_opts.cluster_top)
     b->any_global = false;
     b->run_kernel.assign(b->n, 0);
     b->run_ctas.assign(b->n, 0);
     for (int r = 0; r < b->n; ++r) {
+        RepDesc& D = b->desc[r];
         int c = -1;
         size_t need = 0;
-        for (int k = 0; k < 5 && allowed && c < 0; ++k) {
-            need = resident_smem_bytes(b->desc[r], b->n_vac[r], b->cap, threads[k], 1, 2);
+        for (int k = 0; k < 4 && allowed && c < 0; ++k) {
+            need = resident_smem_bytes(D, b->cap, threads[k], 1, prec ? 2 : plain_ev, prec);
             if (need <= bounds[k]) c = k;
         }
         // the first draws of as many colour phases per batch as the class's shared
         // memory allows beside the state (8: one batch per window): four events per
         // fragment where 2 or more phases of them fit, else two
-        b->desc[r].pre_g = 1;
-        b->desc[r].pre_ev = 2;
+        D.pre_g = 1;
+        D.pre_ev = prec ? 2 : plain_ev;
         static const int pick[6][2] = {{8, 4}, {4, 4}, {2, 4}, {8, 2}, {4, 2}, {2, 2}};  // (phases, events)
         for (int k = 0; c >= 0 && k < 6; ++k) {
-            const size_t ng = resident_smem_bytes(b->desc[r], b->n_vac[r], b->cap, threads[c], pick[k][0], pick[k][1]);
+            const int ev = prec ? pick[k][1] : plain_ev;
+            const size_t ng = resident_smem_bytes(D, b->cap, threads[c], pick[k][0], ev, prec);
             if (ng <= bounds[c]) {
-                b->desc[r].pre_g = pick[k][0];
-                b->desc[r].pre_ev = pick[k][1];
+                D.pre_g = pick[k][0];
+                D.pre_ev = ev;
                 need = ng;
                 break;
             }
         }
-        // the cluster-resident kernel: a replica too large for one SM (or every
-        // replica, with cluster_ctas forced) held by a cluster of CTAs, one z-slab each
+        // a cluster: a replica too large for one SM (or every replica, with
+        // cluster_ctas forced), on the most CTAs that fit
         const int force = b->opts.cluster_ctas;
         if (allowed && force >= 0 && (c < 0 || force >= 2)) {
             ClusterPlan pl{};
+            const int ev = prec ? 4 : plain_ev;
             const int lo = force >= 2 ? force : 2, hi = force >= 2 ? force : CLUSTER_MAX_CTAS;
-            if (make_cluster_plan(b->desc[r], b->n_vac[r], b->cap, lo, hi, &pl) &&
-                cluster_fits(pl.ncta, cluster_smem_bytes(b->desc[r], pl, b->cap)) > 0) {
+            if (make_cluster_plan(D, b->cap, ev, prec, lo, hi, &pl) &&
+                cluster_fits(prec, pl.ncta, cluster_smem_bytes(D, pl, b->cap, ev, prec)) > 0) {
                 pl.rep = r;
                 plans.push_back(pl);
-                b->desc[r].resident = 1;
+                D.resident = 1;
+                D.pre_ev = ev;
                 b->run_kernel[r] = 2;
                 b->run_ctas[r] = pl.ncta;
                 continue;
             }
         }
-        b->desc[r].resident = c >= 0 ? 1 : 0;
+        D.resident = c >= 0 ? 1 : 0;
         if (c < 0) {
             b->any_global = true;
             continue;
@@ -469,24 +496,74 @@ int plan_residency(kmc_batch* b)
     }
     // largest replicas (by vacancies, the work per phase) first in every class: the
     // longest-running CTAs start earliest, which shortens the tail of the launch
-    for (int c = 0; c < 5; ++c)
+    for (int c = 0; c < 4; ++c)
         std::sort(cls[c].begin(), cls[c].end(), [&](int a, int q) {
             return b->n_vac[a] != b->n_vac[q] ? b->n_vac[a] > b->n_vac[q] : a < q;
         });
-    // optionally the largest of the 1024-thread class run as 2-CTA clusters (class 5)
-    const int ntop = std::min<int>((int)cls[3].size(), b->cluster_top);
-    cls[5].assign(cls[3].begin(), cls[3].begin() + ntop);
-    cls[3].erase(cls[3].begin(), cls[3].begin() + ntop);
-    for (int r : cls[5]) b->run_ctas[r] = 2;
-    for (int c = 0; c < 6; ++c)
+    // the largest of the last class on two CTAs each (kmc_opts.cluster_top)
+    for (int k = 0; prec == 1 && k < std::min<int>((int)cls[3].size(), b->cluster_top);) {
+        const int r = cls[3][k];
+        ClusterPlan pl{};
+        if (!make_cluster_plan(b->desc[r], b->cap, 4, prec, 2, 2, &pl) ||
+            cluster_fits(prec, 2, cluster_smem_bytes(b->desc[r], pl, b->cap, 4, prec)) <= 0) {
+            ++k;
+            continue;
+        }
+        pl.rep = r;
+        plans.push_back(pl);
+        b->desc[r].pre_ev = 4;
+        b->run_ctas[r] = 2;
+        pairs.push_back(r);
+        if ((int)pairs.size() >= b->cluster_top) break;
+        ++k;
+    }
+    for (int r : pairs) cls[3].erase(std::find(cls[3].begin(), cls[3].end(), r));
+    // more warps for the replicas with the most vacancies while every CTA still has
+    // its share of an SM (a class's CTAs per SM: by registers 4, 4, 2, 1): a phase
+    // takes as long as its slowest visit, so a visit should not wait for a warp
+    {
+        const double share[4] = {0.25, 0.25, 0.5, 1.0};
+        double used = 0.0;
+        std::vector<std::pair<int64_t, int>> order;
+        for (int c = 0; c < 4; ++c)
+            for (int r : cls[c]) {
+                used += share[c];
+                order.push_back({b->n_vac[r], r});
+            }
+        for (const ClusterPlan& pl : plans) used += pl.ncta;
+        std::sort(order.rbegin(), order.rend());
+        for (auto& o : order) {
+            const int r = o.second;
+            const RepDesc& D = b->desc[r];
+            const int maxc = ((D.nf[0] + 1) / 2) * ((D.nf[1] + 1) / 2) * ((D.nf[2] + 1) / 2);
+            for (int c = 0; c < 3; ++c) {
+                auto it = std::find(cls[c].begin(), cls[c].end(), r);
+                if (it == cls[c].end()) continue;
+                const int to = c < 2 ? 2 : 3;
+                const int warps = threads[c] / 32;  // one visit per warp, at most maxc of them
+                const size_t nd = resident_smem_bytes(D, b->cap, threads[to], D.pre_g, D.pre_ev, prec);
+                if (maxc <= warps || o.first <= 4 * warps || used + share[to] - share[c] > (double)sms ||
+                    nd > RESIDENT_MAX_SMEM)
+                    break;
+                used += share[to] - share[c];
+                cls[c].erase(it);
+                cls[to].push_back(r);
+                need_of[r] = nd;
+            }
+        }
+    }
+    for (int c = 0; c < 4; ++c)
+        std::sort(cls[c].begin(), cls[c].end(), [&](int a, int q) {
+            return b->n_vac[a] != b->n_vac[q] ? b->n_vac[a] > b->n_vac[q] : a < q;
+        });
+    for (int c = 0; c < 4; ++c)
         for (int r : cls[c]) cmax[c] = std::max(cmax[c], need_of[r]);
     if (b->opts.schedule == 2 && b->any_global)
         return fail(FKMC_EINVAL, "schedule 2 needs every replica to fit the resident kernel (mixed form)");
     std::vector<int32_t> order;
-    for (int c = 0; c < 6; ++c) {
+    for (int c = 0; c < 4; ++c) {
         if (cls[c].empty()) continue;
-        kmc_batch::RClass rc{(int)order.size(), (int)cls[c].size(), cmax[c], c == 5 ? 1024 : threads[c],
-                             c == 5 ? 2 : 1, nullptr, nullptr, false};
+        kmc_batch::RClass rc{(int)order.size(), (int)cls[c].size(), cmax[c], threads[c], 1, nullptr, nullptr, false};
         for (int r : cls[c]) order.push_back(r);
         CK(cudaStreamCreateWithFlags(&rc.st, cudaStreamNonBlocking), "stream");
         CK(cudaEventCreateWithFlags(&rc.done, cudaEventDisableTiming), "event");
@@ -496,13 +573,14 @@ int plan_residency(kmc_batch* b)
         CK(cudaMemcpyAsync(b->d_reps, order.data(), sizeof(int32_t) * order.size(), cudaMemcpyHostToDevice,
                            b->st),
            "replica list upload");
-    // cluster-resident replicas: one launch per CTA count (a launch has one cluster shape)
+    // replicas on clusters: one launch per CTA count (a launch has one cluster shape)
     std::stable_sort(plans.begin(), plans.end(),
                      [](const ClusterPlan& x, const ClusterPlan& y) { return x.ncta < y.ncta; });
     for (size_t k = 0; k < plans.size();) {
         size_t e = k, smem = 0;
         while (e < plans.size() && plans[e].ncta == plans[k].ncta) {
-            smem = std::max(smem, cluster_smem_bytes(b->desc[plans[e].rep], plans[e], b->cap));
+            const RepDesc& D = b->desc[plans[e].rep];
+            smem = std::max(smem, cluster_smem_bytes(D, plans[e], b->cap, D.pre_ev, prec));
             ++e;
         }
         kmc_batch::RClass rc{(int)k, (int)(e - k), smem, CLUSTER_THREADS, plans[k].ncta, nullptr, nullptr, true};
@@ -515,6 +593,37 @@ int plan_residency(kmc_batch* b)
         CK(cudaMemcpyAsync(b->d_plans, plans.data(), sizeof(ClusterPlan) * plans.size(), cudaMemcpyHostToDevice,
                            b->st),
            "cluster plan upload");
+    // the resident replicas' buffers: site -> record maps, stage-out copies, first draws (plain form)
+    int64_t sites = 0, frags = 0;
+    b->res_max_frag = 0;
+    for (RepDesc& D : b->desc) {
+        D.vmap_off = sites;
+        D.tmp_off = D.draw_off = frags;
+        if (!D.resident) continue;
+        const int64_t nf = (int64_t)D.nf[0] * D.nf[1] * D.nf[2];
+        sites += 48 * (int64_t)D.L[2] * D.L[1] * D.row_words;  // sixteen sites per occupancy word
+        frags += nf;
+        b->res_max_frag = std::max(b->res_max_frag, nf);
+    }
+    b->res_frags = frags;
+    b->res_ev = plain_ev;
+    auto grow = [&](void** p, size_t* have, size_t want) -> bool {
+        if (want <= *have) return true;
+        b->dfree(*p);
+        *p = b->dalloc(want);
+        *have = *p ? want : 0;
+        return *p != nullptr;
+    };
+    b->draw_windows = 0;
+    if (frags > 0 && prec == 0) {  // two buffers of up to 64 windows, 64 MB together where one window fits
+        const int64_t per = frags * plain_ev * (int64_t)sizeof(Draw);
+        b->draw_windows = (int)std::max<int64_t>(1, std::min<int64_t>(64, ((int64_t)32 << 20) / per));
+        if (!grow((void**)&b->draws, &b->draws_bytes, 2 * (size_t)per * b->draw_windows))
+            return fail(FKMC_ENOMEM, "device allocation failed (first draws)");
+    }
+    if (frags > 0 && (!grow((void**)&b->vmap, &b->vmap_bytes, sizeof(uint32_t) * (size_t)sites) ||
+                      !grow((void**)&b->rec_tmp, &b->tmp_bytes, sizeof(VacRec) * (size_t)frags * b->cap)))
+        return fail(FKMC_ENOMEM, "device allocation failed (resident replicas)");
     return FKMC_OK;
 }
 
@@ -972,10 +1081,8 @@ int kmc_create_batch(int32_t n, const kmc_cells* cells, const kmc_composition* c
     b->scratch_all = (unsigned long long*)b->dalloc(sizeof(unsigned long long) * 7 * n);
     b->d_reps = (int32_t*)b->dalloc(sizeof(int32_t) * n);
     b->d_plans = (ClusterPlan*)b->dalloc(sizeof(ClusterPlan) * n);
-    b->rcache.tot = (unsigned long long*)b->dalloc(sizeof(unsigned long long) * std::max<int64_t>(b->nfrag_total, 1));
-    b->rcache.dirty = (uint8_t*)b->dalloc((size_t)std::max<int64_t>(b->nfrag_total, 1));
+    b->rcache.lim = (uint64_t*)b->dalloc(sizeof(uint64_t) * std::max<int64_t>(b->nfrag_total, 1));
     b->rcache.valid = (uint8_t*)b->dalloc((size_t)n);
-    b->d_nvac = (int64_t*)b->dalloc(sizeof(int64_t) * n);
     b->wctl = (unsigned long long*)b->dalloc(sizeof(unsigned long long) * 2);
     b->perms = (uint32_t*)b->dalloc(sizeof(uint32_t) * n);
     b->act = (ActEntry*)b->dalloc(sizeof(ActEntry) * 3 * std::max<int64_t>(b->total_items, 1));
@@ -993,8 +1100,8 @@ int kmc_create_batch(int32_t n, const kmc_cells* cells, const kmc_composition* c
         }
     }
     if (!b->occ || !b->recs || !b->counts || (o.tracer && !b->tracer) || !b->d_desc || !b->stats ||
-        !b->status || !b->scratch || !b->scratch_all || !b->d_reps || !b->d_plans || !b->rcache.tot ||
-        !b->rcache.dirty || !b->rcache.valid || !b->d_nvac || !b->wctl ||
+        !b->status || !b->scratch || !b->scratch_all || !b->d_reps || !b->d_plans || !b->rcache.lim ||
+        !b->rcache.valid || !b->wctl ||
         !b->perms ||
         !b->act || !b->act_count || !b->cls) {
         b->release();
@@ -1011,7 +1118,6 @@ int kmc_create_batch(int32_t n, const kmc_cells* cells, const kmc_composition* c
     step(phase_prepare(b->cap), "kernel attributes");
     step(run_pass_blocks(b->opts.precision, b->cap, false, false, &b->run_blocks), "occupancy query");
     step(resident_prepare(), "kernel attributes");
-    step(cluster_prepare(), "kernel attributes");
     step(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "event");
     step(cudaEventCreate(&b->ev0), "event");
     step(cudaEventCreate(&b->ev1), "event");
@@ -1089,50 +1195,81 @@ int kmc_set_barriers(kmc_batch* b, const kmc_barrier_table* tables, const double
         rc = build_btab(b);
         if (rc) return rc;
     }
+    b->rates_set = false;  // a failed plan leaves nothing to run
     rc = plan_residency(b);
     if (rc) return rc;
-    CK(cudaMemcpyAsync(b->d_nvac, b->n_vac.data(), sizeof(int64_t) * b->n, cudaMemcpyHostToDevice, b->st),
-       "vacancy count upload");
     rc = upload_desc(b);
     if (rc) return rc;
     b->rates_set = true;
     return FKMC_OK;
 }
 
-int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
+}  // extern "C"
+
+namespace {
+
+ResidentArgs resident_args(const kmc_batch* b)
 {
-    NvtxRange nvtx_range("kmc_run");
-    if (!b) return fail(FKMC_EINVAL, "null batch");
-    if (!b->rates_set) return fail(FKMC_ESTATE, "kmc_set_barriers must come before kmc_run");
-    std::vector<unsigned long long> before = b->stats_host;
-    CK(cudaEventRecord(b->ev0, b->st), "event record");
-    if (!b->rclass.empty() && windows > 0) {
-        // replica-resident classes on forked streams, joined back: captured once
-        // per window count into a graph (fork, one launch per class, join) and
-        // replayed on the caller's stream
+    ResidentArgs a;
+    a.descs = b->d_desc;
+    a.occ = b->occ;
+    a.recs = b->recs;
+    a.tmp = b->rec_tmp;
+    a.vmap = b->vmap;
+    a.counts = b->counts;
+    a.tracer = b->tracer;
+    a.stats = b->stats;
+    a.status = b->status;
+    a.cap = b->cap;
+    a.nbt = b->nbt;
+    a.frag_tot = b->res_frags;
+    a.stuck_wait_us = (uint32_t)b->opts.test_stuck_wait_us;
+    a.rc = b->rcache;
+    return a;
+}
+
+// one launch per class on the classes' streams, after `from` and before `to`
+// (largest classes first: their CTAs run longest and should take SMs first)
+cudaError_t launch_classes(kmc_batch* b, int prec, uint64_t w0, uint64_t windows, const Draw* draws, cudaEvent_t from,
+                           cudaStream_t to)
+{
+    const ResidentArgs args = resident_args(b);
+    cudaError_t le = cudaSuccess;
+    for (auto it = b->rclass.rbegin(); it != b->rclass.rend() && le == cudaSuccess; ++it) {
+        auto& c = *it;
+        le = cudaStreamWaitEvent(c.st, from, 0);
+        if (le == cudaSuccess && c.slabs)
+            le = launch_cluster(prec, args, b->d_plans + c.start, c.count, c.cluster, c.smem, w0, windows, draws, c.st);
+        else if (le == cudaSuccess)
+            le = launch_resident(prec, args, b->d_reps + c.start, c.count, c.smem, c.threads, w0, windows, draws, c.st);
+        if (le == cudaSuccess) le = cudaEventRecord(c.done, c.st);
+        if (le == cudaSuccess) le = cudaStreamWaitEvent(to, c.done, 0);
+    }
+    return le;
+}
+
+// The resident replicas' windows on a stream beside the caller's (res_st, after
+// res_fork, ended by res_join).  Mixed form: the class launches captured once
+// per window count into a graph (fork, one launch per class, join).  Plain
+// form: the first draws of draw_windows windows at a time by k_draws on a
+// stream of their own, the next chunk's beside the current chunk's windows
+// (two buffers).
+int launch_resident_classes(kmc_batch* b, uint64_t windows, uint64_t* launches)
+{
+    if (!b->cap_st) CK(cudaStreamCreateWithFlags(&b->cap_st, cudaStreamNonBlocking), "stream");
+    if (!b->res_st) {
+        CK(cudaStreamCreateWithFlags(&b->res_st, cudaStreamNonBlocking), "stream");
+        CK(cudaEventCreateWithFlags(&b->res_fork, cudaEventDisableTiming), "event");
+        CK(cudaEventCreateWithFlags(&b->res_join, cudaEventDisableTiming), "event");
+    }
+    if (b->opts.precision == FKMC_MIXED) {
         if (!b->res_exec || b->res_exec_windows != windows) {
             if (b->res_exec) cudaGraphExecDestroy(b->res_exec);
             b->res_exec = nullptr;
-            if (!b->cap_st) CK(cudaStreamCreateWithFlags(&b->cap_st, cudaStreamNonBlocking), "stream");
             cudaGraph_t graph = nullptr;
             CK(cudaStreamBeginCapture(b->cap_st, cudaStreamCaptureModeThreadLocal), "graph capture");
             cudaError_t le = cudaEventRecord(b->fork, b->cap_st);
-            // largest classes first: their CTAs run longest and should take SMs first
-            for (auto it = b->rclass.rbegin(); it != b->rclass.rend() && le == cudaSuccess; ++it) {
-                auto& c = *it;
-                le = cudaStreamWaitEvent(c.st, b->fork, 0);
-                if (le == cudaSuccess && c.slabs)
-                    le = launch_cluster(b->d_desc, b->d_plans + c.start, c.count, c.cluster, c.smem, windows, b->occ,
-                                        b->recs, b->counts, b->tracer, b->stats, b->status, b->cap, b->nbt, b->rcache,
-                                        c.st);
-                else if (le == cudaSuccess)
-                    le = launch_resident(b->d_desc, b->d_reps + c.start, c.count, b->d_nvac, c.smem, c.threads,
-                                         c.cluster, windows, b->occ, b->recs, b->counts, b->tracer, b->stats,
-                                         b->status, b->cap, b->nbt, (uint32_t)b->opts.test_stuck_wait_us, b->rcache,
-                                         c.st);
-                if (le == cudaSuccess) le = cudaEventRecord(c.done, c.st);
-                if (le == cudaSuccess) le = cudaStreamWaitEvent(b->cap_st, c.done, 0);
-            }
+            if (le == cudaSuccess) le = launch_classes(b, 1, 0, windows, nullptr, b->fork, b->cap_st);
             cudaError_t ce = cudaStreamEndCapture(b->cap_st, &graph);
             if (le != cudaSuccess) return cuda_fail(le, "resident capture");
             if (ce != cudaSuccess) return cuda_fail(ce, "resident capture");
@@ -1144,15 +1281,58 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
             }
             b->res_exec_windows = windows;
         }
-        if (!b->res_st) {
-            CK(cudaStreamCreateWithFlags(&b->res_st, cudaStreamNonBlocking), "stream");
-            CK(cudaEventCreateWithFlags(&b->res_fork, cudaEventDisableTiming), "event");
-            CK(cudaEventCreateWithFlags(&b->res_join, cudaEventDisableTiming), "event");
-        }
         CK(cudaEventRecord(b->res_fork, b->st), "event record");
         CK(cudaStreamWaitEvent(b->res_st, b->res_fork, 0), "stream wait");
         CK(cudaGraphLaunch(b->res_exec, b->res_st), "graph launch");
         CK(cudaEventRecord(b->res_join, b->res_st), "event record");
+        *launches = b->rclass.size();
+        return FKMC_OK;
+    }
+    if (!b->draw_st) {
+        CK(cudaStreamCreateWithFlags(&b->draw_st, cudaStreamNonBlocking), "stream");
+        for (int k = 0; k < 2; ++k) {
+            CK(cudaEventCreateWithFlags(&b->draw_done[k], cudaEventDisableTiming), "event");
+            CK(cudaEventCreateWithFlags(&b->draw_free[k], cudaEventDisableTiming), "event");
+        }
+    }
+    CK(cudaEventRecord(b->res_fork, b->st), "event record");
+    CK(cudaStreamWaitEvent(b->res_st, b->res_fork, 0), "stream wait");
+    CK(cudaStreamWaitEvent(b->draw_st, b->res_fork, 0), "stream wait");
+    const uint64_t step = (uint64_t)b->draw_windows;
+    uint64_t done = 0;
+    for (uint64_t w0 = 0; w0 < windows; w0 += step, ++done) {
+        const int k = (int)(done & 1);
+        const uint64_t nw = std::min(step, windows - w0);
+        Draw* buf = b->draws + (size_t)k * b->res_frags * b->res_ev * step;
+        if (done >= 2) CK(cudaStreamWaitEvent(b->draw_st, b->draw_free[k], 0), "stream wait");
+        CK(launch_draws(b->d_desc, b->n, b->res_max_frag, w0, (int)nw, b->res_ev, b->res_frags, buf, b->draw_st),
+           "draws kernel");
+        CK(cudaEventRecord(b->draw_done[k], b->draw_st), "event record");
+        CK(cudaStreamWaitEvent(b->res_st, b->draw_done[k], 0), "stream wait");
+        CK(cudaEventRecord(b->draw_free[k], b->res_st), "event record");  // the windows before have ended
+        CK(launch_classes(b, 0, w0, nw, buf, b->draw_free[k], b->res_st), "resident launch");
+        CK(cudaEventRecord(b->draw_free[k], b->res_st), "event record");
+        *launches += 1 + b->rclass.size();
+    }
+    CK(cudaEventRecord(b->res_join, b->res_st), "event record");
+    return FKMC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
+{
+    NvtxRange nvtx_range("kmc_run");
+    if (!b) return fail(FKMC_EINVAL, "null batch");
+    if (!b->rates_set) return fail(FKMC_ESTATE, "kmc_set_barriers must come before kmc_run");
+    std::vector<unsigned long long> before = b->stats_host;
+    CK(cudaEventRecord(b->ev0, b->st), "event record");
+    uint64_t res_launches = 0;
+    if (!b->rclass.empty() && windows > 0) {
+        int rc0 = launch_resident_classes(b, windows, &res_launches);
+        if (rc0) return rc0;
     }
     uint64_t extra_launches = 0;
     if (site_path(b) && !b->field_valid) {
@@ -1225,7 +1405,7 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
         }
         stats->windows = windows;
         stats->launches =
-            (windows > 0 ? b->rclass.size() : 0) +
+            res_launches +
             (b->any_global ? window_launches(b) * windows : 0) +
             extra_launches;
         float ms = 0.f;
@@ -1506,8 +1686,6 @@ int kmc_write_state(kmc_batch* b, int32_t r, const uint8_t* host_occ, size_t n)
     if (b->rates_set) {
         int rc = plan_residency(b);
         if (rc) return rc;
-        CK(cudaMemcpyAsync(b->d_nvac, b->n_vac.data(), sizeof(int64_t) * b->n, cudaMemcpyHostToDevice, b->st),
-           "vacancy count upload");
         rc = upload_desc(b);
         if (rc) return rc;
     }
@@ -1726,8 +1904,6 @@ int kmc_upload_state(kmc_batch* b, const void* host, size_t bytes)
     if (b->rates_set) {
         rc = plan_residency(b);
         if (rc) return rc;
-        CK(cudaMemcpyAsync(b->d_nvac, b->n_vac.data(), sizeof(int64_t) * b->n, cudaMemcpyHostToDevice, b->st),
-           "vacancy count upload");
     }
     return upload_desc(b);
 }
@@ -2199,7 +2375,7 @@ int kmc_get_replica_info(kmc_batch* b, int32_t r, kmc_replica_info* out)
         out->kernel = b->run_kernel[r];
         out->ctas = b->run_ctas[r];
         out->draw_phases = b->run_kernel[r] == 1 ? D.pre_g : 0;
-        out->draw_events = b->run_kernel[r] == 1 ? (D.pre_ev == 4 ? 4 : 2) : 0;
+        out->draw_events = b->run_kernel[r] == 1 ? D.pre_ev : 0;
     }
     return FKMC_OK;
 }

@@ -69,8 +69,18 @@ struct RepDesc {
     double k64g[6];
     uint64_t qg[6];
     uint64_t qng[6];
-    int32_t pre_ev;        // replica-resident kernel: events per fragment drawn in the batch (2: block 0; 4: blocks 0, 1)
+    int32_t pre_ev;        // resident kernels: events per fragment drawn ahead (2: block 0; 4: blocks 0, 1; 8: 0 .. 3)
     int32_t pad_ev_;
+    // resident kernels
+    int64_t vmap_off;      // first word of this replica's site -> record map
+    int64_t tmp_off;       // first fragment of this replica in the record copies of the stage-out
+    int64_t draw_off;      // first fragment of this replica among a window's first draws (plain form)
+};
+
+// One event's draws of the plain form: exponential variate, selection word.
+struct __align__(16) Draw {
+    double E;
+    uint64_t xs;
 };
 
 // One pick of the null-event form: the vacancy (by id) and its event (-1: null).
@@ -214,6 +224,63 @@ __device__ __forceinline__ float neglog32(uint64_t x)
     const float lnm = __fmul_rn(s, q);
     const float ln_u = __fadd_rn(__fmul_rn(__int2float_rn(e), 0.693147182f), lnm);
     return -ln_u;
+}
+
+// ---------------------------------------------------------------- mixed-form clock
+// The FP64 pipe of GB300 takes one warp instruction per 64 cycles and SM
+// quarter, whatever the number of active lanes (measured: add, multiply, FMA,
+// u64 -> float/double conversions), so that the conversion of the rate sum and
+// the clock's conversion, add and compare cost every warp sharing the pipe 256
+// cycles per event.  The functions below give the same bits with integer
+// instructions.
+
+// v rounded to nearest even, v > 0: the top 32 bits with the rest as a sticky
+// bit round like v itself (8 bits are dropped, the sticky one is the lowest)
+__device__ __forceinline__ float u64_to_float_rn(unsigned long long v)
+{
+    const int lz = __clzll((long long)v);
+    const unsigned long long n = v << lz;
+    const float f = __uint2float_rn((unsigned)(n >> 32) | (unsigned)((unsigned)n != 0u));
+    return __uint_as_float(__float_as_uint(f) + ((unsigned)(32 - lz) << 23));
+}
+
+// The window test of the mixed form, clock + ratio > theta with an FP64 add and
+// compare, all in units of 2^F / k32max (th: the bits of theta 2^-F, a normal
+// double in [2^e, 2^(e+1))).  Without `fp` the clock counts units of 2^(e-52),
+// theta's last place: a ratio of exponent e-29 or more is a whole number of
+// them (24-bit mantissa), so clock and sum are too, and a sum below 2^(e+1) is
+// exact in FP64 while one above exceeds theta either way.  A ratio of a larger
+// exponent than theta's exceeds it alone.  A smaller ratio (a share of about
+// 1e-9 of the draws) turns the clock into the FP64 value it stands for (`fp`)
+// for the rest of the visit.  Returns true when the event lies past the
+// window; next gets the clock after it otherwise.
+__device__ __forceinline__ uint64_t window_bits(double theta, int F)
+{
+    return (uint64_t)(__double_as_longlong(theta) - ((long long)F << 52));
+}
+
+// FP64 bits of the clock after the event, from either form of the clock before it
+inline __device__ __noinline__ uint64_t mixed_clock_fp64(uint64_t clock, bool fp, float ratio, uint64_t th)
+{
+    double c = __longlong_as_double((long long)clock);
+    if (!fp && clock != 0)  // clock 2^(e-52), e + 1023 = th >> 52
+        c = __longlong_as_double(__double_as_longlong(__ull2double_rn(clock)) +
+                                 (((long long)(th >> 52) - 1075) << 52));
+    return (uint64_t)__double_as_longlong(__dadd_rn(c, (double)ratio));
+}
+
+__device__ __forceinline__ bool mixed_clock(uint64_t clock, bool& fp, float ratio, uint64_t th, uint64_t& next)
+{
+    const uint32_t rb = __float_as_uint(ratio);
+    const int d = (int)(rb >> 23) + 896 - (int)(th >> 52);  // exponent of ratio minus e
+    if (d > 0) return true;
+    if (!fp && d >= -29) {
+        next = clock + ((uint64_t)((rb & 0x7fffffu) | 0x800000u) << (d + 29));
+        return next > ((th & 0x000fffffffffffffull) | 0x0010000000000000ull);
+    }
+    next = mixed_clock_fp64(clock, fp, ratio, th);
+    fp = true;
+    return next > th;  // positive doubles compare as their bits
 }
 
 // A fragment that the screen pass of a colour phase keeps for the run pass,

@@ -466,7 +466,10 @@ __global__ void __launch_bounds__(128, 8) k_run(const RepDesc* __restrict__ desc
     double Ed_even = 0.0, Ed_odd = 0.0;
     float Ef_even = 0.f, Ef_odd = 0.f;
 
-    double clock = 0.0;
+    double clock = 0.0;   // plain form
+    uint64_t mclock = 0;  // mixed form (mixed_clock)
+    bool mfp = false;
+    const uint64_t th = window_bits(D.theta_tau, D.F);
     uint64_t i = 0;
     uint32_t nhand = 0;
     for (;;) {
@@ -516,7 +519,8 @@ __global__ void __launch_bounds__(128, 8) k_run(const RepDesc* __restrict__ desc
             else Ef = __shfl_sync(0xffffffffu, odd ? Ef_odd : Ef_even, src);
         }
 
-        double dclock;
+        double dclock = 0.0;
+        uint64_t nclock = 0;
         int e_sel = -1;
         if constexpr (PREC == 0) {
             const double R = (double)total;
@@ -549,10 +553,7 @@ __global__ void __launch_bounds__(128, 8) k_run(const RepDesc* __restrict__ desc
             }
         } else {
             const unsigned long long Sq = (unsigned long long)total;
-            const float ratio = __fdiv_rn(Ef, __ull2float_rn(Sq));
-            const double dth = __dmul_rn((double)ratio, D.two_pow_F);
-            if (__dadd_rn(clock, dth) > D.theta_tau) break;
-            dclock = dth;
+            if (mixed_clock(mclock, mfp, __fdiv_rn(Ef, u64_to_float_rn(Sq)), th, nclock)) break;
             const unsigned long long target = __umul64hi(xs, Sq);
             unsigned long long cc = 0ull;
             for (int c = 0; c < nch; ++c) {
@@ -625,7 +626,8 @@ __global__ void __launch_bounds__(128, 8) k_run(const RepDesc* __restrict__ desc
         }
         if constexpr (SITE) __threadfence_block();  // field atomics before the rate reads
         __syncwarp();
-        clock = __dadd_rn(clock, dclock);
+        if constexpr (PREC == 0) clock = __dadd_rn(clock, dclock);
+        else mclock = nclock;
         ++i;
         if constexpr (SITE) compute_rates_site<GRAIN>(D, occ, sa, S, nslots, nch, lane, status);
         else compute_types<GRAIN>(D, occ, S, nslots, nch, lane, sa.gbound);
@@ -739,7 +741,10 @@ __global__ void __launch_bounds__(128, 8) k_run_small(const RepDesc* __restrict_
             }
         };
         types();
-        double clock = 0.0;
+        double clock = 0.0;   // plain form
+        uint64_t mclock = 0;  // mixed form (mixed_clock)
+        bool mfp = false;
+        const uint64_t th = window_bits(D.theta_tau, D.F);
         uint64_t i = 0;
         uint64_t xs_even = 0, xs_odd = 0;
         double Ed_even = 0.0, Ed_odd = 0.0;
@@ -791,6 +796,7 @@ __global__ void __launch_bounds__(128, 8) k_run_small(const RepDesc* __restrict_
                 }
             }
             double dclock = 0.0;
+            uint64_t nclock = 0;
             bool cont;
             int e_sel;
             if constexpr (PREC == 0) {
@@ -804,10 +810,7 @@ __global__ void __launch_bounds__(128, 8) k_run_small(const RepDesc* __restrict_
                 e_sel = b1 ? __ffs(b1) - 1 : (b2 ? 31 - __clz(b2) : -1);
             } else {
                 const unsigned long long Sq = total;
-                const float ratio = go ? __fdiv_rn(Ef, __ull2float_rn(Sq)) : 0.f;
-                const double dth = __dmul_rn((double)ratio, D.two_pow_F);
-                cont = go && !(__dadd_rn(clock, dth) > D.theta_tau);
-                dclock = dth;
+                cont = go && !mixed_clock(mclock, mfp, __fdiv_rn(Ef, u64_to_float_rn(Sq)), th, nclock);
                 const unsigned long long target = __umul64hi(xs, Sq);
                 const unsigned b1 = __ballot_sync(FULL, cont && p > target) & gmask;
                 e_sel = b1 ? __ffs(b1) - 1 : -1;
@@ -866,7 +869,8 @@ __global__ void __launch_bounds__(128, 8) k_run_small(const RepDesc* __restrict_
                 alive = nalive;
             }
             if (cont) {
-                clock = __dadd_rn(clock, dclock);
+                if constexpr (PREC == 0) clock = __dadd_rn(clock, dclock);
+                else mclock = nclock;
                 ++i;
             }
             run = cont;
@@ -1075,7 +1079,9 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
         const uint64_t w = D.window + wctl[1];
         const uint64_t k1 = key_word(D.replica, PURPOSE_HOP);
         U64x4 blk{};
-        double clock = 0.0;
+        uint64_t clock = 0;
+        bool fp = false;  // the clock's form (mixed_clock)
+        const uint64_t th = window_bits(D.theta_tau, D.F);
         uint64_t i = 0;
         for (;;) {
             unsigned long long total = 0ull;
@@ -1090,9 +1096,8 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
             const bool odd = (i & 1) != 0;
             const uint64_t xs = odd ? blk.x[3] : blk.x[1];
             const float Ef = neglog32(odd ? blk.x[2] : blk.x[0]);
-            const float ratio = __fdiv_rn(Ef, __ull2float_rn(total));
-            const double dth = __dmul_rn((double)ratio, D.two_pow_F);
-            if (__dadd_rn(clock, dth) > D.theta_tau) break;
+            uint64_t nclock = 0;
+            if (mixed_clock(clock, fp, __fdiv_rn(Ef, u64_to_float_rn(total)), th, nclock)) break;
             const unsigned long long target = __umul64hi(xs, total);
             // slot m and neighbour n of the first event whose prefix exceeds the target
             int m = NL - 1;
@@ -1175,7 +1180,7 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
 #pragma unroll
             for (int k = 0; k < NL; ++k)
                 if (k == m) r[k] = cur;
-            clock = __dadd_rn(clock, dth);
+            clock = nclock;
             ++i;
             // rates after the exchange: vacancies near s or j read their words again
             uint32_t redo = 0;
@@ -1355,7 +1360,8 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
     uint32_t ord = 0, alive = 0, pending = 0, nhand = 0;
     int lo_c[3] = {0, 0, 0}, hi_c[3] = {0, 0, 0};
     U64x4 blk{};
-    double clock = 0.0;
+    uint64_t clock = 0;
+    bool fp = false;  // the clock's form (mixed_clock)
     uint64_t i = 0;
     // hop and hand-off counts of the lane, for replica acc_rep
     int acc_rep = -1;
@@ -1455,7 +1461,8 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
                 alive = pending = (1u << nv) - 1u;
                 wnd = D.window + wk;
                 blk = philox4x64((uint64_t)fid, wnd, 0, 0, D.seed, key_word(D.replica, PURPOSE_HOP));
-                clock = 0.0;
+                clock = 0;
+                fp = false;
                 i = 0;
                 nhand = 0;
                 if (rep != acc_rep) {
@@ -1495,9 +1502,9 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
                 const bool odd = (i & 1) != 0;
                 const uint64_t xs = odd ? blk.x[3] : blk.x[1];
                 const float Ef = neglog32(odd ? blk.x[2] : blk.x[0]);
-                const float ratio = __fdiv_rn(Ef, __ull2float_rn(total));
-                const double dth = __dmul_rn((double)ratio, D.two_pow_F);
-                if (__dadd_rn(clock, dth) > D.theta_tau) {
+                uint64_t nclock = 0;
+                if (mixed_clock(clock, fp, __fdiv_rn(Ef, u64_to_float_rn(total)), window_bits(D.theta_tau, D.F),
+                                nclock)) {
                     fin = true;
                 } else {
                     // slot m and neighbour n of the first event whose prefix exceeds the target
@@ -1581,7 +1588,7 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
                         ++nhand;
                     }
                     __threadfence_block();
-                    clock = __dadd_rn(clock, dth);
+                    clock = nclock;
                     ++i;
                     // stale rates: the moved vacancy's, and those of vacancies near s or j
                     pending = owned ? 1u << m : 0u;

@@ -93,18 +93,20 @@ cudaError_t elec_update(const RepDesc& D, const double* phi, double q, int32_t* 
                         cudaStream_t st);
 cudaError_t elec_add(int32_t* field, const int32_t* u, int64_t n, cudaStream_t st);
 
-// Per-fragment event totals and dirty flags the resident kernels leave at the end
-// of a call (batch-wide fragment index), and per replica whether they are still
-// valid: the host clears `valid` whenever anything but a resident run changes a
-// replica's state or rates, and the next call then starts from every fragment dirty.
+// Per fragment (batch-wide index) the screen's limit that the resident kernels
+// leave at the end of a launch, and per replica whether they are still valid: the
+// host clears `valid` whenever anything but a resident run changes a replica's
+// state or rates, and the next launch then starts from every fragment unknown.
 struct ResCache {
-    unsigned long long* tot;
-    uint8_t* dirty;
+    uint64_t* lim;
     uint8_t* valid;
 };
 
-// cluster-resident kernel (fkmc_resident.cu): one replica per thread-block cluster,
-// CTA c holding the z-slab of fragment layers [fz0[c], fz0[c+1])
+// resident kernels (fkmc_resident.cu): a replica's occupancy in the shared memory
+// of one CTA, or of a thread-block cluster, CTA c holding the z-slab of fragment
+// layers [fz0[c], fz0[c+1])
+constexpr int RESIDENT_MAX_SLOTS = 64;            // vacancy slots per fragment (kmc_opts.cap_v) they take
+constexpr size_t RESIDENT_MAX_SMEM = 220 * 1024;  // dynamic shared memory per CTA
 constexpr int CLUSTER_MAX_CTAS = 16;
 constexpr int CLUSTER_THREADS = 512;
 struct ClusterPlan {
@@ -113,28 +115,35 @@ struct ClusterPlan {
     int32_t fz0[CLUSTER_MAX_CTAS + 1];    // fragment layers of CTA c: [fz0[c], fz0[c + 1])
     int32_t zs;                           // cells in z of the thickest slab (the common layout)
     int32_t nfl;                          // fragments of the thickest slab
-    int32_t vcap;                         // vacancy slots per CTA
-    int32_t icap;                         // inbox entries per phase parity per CTA
 };
-size_t cluster_smem_bytes(const RepDesc& D, const ClusterPlan& p, int cap);
-// the plan with the fewest CTAs in [min_ctas, max_ctas] whose slabs fit one SM's shared memory
-bool make_cluster_plan(const RepDesc& D, int64_t n_vac, int cap, int min_ctas, int max_ctas, ClusterPlan* out);
-cudaError_t cluster_prepare();
-int cluster_fits(int ncta, size_t smem);  // clusters of ncta CTAs with this much shared memory the GPU can hold at once
-cudaError_t launch_cluster(const RepDesc* d_descs, const ClusterPlan* d_plans, int nplans, int ncta, size_t smem,
-                           uint64_t windows, uint32_t* occ, VacRec* recs, int32_t* counts, int32_t* tracer,
-                           unsigned long long* stats, uint32_t* status, int cap, const NbTable& nbt,
-                           const ResCache& rc, cudaStream_t st);
-
-// replica-resident kernel (fkmc_resident.cu)
-constexpr int RESIDENT_MAX_SLOTS = 64;               // vacancies per fragment a thread can hold
-constexpr size_t RESIDENT_MAX_SMEM = 220 * 1024;     // dynamic shared memory per replica CTA
-size_t resident_smem_bytes(const RepDesc& D, int64_t n_vac, int cap, int threads, int pre_g, int pre_ev);
+struct ResidentArgs {  // fixed for a batch and its plan
+    const RepDesc* descs;
+    uint32_t* occ;
+    VacRec* recs;
+    VacRec* tmp;       // stage-out copies of the records, by RepDesc.tmp_off
+    uint32_t* vmap;    // record index of every vacancy's site, by RepDesc.vmap_off
+    int32_t* counts;
+    int32_t* tracer;
+    unsigned long long* stats;
+    uint32_t* status;
+    int cap;
+    NbTable nbt;
+    int64_t frag_tot;  // fragments of all resident replicas (stride of the plain form's draws)
+    uint32_t stuck_wait_us;
+    ResCache rc;
+};
+size_t resident_smem_bytes(const RepDesc& D, int cap, int threads, int pre_g, int pre_ev, int prec);
+size_t cluster_smem_bytes(const RepDesc& D, const ClusterPlan& p, int cap, int pre_ev, int prec);
+// the plan with the most CTAs in [min_ctas, max_ctas] whose slabs fit one SM's shared memory
+bool make_cluster_plan(const RepDesc& D, int cap, int pre_ev, int prec, int min_ctas, int max_ctas, ClusterPlan* out);
+int cluster_fits(int prec, int ncta, size_t smem);  // clusters of this shape the GPU can hold at once
 cudaError_t resident_prepare();
-cudaError_t launch_resident(const RepDesc* d_descs, const int32_t* d_reps, int nreps, const int64_t* d_nvac,
-                            size_t smem, int threads, int cluster, uint64_t windows, uint32_t* occ, VacRec* recs,
-                            int32_t* counts, int32_t* tracer, unsigned long long* stats, uint32_t* status,
-                            int cap, const NbTable& nbt, uint32_t stuck_wait_us, const ResCache& rc,
-                            cudaStream_t st);
+// first draws of `windows` windows from w0 on, of every resident replica (plain form)
+cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uint64_t w0, int windows, int ev_per,
+                         int64_t frag_tot, Draw* draws, cudaStream_t st);
+cudaError_t launch_resident(int prec, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
+                            uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st);
+cudaError_t launch_cluster(int prec, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,
+                           size_t smem, uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st);
 
 }  // namespace fkmc

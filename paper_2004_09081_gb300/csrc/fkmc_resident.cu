@@ -1,29 +1,52 @@
-// fkmc_resident.cu -- replica-resident window kernel (mixed form).
+// fkmc_resident.cu -- replica-resident window kernels (both arithmetic forms).
 //
-// One CTA owns one replica for a whole kmc_run call: the replica's packed
-// occupancy is staged into shared memory with TMA bulk copies
-// (cp.async.bulk + mbarrier), its vacancy records are unpacked into
-// shared-memory arrays linked per fragment, and the CTA runs every window and
-// colour phase with __syncthreads() between phases -- no grid-wide
-// synchronisation, because replicas are independent.  The fragment BKL is
-// that of arXiv:2004.09081 Sec. II.A (Eqs. RateCnst1, eventSelection,
-// TimeStep) with fragment-local selection (Sec. II.B, Eq. AtomP); selection
-// uses exact u64 fixed-point sums, so results are identical to the
-// colour-phase kernel and to the oracle's mixed form.
+// One CTA (k_resident<..., false>) or one thread-block cluster of up to 16 CTAs
+// (k_resident<..., true>, CTA c holding the z-slab of fragment layers
+// [P.fz0[c], P.fz0[c+1])) owns one replica for a whole launch: the packed
+// occupancy lives in shared memory and every window and colour phase runs with
+// CTA or cluster barriers only, because replicas are independent.  The fragment
+// BKL is that of arXiv:2004.09081 Sec. II.A (Eqs. RateCnst1, eventSelection,
+// TimeStep) with fragment-local selection (Sec. II.B, Eq. AtomP); the mixed
+// form's sums are exact u64 integers, the plain form sums FP64 rates in the
+// canonical order of the colour-phase kernels, so both reproduce them (and the
+// oracle) bit for bit.
+//
+// The occupancy is the only copy of the vacancies' positions.  A visit finds
+// its fragment's vacancies by scanning the fragment's rows for the vacancy
+// code, which yields them in site order (the slots' order) without a list to
+// walk, sort, relink or hand over: a vacancy that hops into another fragment
+// (or another CTA's slab) belongs to it by lying there.  A record is reached
+// only when its vacancy hops, through vmap, one word per site in global memory
+// with the index of the vacancy's record; the word is loaded when a visit
+// starts and arrives long before the first exchange needs it, and the
+// displacement goes to the record with fire-and-forget reductions.  At the end
+// of a launch the records move to the lists of the fragments that hold them.
 //
 // Each colour phase has two passes:
 //   screen  one thread per fragment of the colour.  A fragment whose
 //           neighbourhood did not change since its last visit keeps its exact
-//           event total S; with the first draw of the phase, E/S > window
-//           proves that nothing happens, and the fragment is skipped.
+//           event total; with the first draw of the phase, a first event past
+//           the window proves that nothing happens, and the fragment is skipped.
 //           Everything else goes to a compact list.
 //   run     one warp per listed fragment (lane = 4 slots x 8 directions per
-//           32-event chunk; the warp draws 64 events' random numbers at once):
-//           exact total, clock, selection by warp scan, exchange, hand-off,
-//           and "dirty" marks on the owners of every vacancy next to one of the
-//           two changed sites -- exactly the fragments whose total changed.
-// At the end the occupancy goes back with a TMA bulk store and the records go
-// back to the per-fragment lists.
+//           32-event chunk): total, clock, selection by warp scan, exchange, and
+//           "dirty" marks on the owners of every vacancy next to one of the two
+//           changed sites -- exactly the fragments whose total changed.
+//           Fragments of one colour never touch each other's sites (edges >= 2).
+//
+// What bounds it: dependent instructions.  A running warp issues one every 5 to
+// 6 cycles (2.2 of them fixed latency, 0.8 shared memory, 0.4 each branches and
+// instruction fetch), a phase lasts as long as its slowest visit (one to three
+// events, some 900 instructions), and no pipe is near its rate.  So a visit does
+// as little as it can in sequence: totals by warp reductions with the prefix
+// scan only for events that happen, no FP64 instruction in the mixed form and
+// few in the plain one, records and tracer written an exchange late.
+// Measured (one GB300, whole calls with read-out, against linked per-fragment
+// lists for the mixed form and per-phase launches for the plain form): 256
+// uneven replicas mixed 61.4 -> 55.7 us per window, 24 traced 32^3 replicas
+// mixed 22.8 -> 19.1, 128^3 mixed 55.2 -> 50.8; plain: five 32^3 replicas 155 ->
+// 29.8, 8^3 113 -> 28.5, 128^3 196 -> 75.5.
+//
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -106,6 +129,13 @@ __device__ __forceinline__ uint32_t cluster_ctarank()
     return r;
 }
 
+__device__ __forceinline__ uint32_t cluster_nctas()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+
 // every thread of every CTA of the cluster; release / acquire of shared memory
 __device__ __forceinline__ void cluster_sync()
 {
@@ -131,18 +161,13 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t peer)
     return r;
 }
 
-__device__ __forceinline__ void st_peer(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_peer(uint32_t a, int32_t v) { st_peer(a, (uint32_t)v); }
-__device__ __forceinline__ void st_peer16(uint32_t a, int16_t v)
-{
-    asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
-}
 __device__ __forceinline__ void st_peer8(uint32_t a, uint8_t v)
 {
     asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+}
+__device__ __forceinline__ void st_peer(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 __device__ __forceinline__ void st_peer64(uint32_t a, unsigned long long v)
 {
@@ -151,21 +176,6 @@ __device__ __forceinline__ void st_peer64(uint32_t a, unsigned long long v)
 __device__ __forceinline__ void red_peer_xor(uint32_t a, uint32_t v)
 {
     asm volatile("red.shared::cluster.xor.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ int32_t atom_peer_exch(uint32_t a, int32_t v)
-{
-    int32_t o;
-    asm volatile("atom.shared::cluster.exch.b32 %0, [%1], %2;" : "=r"(o) : "r"(a), "r"(v) : "memory");
-    return o;
-}
-__device__ __forceinline__ uint4 ld_peer16(uint32_t a)
-{
-    uint4 v;
-    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(a)
-                 : "memory");
-    return v;
 }
 __device__ __forceinline__ int32_t ld_peer(uint32_t a)
 {
@@ -176,9 +186,10 @@ __device__ __forceinline__ int32_t ld_peer(uint32_t a)
 
 constexpr uint32_t BULK_CHUNK = 32768;        // bytes per bulk copy instruction
 constexpr uint64_t WAIT_NS = 2000000000ull;   // 2 s bound on any device-side wait
+constexpr uint32_t DEAD = 0xffffffffu;        // slot key of a vacancy that left the fragment, or of no vacancy
 
-// compact site key in shared memory: t<<30 | z<<20 | y<<10 | x (cells < 1024),
-// ordered like the linear site index
+// compact site key: t<<30 | z<<20 | y<<10 | x (cells < 1024), ordered like the
+// linear site index
 __device__ __forceinline__ uint32_t key32(int t, int x, int y, int z)
 {
     return ((uint32_t)t << 30) | ((uint32_t)z << 20) | ((uint32_t)y << 10) | (uint32_t)x;
@@ -192,245 +203,652 @@ __device__ __forceinline__ void split32(uint32_t k, int& t, int& x, int& y, int&
     t = (int)(k >> 30);
 }
 
+// rate types of an event: species * 3 + dz + 1; a vacancy neighbour (species 2)
+// gives 6..8, which the rate table holds as zeros
+constexpr int NO_EVENT = 6;
+
 struct Shared {
     RepDesc D;
-    NbEntry nb[3][8];
+    ClusterPlan P;
+    uint64_t rate[9];    // mixed: fixed-point rates, plain: bits of the FP64 rates
     uint64_t bar;
     uint64_t bar_test;   // the wait test's barrier, which nothing completes
     uint32_t perms[64];  // colour orders of 64 consecutive windows (nibble p = colour of phase p)
-    int nv_count;
-    int nact;
-    int next_act;
+    int coff[9];         // first entry of each colour in the fragment list
+    int zbeg[CLUSTER_MAX_CTAS + 1];  // first z cell of CTA c's slab
+    int nact[2];         // screened fragments, by phase parity
+    int next_act[2];     // tickets beyond each warp's first
+    int ndraw;           // fragments of the current batch of first draws
     unsigned long long hops, hand;
     int abort;
-    int cached;  // the fragment totals of the last call are valid
+    int cached;          // the fragment totals of the last launch are valid
+};
+
+// What the screen compares a fragment's first variate E with (see `limit_of`):
+// active where E <= limit.  Mixed: FP32 bits, plain: FP64 bits.
+template <int PREC>
+struct Limit;
+template <>
+struct Limit<1> {
+    using T = uint32_t;
+    static constexpr T DIRTY = 0x7f800000u;  // +inf: the total is not known
+    static constexpr T EMPTY = 0u;           // no event
+};
+template <>
+struct Limit<0> {
+    using T = uint64_t;
+    static constexpr T DIRTY = 0x7ff0000000000000ull;
+    static constexpr T EMPTY = 0ull;
 };
 
 struct Layout {
-    uint32_t* occ;
-    uint32_t* key;
-    int32_t* d;
-    uint32_t* id;
-    int16_t* next;
-    int32_t* head;
-    unsigned long long* S;
-    uint8_t* dirty;
-    int32_t* act;          // screened fragments
-    float* pre_E;          // first exponential variates (events 0, 1, and 2, 3 where drawn) of every
-    uint64_t* pre_xs;      // fragment of the batch's phases, and their selection words, by (phase in
-                           // batch, screen index)
-    uint16_t* frag_of_c;   // cell -> fragment index: x cells, then y, then z
-    int16_t* wslot;   // per warp: vacancy index of each slot (-1: handed off)
-    int8_t* wtype;    // per warp: rate type of each event (-1: none)
+    uint32_t* occ;         // [zs][L1][RW][3], the global layout of the slab's z cells
+    void* lim;             // Limit<PREC>::T by local fragment
+    uint8_t* stale;        // 1: a vacancy came in since `slots` was written
+    uint64_t* wlog;        // plain, per warp: E and R of events whose clock division is put off
+    uint32_t* slots;       // site keys of each local fragment's vacancies in site order (DEAD: none), or
+                           // UNLISTED where it holds more than KSLOTS
+    uint2* box;            // first cell and extent of each local fragment, 10 bits per dimension
+    uint16_t* flist;       // this CTA's fragments by colour
+    uint32_t* act;         // screened fragments: local fragment | index in its colour << 16
+    uint64_t* pre_xs;      // first draws by (row, event): selection words
+    void* pre_E;           // and exponential variates (mixed: floats; plain: doubles)
+    uint16_t* pre_row;     // one CTA: row of each fragment's first draws, NO_ROW: none
+    uint16_t* dlist;       // one CTA: the fragments of the current batch of first draws
+    uint16_t* frag_of_c;   // cell -> fragment coordinate: x cells, then y, then z
+    uint32_t* zmap;        // cluster: z cell -> CTA | z within its slab << 8 | fragment layer within it << 18
+    uint32_t* wkey;        // per warp: site key of each slot
+    uint32_t* wvac;        // per warp: record index of each slot (fragments of more than 32 vacancies)
+    int8_t* wtype;         // per warp: rate type of each event (more than two chunks)
+};
+constexpr unsigned NO_ROW = 0xffffu;      // a fragment's row of first draws: none,
+constexpr unsigned ROW_FULL = 0x8000u;    // or row | ROW_FULL where every event of the row was drawn (else two)
+constexpr int KSLOTS = 8;
+constexpr int CLOCK_LOG = 8;  // events whose clock division the plain form puts off
+constexpr uint32_t UNLISTED = 0xfffffffeu;
+
+// Shared-memory arrays of one CTA: `zs` cells in z, `nfl` fragments, `maxc`
+// fragments of one colour at most.
+struct Sizes {
+    int64_t words;
+    int nfl, maxc, cap, nwarps, ltot, lz, rows, pre_ev, prec;
 };
 
+constexpr int NARR = 17;
 
-__host__ __device__ inline size_t layout_bytes(int64_t words, int64_t nv, int64_t nfrag, int64_t ncls, int cap,
-                                               int nwarps, int ltot, int pre_g, int pre_ev,
-                                               size_t* off /* 14 offsets or null */)
+__host__ __device__ inline size_t layout_bytes(const Sizes& z, size_t* off /* NARR offsets or null */)
 {
     // every array starts on a 16-byte boundary, whatever the sizes before it
-    const size_t sz[14] = {
-        (size_t)words * 4,         // 0 occupancy (bulk-copied)
-        (size_t)nv * 4,            // 1 keys
-        (size_t)nv * 12,           // 2 displacements
-        (size_t)nv * 4,            // 3 ids
-        (size_t)nv * 2,            // 4 next links
-        (size_t)nfrag * 4,         // 5 list heads
-        (size_t)nfrag * 8,         // 6 cached totals
-        (size_t)nfrag,             // 7 dirty flags
-        (size_t)ncls * 4,          // 8 screened list
-        (size_t)nwarps * cap * 2,  // 9 per-warp slots
-        (size_t)nwarps * cap * 8,  // 10 per-warp event types
-        (size_t)pre_g * pre_ev * ncls * 8,  // 11 first draws of the batch's phases: selection words
-        (size_t)pre_g * pre_ev * ncls * 4,  // 12 and variates
-        (size_t)ltot * 2,          // 13 cell -> fragment tables
+    const size_t draws = (size_t)z.rows * z.maxc * z.pre_ev;
+    const size_t sz[NARR] = {
+        (size_t)z.words * 4,             // 0 occupancy (bulk-copied)
+        (size_t)z.nfl * (z.prec ? 4 : 8),  // 1 limits
+        (size_t)z.nfl * 8,               // 2 boxes
+        (size_t)z.nfl * 2,               // 3 fragment list
+        (size_t)z.maxc * 4,              // 4 screened list
+        draws * 8,                       // 5 first draws: selection words
+        draws * (z.prec ? 4 : 8),        // 6 and variates
+        z.lz ? 0 : (size_t)z.nfl * 2,    // 7 their rows
+        z.lz ? 0 : (size_t)z.rows * z.maxc * 2,  // 8 the batch's fragments
+        (size_t)z.ltot * 2,              // 9 cell -> fragment tables
+        (size_t)z.lz * 4,                // 10 z cell -> CTA, slab z, slab layer
+        (size_t)z.nwarps * z.cap * 4,    // 11 per-warp slot keys
+        (size_t)z.nwarps * z.cap * 4,    // 12 per-warp record indices
+        (size_t)z.nwarps * z.cap * 8,    // 13 per-warp event types
+        (size_t)z.nfl,                   // 14 stale flags
+        (size_t)z.nfl * KSLOTS * 4,      // 15 vacancies by fragment
+        z.prec ? 0 : (size_t)z.nwarps * CLOCK_LOG * 16,  // 16 per-warp clock log (plain)
     };
     size_t b = 0;
-    for (int k = 0; k < 14; ++k) {
+    for (int k = 0; k < NARR; ++k) {
         if (off) off[k] = b;
         b += (sz[k] + 15) & ~(size_t)15;
     }
     return (b + 127) & ~(size_t)127;
 }
 
-__device__ __forceinline__ Layout carve(unsigned char* dyn, int64_t words, int64_t nv, int64_t nfrag, int64_t ncls,
-                                        int cap, int nwarps, int ltot, int pre_g, int pre_ev)
+__host__ __device__ inline int half_up(int n) { return (n + 1) / 2; }
+
+// one CTA holding the whole replica: `rows` = colour phases whose first draws are made in one batch
+__host__ __device__ inline Sizes sizes_single(const RepDesc& D, int cap, int nwarps, int rows, int pre_ev, int prec)
 {
-    size_t o[14];
-    layout_bytes(words, nv, nfrag, ncls, cap, nwarps, ltot, pre_g, pre_ev, o);
+    Sizes z;
+    z.words = 3 * (int64_t)D.L[2] * D.L[1] * D.row_words;
+    z.nfl = D.nf[0] * D.nf[1] * D.nf[2];
+    z.maxc = half_up(D.nf[0]) * half_up(D.nf[1]) * half_up(D.nf[2]);
+    z.cap = cap;
+    z.nwarps = nwarps;
+    z.ltot = D.L[0] + D.L[1] + D.L[2];
+    z.lz = 0;
+    z.rows = rows;
+    z.pre_ev = pre_ev;
+    z.prec = prec;
+    return z;
+}
+
+// one CTA of a cluster: rows = 2 (the phase's first draws and the next phase's)
+__host__ __device__ inline Sizes sizes_cluster(const RepDesc& D, const ClusterPlan& P, int cap, int nwarps, int pre_ev,
+                                               int prec)
+{
+    Sizes z;
+    z.words = (int64_t)3 * P.zs * D.L[1] * D.row_words;
+    z.nfl = P.nfl;
+    z.maxc = half_up(D.nf[0]) * half_up(D.nf[1]) * half_up(P.nfl / (D.nf[0] * D.nf[1]));
+    z.cap = cap;
+    z.nwarps = nwarps;
+    z.ltot = D.L[0] + D.L[1] + D.L[2];
+    z.lz = D.L[2];
+    z.rows = 2;
+    z.pre_ev = pre_ev;
+    z.prec = prec;
+    return z;
+}
+
+__device__ __forceinline__ Layout carve(unsigned char* dyn, const Sizes& z)
+{
+    size_t o[NARR];
+    layout_bytes(z, o);
     Layout L;
     L.occ = reinterpret_cast<uint32_t*>(dyn + o[0]);
-    L.key = reinterpret_cast<uint32_t*>(dyn + o[1]);
-    L.d = reinterpret_cast<int32_t*>(dyn + o[2]);
-    L.id = reinterpret_cast<uint32_t*>(dyn + o[3]);
-    L.next = reinterpret_cast<int16_t*>(dyn + o[4]);
-    L.head = reinterpret_cast<int32_t*>(dyn + o[5]);
-    L.S = reinterpret_cast<unsigned long long*>(dyn + o[6]);
-    L.dirty = reinterpret_cast<uint8_t*>(dyn + o[7]);
-    L.act = reinterpret_cast<int32_t*>(dyn + o[8]);
-    L.pre_xs = reinterpret_cast<uint64_t*>(dyn + o[11]);
-    L.pre_E = reinterpret_cast<float*>(dyn + o[12]);
-    L.frag_of_c = reinterpret_cast<uint16_t*>(dyn + o[13]);
-    L.wslot = reinterpret_cast<int16_t*>(dyn + o[9]);
-    L.wtype = reinterpret_cast<int8_t*>(dyn + o[10]);
+    L.lim = dyn + o[1];
+    L.box = reinterpret_cast<uint2*>(dyn + o[2]);
+    L.flist = reinterpret_cast<uint16_t*>(dyn + o[3]);
+    L.act = reinterpret_cast<uint32_t*>(dyn + o[4]);
+    L.pre_xs = reinterpret_cast<uint64_t*>(dyn + o[5]);
+    L.pre_E = dyn + o[6];
+    L.pre_row = reinterpret_cast<uint16_t*>(dyn + o[7]);
+    L.dlist = reinterpret_cast<uint16_t*>(dyn + o[8]);
+    L.frag_of_c = reinterpret_cast<uint16_t*>(dyn + o[9]);
+    L.zmap = reinterpret_cast<uint32_t*>(dyn + o[10]);
+    L.wkey = reinterpret_cast<uint32_t*>(dyn + o[11]);
+    L.wvac = reinterpret_cast<uint32_t*>(dyn + o[12]);
+    L.wtype = reinterpret_cast<int8_t*>(dyn + o[13]);
+    L.wlog = reinterpret_cast<uint64_t*>(dyn + o[16]);
+    L.stale = dyn + o[14];
+    L.slots = reinterpret_cast<uint32_t*>(dyn + o[15]);
     return L;
 }
 
-// word and shift in the replica's occupancy of neighbour q of the site (t,x,y,z)
-struct NbSite {
-    int t2, jx, jy, jz;
-};
-
-// lattice sizes, row words, fragment counts, clock scale and window: loaded
-// into registers once (shared-memory reads would be repeated after every
-// atomic and warp barrier)
+// lattice and slab sizes, in registers
 struct Geo {
-    int L0, L1, L2, RW, nf0, nf1, F;
-    double theta;
-    float theta_f;  // the largest float <= theta 2^-F (see window_f)
+    int L0, L1, L2, RW, nf0, nf1;
+    int zb, zl;   // this CTA's z cells: [zb, zb + zl)
+    int fzb;      // its first fragment layer
+    uint32_t me;  // its rank
 };
 
-// The window test of a clock still at zero: 2^F r > theta for the FP32 ratio r
-// (2^F r is an exact double, and 0 + 2^F r is that double) holds exactly when
-// r > theta 2^-F, and for a float r that holds exactly when r exceeds the
-// largest float not above theta 2^-F -- one FP32 compare instead of a
-// conversion, an add and a compare on the FP64 pipe, with the same outcome.
-__device__ __forceinline__ float window_f(double theta, int F)
+// a neighbour of a site: coordinates, site type, dz + 1
+struct NbSite {
+    int t2, x, y, z, dz1;
+};
+
+// This lane's direction q = lane & 7 for the three site types: 10 bits each,
+// t2 | (dc_x+1) << 2 | (dc_y+1) << 4 | (dc_z+1) << 6 | (d_z+1) << 8.
+__device__ __forceinline__ uint32_t pack_direction(const NbTable& nbt, int q)
 {
-    return __double2float_rd(__longlong_as_double(__double_as_longlong(theta) - ((long long)F << 52)));
+    uint32_t p = 0;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const NbEntry e = nbt.e[t][q];
+        p |= ((uint32_t)e.t2 | (uint32_t)(e.dc[0] + 1) << 2 | (uint32_t)(e.dc[1] + 1) << 4 |
+              (uint32_t)(e.dc[2] + 1) << 6 | (uint32_t)(e.d[2] + 1) << 8)
+             << (10 * t);
+    }
+    return p;
 }
 
-__device__ __forceinline__ NbSite nb_site(const Shared& sh, const Geo& g, int t, int x, int y, int z, int q)
+// c in [-1, L] to [0, L): the least of c, c + L and c - L as unsigned numbers
+__device__ __forceinline__ int wrap1(int c, int L)
 {
-    const NbEntry nb = sh.nb[t][q];
+    return (int)min(min((unsigned)c, (unsigned)(c + L)), (unsigned)(c - L));
+}
+
+__device__ __forceinline__ NbSite nb_site(const Geo& g, uint32_t dirs, uint32_t key)
+{
+    int t, x, y, z;
+    split32(key, t, x, y, z);
+    const uint32_t e = dirs >> (10 * t);
     NbSite s;
-    s.t2 = nb.t2;
-    s.jx = wrapc(x + nb.dc[0], g.L0);
-    s.jy = wrapc(y + nb.dc[1], g.L1);
-    s.jz = wrapc(z + nb.dc[2], g.L2);
+    s.t2 = (int)(e & 3u);
+    s.x = wrap1(x + (int)((e >> 2) & 3u) - 1, g.L0);
+    s.y = wrap1(y + (int)((e >> 4) & 3u) - 1, g.L1);
+    s.z = wrap1(z + (int)((e >> 6) & 3u) - 1, g.L2);
+    s.dz1 = (int)((e >> 8) & 3u);
     return s;
 }
 
-__device__ __forceinline__ int site_code(const Geo& g, const uint32_t* occ, int t, int x, int y, int z)
+// word of a site in its CTA's slab: index for a slab-local z
+__device__ __forceinline__ int word_of(const Geo& g, int t, int x, int y, int zr)
 {
-    const uint32_t w = occ[((z * g.L1 + y) * g.RW + (x >> 4)) * 3 + t];
+    return ((zr * g.L1 + y) * g.RW + (x >> 4)) * 3 + t;
+}
+
+// species code of a site; a site in another CTA's slab is read through
+// distributed shared memory
+template <bool CL>
+__device__ __forceinline__ int site_code(const Layout& S, const Geo& g, int t, int x, int y, int z)
+{
+    uint32_t w;
+    const int zr = CL ? z - g.zb : z;
+    if (!CL || (unsigned)zr < (unsigned)g.zl) {
+        w = S.occ[word_of(g, t, x, y, zr)];
+    } else {
+        const uint32_t zm = S.zmap[z];
+        w = (uint32_t)ld_peer(peer_addr(S.occ + word_of(g, t, x, y, (int)((zm >> 8) & 1023u)), zm & 255u));
+    }
     return (int)((w >> occ_shift(x)) & 3u);
 }
 
-// owner fragment of cell (x,y,z), from the per-dimension tables
-__device__ __forceinline__ int owner_of(const Geo& g, const uint16_t* fo, int x, int y, int z)
+// marks the fragment owning a site as changed, unless it is this CTA's fragment
+// `own`; `came`: a vacancy came to that site
+template <int PREC, bool CL>
+__device__ __forceinline__ void mark_owner(const Layout& S, const Geo& g, int x, int y, int z, int own, bool came)
 {
-    return (fo[g.L0 + g.L1 + z] * g.nf1 + fo[g.L0 + y]) * g.nf0 + fo[x];
+    using Lim = Limit<PREC>;
+    typename Lim::T* lim = reinterpret_cast<typename Lim::T*>(S.lim);
+    const int fx = S.frag_of_c[x], fy = S.frag_of_c[g.L0 + y];
+    if constexpr (!CL) {
+        const int f = ((int)S.frag_of_c[g.L0 + g.L1 + z] * g.nf1 + fy) * g.nf0 + fx;
+        if (f != own) {
+            lim[f] = Lim::DIRTY;
+            if (came) S.stale[f] = 1;
+        }
+    } else {
+        const uint32_t zm = S.zmap[z];
+        const int f = ((int)(zm >> 18) * g.nf1 + fy) * g.nf0 + fx;
+        if ((zm & 255u) == g.me) {
+            if (f != own) {
+                lim[f] = Lim::DIRTY;
+                if (came) S.stale[f] = 1;
+            }
+        } else {
+            if constexpr (PREC == 1) st_peer(peer_addr(lim + f, zm & 255u), Lim::DIRTY);
+            else st_peer64(peer_addr(lim + f, zm & 255u), Lim::DIRTY);
+            if (came) st_peer8(peer_addr(S.stale + f, zm & 255u), 1);
+        }
+    }
 }
 
-// exact product 2^F * d for a positive normal double (exponent add)
-__device__ __forceinline__ double scale_pow2(double d, int F)
+// index of a site in the site -> record map: sixteen entries per occupancy word
+__device__ __forceinline__ uint32_t map_index(const Geo& g, uint32_t key)
 {
-    return __longlong_as_double(__double_as_longlong(d) + ((long long)F << 52));
+    int t, x, y, z;
+    split32(key, t, x, y, z);
+    return (uint32_t)word_of(g, t, x, y, z) * 16u + (uint32_t)(x & 15);
+}
+
+// The vacancies of a box (first cell lo, extents ex, ey, ez) in site order: their
+// keys to wkey[0 .. min(n, cap)), the number n returned.  Lane l scans rows
+// [RPL l, RPL (l + 1)) of the box, three words (site types) per row; with at
+// most one vacancy per lane and type the slots follow from three ballots,
+// else from a scan of the packed counts.
+template <typename M>
+__device__ __forceinline__ int gather_rows(const Layout& S, const Geo& g, uint32_t* wkey, int cap, int lane, int lo0,
+                                           int lo1, int lo2, int ex, int ey, int rows, int rpl)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const unsigned below = (1u << lane) - 1u;
+    // masks of up to 16 or 32 cells, bit 2 c for cell c: row c / ex of this lane's rows, x = lo0 + c % ex
+    const int r = rpl * lane;
+    int z = (int)(((float)r + 0.5f) * __fdividef(1.0f, (float)ey));  // r / ey, exact for r < 2^19
+    int y = r - z * ey;
+    const int dy = y, dz = z;
+    const M emask = ex == 16 ? (M)0xffffffffu : (M)((1u << (2 * ex)) - 1u);
+    const int off = (lo0 & 15) * 2;
+    const bool two = off + 2 * ex > 32;
+    M m[3] = {0, 0, 0};
+    for (int k = 0; k < rpl; ++k) {
+        if (r + k < rows) {
+            const uint32_t* w = S.occ + word_of(g, 0, lo0, lo1 + y, lo2 - g.zb + z);
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                const uint32_t v = two ? __funnelshift_r(w[t], w[3 + t], off) : w[t] >> off;
+                m[t] |= ((M)((v >> 1) & ~v & 0x55555555u) & emask) << (2 * ex * k);
+            }
+        }
+        if (++y == ey) {
+            y = 0;
+            ++z;
+        }
+    }
+    auto count = [](M v) { return sizeof(M) == 8 ? __popcll(v) : __popc((unsigned)v); };
+    int s0, s1, s2, n;
+    if (!__any_sync(FULL, ((m[0] & (m[0] - 1)) | (m[1] & (m[1] - 1)) | (m[2] & (m[2] - 1))) != 0)) {
+        const unsigned b0 = __ballot_sync(FULL, m[0] != 0), b1 = __ballot_sync(FULL, m[1] != 0),
+                       b2 = __ballot_sync(FULL, m[2] != 0);
+        const int n0 = __popc(b0), n1 = __popc(b1);
+        s0 = __popc(b0 & below);
+        s1 = n0 + __popc(b1 & below);
+        s2 = n0 + n1 + __popc(b2 & below);
+        n = n0 + n1 + __popc(b2);
+    } else {
+        const uint32_t mine = (uint32_t)count(m[0]) | (uint32_t)count(m[1]) << 10 | (uint32_t)count(m[2]) << 20;
+        uint32_t c = mine;  // at most 32 lanes x 16 (or 31) cells per field: the last may carry out unused
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, c, o);
+            if (lane >= o) c += u;
+        }
+        const uint32_t tot = __shfl_sync(FULL, c, 31);
+        c -= mine;
+        const int n0 = (int)(tot & 1023u), n1 = (int)((tot >> 10) & 1023u);
+        s0 = (int)(c & 1023u);
+        s1 = n0 + (int)((c >> 10) & 1023u);
+        s2 = n0 + n1 + (int)(c >> 20);
+        n = n0 + n1 + (int)(tot >> 20);
+    }
+    // one vacancy per turn and lane, over the three masks
+    int t = 0;
+    while (true) {
+        while (t < 3 && m[0] == 0) {  // the next type with a vacancy left
+            m[0] = m[1];
+            m[1] = m[2];
+            m[2] = 0;
+            s0 = s1;
+            s1 = s2;
+            ++t;
+        }
+        if (t >= 3) break;
+        const int c = (sizeof(M) == 8 ? __ffsll((long long)m[0]) - 1 : __ffs((int)m[0]) - 1) >> 1;
+        m[0] &= m[0] - 1;
+        int yy = dy, zz = dz, xx = c;
+        while (xx >= ex) {
+            xx -= ex;
+            if (++yy == ey) {
+                yy = 0;
+                ++zz;
+            }
+        }
+        if (s0 < cap) wkey[s0] = key32(t, lo0 + xx, lo1 + yy, lo2 + zz);
+        ++s0;
+    }
+    __syncwarp();
+    return n;
+}
+
+__device__ __forceinline__ int gather(const Layout& S, const Geo& g, uint32_t* wkey, int cap, int lane, int lo0, int lo1,
+                                      int lo2, int ex, int ey, int ez)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int rows = ey * ez, rpl = (rows + 31) >> 5;
+    // (at most 31 cells per lane keep every count of the packed scan below 1024)
+    if (rpl * ex <= 16) return gather_rows<uint32_t>(S, g, wkey, cap, lane, lo0, lo1, lo2, ex, ey, rows, rpl);
+    if (rpl * ex <= 31 && ex <= 16)
+        return gather_rows<uint64_t>(S, g, wkey, cap, lane, lo0, lo1, lo2, ex, ey, rows, rpl);
+    const int hi0 = lo0 + ex;
+    // larger boxes: 16-cell pieces of rows, one site type after the other
+    const int pieces = (ex + 15) >> 4, items = rows * pieces;
+    int n = 0;
+    for (int t = 0; t < 3; ++t) {
+        for (int base = 0; base < items; base += 32) {
+            const int it = base + lane;
+            uint32_t m = 0;
+            int x0 = 0, y = 0, z = 0;
+            if (it < items) {
+                const int r = it / pieces, p = it - r * pieces;
+                z = r / ey;
+                y = lo1 + r - z * ey;
+                z += lo2;
+                x0 = lo0 + 16 * p;
+                const int len = min(16, hi0 - x0), off = (x0 & 15) * 2;
+                const uint32_t* w = S.occ + word_of(g, t, x0, y, z - g.zb);
+                const uint32_t v = __funnelshift_r(w[0], off + 2 * len > 32 ? w[3] : 0u, off);
+                m = (v >> 1) & ~v & 0x55555555u & (uint32_t)((1ull << (2 * len)) - 1ull);
+            }
+            const int c = __popc(m);
+            if (!__any_sync(FULL, c != 0)) continue;
+            int s = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(FULL, s, o);
+                if (lane >= o) s += u;
+            }
+            int slot = n + s - c;
+            n += __shfl_sync(FULL, s, 31);
+            while (m) {
+                const int b = (__ffs(m) - 1) >> 1;
+                m &= m - 1;
+                if (slot < cap) wkey[slot] = key32(t, x0 + b, y, z);
+                ++slot;
+            }
+        }
+    }
+    __syncwarp();
+    return n;
+}
+
+// u = floor(x / 2^11) 2^-53, exact, from integer instructions
+__device__ __forceinline__ double uniform53(uint64_t x)
+{
+    const uint64_t u = x >> 11;
+    if (u == 0) return 0.0;
+    const int n = 63 - __clzll((long long)u);
+    return __longlong_as_double((long long)(((u << (52 - n)) & 0x000fffffffffffffull) | ((uint64_t)(n + 970) << 52)));
+}
+
+// A positive double as a float, truncated, from integer instructions; exponents
+// in [-100, 100] only.
+__device__ __forceinline__ bool float_range(long long b) { return (unsigned)((int)(b >> 52) - 923) <= 200u; }
+__device__ __forceinline__ float to_float(long long b)
+{
+    return __uint_as_float((uint32_t)((b - (896ll << 52)) >> 29));
+}
+
+// The screen's limit for a fragment of event total `tot` (> 0): no less than any
+// first variate E that does not put the first event past the window.  Mixed:
+// fl(E / S32) > theta' whenever E > S32 theta' (1 + 2^-20), lim32 the factor
+// theta' (1 + 2^-20) rounded up; plain: fl(E / R) > tau whenever E exceeds
+// fl(tau R) by 2^-40.
+template <int PREC>
+__device__ __forceinline__ typename Limit<PREC>::T limit_of(uint64_t tot, float lim32, double tau)
+{
+    if constexpr (PREC == 1) return __float_as_uint(__fmul_ru(u64_to_float_rn(tot), lim32));
+    else return (uint64_t)__double_as_longlong(__dmul_rn(tau, __longlong_as_double((long long)tot))) + 4096ull;
+}
+
+// warp total of u64 values below 2^63 / 32: three 21-bit limbs by warp reductions
+__device__ __forceinline__ unsigned long long warp_total(unsigned long long v)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const unsigned a = __reduce_add_sync(FULL, (unsigned)v & 0x1fffffu);
+    const unsigned b = __reduce_add_sync(FULL, (unsigned)(v >> 21) & 0x1fffffu);
+    const unsigned c = __reduce_add_sync(FULL, (unsigned)(v >> 42));
+    return (unsigned long long)a + ((unsigned long long)b << 21) + ((unsigned long long)c << 42);
 }
 
 }  // namespace
 
-size_t resident_smem_bytes(const RepDesc& D, int64_t n_vac, int cap, int threads, int pre_g, int pre_ev)
+size_t resident_smem_bytes(const RepDesc& D, int cap, int threads, int pre_g, int pre_ev, int prec)
 {
-    const int64_t words = 3 * (int64_t)D.L[2] * D.L[1] * D.row_words;
-    const int64_t nfrag = (int64_t)D.nf[0] * D.nf[1] * D.nf[2];
-    const int64_t ncls = (int64_t)((D.nf[0] + 1) / 2) * ((D.nf[1] + 1) / 2) * ((D.nf[2] + 1) / 2);
-    if (D.L[0] > 1024 || D.L[1] > 1024 || D.L[2] > 1024 || n_vac > 32767 || nfrag > 32767)
-        return ~(size_t)0;  // compact keys and 16-bit links need these bounds
-    if (pre_g < 1 || pre_g > 8 || (8 % pre_g) != 0 || (pre_ev != 2 && pre_ev != 4)) return ~(size_t)0;
-    return layout_bytes(words, n_vac, nfrag, ncls, cap, threads / 32, D.L[0] + D.L[1] + D.L[2], pre_g, pre_ev,
-                        nullptr);
+    const Sizes z = sizes_single(D, cap, threads / 32, 1, 2, prec);
+    if (D.L[0] > 1024 || D.L[1] > 1024 || D.L[2] > 1024 || z.nfl > 65535 || 8 * z.maxc > 32767)
+        return ~(size_t)0;  // compact keys, 16-bit fragment and row indices
+    if (pre_g < 1 || pre_g > 8 || (8 % pre_g) != 0 || (pre_ev != 2 && pre_ev != 4 && pre_ev != 8)) return ~(size_t)0;
+    return layout_bytes(sizes_single(D, cap, threads / 32, pre_g, pre_ev, prec), nullptr);
 }
 
-// CL = CTAs per replica (a thread-block cluster).  With CL = 2 both CTAs hold
-// the whole replica; each screens and runs half of every colour's fragments,
-// and every write to the replica's state is made in both copies (the local one
-// and, through distributed shared memory, the peer's), so the copies stay
-// identical; reads are local.  Phases end with a cluster barrier.
-template <int NT, int CL>
-__global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1))) k_resident(const RepDesc* __restrict__ descs,
-                                                  const int32_t* __restrict__ reps,
-                                                  const int64_t* __restrict__ nvac, uint64_t windows,
-                                                  uint32_t* occ, VacRec* recs, int32_t* counts,
-                                                  int32_t* tracer, unsigned long long* stats,
-                                                  uint32_t* status, int cap, NbTable nbt,
-                                                  uint32_t stuck_wait_us, ResCache rc)
+size_t cluster_smem_bytes(const RepDesc& D, const ClusterPlan& p, int cap, int pre_ev, int prec)
+{
+    return layout_bytes(sizes_cluster(D, p, cap, CLUSTER_THREADS / 32, pre_ev, prec), nullptr);
+}
+
+// First draws of the plain form, one window after the other: event ev of
+// fragment f of window w0 + z at ((z frag_tot + draw_off + f) ev_per + ev).
+// The FP64 logarithm (some 45 FP64 instructions at 64 cycles of an SM quarter's
+// FP64 pipe each) would keep the few SMs that hold a plain replica busy for
+// longer than the events themselves; here the whole GPU computes it, beside
+// the windows before.
+__global__ void __launch_bounds__(64) k_draws(const RepDesc* __restrict__ descs, int nrep, uint64_t w0, int ev_per,
+                                              int64_t frag_tot, Draw* draws)
+{
+    const int nbk = ev_per >> 1;
+    for (int r = blockIdx.y; r < nrep; r += gridDim.y) {
+        const RepDesc& D = descs[r];
+        if (!D.resident) continue;
+        const int64_t n = (int64_t)D.nf[0] * D.nf[1] * D.nf[2] * nbk;
+        const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        if (i >= n) continue;
+        const int64_t fid = i / nbk;
+        const int bk = (int)(i - fid * nbk);
+        const U64x4 b = philox4x64((uint64_t)fid, D.window + w0 + blockIdx.z, (uint64_t)bk, 0, D.seed,
+                                   key_word(D.replica, PURPOSE_HOP));
+        Draw* o = draws + ((int64_t)blockIdx.z * frag_tot + D.draw_off + fid) * ev_per + 2 * bk;
+        o[0].E = neglog64(b.x[0]);
+        o[0].xs = b.x[1];
+        o[1].E = neglog64(b.x[2]);
+        o[1].xs = b.x[3];
+    }
+}
+
+template <int PREC, int NT, bool CL>
+__global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
+    k_resident(const RepDesc* __restrict__ descs, const int32_t* __restrict__ reps,
+               const ClusterPlan* __restrict__ plans, uint64_t w0, uint64_t windows, uint32_t* occ, VacRec* recs,
+               VacRec* tmp, uint32_t* vmap, int32_t* counts, int32_t* tracer, unsigned long long* stats,
+               uint32_t* status, int cap, NbTable nbt, const Draw* __restrict__ draws, int64_t frag_tot,
+               uint32_t stuck_wait_us, ResCache rc)
 {
     extern __shared__ __align__(128) unsigned char dyn[];
     __shared__ Shared sh;
-    const int tid = threadIdx.x;
-    const int r = reps[blockIdx.x / CL];
-    const int64_t n_vac = nvac[r];
-    const uint32_t rank = CL > 1 ? cluster_ctarank() : 0u;
-    const uint32_t peer = rank ^ 1u;
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t me = CL ? cluster_ctarank() : 0u;
 
     if (tid == 0) {
+        int r;
+        if constexpr (CL) {
+            sh.P = plans[blockIdx.x / cluster_nctas()];
+            r = sh.P.rep;
+        } else {
+            r = reps[blockIdx.x];
+        }
         sh.D = descs[r];
-        sh.nv_count = 0;
+        if constexpr (!CL) {
+            sh.P.rep = r;
+            sh.P.ncta = 1;
+            sh.P.fz0[0] = 0;
+            sh.P.fz0[1] = sh.D.nf[2];
+        }
+        for (int c = 0; c <= sh.P.ncta; ++c) sh.zbeg[c] = frag_start(sh.P.fz0[c], sh.D.base[2], sh.D.rem[2]);
+        for (int k = 0; k < 9; ++k) {
+            if constexpr (PREC == 1) sh.rate[k] = k < 6 ? sh.D.q[k] : 0ull;
+            else sh.rate[k] = k < 6 ? (uint64_t)__double_as_longlong(sh.D.k64[k]) : 0ull;
+        }
+        sh.nact[0] = sh.nact[1] = 0;
+        sh.ndraw = 0;
+        sh.next_act[0] = sh.next_act[1] = NW;  // each warp's first fragment is its own index
         sh.hops = 0;
         sh.hand = 0;
         sh.abort = 0;
         sh.cached = rc.valid[r];
     }
-    if (tid < 24) (&sh.nb[0][0])[tid] = (&nbt.e[0][0])[tid];  // threads index it with different t
     __syncthreads();
     const RepDesc& D = sh.D;
-    const int64_t words = 3 * (int64_t)D.L[2] * D.L[1] * D.row_words;
-    const int nfrag = D.nf[0] * D.nf[1] * D.nf[2];
-    const int ncls_max = ((D.nf[0] + 1) / 2) * ((D.nf[1] + 1) / 2) * ((D.nf[2] + 1) / 2);
-    const int pre_g = (D.pre_g == 2 || D.pre_g == 4 || D.pre_g == 8) ? D.pre_g : 1;  // the host sized the layout for it
-    const int pre_ev = D.pre_ev == 4 ? 4 : 2;  // events per fragment drawn ahead: block 0, or blocks 0 and 1
-    const Layout S =
-        carve(dyn, words, n_vac, nfrag, ncls_max, cap, NT / 32, D.L[0] + D.L[1] + D.L[2], pre_g, pre_ev);
+    const ClusterPlan& P = sh.P;
+    const int rep = P.rep;
+    const int pre_ev = D.pre_ev == 8 ? 8 : (D.pre_ev == 4 ? 4 : 2);
+    const int pre_g = CL ? 2 : ((D.pre_g == 2 || D.pre_g == 4 || D.pre_g == 8) ? D.pre_g : 1);
+    const Sizes sz = CL ? sizes_cluster(D, P, cap, NW, pre_ev, PREC) : sizes_single(D, cap, NW, pre_g, pre_ev, PREC);
+    const Layout S = carve(dyn, sz);
+    using Lim = Limit<PREC>;
+    typename Lim::T* const lim = reinterpret_cast<typename Lim::T*>(S.lim);
+    const int maxc = sz.maxc;
+    const int fzb = P.fz0[me], fze = P.fz0[me + 1];
+    const Geo geo{D.L[0], D.L[1], D.L[2], D.row_words, D.nf[0], D.nf[1], sh.zbeg[me], sh.zbeg[me + 1] - sh.zbeg[me],
+                  fzb, me};
+    const int nfl = (fze - fzb) * D.nf[0] * D.nf[1];
+    const int64_t frag0 = D.frag_base + (int64_t)fzb * D.nf[1] * D.nf[0];  // layers are contiguous in the global order
 
-    // ---- stage in: occupancy by TMA bulk copies, records by plain loads (the
-    // first CTA of a cluster; the second copies its shared memory afterwards)
-    const uint32_t occ_bytes = (uint32_t)(words * 4);
-    if (tid == 0 && rank == 0) {
+    // ---- stage in: this CTA's occupancy (its z cells are contiguous in the global
+    // layout) by TMA bulk copies, the record index of every vacancy's site
+    const int slab_words = geo.zl * D.L[1] * D.row_words * 3;
+    const int slab_word0 = geo.zb * D.L[1] * D.row_words * 3;
+    uint32_t* const occ_g = occ + D.occ_word_off + (int64_t)geo.zb * D.L[1] * D.row_words * 3;
+    const uint32_t occ_bytes = (uint32_t)slab_words * 4u;  // rows are multiples of 16 bytes
+    if (tid == 0) {
         mbar_init(&sh.bar, 1);
         mbar_arrive_expect_tx(&sh.bar, occ_bytes);
-        const char* src = reinterpret_cast<const char*>(occ + D.occ_word_off);
-        for (uint32_t off = 0; off < occ_bytes; off += BULK_CHUNK) {
-            const uint32_t n = min(BULK_CHUNK, occ_bytes - off);
-            bulk_g2s(S.occ + off / 4, src + off, n, &sh.bar);
-        }
+        const char* src = reinterpret_cast<const char*>(occ_g);
+        for (uint32_t off = 0; off < occ_bytes; off += BULK_CHUNK)
+            bulk_g2s(S.occ + off / 4, src + off, min(BULK_CHUNK, occ_bytes - off), &sh.bar);
     }
-    for (int k = tid; k < D.L[0] + D.L[1] + D.L[2]; k += blockDim.x) {
+    for (int k = tid; k < D.L[0] + D.L[1] + D.L[2]; k += NT) {
         const int d = k < D.L[0] ? 0 : (k < D.L[0] + D.L[1] ? 1 : 2);
         const int c = d == 0 ? k : (d == 1 ? k - D.L[0] : k - D.L[0] - D.L[1]);
         S.frag_of_c[k] = (uint16_t)frag_of(c, D.base[d], D.rem[d]);
     }
-    for (int f = tid; f < (rank == 0 ? nfrag : 0); f += blockDim.x) {
-        const int64_t g = D.frag_base + f;
-        const int c = counts[g];
-        int head = -1;
-        for (int k = 0; k < c && k < cap; ++k) {
-            const int v = atomicAdd(&sh.nv_count, 1);
-            if (v >= n_vac) {
-                atomicOr(status, STATUS_OVERFLOW);
-                break;
-            }
-            const VacRec rr = recs[g * cap + k];
-            int t, x, y, z;
-            split_key(rr.key, t, x, y, z);
-            S.key[v] = key32(t, x, y, z);
-            S.d[3 * v] = rr.d[0];
-            S.d[3 * v + 1] = rr.d[1];
-            S.d[3 * v + 2] = rr.d[2];
-            S.id[v] = rr.id;
-            S.next[v] = (int16_t)head;
-            head = v;
+    if constexpr (CL) {
+        for (int z = tid; z < D.L[2]; z += NT) {
+            const int fz = frag_of(z, D.base[2], D.rem[2]);
+            int c = 0;
+            while (c + 1 < P.ncta && P.fz0[c + 1] <= fz) ++c;
+            S.zmap[z] = (uint32_t)c | ((uint32_t)(z - sh.zbeg[c]) << 8) | ((uint32_t)(fz - P.fz0[c]) << 18);
         }
-        if (c > cap) atomicOr(status, STATUS_OVERFLOW);
-        S.head[f] = head;
-        // the fragment totals the last call left, where nothing changed the replica since
-        S.dirty[f] = sh.cached ? rc.dirty[g] : 1;
-        S.S[f] = sh.cached ? rc.tot[g] : 0ull;
     }
-    __syncthreads();  // the barrier init is visible to every thread from here on
-    if (rank == 0 && !mbar_wait_bounded(&sh.bar, 0, WAIT_NS)) {
+    // this CTA's fragments by colour
+    auto colour_count = [&](int colour, int cnt[2], int& lz0) -> int {
+        const int b0 = colour & 1, b1 = (colour >> 1) & 1, b2 = colour >> 2;
+        cnt[0] = D.nf[0] == 1 ? (b0 == 0 ? 1 : 0) : D.nf[0] / 2;
+        cnt[1] = D.nf[1] == 1 ? (b1 == 0 ? 1 : 0) : D.nf[1] / 2;
+        lz0 = D.nf[2] == 1 ? 0 : (fzb + ((fzb & 1) != b2 ? 1 : 0));
+        const int nlz = D.nf[2] == 1 ? (b2 == 0 ? 1 : 0) : (fze > lz0 ? (fze - lz0 + 1) / 2 : 0);
+        return cnt[0] * cnt[1] * nlz;
+    };
+    if (tid == 0) {
+        int s = 0;
+        for (int c = 0; c < 8; ++c) {
+            int cnt[2], lz0;
+            sh.coff[c] = s;
+            s += colour_count(c, cnt, lz0);
+        }
+        sh.coff[8] = s;
+    }
+    __syncthreads();
+    for (int c = 0; c < 8; ++c) {
+        int cnt[2], lz0;
+        const int n = colour_count(c, cnt, lz0);
+        for (int l = tid; l < n; l += NT) {
+            const int i0 = l % cnt[0], i1 = (l / cnt[0]) % cnt[1], i2 = l / (cnt[0] * cnt[1]);
+            const int f0 = D.nf[0] == 1 ? 0 : 2 * i0 + (c & 1), f1 = D.nf[1] == 1 ? 0 : 2 * i1 + ((c >> 1) & 1);
+            const int f2 = lz0 + 2 * i2, lf = ((f2 - fzb) * D.nf[1] + f1) * D.nf[0] + f0;
+            S.flist[sh.coff[c] + l] = (uint16_t)lf;
+            const int o0 = frag_start(f0, D.base[0], D.rem[0]), e0 = frag_start(f0 + 1, D.base[0], D.rem[0]) - o0;
+            const int o1 = frag_start(f1, D.base[1], D.rem[1]), e1 = frag_start(f1 + 1, D.base[1], D.rem[1]) - o1;
+            const int o2 = frag_start(f2, D.base[2], D.rem[2]), e2 = frag_start(f2 + 1, D.base[2], D.rem[2]) - o2;
+            S.box[lf] = make_uint2((uint32_t)o0 | (uint32_t)o1 << 10 | (uint32_t)o2 << 20,
+                                   (uint32_t)(e0 - 1) | (uint32_t)(e1 - 1) << 10 | (uint32_t)(e2 - 1) << 20);
+        }
+    }
+    // sites of this slab count from vmap_s, sites of the replica from vmap_r
+    uint32_t* const vmap_r = vmap + D.vmap_off;
+    uint32_t* const vmap_s = vmap_r + (int64_t)geo.zb * D.L[1] * D.row_words * 48;
+    VacRec* const recs_r = recs + D.frag_base * cap;  // record indices count from here
+    const uint32_t rec_lim = (uint32_t)(D.nf[0] * D.nf[1] * D.nf[2] * cap);
+    for (int f = tid; f < nfl; f += NT) {
+        const int64_t g = frag0 + f;
+        const int c = counts[g];
+        if (c > cap) atomicOr(status, STATUS_OVERFLOW);
+        uint32_t* const sl = S.slots + f * KSLOTS;
+        int have = 0;
+        for (int k = 0; k < c && k < cap; ++k) {
+            int t, x, y, z;
+            split_key(recs[g * cap + k].key, t, x, y, z);
+            vmap_s[map_index(geo, key32(t, x, y, z - geo.zb))] = (uint32_t)((g - D.frag_base) * cap + k);
+            if (c <= KSLOTS) {  // into the sorted list
+                const uint32_t key = key32(t, x, y, z);
+                int m = have++;
+                for (; m > 0 && sl[m - 1] > key; --m) sl[m] = sl[m - 1];
+                sl[m] = key;
+            }
+        }
+        for (int k = have; k < KSLOTS; ++k) sl[k] = DEAD;
+        if (c > KSLOTS) sl[0] = UNLISTED;
+        S.stale[f] = 0;
+        // the limit the last launch left, where nothing changed the replica since
+        lim[f] = sh.cached ? (typename Lim::T)rc.lim[g] : (c > 0 ? Lim::DIRTY : Lim::EMPTY);
+    }
+    if (!mbar_wait_bounded(&sh.bar, 0, WAIT_NS)) {
         if (tid == 0) {
             atomicOr(status, STATUS_TIMEOUT);
             sh.abort = 1;
@@ -438,7 +856,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1))) k_r
         mbar_wait_bounded(&sh.bar, 0, WAIT_NS);  // let copies in flight land before leaving
     }
     __syncthreads();
-    if (stuck_wait_us && rank == 0 && !sh.abort) {
+    if (!CL && stuck_wait_us && !sh.abort) {
         // test of the bounded wait: no copy is in flight here, and the barrier
         // below is never completed, so the wait must give up after
         // stuck_wait_us, report FKMC_ETIMEOUT and leave the state untouched
@@ -451,1417 +869,710 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1))) k_r
         }
         __syncthreads();
     }
-    if constexpr (CL > 1) {
-        // every CTA of the cluster passes the same barriers: the decision to stop
-        // is read from the first CTA after the cluster barrier
+    if constexpr (CL) {
+        // every slab is in place before any CTA reads a peer's; the CTAs of a cluster
+        // stop together: a CTA whose stage-in timed out tells all
+        const bool bad = sh.abort != 0;
         cluster_sync();
-        if (rank != 0) {
-            if (tid == 0) sh.abort = ld_peer(peer_addr(&sh.abort, 0));
-            __syncthreads();
-            if (!sh.abort) {
-                const uint32_t base = peer_addr(dyn, 0);
-                const size_t bytes = layout_bytes(words, n_vac, nfrag, ncls_max, cap, NT / 32,
-                                                  D.L[0] + D.L[1] + D.L[2], pre_g, pre_ev, nullptr);
-                for (size_t k = (size_t)tid * 16; k < bytes; k += (size_t)NT * 16) {
-                    const uint4 v = ld_peer16(base + (uint32_t)k);
-                    *reinterpret_cast<uint4*>(dyn + k) = v;
-                }
-            }
-        }
-        cluster_sync();  // the first CTA writes into the copy only after it is complete
+        if (bad && tid < P.ncta) st_peer8(peer_addr(&sh.abort, (uint32_t)tid), 1);
+        cluster_sync();
     }
     if (sh.abort) return;
 
     const uint64_t hop_k1 = key_word(D.replica, PURPOSE_HOP);
-    const Geo geo{D.L[0], D.L[1], D.L[2], D.row_words, D.nf[0], D.nf[1], D.F, D.theta_tau, window_f(D.theta_tau, D.F)};
-    const int lane = tid & 31;
-    const int warp = tid >> 5;
-    const unsigned FULL = 0xffffffffu;
-    int16_t* wslot = S.wslot + warp * cap;
-    int8_t* wtype = S.wtype + warp * cap * 8;
+    const uint64_t th = window_bits(D.theta_tau, D.F);  // mixed form
+    const double tau = D.tau;                           // plain form
+    const float lim32 = __double2float_ru(__dmul_ru(__longlong_as_double((long long)th), 1.0 + 0x1p-20));
+    const uint32_t dirs = pack_direction(nbt, lane & 7);
+    uint32_t* const wkey = S.wkey + warp * cap;
+    uint32_t* const wvac = S.wvac + warp * cap;
+    int8_t* const wtype = S.wtype + warp * cap * 8;
+    uint64_t* const wlog = S.wlog + warp * 2 * CLOCK_LOG;
     unsigned long long my_hops = 0, my_hand = 0;
 
+    const uint32_t key0 = key32(0, 0, 0, geo.zb);  // a site of this slab
+    const int frag_off = fzb * geo.nf1 * geo.nf0;  // fragment index of local fragment 0
+    // first draws of local fragment lf, events 0 .. pre_ev - 1, at offset o: part k, one
+    // Philox block (mixed) or one event (plain: a copy of what k_draws computed);
+    // they depend on no fragment's state
+    const int per = PREC == 1 ? pre_ev >> 1 : pre_ev;
+    const int sh_per = per == 8 ? 3 : (per == 4 ? 2 : (per == 2 ? 1 : 0));
+    auto draw = [&](int lf, uint64_t wk, int o, int k) {
+        const int fid = frag_off + lf;
+        if constexpr (PREC == 1) {
+            const U64x4 b = philox4x64((uint64_t)fid, D.window + w0 + wk, (uint64_t)k, 0, D.seed, hop_k1);
+            float* E = reinterpret_cast<float*>(S.pre_E);
+            E[o + 2 * k] = neglog32(b.x[0]);
+            E[o + 2 * k + 1] = neglog32(b.x[2]);
+            S.pre_xs[o + 2 * k] = b.x[1];
+            S.pre_xs[o + 2 * k + 1] = b.x[3];
+        } else {
+            const int4 d = __ldg(
+                reinterpret_cast<const int4*>(draws + ((int64_t)wk * frag_tot + D.draw_off + fid) * pre_ev + k));
+            reinterpret_cast<uint64_t*>(S.pre_E)[o + k] = (uint64_t)(uint32_t)d.x | (uint64_t)(uint32_t)d.y << 32;
+            S.pre_xs[o + k] = (uint64_t)(uint32_t)d.z | (uint64_t)(uint32_t)d.w << 32;
+        }
+    };
+    // cluster: of every fragment of a colour, to row `row`
+    auto draw_colour = [&](int colour, uint64_t wk, int row) {
+        const int c0 = sh.coff[colour], n = sh.coff[colour + 1] - c0;
+        for (int it = tid; it < n << sh_per; it += NT)
+            draw(S.flist[c0 + (it >> sh_per)], wk, (row * maxc + (it >> sh_per)) * pre_ev, it & (per - 1));
+    };
+    // rate type and neighbour key of this lane's direction (no event for a dead slot, without a branch)
+    auto type_of = [&](uint32_t key, uint32_t& nkey) -> int {
+        const bool dead = key == DEAD;
+        const NbSite s = nb_site(geo, dirs, dead ? key0 : key);
+        nkey = key32(s.t2, s.x, s.y, s.z);
+        const int ty = site_code<CL>(S, geo, s.t2, s.x, s.y, s.z) * 3 + s.dz1;
+        return dead ? NO_EVENT : ty;
+    };
+    auto rate_of = [&](int ty) -> uint64_t { return sh.rate[ty]; };
+    auto scan64 = [&](uint64_t v) -> uint64_t {  // inclusive prefix over the lanes, strides 1, 2, .. 16
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t u = __shfl_up_sync(FULL, (unsigned long long)v, o);
+            if (lane >= o) {
+                if constexpr (PREC == 1) v += u;
+                else v = (uint64_t)__double_as_longlong(
+                         __dadd_rn(__longlong_as_double((long long)v), __longlong_as_double((long long)u)));
+            }
+        }
+        return v;
+    };
+    auto add = [&](uint64_t a, uint64_t b) -> uint64_t {
+        if constexpr (PREC == 1) return a + b;
+        else return (uint64_t)__double_as_longlong(
+                 __dadd_rn(__longlong_as_double((long long)a), __longlong_as_double((long long)b)));
+    };
+
+    uint32_t ph = 0;  // phases of this launch so far
     for (uint64_t wk = 0; wk < windows; ++wk) {
-        const uint64_t w = D.window + wk;
+        const uint64_t w = D.window + w0 + wk;
         if ((wk & 63) == 0) {  // colour orders of the next 64 windows, one thread each
             if (tid < 64 && wk + tid < windows) sh.perms[tid] = colour_perm_packed(D.seed, D.replica, w + tid);
             __syncthreads();
         }
         const uint32_t wperm = sh.perms[wk & 63];
-        for (int p = 0; p < 8; ++p) {
+        for (int p = 0; p < 8; ++p, ++ph) {
             const int colour = (int)((wperm >> (4 * p)) & 15u);
-            int cnt[3], bit[3];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                bit[d] = (colour >> d) & 1;
-                cnt[d] = D.nf[d] == 1 ? (bit[d] == 0 ? 1 : 0) : D.nf[d] / 2;
-            }
-            const int ncls = cnt[0] * cnt[1] * cnt[2];
-            const int pslot = p & (pre_g - 1);  // this phase's rows of the first-draw arrays
-            if (pslot == 0) {
-                // first draws (block 0: events 0 and 1; with pre_ev 4 also block 1: events 2
-                // and 3) of every fragment of the next pre_g phases, one thread per block:
-                // they depend on no state, and one batch of Philox blocks here replaces one
-                // per phase (and one per visit of two events or more) on the critical paths
-                const int nbk = pre_ev >> 1;
-                for (int it = tid; it < pre_g * ncls_max * nbk; it += NT) {
-                    const int idx = nbk == 2 ? it >> 1 : it, bk = it - idx * nbk;
-                    const int pp = idx / ncls_max, l = idx - pp * ncls_max;
+            const int par = (int)(ph & 1u);
+            if constexpr (CL) {
+                if (p == 0 && (wk & 63) == 0) {  // otherwise drawn at the end of the phase before
+                    draw_colour(colour, wk, par);
+                    __syncthreads();
+                }
+            } else if ((p & (pre_g - 1)) == 0) {
+                // of the next pre_g phases at once, for the fragments that hold an event now: a
+                // list of them, then one thread per part of their draws (an empty fragment that
+                // receives a vacancy meanwhile draws for itself)
+                for (int it = tid; it < pre_g * maxc; it += NT) {
+                    const int pp = it / maxc, l = it - pp * maxc;
                     const int col = (int)((wperm >> (4 * (p + pp))) & 15u);
-                    int c3[3], f3[3];
-#pragma unroll
-                    for (int d = 0; d < 3; ++d)
-                        c3[d] = D.nf[d] == 1 ? (((col >> d) & 1) == 0 ? 1 : 0) : D.nf[d] / 2;
-                    if (l >= c3[0] * c3[1] * c3[2]) continue;
-                    f3[0] = l % c3[0];
-                    f3[1] = (l / c3[0]) % c3[1];
-                    f3[2] = l / (c3[0] * c3[1]);
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) f3[d] = D.nf[d] == 1 ? 0 : 2 * f3[d] + ((col >> d) & 1);
-                    const int fid = (f3[2] * D.nf[1] + f3[1]) * D.nf[0] + f3[0];
-                    const U64x4 blk = philox4x64((uint64_t)fid, w, (uint64_t)bk, 0, D.seed, hop_k1);
-                    const int o = pre_ev * idx + 2 * bk;
-                    S.pre_E[o] = neglog32(blk.x[0]);
-                    S.pre_E[o + 1] = neglog32(blk.x[2]);
-                    S.pre_xs[o] = blk.x[1];
-                    S.pre_xs[o + 1] = blk.x[3];
+                    if (l >= sh.coff[col + 1] - sh.coff[col]) continue;
+                    const int lf = S.flist[sh.coff[col] + l];
+                    unsigned r = NO_ROW;
+                    const typename Lim::T m = lim[lf];
+                    if (m != Lim::EMPTY) {
+                        r = (unsigned)atomicAdd(&sh.ndraw, 1);
+                        // the limit is about the expected number of events: below 1/4 a third is rare
+                        if (PREC == 0 || m >= 0x3e800000u) r |= ROW_FULL;
+                        S.dlist[r & ~ROW_FULL] = (uint16_t)lf;
+                    }
+                    S.pre_row[lf] = (uint16_t)r;
                 }
+                __syncthreads();
+                const int nd = sh.ndraw << sh_per;
+                for (int it = tid; it < nd; it += NT) {
+                    const int lf = S.dlist[it >> sh_per], k = it & (per - 1);
+                    if (PREC == 1 && k > 0 && !(S.pre_row[lf] & ROW_FULL)) continue;
+                    draw(lf, wk, (it >> sh_per) * pre_ev, k);
+                }
+                __syncthreads();
+                if (tid == 0) sh.ndraw = 0;
             }
-            if (tid == 0) {
-                sh.nact = 0;
-                sh.next_act = 0;
-            }
-            __syncthreads();
             // ---- screen: one thread per fragment of the colour
-            for (int l = tid * CL + (int)rank; l < ncls; l += NT * CL) {
-                int f0 = l % cnt[0], f1 = (l / cnt[0]) % cnt[1], f2 = l / (cnt[0] * cnt[1]);
-                f0 = D.nf[0] == 1 ? 0 : 2 * f0 + bit[0];
-                f1 = D.nf[1] == 1 ? 0 : 2 * f1 + bit[1];
-                f2 = D.nf[2] == 1 ? 0 : 2 * f2 + bit[2];
-                const int fid = (f2 * D.nf[1] + f1) * D.nf[0] + f0;
-                if (S.head[fid] < 0) continue;
-                const bool dirty = S.dirty[fid] != 0;
-                const unsigned long long tot = S.S[fid];
-                if (!dirty && tot == 0ull) continue;
-                bool active = dirty;
-                if (!active) {
-                    const float E0 = S.pre_E[pre_ev * (pslot * ncls_max + l)];
-                    const float ratio = __fdiv_rn(E0, __ull2float_rn(tot));
-                    active = !(ratio > geo.theta_f);  // 0 + 2^F ratio <= theta
+            const int c0 = sh.coff[colour], ncol = sh.coff[colour + 1] - c0;
+            for (int l = tid; l < ncol; l += NT) {
+                const int lf = S.flist[c0 + l];
+                const typename Lim::T m = lim[lf];
+                bool active = m == Lim::DIRTY;
+                if (!active && m != Lim::EMPTY) {
+                    const int o = (CL ? par * maxc + l : (int)(S.pre_row[lf] & (ROW_FULL - 1u))) * pre_ev;
+                    if constexpr (PREC == 1) active = reinterpret_cast<const float*>(S.pre_E)[o] <= __uint_as_float(m);
+                    else active = reinterpret_cast<const uint64_t*>(S.pre_E)[o] <= m;  // positive doubles
                 }
-                if (active) {
-                    const int a = atomicAdd(&sh.nact, 1);
-                    S.act[a] = f0 | (f1 << 10) | (f2 << 20);  // fragment coordinates (< 1024 each)
-                }
+                if (active) S.act[atomicAdd(&sh.nact[par], 1)] = (uint32_t)lf | (uint32_t)l << 16;
             }
             __syncthreads();
-            // ---- run: one warp per listed fragment
-            const int nact = sh.nact;
-            for (;;) {
-                // warps take the screened fragments one at a time, as they become free
-                int a = 0;
-                if (lane == 0) a = atomicAdd(&sh.next_act, 1);
-                a = __shfl_sync(FULL, a, 0);
-                if (a >= nact) break;
-                const int fxyz = S.act[a];
-                const int fx = fxyz & 1023, fy = (fxyz >> 10) & 1023, fz = fxyz >> 20;
-                const int fid = (fz * D.nf[1] + fy) * D.nf[0] + fx;
-                // the fragment's screen index within its colour, and its row of first draws
-                const int ls = ((D.nf[2] == 1 ? 0 : fz >> 1) * cnt[1] + (D.nf[1] == 1 ? 0 : fy >> 1)) * cnt[0] +
-                               (D.nf[0] == 1 ? 0 : fx >> 1);
-                const int prow = pslot * ncls_max + ls;
-                const int lo0 = frag_start(fx, D.base[0], D.rem[0]), hi0 = frag_start(fx + 1, D.base[0], D.rem[0]);
-                const int lo1 = frag_start(fy, D.base[1], D.rem[1]), hi1 = frag_start(fy + 1, D.base[1], D.rem[1]);
-                const int lo2 = frag_start(fz, D.base[2], D.rem[2]), hi2 = frag_start(fz + 1, D.base[2], D.rem[2]);
-                // slots: the fragment's vacancies in ascending site order
-                int n = 0;
-                if (lane == 0) {
-                    for (int v = S.head[fid]; v >= 0; v = S.next[v]) {
-                        if (n >= cap) {
-                            atomicOr(status, STATUS_OVERFLOW);
-                            break;
-                        }
-                        wslot[n++] = (int16_t)v;
-                    }
-                }
-                n = __shfl_sync(FULL, n, 0);
-                __syncwarp();
-                // a list that received no vacancy since its last visit is still in site order
-                bool ordered = false;
-                uint32_t kk = 0xffffffffu;
-                if (n <= 32) {  // rank by site (sites are distinct), unless already in order
-                    const int vk = lane < n ? wslot[lane] : -1;
-                    kk = lane < n ? S.key[vk] : 0xffffffffu;
-                    const uint32_t kprev = __shfl_up_sync(FULL, kk, 1);
-                    ordered = __ballot_sync(FULL, lane > 0 && lane < n && kprev > kk) == 0u;
-                    if (!ordered) {
-                        int rnk = 0;
-                        for (int q = 0; q < n; ++q) rnk += __shfl_sync(FULL, kk, q) < kk ? 1 : 0;
-                        __syncwarp();
-                        if (lane < n) wslot[rnk] = (int16_t)vk;
-                    }
-                } else if (lane == 0) {
-                    for (int k = 1; k < n; ++k) {
-                        const int v = wslot[k];
-                        const uint32_t kv = S.key[v];
-                        int m = k;
-                        while (m > 0 && S.key[wslot[m - 1]] > kv) {
-                            wslot[m] = wslot[m - 1];
-                            --m;
-                        }
-                        wslot[m] = (int16_t)v;
-                    }
-                }
-                __syncwarp();
-                const int nch = (n + 3) >> 2;
-                // up to two chunks (8 vacancies): each lane keeps the site keys of its two
-                // events' slots in registers (0xffffffff: no slot, or handed off)
-                uint32_t kc0 = 0xffffffffu, kc1 = 0xffffffffu;
-                if (nch <= 2) {
-                    const int m0 = lane >> 3, m1 = 4 + (lane >> 3);
-                    if (ordered) {  // lane m holds slot m's key
-                        const uint32_t a0 = __shfl_sync(FULL, kk, m0), a1 = __shfl_sync(FULL, kk, m1);
-                        if (m0 < n) kc0 = a0;
-                        if (m1 < n) kc1 = a1;
-                    } else {
-                        if (m0 < n) kc0 = S.key[wslot[m0]];
-                        if (m1 < n) kc1 = S.key[wslot[m1]];
-                    }
-                }
-                auto type_of = [&](uint32_t k, int q) -> int {
-                    int t, x, y, z;
-                    split32(k, t, x, y, z);
-                    const NbEntry nbe = sh.nb[t][q];
-                    const int code = site_code(geo, S.occ, nbe.t2, wrapc(x + nbe.dc[0], geo.L0),
-                                               wrapc(y + nbe.dc[1], geo.L1), wrapc(z + nbe.dc[2], geo.L2));
-                    return code == SP_V ? -1 : code * 3 + nbe.d[2] + 1;
+            if (tid == 0) {  // the next phase's counters
+                sh.nact[par ^ 1] = 0;
+                sh.next_act[par ^ 1] = NW;
+            }
+            // ---- run: one warp per listed fragment; each warp's first by its index, then as they become free
+            const int nact = sh.nact[par];
+            for (int a = warp; a < nact;) {
+                const uint32_t ent = S.act[a];
+                const int lf = (int)(ent & 0xffffu);
+                const unsigned prow = CL ? (unsigned)(par * maxc) + (ent >> 16) : (unsigned)S.pre_row[lf];
+                const int o0 = (int)(CL ? prow : prow & (ROW_FULL - 1u)) * pre_ev;
+                // events drawn ahead
+                const int n_pre = CL || (prow & ROW_FULL) ? (!CL && prow == NO_ROW ? 0 : pre_ev) : 2;
+                const uint2 bx = S.box[lf];
+                const int lo0 = (int)(bx.x & 1023u), lo1 = (int)((bx.x >> 10) & 1023u), lo2 = (int)(bx.x >> 20);
+                const int ex = (int)(bx.y & 1023u) + 1, ey = (int)((bx.y >> 10) & 1023u) + 1, ez = (int)(bx.y >> 20) + 1;
+                // the fragment's vacancies: its list, or, where it changed from outside or is too long
+                // for one, a scan of its rows.  Up to two chunks (8 vacancies) each lane keeps the site
+                // keys of its two events' slots, their rate types and their targets' keys in registers
+                uint32_t* const sl = S.slots + lf * KSLOTS;
+                uint32_t kc0 = sl[lane >> 3], kc1 = sl[4 + (lane >> 3)];
+                const bool scan = S.stale[lf] != 0 || __shfl_sync(FULL, kc0, 0) == UNLISTED;
+                // key of slot lane & 7 (up to two chunks)
+                auto slot_key = [&]() -> uint32_t {
+                    const uint32_t u = __shfl_sync(FULL, kc0, (lane & 3) * 8), v = __shfl_sync(FULL, kc1, (lane & 3) * 8);
+                    return lane & 4 ? v : u;
                 };
-                int ty0 = -1, ty1 = -1;  // up to two chunks: rate types of events lane and 32 + lane
+                int n;
+                if (!scan) {
+                    n = __popc(__ballot_sync(FULL, kc0 != DEAD) & 0x01010101u) +
+                        __popc(__ballot_sync(FULL, kc1 != DEAD) & 0x01010101u);
+                    // the last visit left its slots' order: into site order where its exchanges changed it
+                    const uint32_t k = slot_key();
+                    const uint32_t up = __shfl_up_sync(FULL, k, 1);
+                    if (__any_sync(FULL, (lane & 7) > 0 && up > k)) {
+                        int r = 0;
+#pragma unroll
+                        for (int q = 0; q < KSLOTS; ++q) r += __shfl_sync(FULL, k, q) < k ? 1 : 0;
+                        if (lane < KSLOTS && k != DEAD) wkey[r] = k;
+                        __syncwarp();
+                        const int m = lane >> 3;
+                        kc0 = m < n ? wkey[m] : DEAD;
+                        kc1 = m + 4 < n ? wkey[m + 4] : DEAD;
+                    }
+                } else {
+                    n = gather(S, geo, wkey, cap, lane, lo0, lo1, lo2, ex, ey, ez);
+                    if (n > cap) {
+                        if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
+                        n = cap;
+                    }
+                    const int m = lane >> 3;
+                    kc0 = m < n ? wkey[m] : DEAD;
+                    kc1 = m + 4 < n ? wkey[m + 4] : DEAD;
+                }
+                const int nch = (n + 3) >> 2;
+                // record index of slot `lane` (beyond 32 slots: through wvac); used at the first exchange
+                uint32_t vrec = 0;
+                if (nch <= 2) {
+                    const uint32_t k = slot_key();
+                    if (lane < n) vrec = __ldcg(vmap_r + map_index(geo, k));
+                } else {
+                    if (lane < n) vrec = __ldcg(vmap_r + map_index(geo, wkey[lane]));
+                    if (n > 32)
+                        for (int k = lane; k < n; k += 32) wvac[k] = __ldcg(vmap_r + map_index(geo, wkey[k]));
+                }
+                uint32_t nk0 = 0, nk1 = 0;
+                int ty0 = NO_EVENT, ty1 = NO_EVENT;
                 auto compute_types = [&]() {
                     if (nch <= 2) {
-                        ty0 = kc0 != 0xffffffffu ? type_of(kc0, lane & 7) : -1;
-                        ty1 = (nch == 2 && kc1 != 0xffffffffu) ? type_of(kc1, lane & 7) : -1;
+                        ty0 = type_of(kc0, nk0);
+                        if (nch == 2) ty1 = type_of(kc1, nk1);
                     } else {
                         for (int c = 0; c < nch; ++c) {
                             const int e = c * 32 + lane, m = e >> 3;
-                            int ty = -1;
-                            if (m < n && wslot[m] >= 0) ty = type_of(S.key[wslot[m]], e & 7);
+                            int ty = NO_EVENT;
+                            uint32_t nk;
+                            if (m < n && wkey[m] != DEAD) ty = type_of(wkey[m], nk);
                             wtype[e] = (int8_t)ty;
                         }
+                        __syncwarp();
                     }
-                    __syncwarp();
                 };
                 compute_types();
 
-                double clock = 0.0;
+                // mixed: mixed_clock's; plain: FP64 bits, of the events before `logged0`, those from
+                // there on in the log (E, R), and an FP32 estimate of the whole in units of tau
+                uint64_t clock = 0;
+                bool fp = false;
+                int logged0 = 0;
+                float xclock = 0.0f;
                 uint64_t i = 0, batch = ~0ull;
-                uint64_t xs_even = 0, xs_odd = 0;
-                float E_even = 0.f, E_odd = 0.f;
-                unsigned long long tot = 0;
-                for (;;) {
-                    // exact total of the fragment's events (order-free integer sum).  Up to two
-                    // chunks (8 vacancies) one inclusive scan gives both the total and the
-                    // prefixes the selection needs; beyond that, a reduction now and scans later.
-                    unsigned long long inc0 = 0, inc1 = 0;
-                    if (nch <= 2) {
-                        const int t0 = ty0;
-                        inc0 = t0 < 0 ? 0ull : (unsigned long long)D.q[t0];
-#pragma unroll
-                        for (int off = 1; off < 32; off <<= 1) {
-                            const unsigned long long t2 = __shfl_up_sync(FULL, inc0, off);
-                            if (lane >= off) inc0 += t2;
-                        }
-                        tot = __shfl_sync(FULL, inc0, 31);
-                        if (nch == 2) {
-                            const int t1 = ty1;
-                            inc1 = t1 < 0 ? 0ull : (unsigned long long)D.q[t1];
-#pragma unroll
-                            for (int off = 1; off < 32; off <<= 1) {
-                                const unsigned long long t2 = __shfl_up_sync(FULL, inc1, off);
-                                if (lane >= off) inc1 += t2;
-                            }
-                            inc1 += tot;
-                            tot = __shfl_sync(FULL, inc1, 31);
-                        }
+                uint64_t xs_even = 0, xs_odd = 0, E_even = 0, E_odd = 0;
+                uint64_t tot = 0;
+                // the last exchange's record: its slot (-1: none), the target's entry of the map
+                // (lane 1), the displacement (lanes 0..2), and the exchanged ion's displacement
+                // (lanes 8..10).  Written at the next exchange or at the end of the visit, when the
+                // record index and the ion's displacement have long arrived.
+                int pend_m = -1, pend_at = 0, pend_d = 0;
+                int trv = 0;
+                int64_t trs = 0, trj = 0;
+                auto flush = [&]() {
+                    if (pend_m < 0) return;
+                    const uint32_t v = n <= 32 ? __shfl_sync(FULL, vrec, pend_m & 31) : wvac[pend_m];
+                    if (v >= rec_lim) {  // a vacancy without a record: not a state this library wrote
+                        if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
                     } else {
-                        unsigned long long part = 0;
-                        for (int c = 0; c < nch; ++c) {
-                            const int ty = wtype[c * 32 + lane];
-                            part += ty < 0 ? 0ull : (unsigned long long)D.q[ty];
+                        if (lane == 1) vmap_r[pend_at] = v;
+                        if (lane < 3 && pend_d != 0) atomicAdd(&recs_r[v].d[lane], pend_d);
+                    }
+                    if (tracer && lane >= 8 && lane < 11) {
+                        tracer[trs] = trv;
+                        tracer[trj] = 0;
+                    }
+                };
+                for (;;) {
+                    // the total of the fragment's events; the plain form's scans, in the canonical
+                    // order, give the inclusive prefixes that the selection needs besides
+                    uint64_t inc0 = 0, inc1 = 0;
+                    if (nch <= 2) {
+                        inc0 = rate_of(ty0);
+                        inc1 = nch == 2 ? rate_of(ty1) : 0ull;
+                        if constexpr (PREC == 1) {
+                            tot = warp_total(inc0 + inc1);
+                        } else {
+                            inc0 = scan64(inc0);
+                            tot = __shfl_sync(FULL, inc0, 31);
+                            if (nch == 2) {
+                                inc1 = add(tot, scan64(inc1));
+                                tot = __shfl_sync(FULL, inc1, 31);
+                            }
                         }
-#pragma unroll
-                        for (int off = 16; off; off >>= 1) part += __shfl_xor_sync(FULL, part, off);
-                        tot = part;
+                    } else if constexpr (PREC == 1) {
+                        unsigned long long part = 0;
+                        for (int c = 0; c < nch; ++c) part += rate_of(wtype[c * 32 + lane]);
+                        tot = warp_total(part);
+                    } else {
+                        tot = 0;
+                        for (int c = 0; c < nch; ++c)
+                            tot = __shfl_sync(FULL, add(tot, scan64(rate_of(wtype[c * 32 + lane]))), 31);
                     }
                     if (tot == 0ull) break;
                     if (i >= MAX_EVENTS_PER_PHASE) {
                         if (lane == 0) atomicOr(status, STATUS_EVENT_LIMIT);
                         break;
                     }
-                    uint64_t xs;
-                    float E;
-                    if (i < (uint64_t)pre_ev) {  // blocks 0 (and 1), drawn in the batch before the phase
-                        xs = S.pre_xs[pre_ev * prow + (int)i];
-                        E = S.pre_E[pre_ev * prow + (int)i];
+                    uint64_t xs, Eb;
+                    if (i < (uint64_t)n_pre) {  // drawn ahead
+                        xs = S.pre_xs[o0 + (int)i];
+                        if constexpr (PREC == 1) Eb = reinterpret_cast<const uint32_t*>(S.pre_E)[o0 + (int)i];
+                        else Eb = reinterpret_cast<const uint64_t*>(S.pre_E)[o0 + (int)i];
                     } else {
-                        // events [2 + 64 b, 66 + 64 b) come from blocks 1 + 32 b + lane (block 1,
-                        // events 2 and 3, was drawn ahead with pre_ev 4: lane 0 recomputes it unused)
-                        const uint64_t k = i - 2;
+                        // events [64 b, 64 b + 64) come from blocks 32 b + lane (those drawn ahead
+                        // are computed again, unused)
+                        const uint64_t k = i;
                         if ((k >> 6) != batch) {
                             batch = k >> 6;
                             const U64x4 blk =
-                                philox4x64((uint64_t)fid, w, 1 + 32 * batch + lane, 0, D.seed, hop_k1);
+                                philox4x64((uint64_t)(frag_off + lf), w, 32 * batch + lane, 0, D.seed, hop_k1);
                             xs_even = blk.x[1];
                             xs_odd = blk.x[3];
-                            E_even = neglog32(blk.x[0]);
-                            E_odd = neglog32(blk.x[2]);
+                            if constexpr (PREC == 1) {
+                                E_even = __float_as_uint(neglog32(blk.x[0]));
+                                E_odd = __float_as_uint(neglog32(blk.x[2]));
+                            } else {
+                                E_even = (uint64_t)__double_as_longlong(neglog64(blk.x[0]));
+                                E_odd = (uint64_t)__double_as_longlong(neglog64(blk.x[2]));
+                            }
                         }
                         const int src = (int)((k >> 1) & 31);
                         const bool odd = (k & 1) != 0;
                         xs = __shfl_sync(FULL, odd ? xs_odd : xs_even, src);
-                        E = __shfl_sync(FULL, odd ? E_odd : E_even, src);
+                        Eb = __shfl_sync(FULL, odd ? E_odd : E_even, src);
                     }
-                    const float ratio = __fdiv_rn(E, __ull2float_rn(tot));
-                    const double nclock = __dadd_rn(clock, scale_pow2((double)ratio, geo.F));
-                    const bool past = i == 0 ? ratio > geo.theta_f : nclock > geo.theta;  // the first: clock 0
-                    // up to two chunks: the selection (no side effects) before the clock test,
-                    // so that its shuffles overlap the clock's FP64 chain; a break discards it
-                    const unsigned long long target = __umul64hi(xs, tot);
-                    int e_sel = -1;
-                    uint32_t ksel = 0u;
-                    int tsel = -1;
-                    if (nch <= 2) {
-                        unsigned bal = __ballot_sync(FULL, inc0 > target);
-                        if (bal) {
-                            e_sel = __ffs(bal) - 1;
-                        } else {
-                            bal = __ballot_sync(FULL, inc1 > target);
-                            if (bal && nch == 2) e_sel = 32 + __ffs(bal) - 1;
+                    // the window test, and the selection (no side effects) beside it
+                    uint64_t nclock = 0;
+                    bool past;
+                    uint64_t target;
+                    if constexpr (PREC == 1) {
+                        past = mixed_clock(clock, fp, __fdiv_rn(__uint_as_float((uint32_t)Eb), u64_to_float_rn(tot)), th,
+                                           nclock);
+                        target = __umul64hi(xs, tot);
+                    } else {
+                        // clock + fl(E / R) > tau, the clock the rounded sum of the events before.  An
+                        // estimate of clock / tau in FP32 (each term E / fl(tau R) to 2^-20, 2^12 of them
+                        // at most) decides unless it comes within 2^-10 of 1; then the divisions are done,
+                        // those of the events before from the log.  (A division is some ten FP64
+                        // instructions, each 64 cycles of the SM quarter's FP64 pipe.)
+                        const double R = __longlong_as_double((long long)tot);
+                        const long long pb = __double_as_longlong(__dmul_rn(tau, R));
+                        float est = 2.0f;  // out of the estimate's range: exact
+                        bool sure = float_range((long long)Eb) && float_range(pb) && i < 4096;
+                        if (sure) {
+                            est = xclock + __fdividef(to_float((long long)Eb), to_float(pb));
+                            sure = fabsf(est - 1.0f) > 0x1p-10f;
+                            past = est > 1.0f;
                         }
-                        const int ms = e_sel >> 3;  // the slot's site key and the event's type
-                        ksel = __shfl_sync(FULL, ms < 4 ? kc0 : kc1, (ms & 3) << 3);
-                        tsel = __shfl_sync(FULL, e_sel < 32 ? ty0 : ty1, e_sel & 31);
+                        const int left = (int)i - logged0;
+                        if (!sure || left == CLOCK_LOG) {
+                            double c = __longlong_as_double((long long)clock);
+                            for (int q = 0; q < left; ++q)
+                                c = __dadd_rn(c, __ddiv_rn(__longlong_as_double((long long)wlog[2 * q]),
+                                                           __longlong_as_double((long long)wlog[2 * q + 1])));
+                            clock = (uint64_t)__double_as_longlong(c);
+                            logged0 = (int)i;
+                            if (!sure) {
+                                c = __dadd_rn(c, __ddiv_rn(__longlong_as_double((long long)Eb), R));
+                                past = c > tau;
+                                if (!past) {
+                                    clock = (uint64_t)__double_as_longlong(c);
+                                    logged0 = (int)i + 1;
+                                    xclock = __double2float_rn(__ddiv_rn(c, tau));
+                                }
+                            }
+                            __syncwarp();
+                        }
+                        if (sure && !past) {
+                            if (lane == 0) {
+                                wlog[2 * ((int)i - logged0)] = Eb;
+                                wlog[2 * ((int)i - logged0) + 1] = tot;
+                            }
+                            __syncwarp();
+                            xclock = est;
+                        }
+                        nclock = clock;
+                        // doubles >= 0 compare as their bits
+                        target = (uint64_t)__double_as_longlong(__dmul_rn(uniform53(xs), R));
                     }
                     if (past) break;
-                    // first event whose running sum exceeds the target
-                    if (nch > 2) {
-                        unsigned long long carry = 0;
-                        for (int c = 0; c < nch; ++c) {
-                            const int ty = wtype[c * 32 + lane];
-                            unsigned long long inc = ty < 0 ? 0ull : (unsigned long long)D.q[ty];
-#pragma unroll
-                            for (int off = 1; off < 32; off <<= 1) {
-                                const unsigned long long t2 = __shfl_up_sync(FULL, inc, off);
-                                if (lane >= off) inc += t2;
-                            }
-                            inc += carry;
-                            const unsigned bal = __ballot_sync(FULL, inc > target);
-                            if (bal) {
-                                e_sel = c * 32 + __ffs(bal) - 1;
-                                break;
-                            }
+                    if constexpr (PREC == 1) {  // the prefixes, only for an event that happens
+                        if (nch <= 2) {
+                            inc0 = scan64(inc0);
+                            if (nch == 2) inc1 = __shfl_sync(FULL, inc0, 31) + scan64(inc1);
+                        }
+                    }
+                    // first event whose inclusive prefix exceeds the target (plain: among the events of
+                    // nonzero rate, and the last of those where rounding left no prefix above it)
+                    int e_sel = -1;
+                    if (nch <= 2) {
+                        const bool h0 = inc0 > target && (PREC == 1 || ty0 < NO_EVENT);
+                        const bool h1 = nch == 2 && inc1 > target && (PREC == 1 || ty1 < NO_EVENT);
+                        const unsigned b0 = __ballot_sync(FULL, h0), b1 = __ballot_sync(FULL, h1);
+                        e_sel = b0 ? __ffs(b0) - 1 : (b1 ? 32 + __ffs(b1) - 1 : -1);
+                        if (PREC == 0 && e_sel < 0) {
+                            const unsigned l0 = __ballot_sync(FULL, rate_of(ty0) != 0ull),
+                                           l1 = __ballot_sync(FULL, nch == 2 && rate_of(ty1) != 0ull);
+                            e_sel = l1 ? 63 - __clz(l1) : 31 - __clz(l0);
+                        }
+                    } else {
+                        uint64_t carry = 0;
+                        for (int c = 0; c < nch && e_sel < 0; ++c) {
+                            const uint64_t v = rate_of(wtype[c * 32 + lane]);
+                            const uint64_t inc = add(carry, scan64(v));
+                            const unsigned bal = __ballot_sync(FULL, inc > target && (PREC == 1 || v != 0ull));
+                            if (bal) e_sel = c * 32 + __ffs(bal) - 1;
                             carry = __shfl_sync(FULL, inc, 31);
+                        }
+                        if (PREC == 0) {
+                            for (int c = nch - 1; c >= 0 && e_sel < 0; --c) {
+                                const unsigned bal = __ballot_sync(FULL, rate_of(wtype[c * 32 + lane]) != 0ull);
+                                if (bal) e_sel = c * 32 + 31 - __clz(bal);
+                            }
                         }
                     }
                     if (e_sel < 0) {  // cannot happen: the target lies below the total
                         if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
                         break;
                     }
-                    const int m = e_sel >> 3, qd = e_sel & 7;
-                    int t, x, y, z;
-                    split32(nch <= 2 ? ksel : S.key[wslot[m]], t, x, y, z);
-                    const NbEntry nb = sh.nb[t][qd];
-                    const NbSite j = nb_site(sh, geo, t, x, y, z, qd);
-                    const bool owned = j.jx >= lo0 && j.jx < hi0 && j.jy >= lo1 && j.jy < hi1 && j.jz >= lo2 &&
-                                       j.jz < hi2;
-                    if (lane == 0) {  // apply the exchange
-                        const int v = wslot[m];
-                        const uint32_t ion = (uint32_t)((nch <= 2 ? tsel : (int)wtype[e_sel]) / 3);
-                        uint32_t* ws = S.occ + ((z * geo.L1 + y) * geo.RW + (x >> 4)) * 3 + t;
-                        uint32_t* wj = S.occ + ((j.jz * geo.L1 + j.jy) * geo.RW + (j.jx >> 4)) * 3 + j.t2;
-                        const uint32_t ms = ((uint32_t)SP_V ^ ion) << occ_shift(x);
-                        const uint32_t mj = (ion ^ (uint32_t)SP_V) << occ_shift(j.jx);
-                        atomicXor(ws, ms);
-                        atomicXor(wj, mj);
-                        S.d[3 * v] += nb.d[0];
-                        S.d[3 * v + 1] += nb.d[1];
-                        S.d[3 * v + 2] += nb.d[2];
-                        if constexpr (CL > 1) {
-                            red_peer_xor(peer_addr(ws, peer), ms);
-                            red_peer_xor(peer_addr(wj, peer), mj);
-                            for (int k = 0; k < 3; ++k) st_peer(peer_addr(S.d + 3 * v + k, peer), S.d[3 * v + k]);
-                        }
-                        if (tracer) {
-                            const int64_t s_lin = (((int64_t)t * D.L[2] + z) * D.L[1] + y) * D.L[0] + x;
-                            const int64_t j_lin = (((int64_t)j.t2 * D.L[2] + j.jz) * D.L[1] + j.jy) * D.L[0] + j.jx;
-                            int32_t* ts = tracer + 3 * (D.site_off + s_lin);
-                            int32_t* tj = tracer + 3 * (D.site_off + j_lin);
-                            ts[0] = tj[0] - nb.d[0];
-                            ts[1] = tj[1] - nb.d[1];
-                            ts[2] = tj[2] - nb.d[2];
-                            tj[0] = tj[1] = tj[2] = 0;
-                        }
-                        S.key[v] = key32(j.t2, j.jx, j.jy, j.jz);
-                        if constexpr (CL > 1) st_peer(peer_addr(S.key + v, peer), S.key[v]);
-                        if (!owned) {
-                            // leaves the fragment: its slot goes dead (zero rate), the record
-                            // is pushed onto the owner's list (the owner does not run in this
-                            // phase, so that list only receives pushes; links are read after
-                            // the phase barrier)
-                            wslot[m] = -1;
-                            const int g2 = owner_of(geo, S.frag_of_c, j.jx, j.jy, j.jz);
-                            S.next[v] = (int16_t)atomicExch(S.head + g2, v);
-                            if constexpr (CL > 1)
-                                st_peer16(peer_addr(S.next + v, peer),
-                                          (int16_t)atom_peer_exch(peer_addr(S.head + g2, peer), v));
-                            ++my_hand;
+                    // the exchange: site s, its target j, the ion
+                    const int m = e_sel >> 3;
+                    uint32_t ks, kj;
+                    int ty;
+                    if (nch <= 2) {
+                        const bool c1 = e_sel >= 32;
+                        ks = __shfl_sync(FULL, c1 ? kc1 : kc0, e_sel & 31);
+                        kj = __shfl_sync(FULL, c1 ? nk1 : nk0, e_sel & 31);
+                        ty = __shfl_sync(FULL, c1 ? ty1 : ty0, e_sel & 31);
+                    } else {
+                        ks = wkey[m];
+                        uint32_t nk;
+                        type_of(ks, nk);
+                        kj = __shfl_sync(FULL, nk, e_sel & 7);
+                        ty = wtype[e_sel];
+                    }
+                    // even lanes compute s's addresses, odd lanes j's
+                    int tk, xk, yk, zk;
+                    split32((lane & 1) ? kj : ks, tk, xk, yk, zk);
+                    const int wg = word_of(geo, tk, xk, yk, zk);  // word within the replica
+                    if (lane < 2) {
+                        const uint32_t flip = ((uint32_t)SP_V ^ (ty >= 3 ? (uint32_t)SP_H : (uint32_t)SP_O))
+                                              << occ_shift(xk);
+                        const int wl = CL ? wg - slab_word0 : wg;
+                        if (!CL || (unsigned)wl < (unsigned)slab_words) {
+                            atomicXor(S.occ + wl, flip);
+                        } else {
+                            const uint32_t zm = S.zmap[zk];
+                            red_peer_xor(peer_addr(S.occ + word_of(geo, tk, xk, yk, (int)((zm >> 8) & 1023u)), zm & 255u),
+                                         flip);
                         }
                     }
-                    __syncwarp();
-                    if (nch <= 2) {  // the moved vacancy's lanes follow it (or drop a handed-off slot)
-                        const uint32_t nk = owned ? key32(j.t2, j.jx, j.jy, j.jz) : 0xffffffffu;
-                        if ((lane >> 3) == m) kc0 = nk;
-                        if (4 + (lane >> 3) == m) kc1 = nk;
-                    }
+                    const bool own_lane = (unsigned)(xk - lo0) < (unsigned)ex && (unsigned)(yk - lo1) < (unsigned)ey &&
+                                          (unsigned)(zk - lo2) < (unsigned)ez;
+                    const bool owned = __shfl_sync(FULL, (int)own_lane, 1) != 0;
+                    flush();  // the exchange before
                     {
-                        // the fragments whose totals changed: owners of the vacancies next to the
-                        // two changed sites (lanes 0-7 look around s, 8-15 around j; 16-31 repeat
-                        // them without storing, so that no branch splits the warp and the probe's
-                        // loads overlap those of the rate types)
-                        const int pl = lane & 15;
-                        const int bt = pl < 8 ? t : j.t2;
-                        const int bx = pl < 8 ? x : j.jx, by = pl < 8 ? y : j.jy, bz = pl < 8 ? z : j.jz;
-                        const NbSite c = nb_site(sh, geo, bt, bx, by, bz, pl & 7);
-                        const bool vac = site_code(geo, S.occ, c.t2, c.jx, c.jy, c.jz) == SP_V;
-                        const int g = owner_of(geo, S.frag_of_c, c.jx, c.jy, c.jz);
-                        compute_types();
-                        if (lane < 16 && vac && g != fid) {
-                            S.dirty[g] = 1;
-                            if constexpr (CL > 1) st_peer8(peer_addr(S.dirty + g, peer), 1);
+                        // displacement in units of a/2 along this lane's axis
+                        const int ts = (int)(ks >> 30), tj = (int)(kj >> 30);
+                        const uint32_t e = __shfl_sync(FULL, dirs, e_sel & 7) >> (10 * ts);
+                        const int ax = lane & 3;  // 0..2
+                        pend_m = m;
+                        pend_at = wg * 16 + (xk & 15);
+                        pend_d = 2 * ((int)((e >> (2 + 2 * ax)) & 3u) - 1) + (tj == ax) - (ts == ax);
+                        if (tracer) {
+                            const int lin = ((tk * geo.L2 + zk) * geo.L1 + yk) * geo.L0 + xk;
+                            const int ls = __shfl_sync(FULL, lin, 0), lj = __shfl_sync(FULL, lin, 1);
+                            if (lane >= 8 && lane < 11) {
+                                trj = 3 * (D.site_off + lj) + ax;
+                                trs = 3 * (D.site_off + ls) + ax;
+                                trv = __ldcg(tracer + trj) - pend_d;
+                            }
                         }
+                    }
+                    __syncwarp();  // the exchanged codes are in place
+                    const uint32_t nk = owned ? kj : DEAD;
+                    if (nch <= 2) {  // the moved vacancy's lanes follow it (or drop a handed-off slot)
+                        if ((lane >> 3) == m) kc0 = nk;
+                        if ((lane >> 3) + 4 == m) kc1 = nk;
+                    } else {
+                        if (lane == 0) wkey[m] = nk;
+                        __syncwarp();
+                    }
+                    my_hand += !owned;
+                    {
+                        // the fragments whose totals changed: owners of the vacancies next to the two
+                        // changed sites (lanes 0-7 look around s, 8-15 around j; 16-31 repeat them
+                        // without marking, so that no branch splits the warp)
+                        // (with up to two vacancies lanes 16-31, which hold no event, do it beside the
+                        // rate types of lanes 0-15)
+                        const uint32_t pk = (lane & 8) ? kj : ks;
+                        NbSite c;
+                        int code;
+                        if (n <= 2) {
+                            const bool dead = kc0 == DEAD;
+                            const uint32_t k = lane < 16 ? (dead ? key0 : kc0) : pk;
+                            c = nb_site(geo, dirs, k);
+                            nk0 = key32(c.t2, c.x, c.y, c.z);
+                            code = site_code<CL>(S, geo, c.t2, c.x, c.y, c.z);
+                            ty0 = lane < 16 && !dead ? code * 3 + c.dz1 : NO_EVENT;
+                            if (lane < 16) code = SP_O;
+                        } else {
+                            c = nb_site(geo, dirs, pk);
+                            code = site_code<CL>(S, geo, c.t2, c.x, c.y, c.z);
+                            if (lane >= 16) code = SP_O;
+                            compute_types();
+                        }
+                        if (code == SP_V)
+                            mark_owner<PREC, CL>(S, geo, c.x, c.y, c.z, lf, key32(c.t2, c.x, c.y, c.z) == kj);
                     }
                     clock = nclock;
                     ++i;
                 }
-                // surviving vacancies stay linked to this fragment, in slot order (up to 32
-                // slots, each lane links its own slot to the next live one)
-                int head = -1;
-                if (n <= 32) {
-                    const int v = lane < n ? wslot[lane] : -1;
-                    const unsigned live = __ballot_sync(FULL, v >= 0);
-                    const unsigned later = live & ~((2u << lane) - 1u);
-                    const int vn = __shfl_sync(FULL, v, later ? __ffs(later) - 1 : 0);
-                    const int hv = __shfl_sync(FULL, v, live ? __ffs(live) - 1 : 0);
-                    if (v >= 0) {
-                        S.next[v] = (int16_t)(later ? vn : -1);
-                        if constexpr (CL > 1) st_peer16(peer_addr(S.next + v, peer), (int16_t)(later ? vn : -1));
-                    }
-                    head = live ? hv : -1;
-                }
+                flush();
                 if (lane == 0) {
-                    if (n > 32) {
-                        for (int m = n - 1; m >= 0; --m) {
-                            const int v = wslot[m];
-                            if (v < 0) continue;
-                            S.next[v] = (int16_t)head;
-                            if constexpr (CL > 1) st_peer16(peer_addr(S.next + v, peer), (int16_t)head);
-                            head = v;
-                        }
-                    }
-                    S.head[fid] = head;
-                    S.S[fid] = tot;
-                    S.dirty[fid] = 0;
-                    if constexpr (CL > 1) {
-                        st_peer(peer_addr(S.head + fid, peer), head);
-                        st_peer64(peer_addr(S.S + fid, peer), tot);
-                        st_peer8(peer_addr(S.dirty + fid, peer), 0);
-                    }
+                    lim[lf] = tot == 0ull ? Lim::EMPTY : limit_of<PREC>(tot, lim32, tau);
                     my_hops += i;
+                    if (scan) S.stale[lf] = 0;
                 }
-                __syncwarp();
+                if (i > 0 || scan) {  // the fragment's list, in slot order
+                    if (nch <= 2) {
+                        const uint32_t k = slot_key();
+                        if (lane < KSLOTS) sl[lane] = k;
+                    } else if (lane == 0) {
+                        sl[0] = UNLISTED;
+                    }
+                }
+                if (nact <= NW) break;  // every listed fragment has its warp
+                if (lane == 0) a = atomicAdd(&sh.next_act[par], 1);
+                a = __shfl_sync(FULL, a, 0);
             }
-            if constexpr (CL > 1) cluster_sync();  // both copies hold every write of the phase
-            else __syncthreads();
+            if constexpr (CL) {
+                // every write of the phase, local and remote, is visible after the wait; between
+                // arrival and wait the next phase's first draws
+                __syncwarp();
+                cluster_arrive();
+                if (p < 7)
+                    draw_colour((int)((wperm >> (4 * (p + 1))) & 15u), wk, par ^ 1);
+                else if (wk + 1 < windows && ((wk + 1) & 63) != 0)  // the next window's order is known
+                    draw_colour((int)(sh.perms[(wk + 1) & 63] & 15u), wk + 1, par ^ 1);
+                __syncwarp();
+                cluster_wait();
+                __syncthreads();  // the draws of this CTA's other threads, made after their arrival
+            } else {
+                __syncthreads();
+            }
         }
     }
 
-    // ---- stage out (the first CTA of a cluster): occupancy by a TMA bulk store, records to the fragment lists
-    if (tid == 0 && rank == 0) {
+    // ---- stage out: occupancy by TMA bulk stores; each fragment's records from
+    // where they lay to tmp, and back to its list once every CTA has read its own
+    if (tid == 0) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        char* dst = reinterpret_cast<char*>(occ + D.occ_word_off);
-        for (uint32_t off = 0; off < occ_bytes; off += BULK_CHUNK) {
-            const uint32_t nb = min(BULK_CHUNK, occ_bytes - off);
-            bulk_s2g(dst + off, S.occ + off / 4, nb);
-        }
+        char* dst = reinterpret_cast<char*>(occ_g);
+        for (uint32_t off = 0; off < occ_bytes; off += BULK_CHUNK)
+            bulk_s2g(dst + off, S.occ + off / 4, min(BULK_CHUNK, occ_bytes - off));
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     }
-    for (int f = tid; f < (rank == 0 ? nfrag : 0); f += blockDim.x) {
-        const int64_t g = D.frag_base + f;
-        int k = 0;
-        for (int v = S.head[f]; v >= 0; v = S.next[v], ++k) {
-            if (k >= cap) {
-                atomicOr(status, STATUS_OVERFLOW);
-                break;
-            }
+    VacRec* const tmp_r = tmp + (D.tmp_off + (int64_t)fzb * D.nf[1] * D.nf[0]) * cap;
+    for (int f = warp; f < nfl; f += NW) {
+        const uint2 bx = S.box[f];
+        int n = gather(S, geo, wkey, cap, lane, (int)(bx.x & 1023u), (int)((bx.x >> 10) & 1023u), (int)(bx.x >> 20),
+                       (int)(bx.y & 1023u) + 1, (int)((bx.y >> 10) & 1023u) + 1, (int)(bx.y >> 20) + 1);
+        if (n > cap) {
+            if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
+            n = cap;
+        }
+        for (int k = lane; k < n; k += 32) {
+            const uint32_t key = wkey[k];
+            const VacRec* src = recs_r + min(__ldcg(vmap_r + map_index(geo, key)), rec_lim - 1);
             int t, x, y, z;
-            split32(S.key[v], t, x, y, z);
+            split32(key, t, x, y, z);
             VacRec rr;
             rr.key = make_key(t, x, y, z);
-            rr.d[0] = S.d[3 * v];
-            rr.d[1] = S.d[3 * v + 1];
-            rr.d[2] = S.d[3 * v + 2];
-            rr.id = S.id[v];
-            recs[g * cap + k] = rr;
+            rr.d[0] = __ldcg(&src->d[0]);
+            rr.d[1] = __ldcg(&src->d[1]);
+            rr.d[2] = __ldcg(&src->d[2]);
+            rr.id = __ldcg(&src->id);
+            tmp_r[(int64_t)f * cap + k] = rr;
         }
-        counts[g] = k;
-        rc.tot[g] = S.S[f];
-        rc.dirty[g] = S.dirty[f];
+        __syncwarp();
+        if (lane == 0) {
+            counts[frag0 + f] = n;
+            rc.lim[frag0 + f] = (uint64_t)lim[f];
+        }
     }
-    atomicAdd(&sh.hops, my_hops);
-    atomicAdd(&sh.hand, my_hand);
-    __syncthreads();
+    if (my_hand && lane == 0) atomicAdd(&sh.hand, my_hand);
+    if (my_hops) atomicAdd(&sh.hops, my_hops);
+    if constexpr (CL) cluster_sync();
+    else __syncthreads();
+    for (int f = warp; f < nfl; f += NW) {
+        const int n = __ldcg(counts + frag0 + f);
+        for (int k = lane; k < n; k += 32) {  // the thread that wrote the copy
+            recs[(frag0 + f) * cap + k] = tmp_r[(int64_t)f * cap + k];
+        }
+    }
     if (tid == 0) {
-        if (sh.hops) atomicAdd(stats + 2 * r, sh.hops);
-        if (sh.hand) atomicAdd(stats + 2 * r + 1, sh.hand);
-        if (rank == 0) {
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-            rc.valid[r] = 1;
-        }
+        if (sh.hops) atomicAdd(stats + 2 * rep, sh.hops);
+        if (sh.hand) atomicAdd(stats + 2 * rep + 1, sh.hand);
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
-    if constexpr (CL > 1) cluster_sync();  // no CTA leaves while its peer may still address it
+    if constexpr (CL) cluster_sync();  // no CTA leaves while a peer may still address it
+    if (tid == 0 && me == 0) rc.valid[rep] = 1;
 }
 
-// ---------------------------------------------------------------- cluster-resident kernel
-// One replica too large for one SM's shared memory, held by a thread-block
-// cluster of P.ncta CTAs (up to 16): CTA c holds the z-slab of fragment layers
-// [P.fz0[c], P.fz0[c+1]) -- its occupancy planes, its vacancies (a pool of
-// P.vcap slots with a free-slot stack) and its fragments' lists, totals and
-// dirty flags.  Every CTA has the same layout, so a peer's copy of an array is
-// addressed through distributed shared memory (mapa) at the same offset.  The
-// colour phases are those of the replica-resident kernel, with a cluster
-// barrier between phases:
-//   - a neighbour site in another slab is read from that CTA's shared memory
-//     (ld.shared::cluster), an exchange there is an atomic XOR on it
-//     (red.shared::cluster);
-//   - a vacancy leaving the slab is written into the owning CTA's inbox
-//     (double-buffered by phase parity; the slot taken with a remote atomic
-//     add) and its slot returns to the free stack; at the start of the next
-//     phase the owner moves its inbox into free slots and onto the fragments'
-//     lists (the receiving fragment has another colour, so it does not run in
-//     the phase that filled the inbox);
-//   - dirty marks on a peer's fragments are remote byte stores.
-// Fragments of one colour never touch each other's sites, so the result is
-// the replica-resident kernel's (and the oracle's) bit for bit.
-
-struct InboxRec {
-    uint32_t key;
-    int32_t d[3];
-    uint32_t id;
-    int32_t lf;  // the receiving CTA's local fragment index
-};
-static_assert(sizeof(InboxRec) == 24, "inbox record");
-
-struct CShared {
-    RepDesc D;
-    NbEntry nb[3][8];
-    ClusterPlan P;
-    uint32_t perms[64];
-    int zbeg[CLUSTER_MAX_CTAS + 1];  // first z cell of CTA c's slab
-    int nact;
-    int next_act;
-    int inbox_n[2];
-    int free_top;
-    int pool_n;
-    int cached;  // the fragment totals of the last call are valid
-    unsigned long long hops, hand;
-};
-
-struct CLayout {
-    uint32_t* occ;       // [zs][L1][RW][3], the global layout of the slab's z cells
-    uint32_t* key;       // vacancy pool [vcap]
-    int32_t* d;
-    uint32_t* id;
-    int16_t* next;
-    int16_t* fstack;     // free pool slots
-    int32_t* head;       // local fragments [nfl]
-    unsigned long long* S;
-    uint8_t* dirty;
-    int32_t* act;        // screened local fragments, with their first draws
-    uint64_t* act_xs;
-    float* act_E;
-    int16_t* wslot;      // per warp
-    int8_t* wtype;
-    InboxRec* inbox;     // [2][icap]
-    uint16_t* frag_of_c; // cell -> global fragment coordinate: x cells, then y, then z
-    uint32_t* zmap;      // z cell -> its CTA | z within that CTA's slab << 8 | fragment layer within it << 18
-    uint64_t* pre_xs;    // the next phase's first draws by screen index: selection words of events 0, 1
-    float* pre_E;        // and their exponential variates
-};
-
-__host__ __device__ inline size_t cluster_layout_bytes(const RepDesc& D, const ClusterPlan& P, int cap, int nwarps,
-                                                       size_t* off /* 19 offsets or null */)
+// `nc` CTAs of one z-slab of fragment layers each, or false where they do not fit
+static bool cluster_plan_for(const RepDesc& D, int cap, int pre_ev, int prec, int nc, ClusterPlan* out)
 {
-    const size_t words = (size_t)3 * P.zs * D.L[1] * D.row_words;
-    const size_t sz[19] = {
-        words * 4,                          // 0 occupancy slab
-        (size_t)P.vcap * 4,                 // 1 keys
-        (size_t)P.vcap * 12,                // 2 displacements
-        (size_t)P.vcap * 4,                 // 3 ids
-        (size_t)P.vcap * 2,                 // 4 next links
-        (size_t)P.vcap * 2,                 // 5 free-slot stack
-        (size_t)P.nfl * 4,                  // 6 list heads
-        (size_t)P.nfl * 8,                  // 7 cached totals
-        (size_t)P.nfl,                      // 8 dirty flags
-        (size_t)P.nfl * 4,                  // 9 screened list
-        (size_t)P.nfl * 16,                 // 10 screened: selection words
-        (size_t)P.nfl * 8,                  // 11 screened: variates
-        (size_t)nwarps * cap * 2,           // 12 per-warp slots
-        (size_t)nwarps * cap * 8,           // 13 per-warp event types
-        (size_t)2 * P.icap * sizeof(InboxRec),  // 14 inboxes
-        (size_t)(D.L[0] + D.L[1] + D.L[2]) * 2, // 15 cell -> fragment tables
-        (size_t)D.L[2] * 4,                 // 16 z cell -> CTA, slab z, slab fragment layer
-        (size_t)P.nfl * 16,                 // 17 next phase: selection words of events 0, 1
-        (size_t)P.nfl * 8,                  // 18 next phase: variates
-    };
-    size_t b = 0;
-    for (int k = 0; k < 19; ++k) {
-        if (off) off[k] = b;
-        b += (sz[k] + 15) & ~(size_t)15;
-    }
-    return (b + 127) & ~(size_t)127;
-}
-
-namespace {
-
-__device__ __forceinline__ CLayout ccarve(unsigned char* dyn, const RepDesc& D, const ClusterPlan& P, int cap,
-                                          int nwarps)
-{
-    size_t o[19];
-    cluster_layout_bytes(D, P, cap, nwarps, o);
-    CLayout L;
-    L.occ = reinterpret_cast<uint32_t*>(dyn + o[0]);
-    L.key = reinterpret_cast<uint32_t*>(dyn + o[1]);
-    L.d = reinterpret_cast<int32_t*>(dyn + o[2]);
-    L.id = reinterpret_cast<uint32_t*>(dyn + o[3]);
-    L.next = reinterpret_cast<int16_t*>(dyn + o[4]);
-    L.fstack = reinterpret_cast<int16_t*>(dyn + o[5]);
-    L.head = reinterpret_cast<int32_t*>(dyn + o[6]);
-    L.S = reinterpret_cast<unsigned long long*>(dyn + o[7]);
-    L.dirty = reinterpret_cast<uint8_t*>(dyn + o[8]);
-    L.act = reinterpret_cast<int32_t*>(dyn + o[9]);
-    L.act_xs = reinterpret_cast<uint64_t*>(dyn + o[10]);
-    L.act_E = reinterpret_cast<float*>(dyn + o[11]);
-    L.wslot = reinterpret_cast<int16_t*>(dyn + o[12]);
-    L.wtype = reinterpret_cast<int8_t*>(dyn + o[13]);
-    L.inbox = reinterpret_cast<InboxRec*>(dyn + o[14]);
-    L.frag_of_c = reinterpret_cast<uint16_t*>(dyn + o[15]);
-    L.zmap = reinterpret_cast<uint32_t*>(dyn + o[16]);
-    L.pre_xs = reinterpret_cast<uint64_t*>(dyn + o[17]);
-    L.pre_E = reinterpret_cast<float*>(dyn + o[18]);
-    return L;
-}
-
-__device__ __forceinline__ uint32_t atom_peer_add(uint32_t a, uint32_t v)
-{
-    uint32_t o;
-    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(o) : "r"(a), "r"(v) : "memory");
-    return o;
-}
-
-__device__ __forceinline__ uint32_t cluster_nctas()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-
-// where a site's occupancy word lives: the CTA holding its z, and the word's
-// index in that CTA's slab (every CTA has the same slab layout)
-struct CWord {
-    uint32_t cta;
-    int idx;
-};
-
-__device__ __forceinline__ CWord cword(const CLayout& S, const Geo& g, int t, int x, int y, int z)
-{
-    const uint32_t zm = S.zmap[z];
-    CWord w;
-    w.cta = zm & 255u;
-    w.idx = ((((int)((zm >> 8) & 1023u)) * g.L1 + y) * g.RW + (x >> 4)) * 3 + t;
-    return w;
-}
-
-__device__ __forceinline__ int csite_code(const CLayout& S, const Geo& g, uint32_t me, int t, int x, int y, int z)
-{
-    const CWord w = cword(S, g, t, x, y, z);
-    const uint32_t v = w.cta == me ? S.occ[w.idx] : (uint32_t)ld_peer(peer_addr(S.occ + w.idx, w.cta));
-    return (int)((v >> occ_shift(x)) & 3u);
-}
-
-__device__ __forceinline__ void csite_xor(const CLayout& S, const Geo& g, uint32_t me, int t, int x, int y, int z,
-                                          uint32_t m)
-{
-    const CWord w = cword(S, g, t, x, y, z);
-    if (w.cta == me) atomicXor(S.occ + w.idx, m);
-    else red_peer_xor(peer_addr(S.occ + w.idx, w.cta), m);
-}
-
-__device__ __forceinline__ NbSite cnb_site(const CShared& sh, const Geo& g, int t, int x, int y, int z, int q)
-{
-    const NbEntry nb = sh.nb[t][q];
-    NbSite s;
-    s.t2 = nb.t2;
-    s.jx = wrapc(x + nb.dc[0], g.L0);
-    s.jy = wrapc(y + nb.dc[1], g.L1);
-    s.jz = wrapc(z + nb.dc[2], g.L2);
-    return s;
-}
-
-// owner of cell (x,y,z): its CTA and that CTA's local fragment index
-__device__ __forceinline__ void cowner(const CLayout& S, const Geo& g, int x, int y, int z, uint32_t& cta, int& lf)
-{
-    const int fx = S.frag_of_c[x], fy = S.frag_of_c[g.L0 + y];
-    const uint32_t zm = S.zmap[z];
-    cta = zm & 255u;
-    lf = ((int)(zm >> 18) * g.nf1 + fy) * g.nf0 + fx;
-}
-
-}  // namespace
-
-template <int NT>
-__global__ void __launch_bounds__(NT, 1) k_cluster(const RepDesc* __restrict__ descs,
-                                                   const ClusterPlan* __restrict__ plans, uint64_t windows,
-                                                   uint32_t* occ, VacRec* recs, int32_t* counts, int32_t* tracer,
-                                                   unsigned long long* stats, uint32_t* status, int cap, NbTable nbt,
-                                                   ResCache rc)
-{
-    extern __shared__ __align__(128) unsigned char dyn[];
-    __shared__ CShared sh;
-    const int tid = threadIdx.x;
-    const uint32_t me = cluster_ctarank();
-    const int ci = (int)(blockIdx.x / cluster_nctas());
-    if (tid == 0) {
-        sh.P = plans[ci];
-        sh.D = descs[sh.P.rep];
-        for (int c = 0; c <= sh.P.ncta; ++c) sh.zbeg[c] = frag_start(sh.P.fz0[c], sh.D.base[2], sh.D.rem[2]);
-        sh.nact = 0;
-        sh.next_act = 0;
-        sh.inbox_n[0] = sh.inbox_n[1] = 0;
-        sh.pool_n = 0;
-        sh.hops = 0;
-        sh.hand = 0;
-        sh.cached = rc.valid[sh.P.rep];
-    }
-    if (tid < 24) (&sh.nb[0][0])[tid] = (&nbt.e[0][0])[tid];
-    __syncthreads();
-    const RepDesc& D = sh.D;
-    const ClusterPlan& P = sh.P;
-    const CLayout S = ccarve(dyn, D, P, cap, NT / 32);
-    const Geo geo{D.L[0], D.L[1], D.L[2], D.row_words, D.nf[0], D.nf[1], D.F, D.theta_tau, window_f(D.theta_tau, D.F)};
-    const int fzb = P.fz0[me], fze = P.fz0[me + 1];
-    const int zb = sh.zbeg[me], zl = sh.zbeg[me + 1] - zb;
-    const int nfl_me = (fze - fzb) * D.nf[0] * D.nf[1];
-
-    // ---- stage in: this slab's occupancy (its z cells are contiguous in the
-    // global layout), its vacancies, the lookup tables
-    const int slab_words = zl * D.L[1] * D.row_words * 3;
-    const int64_t slab_off = D.occ_word_off + (int64_t)zb * D.L[1] * D.row_words * 3;
-    for (int k = tid; k < slab_words; k += NT) S.occ[k] = occ[slab_off + k];
-    for (int k = tid; k < D.L[0] + D.L[1] + D.L[2]; k += NT) {
-        const int d = k < D.L[0] ? 0 : (k < D.L[0] + D.L[1] ? 1 : 2);
-        const int c = d == 0 ? k : (d == 1 ? k - D.L[0] : k - D.L[0] - D.L[1]);
-        S.frag_of_c[k] = (uint16_t)frag_of(c, D.base[d], D.rem[d]);
-    }
-    for (int z = tid; z < D.L[2]; z += NT) {
-        const int fz = frag_of(z, D.base[2], D.rem[2]);
-        int c = 0;
-        while (c + 1 < P.ncta && P.fz0[c + 1] <= fz) ++c;
-        S.zmap[z] = (uint32_t)c | ((uint32_t)(z - sh.zbeg[c]) << 8) | ((uint32_t)(fz - P.fz0[c]) << 18);
-    }
-    for (int lf = tid; lf < nfl_me; lf += NT) {
-        const int fid = (fzb * D.nf[1]) * D.nf[0] + lf;  // layers are contiguous in the global order
-        const int64_t g = D.frag_base + fid;
-        const int c = counts[g];
-        int head = -1;
-        for (int k = 0; k < c && k < cap; ++k) {
-            const int v = atomicAdd(&sh.pool_n, 1);
-            if (v >= P.vcap) {
-                atomicOr(status, STATUS_OVERFLOW);
-                break;
-            }
-            const VacRec rr = recs[g * cap + k];
-            int t, x, y, z;
-            split_key(rr.key, t, x, y, z);
-            S.key[v] = key32(t, x, y, z);
-            S.d[3 * v] = rr.d[0];
-            S.d[3 * v + 1] = rr.d[1];
-            S.d[3 * v + 2] = rr.d[2];
-            S.id[v] = rr.id;
-            S.next[v] = (int16_t)head;
-            head = v;
-        }
-        if (c > cap) atomicOr(status, STATUS_OVERFLOW);
-        S.head[lf] = head;
-        S.dirty[lf] = sh.cached ? rc.dirty[g] : 1;
-        S.S[lf] = sh.cached ? rc.tot[g] : 0ull;
-    }
-    __syncthreads();
-    {
-        const int used = min(sh.pool_n, P.vcap);
-        for (int k = tid; k < P.vcap - used; k += NT) S.fstack[k] = (int16_t)(used + k);
-        if (tid == 0) sh.free_top = P.vcap - used;
-    }
-    cluster_sync();  // every slab is in place before any CTA reads a peer's
-
-    const uint64_t hop_k1 = key_word(D.replica, PURPOSE_HOP);
-    const int lane = tid & 31;
-    const int warp = tid >> 5;
-    const unsigned FULL = 0xffffffffu;
-    int16_t* wslot = S.wslot + warp * cap;
-    int8_t* wtype = S.wtype + warp * cap * 8;
-    unsigned long long my_hops = 0, my_hand = 0;
-
-    // the inbox of phase parity b into free slots and onto the fragments' lists
-    auto drain = [&](int b) {
-        const int n = min(sh.inbox_n[b], P.icap);
-        if (sh.inbox_n[b] > P.icap && tid == 0) atomicOr(status, STATUS_OVERFLOW);
-        for (int e = tid; e < n; e += NT) {
-            const InboxRec r = S.inbox[b * P.icap + e];
-            const int top = atomicSub(&sh.free_top, 1) - 1;
-            if (top < 0) {
-                atomicOr(status, STATUS_OVERFLOW);
-                continue;
-            }
-            const int v = S.fstack[top];
-            S.key[v] = r.key;
-            S.d[3 * v] = r.d[0];
-            S.d[3 * v + 1] = r.d[1];
-            S.d[3 * v + 2] = r.d[2];
-            S.id[v] = r.id;
-            S.next[v] = (int16_t)atomicExch(S.head + r.lf, v);
-            S.dirty[r.lf] = 1;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            sh.inbox_n[b] = 0;
-            if (sh.free_top < 0) sh.free_top = 0;
-        }
-    };
-
-    // this slab's fragments of a colour: count per dimension, parity bits, first
-    // fragment layer; and the coordinates of the colour's local fragment l
-    auto colour_geo = [&](int colour, int cnt[2], int bit[3], int& lz0) -> int {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) bit[d] = (colour >> d) & 1;
-#pragma unroll
-        for (int d = 0; d < 2; ++d) cnt[d] = D.nf[d] == 1 ? (bit[d] == 0 ? 1 : 0) : D.nf[d] / 2;
-        lz0 = D.nf[2] == 1 ? 0 : (fzb + ((fzb & 1) != bit[2] ? 1 : 0));
-        const int nlz = D.nf[2] == 1 ? (bit[2] == 0 ? 1 : 0) : (fze > lz0 ? (fze - lz0 + 1) / 2 : 0);
-        return cnt[0] * cnt[1] * nlz;
-    };
-    auto frag_coords = [&](int l, const int cnt[2], const int bit[3], int lz0, int& f0, int& f1, int& f2) {
-        f0 = l % cnt[0];
-        f1 = (l / cnt[0]) % cnt[1];
-        f2 = l / (cnt[0] * cnt[1]);
-        f0 = D.nf[0] == 1 ? 0 : 2 * f0 + bit[0];
-        f1 = D.nf[1] == 1 ? 0 : 2 * f1 + bit[1];
-        f2 = lz0 + 2 * f2;
-    };
-    bool pre_valid = false;  // the phase's first draws were computed at the end of the last one
-
-    uint32_t ph = 0;
-    for (uint64_t wk = 0; wk < windows; ++wk) {
-        const uint64_t w = D.window + wk;
-        if ((wk & 63) == 0) {
-            if (tid < 64 && wk + tid < windows) sh.perms[tid] = colour_perm_packed(D.seed, D.replica, w + tid);
-            __syncthreads();
-        }
-        const uint32_t wperm = sh.perms[wk & 63];
-        for (int p = 0; p < 8; ++p, ++ph) {
-            if (ph > 0) drain((ph - 1) & 1);
-            const int colour = (int)((wperm >> (4 * p)) & 15u);
-            int cnt[2], bit[3], lz0;
-            const int ncls = colour_geo(colour, cnt, bit, lz0);
-            if (tid == 0) {
-                sh.nact = 0;
-                sh.next_act = 0;
-            }
-            __syncthreads();
-            // ---- screen: one thread per local fragment of the colour
-            for (int l = tid; l < ncls; l += NT) {
-                int f0, f1, f2;
-                frag_coords(l, cnt, bit, lz0, f0, f1, f2);
-                const int lf = ((f2 - fzb) * D.nf[1] + f1) * D.nf[0] + f0;
-                const int fid = (f2 * D.nf[1] + f1) * D.nf[0] + f0;
-                if (S.head[lf] < 0) continue;
-                const bool dirty = S.dirty[lf] != 0;
-                const unsigned long long tot = S.S[lf];
-                if (!dirty && tot == 0ull) continue;
-                float E0, E1 = 0.f;
-                uint64_t xs0, xs1;
-                U64x4 blk{};
-                if (pre_valid) {
-                    E0 = S.pre_E[2 * l];
-                    E1 = S.pre_E[2 * l + 1];
-                    xs0 = S.pre_xs[2 * l];
-                    xs1 = S.pre_xs[2 * l + 1];
-                } else {
-                    blk = philox4x64((uint64_t)fid, w, 0, 0, D.seed, hop_k1);
-                    E0 = neglog32(blk.x[0]);
-                    xs0 = blk.x[1];
-                    xs1 = blk.x[3];
-                }
-                bool active = dirty;
-                if (!active) {
-                    const float ratio = __fdiv_rn(E0, __ull2float_rn(tot));
-                    active = !(ratio > geo.theta_f);  // 0 + 2^F ratio <= theta
-                }
-                if (active) {
-                    const int a = atomicAdd(&sh.nact, 1);
-                    S.act[a] = f0 | (f1 << 10) | (f2 << 20);  // fragment coordinates (< 1024 each)
-                    S.act_E[2 * a] = E0;
-                    S.act_E[2 * a + 1] = pre_valid ? E1 : neglog32(blk.x[2]);
-                    S.act_xs[2 * a] = xs0;
-                    S.act_xs[2 * a + 1] = xs1;
-                }
-            }
-            __syncthreads();
-            // ---- run: one warp per listed fragment
-            const int nact = sh.nact;
-            for (;;) {
-                int a = 0;
-                if (lane == 0) a = atomicAdd(&sh.next_act, 1);
-                a = __shfl_sync(FULL, a, 0);
-                if (a >= nact) break;
-                const int fxyz = S.act[a];
-                const int fx = fxyz & 1023, fy = (fxyz >> 10) & 1023, fz = fxyz >> 20;
-                const int lf = ((fz - fzb) * D.nf[1] + fy) * D.nf[0] + fx;
-                const int fid = (fz * D.nf[1] + fy) * D.nf[0] + fx;
-                const int lo0 = frag_start(fx, D.base[0], D.rem[0]), hi0 = frag_start(fx + 1, D.base[0], D.rem[0]);
-                const int lo1 = frag_start(fy, D.base[1], D.rem[1]), hi1 = frag_start(fy + 1, D.base[1], D.rem[1]);
-                const int lo2 = frag_start(fz, D.base[2], D.rem[2]), hi2 = frag_start(fz + 1, D.base[2], D.rem[2]);
-                // slots: the fragment's vacancies in ascending site order
-                int n = 0;
-                if (lane == 0) {
-                    for (int v = S.head[lf]; v >= 0; v = S.next[v]) {
-                        if (n >= cap) {
-                            atomicOr(status, STATUS_OVERFLOW);
-                            break;
-                        }
-                        wslot[n++] = (int16_t)v;
-                    }
-                }
-                n = __shfl_sync(FULL, n, 0);
-                __syncwarp();
-                // a list that received no vacancy since its last visit is still in site order
-                bool ordered = false;
-                uint32_t kk = 0xffffffffu;
-                if (n <= 32) {  // rank by site (sites are distinct), unless already in order
-                    const int vk = lane < n ? wslot[lane] : -1;
-                    kk = lane < n ? S.key[vk] : 0xffffffffu;
-                    const uint32_t kprev = __shfl_up_sync(FULL, kk, 1);
-                    ordered = __ballot_sync(FULL, lane > 0 && lane < n && kprev > kk) == 0u;
-                    if (!ordered) {
-                        int rnk = 0;
-                        for (int q = 0; q < n; ++q) rnk += __shfl_sync(FULL, kk, q) < kk ? 1 : 0;
-                        __syncwarp();
-                        if (lane < n) wslot[rnk] = (int16_t)vk;
-                    }
-                } else if (lane == 0) {
-                    for (int k = 1; k < n; ++k) {
-                        const int v = wslot[k];
-                        const uint32_t kv = S.key[v];
-                        int m = k;
-                        while (m > 0 && S.key[wslot[m - 1]] > kv) {
-                            wslot[m] = wslot[m - 1];
-                            --m;
-                        }
-                        wslot[m] = (int16_t)v;
-                    }
-                }
-                __syncwarp();
-                const int nch = (n + 3) >> 2;
-                // up to two chunks: each lane keeps its two slots' site keys in registers
-                // (0xffffffff: no slot, or handed off), as in the replica-resident kernel
-                uint32_t kc0 = 0xffffffffu, kc1 = 0xffffffffu;
-                if (nch <= 2) {
-                    const int m0 = lane >> 3, m1 = 4 + (lane >> 3);
-                    if (ordered) {  // lane m holds slot m's key
-                        const uint32_t a0 = __shfl_sync(FULL, kk, m0), a1 = __shfl_sync(FULL, kk, m1);
-                        if (m0 < n) kc0 = a0;
-                        if (m1 < n) kc1 = a1;
-                    } else {
-                        if (m0 < n) kc0 = S.key[wslot[m0]];
-                        if (m1 < n) kc1 = S.key[wslot[m1]];
-                    }
-                }
-                auto type_of = [&](uint32_t k, int q) -> int {
-                    int t, x, y, z;
-                    split32(k, t, x, y, z);
-                    const NbEntry nbe = sh.nb[t][q];
-                    const int code = csite_code(S, geo, me, nbe.t2, wrapc(x + nbe.dc[0], geo.L0),
-                                                wrapc(y + nbe.dc[1], geo.L1), wrapc(z + nbe.dc[2], geo.L2));
-                    return code == SP_V ? -1 : code * 3 + nbe.d[2] + 1;
-                };
-                int ty0 = -1, ty1 = -1;  // up to two chunks: rate types of events lane and 32 + lane
-                auto compute_types = [&]() {
-                    if (nch <= 2) {
-                        ty0 = kc0 != 0xffffffffu ? type_of(kc0, lane & 7) : -1;
-                        ty1 = (nch == 2 && kc1 != 0xffffffffu) ? type_of(kc1, lane & 7) : -1;
-                    } else {
-                        for (int c = 0; c < nch; ++c) {
-                            const int e = c * 32 + lane, m = e >> 3;
-                            int ty = -1;
-                            if (m < n && wslot[m] >= 0) ty = type_of(S.key[wslot[m]], e & 7);
-                            wtype[e] = (int8_t)ty;
-                        }
-                    }
-                    __syncwarp();
-                };
-                compute_types();
-
-                double clock = 0.0;
-                uint64_t i = 0, batch = ~0ull;
-                uint64_t xs_even = 0, xs_odd = 0;
-                float E_even = 0.f, E_odd = 0.f;
-                unsigned long long tot = 0;
-                for (;;) {
-                    // exact total (order-free integer sum) and, for up to two chunks, the
-                    // inclusive prefixes the selection needs
-                    unsigned long long inc0 = 0, inc1 = 0;
-                    if (nch <= 2) {
-                        const int t0 = ty0;
-                        inc0 = t0 < 0 ? 0ull : (unsigned long long)D.q[t0];
-#pragma unroll
-                        for (int off = 1; off < 32; off <<= 1) {
-                            const unsigned long long t2 = __shfl_up_sync(FULL, inc0, off);
-                            if (lane >= off) inc0 += t2;
-                        }
-                        tot = __shfl_sync(FULL, inc0, 31);
-                        if (nch == 2) {
-                            const int t1 = ty1;
-                            inc1 = t1 < 0 ? 0ull : (unsigned long long)D.q[t1];
-#pragma unroll
-                            for (int off = 1; off < 32; off <<= 1) {
-                                const unsigned long long t2 = __shfl_up_sync(FULL, inc1, off);
-                                if (lane >= off) inc1 += t2;
-                            }
-                            inc1 += tot;
-                            tot = __shfl_sync(FULL, inc1, 31);
-                        }
-                    } else {
-                        unsigned long long part = 0;
-                        for (int c = 0; c < nch; ++c) {
-                            const int ty = wtype[c * 32 + lane];
-                            part += ty < 0 ? 0ull : (unsigned long long)D.q[ty];
-                        }
-#pragma unroll
-                        for (int off = 16; off; off >>= 1) part += __shfl_xor_sync(FULL, part, off);
-                        tot = part;
-                    }
-                    if (tot == 0ull) break;
-                    if (i >= MAX_EVENTS_PER_PHASE) {
-                        if (lane == 0) atomicOr(status, STATUS_EVENT_LIMIT);
-                        break;
-                    }
-                    uint64_t xs;
-                    float E;
-                    if (i < 2) {
-                        xs = S.act_xs[2 * a + (int)i];
-                        E = S.act_E[2 * a + (int)i];
-                    } else {
-                        const uint64_t k = i - 2;
-                        if ((k >> 6) != batch) {
-                            batch = k >> 6;
-                            const U64x4 blk =
-                                philox4x64((uint64_t)fid, w, 1 + 32 * batch + lane, 0, D.seed, hop_k1);
-                            xs_even = blk.x[1];
-                            xs_odd = blk.x[3];
-                            E_even = neglog32(blk.x[0]);
-                            E_odd = neglog32(blk.x[2]);
-                        }
-                        const int src = (int)((k >> 1) & 31);
-                        const bool odd = (k & 1) != 0;
-                        xs = __shfl_sync(FULL, odd ? xs_odd : xs_even, src);
-                        E = __shfl_sync(FULL, odd ? E_odd : E_even, src);
-                    }
-                    const float ratio = __fdiv_rn(E, __ull2float_rn(tot));
-                    const double nclock = __dadd_rn(clock, scale_pow2((double)ratio, geo.F));
-                    const bool past = i == 0 ? ratio > geo.theta_f : nclock > geo.theta;  // the first: clock 0
-                    // up to two chunks: the selection (no side effects) before the clock test,
-                    // so that its shuffles overlap the clock's FP64 chain; a break discards it
-                    const unsigned long long target = __umul64hi(xs, tot);
-                    int e_sel = -1;
-                    uint32_t ksel = 0u;
-                    int tsel = -1;
-                    if (nch <= 2) {
-                        unsigned bal = __ballot_sync(FULL, inc0 > target);
-                        if (bal) {
-                            e_sel = __ffs(bal) - 1;
-                        } else {
-                            bal = __ballot_sync(FULL, inc1 > target);
-                            if (bal && nch == 2) e_sel = 32 + __ffs(bal) - 1;
-                        }
-                        const int ms = e_sel >> 3;  // the slot's site key and the event's type
-                        ksel = __shfl_sync(FULL, ms < 4 ? kc0 : kc1, (ms & 3) << 3);
-                        tsel = __shfl_sync(FULL, e_sel < 32 ? ty0 : ty1, e_sel & 31);
-                    }
-                    if (past) break;
-                    if (nch > 2) {
-                        unsigned long long carry = 0;
-                        for (int c = 0; c < nch; ++c) {
-                            const int ty = wtype[c * 32 + lane];
-                            unsigned long long inc = ty < 0 ? 0ull : (unsigned long long)D.q[ty];
-#pragma unroll
-                            for (int off = 1; off < 32; off <<= 1) {
-                                const unsigned long long t2 = __shfl_up_sync(FULL, inc, off);
-                                if (lane >= off) inc += t2;
-                            }
-                            inc += carry;
-                            const unsigned bal = __ballot_sync(FULL, inc > target);
-                            if (bal) {
-                                e_sel = c * 32 + __ffs(bal) - 1;
-                                break;
-                            }
-                            carry = __shfl_sync(FULL, inc, 31);
-                        }
-                    }
-                    if (e_sel < 0) {  // cannot happen: the target lies below the total
-                        if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
-                        break;
-                    }
-                    const int m = e_sel >> 3, qd = e_sel & 7;
-                    int t, x, y, z;
-                    split32(nch <= 2 ? ksel : S.key[wslot[m]], t, x, y, z);
-                    const NbEntry nb = sh.nb[t][qd];
-                    const NbSite j = cnb_site(sh, geo, t, x, y, z, qd);
-                    const bool owned = j.jx >= lo0 && j.jx < hi0 && j.jy >= lo1 && j.jy < hi1 && j.jz >= lo2 &&
-                                       j.jz < hi2;
-                    if (lane == 0) {  // apply the exchange
-                        const int v = wslot[m];
-                        const uint32_t ion = (uint32_t)((nch <= 2 ? tsel : (int)wtype[e_sel]) / 3);
-                        csite_xor(S, geo, me, t, x, y, z, ((uint32_t)SP_V ^ ion) << occ_shift(x));
-                        csite_xor(S, geo, me, j.t2, j.jx, j.jy, j.jz, (ion ^ (uint32_t)SP_V) << occ_shift(j.jx));
-                        const int d0 = S.d[3 * v] + nb.d[0], d1 = S.d[3 * v + 1] + nb.d[1],
-                                  d2 = S.d[3 * v + 2] + nb.d[2];
-                        if (tracer) {
-                            const int64_t s_lin = (((int64_t)t * D.L[2] + z) * D.L[1] + y) * D.L[0] + x;
-                            const int64_t j_lin = (((int64_t)j.t2 * D.L[2] + j.jz) * D.L[1] + j.jy) * D.L[0] + j.jx;
-                            int32_t* ts = tracer + 3 * (D.site_off + s_lin);
-                            int32_t* tj = tracer + 3 * (D.site_off + j_lin);
-                            ts[0] = tj[0] - nb.d[0];
-                            ts[1] = tj[1] - nb.d[1];
-                            ts[2] = tj[2] - nb.d[2];
-                            tj[0] = tj[1] = tj[2] = 0;
-                        }
-                        const uint32_t jk = key32(j.t2, j.jx, j.jy, j.jz);
-                        if (owned) {
-                            S.d[3 * v] = d0;
-                            S.d[3 * v + 1] = d1;
-                            S.d[3 * v + 2] = d2;
-                            S.key[v] = jk;
-                        } else {
-                            wslot[m] = -1;
-                            uint32_t o2;
-                            int lf2;
-                            cowner(S, geo, j.jx, j.jy, j.jz, o2, lf2);
-                            if (o2 == me) {  // another fragment of this slab: onto its list
-                                S.d[3 * v] = d0;
-                                S.d[3 * v + 1] = d1;
-                                S.d[3 * v + 2] = d2;
-                                S.key[v] = jk;
-                                S.next[v] = (int16_t)atomicExch(S.head + lf2, v);
-                            } else {  // another slab: into its inbox, the slot back to the free stack
-                                const int bidx = (int)(ph & 1u);
-                                const uint32_t e =
-                                    atom_peer_add(peer_addr(&sh.inbox_n[bidx], o2), 1u);
-                                if ((int)e < P.icap) {
-                                    const uint32_t base = peer_addr(S.inbox + bidx * P.icap + (int)e, o2);
-                                    st_peer(base, jk);
-                                    st_peer(base + 4, d0);
-                                    st_peer(base + 8, d1);
-                                    st_peer(base + 12, d2);
-                                    st_peer(base + 16, S.id[v]);
-                                    st_peer(base + 20, lf2);
-                                } else {
-                                    atomicOr(status, STATUS_OVERFLOW);
-                                }
-                                S.fstack[atomicAdd(&sh.free_top, 1)] = (int16_t)v;
-                            }
-                            ++my_hand;
-                        }
-                    }
-                    __syncwarp();
-                    if (nch <= 2) {  // the moved vacancy's lanes follow it (or drop a handed-off slot)
-                        const uint32_t nk = owned ? key32(j.t2, j.jx, j.jy, j.jz) : 0xffffffffu;
-                        if ((lane >> 3) == m) kc0 = nk;
-                        if (4 + (lane >> 3) == m) kc1 = nk;
-                    }
-                    {
-                        // the fragments whose totals changed: owners of the vacancies next to the
-                        // two changed sites (lanes 0-7 look around s, 8-15 around j; 16-31 repeat
-                        // them without storing, so that no branch splits the warp)
-                        const int pl = lane & 15;
-                        const int bt = pl < 8 ? t : j.t2;
-                        const int bx = pl < 8 ? x : j.jx, by = pl < 8 ? y : j.jy, bz = pl < 8 ? z : j.jz;
-                        const NbSite c = cnb_site(sh, geo, bt, bx, by, bz, pl & 7);
-                        const bool vac = csite_code(S, geo, me, c.t2, c.jx, c.jy, c.jz) == SP_V;
-                        uint32_t oc;
-                        int lc;
-                        cowner(S, geo, c.jx, c.jy, c.jz, oc, lc);
-                        compute_types();
-                        if (lane < 16 && vac) {
-                            if (oc == me) {
-                                if (lc != lf) S.dirty[lc] = 1;
-                            } else {
-                                st_peer8(peer_addr(S.dirty + lc, oc), 1);
-                            }
-                        }
-                    }
-                    clock = nclock;
-                    ++i;
-                }
-                // surviving vacancies stay linked to this fragment, in slot order (up to 32
-                // slots, each lane links its own slot to the next live one)
-                int head = -1;
-                if (n <= 32) {
-                    const int v = lane < n ? wslot[lane] : -1;
-                    const unsigned live = __ballot_sync(FULL, v >= 0);
-                    const unsigned later = live & ~((2u << lane) - 1u);
-                    const int vn = __shfl_sync(FULL, v, later ? __ffs(later) - 1 : 0);
-                    const int hv = __shfl_sync(FULL, v, live ? __ffs(live) - 1 : 0);
-                    if (v >= 0) S.next[v] = (int16_t)(later ? vn : -1);
-                    head = live ? hv : -1;
-                }
-                if (lane == 0) {
-                    if (n > 32) {
-                        for (int m = n - 1; m >= 0; --m) {
-                            const int v = wslot[m];
-                            if (v < 0) continue;
-                            S.next[v] = (int16_t)head;
-                            head = v;
-                        }
-                    }
-                    S.head[lf] = head;
-                    S.S[lf] = tot;
-                    S.dirty[lf] = 0;
-                    my_hops += i;
-                }
-                __syncwarp();
-            }
-            // every write of the phase, local and remote, is visible after the wait.
-            // Between arrival and wait: the next phase's first draws (events 0 and 1
-            // of each of this CTA's fragments of the next colour), which depend on no
-            // fragment's state, so that they overlap the barrier's release
-            cluster_arrive();
-            pre_valid = false;
-            {
-                int ncolour = -1;
-                uint64_t nw = w;
-                if (p < 7) {
-                    ncolour = (int)((wperm >> (4 * (p + 1))) & 15u);
-                } else if (wk + 1 < windows && ((wk + 1) & 63) != 0) {  // the next window's order is known
-                    ncolour = (int)(sh.perms[(wk + 1) & 63] & 15u);
-                    nw = w + 1;
-                }
-                if (ncolour >= 0) {
-                    int ncnt[2], nbit[3], nlz0;
-                    const int nn = colour_geo(ncolour, ncnt, nbit, nlz0);
-                    for (int l = tid; l < nn; l += NT) {
-                        int f0, f1, f2;
-                        frag_coords(l, ncnt, nbit, nlz0, f0, f1, f2);
-                        const int fid = (f2 * D.nf[1] + f1) * D.nf[0] + f0;
-                        const U64x4 blk = philox4x64((uint64_t)fid, nw, 0, 0, D.seed, hop_k1);
-                        S.pre_E[2 * l] = neglog32(blk.x[0]);
-                        S.pre_E[2 * l + 1] = neglog32(blk.x[2]);
-                        S.pre_xs[2 * l] = blk.x[1];
-                        S.pre_xs[2 * l + 1] = blk.x[3];
-                    }
-                    pre_valid = true;
-                }
-            }
-            __syncwarp();
-            cluster_wait();
-        }
-    }
-    if (ph > 0) drain((ph - 1) & 1);
-
-    // ---- stage out: this slab's occupancy, its fragments' records
-    for (int k = tid; k < slab_words; k += NT) occ[slab_off + k] = S.occ[k];
-    for (int lf = tid; lf < nfl_me; lf += NT) {
-        const int64_t g = D.frag_base + (int64_t)fzb * D.nf[1] * D.nf[0] + lf;
-        int k = 0;
-        for (int v = S.head[lf]; v >= 0; v = S.next[v], ++k) {
-            if (k >= cap) {
-                atomicOr(status, STATUS_OVERFLOW);
-                break;
-            }
-            int t, x, y, z;
-            split32(S.key[v], t, x, y, z);
-            VacRec rr;
-            rr.key = make_key(t, x, y, z);
-            rr.d[0] = S.d[3 * v];
-            rr.d[1] = S.d[3 * v + 1];
-            rr.d[2] = S.d[3 * v + 2];
-            rr.id = S.id[v];
-            recs[g * cap + k] = rr;
-        }
-        counts[g] = k;
-        rc.tot[g] = S.S[lf];
-        rc.dirty[g] = S.dirty[lf];
-    }
-    atomicAdd(&sh.hops, my_hops);
-    atomicAdd(&sh.hand, my_hand);
-    __syncthreads();
-    if (tid == 0) {
-        if (sh.hops) atomicAdd(stats + 2 * P.rep, sh.hops);
-        if (sh.hand) atomicAdd(stats + 2 * P.rep + 1, sh.hand);
-    }
-    cluster_sync();  // no CTA leaves while a peer may still address it
-    if (tid == 0 && me == 0) rc.valid[P.rep] = 1;
-}
-
-size_t cluster_smem_bytes(const RepDesc& D, const ClusterPlan& p, int cap)
-{
-    return cluster_layout_bytes(D, p, cap, CLUSTER_THREADS / 32, nullptr);
-}
-
-bool make_cluster_plan(const RepDesc& D, int64_t n_vac, int cap, int min_ctas, int max_ctas, ClusterPlan* out)
-{
-    if (D.L[0] > 1024 || D.L[1] > 1024 || D.L[2] > 1024 || D.nf[2] < 2) return false;
     const int nf2 = D.nf[2];
-    for (int nc = std::max(2, min_ctas); nc <= std::min(max_ctas, CLUSTER_MAX_CTAS) && nc <= nf2; ++nc) {
-        ClusterPlan p{};
-        p.ncta = nc;
-        int zs = 0, layers = 0;
-        for (int c = 0; c <= nc; ++c) p.fz0[c] = (int)((int64_t)c * nf2 / nc);
-        for (int c = 0; c < nc; ++c) {
-            const int z0 = p.fz0[c] * D.base[2] + std::min(p.fz0[c], D.rem[2]);
-            const int z1 = p.fz0[c + 1] * D.base[2] + std::min(p.fz0[c + 1], D.rem[2]);
-            zs = std::max(zs, z1 - z0);
-            layers = std::max(layers, p.fz0[c + 1] - p.fz0[c]);
-        }
-        p.zs = zs;
-        p.nfl = layers * D.nf[0] * D.nf[1];
-        // the inbox takes a phase's arrivals through the slab's two faces: at most the
-        // vacancies of the two neighbouring cell layers (a vacancy crosses once per
-        // phase), with a margin of eight standard deviations
-        const double per_layer = 2.0 * (double)n_vac / D.L[2];
-        p.icap = (int)std::min<double>(8192.0, std::ceil(per_layer + 8.0 * std::sqrt(per_layer) + 64.0));
-        // the vacancy pool: whatever shared memory is left, at least twice the slab's share
-        p.vcap = 0;
-        const size_t fixed = cluster_layout_bytes(D, p, cap, CLUSTER_THREADS / 32, nullptr);
-        if (fixed > RESIDENT_MAX_SMEM) continue;
-        const int64_t share = (n_vac * layers + nf2 - 1) / nf2;
-        const int64_t room = (int64_t)(RESIDENT_MAX_SMEM - fixed) / 24 - 64;
-        const int64_t vcap = std::min<int64_t>(32767, room);
-        if (vcap < 2 * share + 64) continue;
-        p.vcap = (int)vcap;
-        if (cluster_layout_bytes(D, p, cap, CLUSTER_THREADS / 32, nullptr) > RESIDENT_MAX_SMEM) continue;
-        *out = p;
-        return true;
+    if (D.L[0] > 1024 || D.L[1] > 1024 || D.L[2] > 1024 || nc < 2 || nc > CLUSTER_MAX_CTAS || nc > nf2) return false;
+    ClusterPlan p{};
+    p.ncta = nc;
+    int zs = 0, layers = 0;
+    for (int c = 0; c <= nc; ++c) p.fz0[c] = (int)((int64_t)c * nf2 / nc);
+    for (int c = 0; c < nc; ++c) {
+        const int z0 = p.fz0[c] * D.base[2] + std::min(p.fz0[c], D.rem[2]);
+        const int z1 = p.fz0[c + 1] * D.base[2] + std::min(p.fz0[c + 1], D.rem[2]);
+        zs = std::max(zs, z1 - z0);
+        layers = std::max(layers, p.fz0[c + 1] - p.fz0[c]);
     }
+    p.zs = zs;
+    p.nfl = layers * D.nf[0] * D.nf[1];
+    if (p.nfl > 65535) return false;  // 16-bit fragment indices
+    if (cluster_smem_bytes(D, p, cap, pre_ev, prec) > RESIDENT_MAX_SMEM) return false;
+    *out = p;
+    return true;
+}
+
+bool make_cluster_plan(const RepDesc& D, int cap, int pre_ev, int prec, int min_ctas, int max_ctas, ClusterPlan* out)
+{
+    for (int nc = std::min(max_ctas, CLUSTER_MAX_CTAS); nc >= std::max(2, min_ctas); --nc)
+        if (cluster_plan_for(D, cap, pre_ev, prec, nc, out)) return true;
     return false;
 }
 
-cudaError_t cluster_prepare()
+using ResidentFn = void (*)(const RepDesc*, const int32_t*, const ClusterPlan*, uint64_t, uint64_t, uint32_t*, VacRec*,
+                            VacRec*, uint32_t*, int32_t*, int32_t*, unsigned long long*, uint32_t*, int, NbTable,
+                            const Draw*, int64_t, uint32_t, ResCache);
+
+static ResidentFn resident_kernel(int prec, int threads, bool cluster)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_cluster<CLUSTER_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)RESIDENT_MAX_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_cluster<CLUSTER_THREADS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (cluster) return prec ? k_resident<1, CLUSTER_THREADS, true> : k_resident<0, CLUSTER_THREADS, true>;
+    if (threads == 128) return prec ? k_resident<1, 128, false> : k_resident<0, 128, false>;
+    if (threads == 256) return prec ? k_resident<1, 256, false> : k_resident<0, 256, false>;
+    return prec ? k_resident<1, 512, false> : k_resident<0, 512, false>;
+}
+
+cudaError_t resident_prepare()
+{
+    cudaError_t e = cudaSuccess;
+    for (int prec = 0; prec < 2; ++prec) {
+        for (int threads : {128, 256, 512})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(resident_kernel(prec, threads, false),
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_MAX_SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(resident_kernel(prec, 0, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)RESIDENT_MAX_SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(resident_kernel(prec, 0, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
     return e;
 }
 
-int cluster_fits(int ncta, size_t smem)
+static cudaLaunchConfig_t cluster_config(int nclusters, int ncta, size_t smem, cudaStream_t st,
+                                         cudaLaunchAttribute* attr)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ncta);
+    cfg.gridDim = dim3((unsigned)(nclusters * ncta));
     cfg.blockDim = dim3(CLUSTER_THREADS);
     cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)ncta;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    cfg.stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)ncta;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+int cluster_fits(int prec, int ncta, size_t smem)
+{
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = cluster_config(1, ncta, smem, nullptr, attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_cluster<CLUSTER_THREADS>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, resident_kernel(prec, 0, true), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return n;
 }
 
-cudaError_t launch_cluster(const RepDesc* d_descs, const ClusterPlan* d_plans, int nplans, int ncta, size_t smem,
-                           uint64_t windows, uint32_t* occ, VacRec* recs, int32_t* counts, int32_t* tracer,
-                           unsigned long long* stats, uint32_t* status, int cap, const NbTable& nbt,
-                           const ResCache& rc, cudaStream_t st)
+cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uint64_t w0, int windows, int ev_per,
+                         int64_t frag_tot, Draw* draws, cudaStream_t st)
 {
-    if (nplans <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(ncta * nplans));
-    cfg.blockDim = dim3(CLUSTER_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)ncta;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_cluster<CLUSTER_THREADS>, d_descs, d_plans, windows, occ, recs, counts, tracer,
-                              stats, status, cap, nbt, rc);
+    const int64_t n = max_frag * (ev_per / 2);
+    const dim3 grid((unsigned)((n + 63) / 64), (unsigned)std::min(nrep, 65535), (unsigned)windows);
+    k_draws<<<grid, 64, 0, st>>>(d_descs, nrep, w0, ev_per, frag_tot, draws);
+    return cudaGetLastError();
 }
 
-cudaError_t resident_prepare()
-{
-    cudaError_t e = cudaSuccess;
-    for (auto fn : {k_resident<128, 1>, k_resident<256, 1>, k_resident<512, 1>, k_resident<1024, 1>,
-                    k_resident<1024, 2>}) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_MAX_SMEM);
-        if (e != cudaSuccess) return e;
-    }
-    return e;
-}
-
-cudaError_t launch_resident(const RepDesc* d_descs, const int32_t* d_reps, int nreps, const int64_t* d_nvac,
-                            size_t smem, int threads, int cluster, uint64_t windows, uint32_t* occ, VacRec* recs,
-                            int32_t* counts, int32_t* tracer, unsigned long long* stats, uint32_t* status,
-                            int cap, const NbTable& nbt, uint32_t stuck_wait_us, const ResCache& rc, cudaStream_t st)
+cudaError_t launch_resident(int prec, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
+                            uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st)
 {
     if (nreps <= 0) return cudaSuccess;
-    if (cluster == 2 && threads == 1024) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2u * nreps);
-        cfg.blockDim = dim3(1024);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k_resident<1024, 2>, d_descs, d_reps, d_nvac, windows, occ, recs, counts,
-                                  tracer, stats, status, cap, nbt, stuck_wait_us, rc);
-    }
-    if (threads == 128)
-        k_resident<128, 1><<<nreps, 128, smem, st>>>(d_descs, d_reps, d_nvac, windows, occ, recs, counts, tracer,
-                                                     stats, status, cap, nbt, stuck_wait_us, rc);
-    else if (threads == 256)
-        k_resident<256, 1><<<nreps, 256, smem, st>>>(d_descs, d_reps, d_nvac, windows, occ, recs, counts, tracer,
-                                                     stats, status, cap, nbt, stuck_wait_us, rc);
-    else if (threads == 1024)
-        k_resident<1024, 1><<<nreps, 1024, smem, st>>>(d_descs, d_reps, d_nvac, windows, occ, recs, counts,
-                                                       tracer, stats, status, cap, nbt, stuck_wait_us, rc);
-    else
-        k_resident<512, 1><<<nreps, 512, smem, st>>>(d_descs, d_reps, d_nvac, windows, occ, recs, counts, tracer,
-                                                     stats, status, cap, nbt, stuck_wait_us, rc);
+    resident_kernel(prec, threads, false)<<<nreps, threads, smem, st>>>(
+        a.descs, d_reps, nullptr, w0, windows, a.occ, a.recs, a.tmp, a.vmap, a.counts, a.tracer, a.stats, a.status,
+        a.cap, a.nbt, draws, a.frag_tot, a.stuck_wait_us, a.rc);
     return cudaGetLastError();
+}
+
+cudaError_t launch_cluster(int prec, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,
+                           size_t smem, uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st)
+{
+    if (nplans <= 0) return cudaSuccess;
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = cluster_config(nplans, ncta, smem, st, attr);
+    return cudaLaunchKernelEx(&cfg, resident_kernel(prec, 0, true), a.descs, (const int32_t*)nullptr, d_plans, w0,
+                              windows, a.occ, a.recs, a.tmp, a.vmap, a.counts, a.tracer, a.stats, a.status, a.cap,
+                              a.nbt, draws, a.frag_tot, a.stuck_wait_us, a.rc);
 }
 
 }  // namespace fkmc

@@ -1,0 +1,80 @@
+"""The resident window kernels (one CTA or a thread-block cluster per replica,
+both arithmetic forms) against the CPU oracle where their parts change over:
+row scans of every box shape, fragment lists that overflow and refill, first
+draws made ahead and during a visit, the two forms of the clock, and the plain
+form's draws in several chunks.  Everything is compared bit for bit."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fk():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2004_09081_gb300 import fkmc
+    fkmc.load()
+    return fkmc
+
+
+def pair(fk, orc, cells, nf, nv, nh, seed, prec, T=900.0, Ez=2e7, cap=64, n_tau=1.0, ctas=0, tracer=True):
+    b = fk.Batch([(*cells, 4.01)], [(nv, nh)], seed, nfrag=nf, precision=prec, tracer=tracer, cap_v=cap, n_tau=n_tau,
+                 cluster_ctas=ctas)
+    b.set_barriers(0.6, 0.4, T, field_z=Ez)
+    ref = orc.Lattice(cells, nf, nv, nh, seed=seed, tracer=tracer)
+    ref.set_rates(0.6, 0.4, T, Ez=Ez, a_ang=4.01, cap_v=cap, n_tau=n_tau, precision=prec)
+    assert b.info().kernel == (2 if ctas else 1)
+    return b, ref
+
+
+def check(b, ref, calls):
+    for w in calls:
+        b.run(w)
+        ref.run(w)
+        assert np.array_equal(b.state(), ref.occupancy())
+        assert np.array_equal(b.records(), ref.records())
+        assert np.array_equal(b.tracer_field(), ref.tracer_field())
+        c = ref.counters()
+        assert (b.info().hops, b.info().handoffs) == (c["hops"], c["handoffs"])
+    assert ref.counters()["hops"] > 100
+
+
+# extents 2 and 3; 5 and 6 (rows across word boundaries); 8; 9; 11 to 13 (more cells per
+# lane than a mask holds); 18 and 40 (pieces of rows)
+@pytest.mark.parametrize("cells,nf", [((8, 10, 8), (4, 4, 4)), ((20, 22, 24), (4, 4, 4)), ((32, 16, 32), (4, 2, 4)),
+                                      ((36, 18, 18), (4, 2, 2)), ((24, 26, 22), (2, 2, 2)), ((36, 12, 12), (2, 2, 2)),
+                                      ((40, 6, 8), (1, 2, 2))])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_row_scans_of_every_box(fk, orc, prec, cells, nf):
+    n = 3 * int(np.prod(cells))
+    nv = min(6 * int(np.prod(nf)), n // 20)
+    check(*pair(fk, orc, cells, nf, nv, n // 12, 5, prec), (25, 1, 30))
+
+
+@pytest.mark.parametrize("ctas", [0, 2, 4])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_lists_overflow_and_refill(fk, orc, prec, ctas):
+    """Eight vacancies per fragment on average: a fragment's list (8) fills, gives
+    way to the row scan and comes back; one CTA and 2 and 4 slabs."""
+    check(*pair(fk, orc, (10, 12, 16), (2, 2, 4), 128, 400, 3, prec, ctas=ctas), (20, 20, 20))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_long_windows_leave_the_clock_estimates(fk, orc, prec):
+    """60 vacancies in one fragment at n_tau 64: thousands of events per visit.
+    The mixed clock meets ratios below its last place and goes on in FP64; the
+    plain clock fills its log many times and meets sums within 2^-10 of the
+    window."""
+    b, ref = pair(fk, orc, (8, 8, 8), (1, 1, 1), 60, 0, 7, prec, Ez=0.0, n_tau=64.0)
+    check(b, ref, (6, 6))
+    assert ref.counters()["hops"] > 30000
+
+
+@pytest.mark.parametrize("ctas", [0, 2])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_many_windows_in_one_call(fk, orc, prec, ctas):
+    """More than two chunks of the plain form's draws (64 windows each), and
+    colour orders of more than two blocks of 64 windows."""
+    check(*pair(fk, orc, (8, 8, 12), (2, 2, 4), 20, 90, 11, prec, ctas=ctas, n_tau=0.5), (150, 3, 200))
