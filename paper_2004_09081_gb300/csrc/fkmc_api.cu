@@ -243,6 +243,9 @@ struct kmc_batch {
     double* nE = nullptr;                  // the current step's clock variate per replica
     unsigned long long* nctl = nullptr;    // [0] steps of this call so far, [1] current step, [2] blocks done
     std::vector<double> theta_host;
+    uint32_t* null_types = nullptr;        // one launch for many steps: packed event types per vacancy
+    void* null_log = nullptr;              // and each replica's barrier and sums per step
+    size_t null_types_bytes = 0;
     cudaGraphExec_t null_exec = nullptr;
     int64_t null_exec_picks = -1, null_exec_vac = -1;
     bool null_exec_grains = false;
@@ -1465,6 +1468,13 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
         CK(cudaMemcpyAsync(b->theta, b->theta_host.data(), sizeof(double) * b->n, cudaMemcpyHostToDevice, b->st),
            "clock upload");
     }
+    if (sizeof(uint32_t) * (size_t)total_vac > b->null_types_bytes || !b->null_log) {
+        b->dfree(b->null_types);
+        b->null_types = (uint32_t*)b->dalloc(sizeof(uint32_t) * (size_t)total_vac);
+        b->null_types_bytes = b->null_types ? sizeof(uint32_t) * (size_t)total_vac : 0;
+        if (!b->null_log) b->null_log = b->dalloc(null_log_bytes(b->n));
+        if (!b->null_types || !b->null_log) return fail(FKMC_ENOMEM, "device allocation failed (null-event buffers)");
+    }
     if (total_picks > b->props_cap) {
         if (b->null_exec) cudaGraphExecDestroy(b->null_exec);
         b->null_exec = nullptr;
@@ -1487,7 +1497,21 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
     CK(launch_null_gather(b->d_desc, b->n, b->recs, b->counts, b->nfrag_total, b->cap, b->vac, b->status, b->st),
        "null gather");
     ++launches;
-    if (steps > 0 && total_vac > 0) {
+    NullStepsPlan plan;
+    int64_t max_vac = 0, max_sites = 0;
+    for (int r = 0; r < b->n; ++r) {
+        max_vac = std::max(max_vac, b->n_vac[r]);
+        max_sites = std::max(max_sites, b->desc[r].nsite);
+    }
+    if (steps > 0 && null_steps_plan(b->n, max_vac, max_sites, &plan)) {
+        for (uint64_t k = 0; k < steps; k += NULL_LOG_STEPS) {
+            CK(launch_null_steps(plan, b->d_desc, b->n, k, (int)std::min<uint64_t>(NULL_LOG_STEPS, steps - k), b->vac,
+                                 b->null_types, b->occ, b->grains_on ? b->gbound : nullptr, b->claims, b->tracer,
+                                 b->null_log, b->theta, b->stats, b->status, b->st),
+               "null-event steps");
+            launches += 2;
+        }
+    } else if (steps > 0 && total_vac > 0) {
         if (!b->null_exec || b->null_exec_picks != total_picks || b->null_exec_vac != total_vac ||
             b->null_exec_grains != b->grains_on) {
             if (b->null_exec) cudaGraphExecDestroy(b->null_exec);

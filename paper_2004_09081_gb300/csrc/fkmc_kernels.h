@@ -55,6 +55,17 @@ cudaError_t launch_null_step(const RepDesc* d_descs, int nrep, int64_t total_vac
                              NullProp* props,
                              unsigned long long* claims, int32_t* tracer, double* theta, double* nE,
                              unsigned long long* stats, unsigned long long* nctl, cudaStream_t st);
+// the same steps by one cooperative launch for up to NULL_LOG_STEPS of them (where the plan holds)
+constexpr int NULL_LOG_STEPS = 4096;
+struct NullStepsPlan {
+    int ctas, per;  // CTAs per replica, vacancies and picks per thread
+};
+size_t null_log_bytes(int nrep);
+bool null_steps_plan(int nrep, int64_t max_vac, int64_t max_sites, NullStepsPlan* out);
+cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, int nrep, uint64_t k0, int steps,
+                              VacRec* vac, uint32_t* types, uint32_t* occ, const uint8_t* gb,
+                              unsigned long long* claims, int32_t* tracer, void* log_mem, double* theta,
+                              unsigned long long* stats, uint32_t* status, cudaStream_t st);
 cudaError_t launch_moments(const RepDesc& D, int species, const uint32_t* occ, const VacRec* recs,
                            const int32_t* counts, const int32_t* tracer, int cap,
                            unsigned long long* out, cudaStream_t st);

@@ -1,6 +1,6 @@
 // fkmc_null.cu -- the atom-based fragment kMC with null events of
 // arXiv:2004.09081 Sec. II.B (Eqs. AtomP, TimeStepFrg), the atoms being the
-// vacancies.  One step over every replica of the batch, four launches:
+// vacancies.  One step over every replica of the batch, three parts:
 //
 //   k_null_rates    R_I of every vacancy; R_tot = sum, R_max = max (exact u64)
 //   k_null_propose  N_frg picks (keyed bijection of the vacancy ids: an
@@ -13,6 +13,9 @@
 //                   updated exchanges are disjoint and commute.  The last
 //                   block to finish advances every replica's clock,
 //                   clock += -ln(r') / R_tot * N_updated (Eq. TimeStepFrg)
+//
+// The parts run in one launch for many steps (k_null_steps, below), or, for more
+// vacancies than the GPU holds threads for, as three launches per step in a graph.
 //
 // Rates are the mixed form's fixed point with F_null = 63 - ceil(log2(8 N_V)),
 // so every sum is an exact integer and no reduction order enters the result.
@@ -345,6 +348,303 @@ __global__ void __launch_bounds__(256) k_null_apply(const RepDesc* __restrict__ 
     if (threadIdx.x == 0) nctl[2] = 0ull;
 }
 
+// ---------------------------------------------------------------- one launch for many steps
+// The same steps by one cooperative launch for a whole range of steps, `ctas`
+// CTAs per replica: a step's three parts are separated by barriers among a
+// replica's CTAs instead of kernel launches: 24.7 -> 12.8 us per step on the 128^3
+// lattice's 18,874 vacancies (148 CTAs).  What bounds a step is its chain
+// of dependent L2 round trips: about 0.4 us each for a vacancy's key, its
+// neighbour words, a pick's key and types, its claims, and some 1 us per barrier.
+// The picks' hashes and draws, which depend on no state, are computed while the
+// rates' reads are in flight; the rates pass leaves the eight events' types packed
+// in a word, so that a pick reads one word instead of eight.  A thread-block
+// cluster of 16 CTAs with hardware barriers took 40 us per step: the uncoalesced
+// reads of 16 SMs are what bounds it then, so the work is spread over every SM.
+constexpr int CT = 128;  // threads per CTA
+
+// One step's sums of a replica.
+struct NullStep {
+    unsigned long long tot, max, updated, pad;
+};
+// A replica's barrier: arrivals since the launch, and whether a wait ran out.
+struct NullBarrier {
+    unsigned int count, stop;
+};
+
+constexpr unsigned long long NULL_WAIT_NS = 2000000000ull;  // bound on one barrier wait
+
+// Barrier number `target / ctas` of the replica's CTAs; false when a wait ran
+// out (here or elsewhere), after which every CTA leaves.
+__device__ __forceinline__ bool null_barrier(NullBarrier* bar, unsigned target)
+{
+    __shared__ int stop;
+    __threadfence();  // this thread's writes before the arrival
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned c;
+        asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(c) : "l"(&bar->count) : "memory");
+        unsigned long long t0, t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+        int out = 0;
+        ++c;
+        while ((int)(c - target) < 0) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&bar->count) : "memory");
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+            if (t - t0 > NULL_WAIT_NS) {
+                atomicExch(&bar->stop, 1u);
+                out = 1;
+                break;
+            }
+        }
+        stop = out || *reinterpret_cast<volatile unsigned*>(&bar->stop) != 0u;
+    }
+    __syncthreads();
+    return stop == 0;
+}
+
+// Sum and maximum over a warp of values below 2^63, by 32-bit warp reductions.
+__device__ __forceinline__ void warp_sum_max(unsigned long long v, unsigned long long& sum, unsigned long long& mx)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const unsigned a = __reduce_add_sync(FULL, (unsigned)v & 0x1fffffu);
+    const unsigned b = __reduce_add_sync(FULL, (unsigned)(v >> 21) & 0x1fffffu);
+    const unsigned c = __reduce_add_sync(FULL, (unsigned)(v >> 42));
+    sum = (unsigned long long)a + ((unsigned long long)b << 21) + ((unsigned long long)c << 42);
+    const unsigned hi = __reduce_max_sync(FULL, (unsigned)(v >> 32));
+    const unsigned lo = __reduce_max_sync(FULL, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+    mx = ((unsigned long long)hi << 32) | lo;
+}
+
+// Steps k0 .. k0 + steps - 1 of every replica (CTAs [r ctas, (r + 1) ctas): replica
+// r).  types: one word per vacancy, nibble n = rate type of event n + 1 (0: no
+// event).  log: per replica and step, cleared by the caller, as are the barriers.
+template <int PER>
+__global__ void __launch_bounds__(CT)
+    k_null_steps(const RepDesc* __restrict__ descs, int ctas, uint64_t k0, int steps, VacRec* vac, uint32_t* types,
+                 uint32_t* occ, const uint8_t* __restrict__ gb, unsigned long long* claims, int32_t* tracer,
+                 NullStep* log, int log_stride, NullBarrier* bars, uint32_t* status)
+{
+    __shared__ RepDesc D;
+    __shared__ PickKeys pk[2];           // by step parity
+    __shared__ unsigned long long q[16]; // rate of type t at t + 1, 0 for no event
+    __shared__ unsigned long long part[2][CT / 32];
+    __shared__ unsigned long long rmax;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rep = (int)(blockIdx.x / ctas), me = (int)(blockIdx.x - rep * ctas);
+    NullBarrier* const bar = bars + rep;
+    unsigned target = 0;
+    if (tid == 0) D = descs[rep];
+    __syncthreads();
+    if (tid < 16) q[tid] = tid == 0 || tid > 12 ? 0ull : (tid <= 6 ? D.qn[tid - 1] : D.qng[tid - 7]);
+    const int nv = (int)D.null_nv, np = (int)D.null_nfrg;
+    VacRec* const vr = vac + D.vac_off;
+    uint32_t* const ty_r = types + D.vac_off;
+    uint32_t* const occ_r = occ + D.occ_word_off;
+    unsigned long long* const cl = claims + D.site_off;
+    const uint64_t key_null = key_word(D.replica, PURPOSE_NULL);
+    const int first = me * CT + tid, stride = ctas * CT;
+    auto keys_of = [&](uint64_t step) {  // one Philox block per thread of lanes 0 .. 2 of the last warp
+        if (warp == CT / 32 - 1 && lane < NULL_PICK_ROUNDS / 4) {
+            const U64x4 b = philox4x64(step, (uint64_t)lane, 0, 0, D.seed, key_word(D.replica, PURPOSE_PICK));
+            for (int i = 0; i < 4; ++i) pk[step & 1].k[4 * lane + i] = b.x[i];
+        }
+    };
+    keys_of(D.null_step + k0);
+    __syncthreads();
+    for (int s = 0; s < steps; ++s) {
+        const uint64_t k = k0 + s, step = D.null_step + k;
+        NullStep* const st = log + (int64_t)rep * log_stride + s;
+        // ---- rates
+        unsigned long long sum = 0ull, mx = 0ull;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int i = first + u * stride;
+            unsigned long long R = 0ull;
+            if (i < nv) {
+                int t, x, y, z;
+                split_key(__ldcg(&vr[i].key), t, x, y, z);
+                uint32_t w[8];
+                int sh[8], base[8];
+                bool bnd[8];
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    const NbEntry nb = null_nb(t, n);
+                    const int jx = wrapc(x + nb.dc[0], D.L[0]);
+                    const int jy = wrapc(y + nb.dc[1], D.L[1]);
+                    const int jz = wrapc(z + nb.dc[2], D.L[2]);
+                    w[n] = __ldcg(occ_r + occ_index(D.row_words, D.L[1], nb.t2, jx, jy, jz));
+                    sh[n] = occ_shift(jx);
+                    base[n] = nb.d[2] + 2;
+                    bnd[n] = gb && gb[cell_index(D, jx, jy, jz)];
+                }
+                const bool own = gb && gb[cell_index(D, x, y, z)];
+                uint32_t packed = 0;
+#pragma unroll
+                for (int n = 0; n < 8; ++n) {
+                    const int code = (int)((w[n] >> sh[n]) & 3u);
+                    const int e = code == SP_V ? 0 : code * 3 + base[n] + ((own || bnd[n]) ? 6 : 0);
+                    packed |= (uint32_t)e << (4 * n);
+                    R += q[e];
+                }
+                ty_r[i] = packed;
+            }
+            unsigned long long ws, wm;
+            warp_sum_max(R, ws, wm);
+            sum += ws;
+            mx = max(mx, wm);
+        }
+        if (lane == 0) {
+            part[0][warp] = sum;
+            part[1][warp] = mx;
+        }
+        // this thread's picks and their draws: they depend on no state
+        int id[PER];
+        uint64_t xs[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int p = first + u * stride;
+            id[u] = -1;
+            xs[u] = 0;
+            if (p < np) {
+                id[u] = (int)null_pick((uint64_t)p, (uint64_t)nv, pk[step & 1]);
+                xs[u] = philox4x64(step, (uint64_t)p, 0, 0, D.seed, key_null).x[0];
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            unsigned long long t2 = 0ull, m2 = 0ull;
+            for (int w = 0; w < CT / 32; ++w) {
+                t2 += part[0][w];
+                m2 = max(m2, part[1][w]);
+            }
+            atomicAdd(&st->tot, t2);
+            atomicMax(&st->max, m2);
+        }
+        keys_of(step + 1);
+        if (!null_barrier(bar, target += ctas)) break;
+        // ---- picks: event or null event, claims
+        if (tid == 0) rmax = __ldcg(&st->max);
+        uint64_t key[PER];
+        uint32_t pt[PER];
+        int sel[PER], ls[PER], lj[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            key[u] = 0;
+            pt[u] = 0;
+            if (id[u] >= 0) {
+                key[u] = __ldcg(&vr[id[u]].key);
+                pt[u] = __ldcg(ty_r + id[u]);
+            }
+        }
+        __syncthreads();
+        const unsigned long long Rmax = rmax;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            sel[u] = -1;
+            ls[u] = lj[u] = 0;
+            if (id[u] < 0) continue;
+            const unsigned long long target = __umul64hi(xs[u], Rmax);
+            unsigned long long P = 0ull;
+#pragma unroll
+            for (int n = 0; n < 8; ++n) {
+                P += q[(pt[u] >> (4 * n)) & 15u];
+                if (sel[u] < 0 && P > target) sel[u] = n;
+            }
+            if (sel[u] < 0) continue;
+            int t, x, y, z;
+            split_key(key[u], t, x, y, z);
+            const NbEntry nb = null_nb(t, sel[u]);
+            ls[u] = (int)lin(D, t, x, y, z);
+            lj[u] = (int)lin(D, nb.t2, wrapc(x + nb.dc[0], D.L[0]), wrapc(y + nb.dc[1], D.L[1]),
+                             wrapc(z + nb.dc[2], D.L[2]));
+            const unsigned long long mine = claim_of(k, first + u * stride);
+            atomicMin(cl + ls[u], mine);
+            atomicMin(cl + lj[u], mine);
+        }
+        if (!null_barrier(bar, target += ctas)) break;
+        // ---- exchanges of the picks that hold both their claims
+        unsigned done = 0;
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            bool did = false;
+            if (sel[u] >= 0) {
+                const unsigned long long mine = claim_of(k, first + u * stride);
+                const unsigned long long c0 = __ldcg(cl + ls[u]), c1 = __ldcg(cl + lj[u]);
+                if (c0 == mine && c1 == mine) {
+                    did = true;
+                    int t, x, y, z;
+                    split_key(key[u], t, x, y, z);
+                    const NbEntry nb = null_nb(t, sel[u]);
+                    const int jx = wrapc(x + nb.dc[0], D.L[0]);
+                    const int jy = wrapc(y + nb.dc[1], D.L[1]);
+                    const int jz = wrapc(z + nb.dc[2], D.L[2]);
+                    const uint32_t ion = ((((pt[u] >> (4 * sel[u])) & 15u) - 1u) % 6u) / 3u;
+                    atomicXor(occ_r + occ_index(D.row_words, D.L[1], t, x, y, z), ((uint32_t)SP_V ^ ion) << occ_shift(x));
+                    atomicXor(occ_r + occ_index(D.row_words, D.L[1], nb.t2, jx, jy, jz),
+                              (ion ^ (uint32_t)SP_V) << occ_shift(jx));
+                    VacRec* v = vr + id[u];
+                    v->key = make_key(nb.t2, jx, jy, jz);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d)
+                        if (nb.d[d]) atomicAdd(&v->d[d], (int)nb.d[d]);
+                    if (tracer) {
+                        int32_t* ts = tracer + 3 * (D.site_off + ls[u]);
+                        int32_t* tj = tracer + 3 * (D.site_off + lj[u]);
+#pragma unroll
+                        for (int d = 0; d < 3; ++d) {
+                            ts[d] = __ldcg(tj + d) - nb.d[d];
+                            tj[d] = 0;
+                        }
+                    }
+                }
+            }
+            done += __popc(__ballot_sync(FULL, did));
+        }
+        if (lane == 0 && done) atomicAdd(&st->updated, (unsigned long long)done);
+        if (!null_barrier(bar, target += ctas)) break;
+    }
+    if (tid == 0 && *reinterpret_cast<volatile unsigned*>(&bar->stop) != 0u) atomicOr(status, STATUS_TIMEOUT);
+}
+
+// The clocks and hop counters of `steps` steps from their log, one block per
+// replica: clock += -ln(r') / R_tot * N_updated step by step (Eq. TimeStepFrg),
+// the terms computed side by side, the sum in order.
+__global__ void __launch_bounds__(256) k_null_clock(const RepDesc* __restrict__ descs, uint64_t k0, int steps,
+                                                    const NullStep* __restrict__ log, int log_stride, double* theta,
+                                                    unsigned long long* stats)
+{
+    __shared__ double term[256];
+    __shared__ unsigned long long hops;
+    const int r = blockIdx.x, tid = threadIdx.x;
+    const RepDesc& D = descs[r];
+    if (tid == 0) hops = 0ull;
+    double th = theta[r];
+    for (int s0 = 0; s0 < steps; s0 += 256) {
+        const int s = s0 + tid;
+        double dth = 0.0;
+        __syncthreads();
+        if (s < steps) {
+            const NullStep l = log[(int64_t)r * log_stride + s];
+            if (l.tot > 0ull) {
+                const U64x4 b = philox4x64(D.null_step + k0 + s, ~0ull, 0, 0, D.seed, key_word(D.replica, PURPOSE_NULL));
+                dth = __dmul_rn(__dmul_rn(__ddiv_rn(neglog64(b.x[0]), __ull2double_rn(l.tot)), D.two_pow_Fn),
+                                __ull2double_rn(l.updated));
+            }
+            if (l.updated) atomicAdd(&hops, l.updated);
+        }
+        term[tid] = dth;
+        __syncthreads();
+        if (tid == 0)
+            for (int q = 0; q < min(256, steps - s0); ++q) th = __dadd_rn(th, term[q]);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        theta[r] = th;
+        stats[2 * r] += hops;
+    }
+}
+
 constexpr int NT = 256;
 
 unsigned grid_of(int64_t n)
@@ -391,6 +691,66 @@ cudaError_t launch_null_step(const RepDesc* d_descs, int nrep, int64_t total_vac
                                                         claims, nE, nctl);
     k_null_apply<<<grid_of(total_picks), NT, 0, st>>>(d_descs, nrep, total_picks, vac, occ, props, claims, tracer,
                                                       acc, theta, stats, nE, nctl);
+    return cudaGetLastError();
+}
+
+using NullStepsFn = void (*)(const RepDesc*, int, uint64_t, int, VacRec*, uint32_t*, uint32_t*, const uint8_t*,
+                             unsigned long long*, int32_t*, NullStep*, int, NullBarrier*, uint32_t*);
+
+static NullStepsFn null_steps_kernel(int per)
+{
+    return per == 1 ? k_null_steps<1> : (per == 2 ? k_null_steps<2> : k_null_steps<4>);
+}
+
+size_t null_log_bytes(int nrep) { return (sizeof(NullStep) * NULL_LOG_STEPS + sizeof(NullBarrier)) * (size_t)nrep + 32; }
+
+// One launch for many steps: the CTAs that hold the largest replica at the
+// fewest vacancies and picks per thread (1, 2 or 4), all replicas' CTAs resident
+// at once, and 32-bit site indices.  Beyond that (several hundred thousand
+// vacancies) a step is bound by its reads, and the launches are as good.
+bool null_steps_plan(int nrep, int64_t max_vac, int64_t max_sites, NullStepsPlan* out)
+{
+    if (max_vac < 1 || max_vac > (1 << 22) || max_sites > 0x7fffffffll) return false;
+    int dev = 0, sms = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) {
+        cudaGetLastError();
+        return false;
+    }
+    for (int per = 1; per <= 4; per *= 2) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, null_steps_kernel(per), CT, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        const int64_t ctas = (max_vac + (int64_t)CT * per - 1) / ((int64_t)CT * per);
+        if (ctas * nrep > (int64_t)sms * per_sm) continue;
+        out->ctas = (int)ctas;
+        out->per = per;
+        return true;
+    }
+    return false;
+}
+
+cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, int nrep, uint64_t k0, int steps,
+                              VacRec* vac, uint32_t* types, uint32_t* occ, const uint8_t* gb,
+                              unsigned long long* claims, int32_t* tracer, void* log_mem, double* theta,
+                              unsigned long long* stats, uint32_t* status, cudaStream_t st)
+{
+    NullBarrier* bars = reinterpret_cast<NullBarrier*>(log_mem);
+    NullStep* log = reinterpret_cast<NullStep*>(reinterpret_cast<char*>(log_mem) + ((sizeof(NullBarrier) * nrep + 31) & ~(size_t)31));
+    int stride = steps;
+    cudaError_t e = cudaMemsetAsync(log_mem, 0, (((sizeof(NullBarrier) * nrep + 31) & ~(size_t)31) +
+                                                 sizeof(NullStep) * (size_t)nrep * stride), st);
+    if (e != cudaSuccess) return e;
+    int ctas = p.ctas;
+    void* args[] = {(void*)&d_descs, &ctas, &k0, &steps, &vac, &types, &occ, (void*)&gb, &claims, &tracer, &log,
+                    &stride, &bars, &status};
+    e = cudaLaunchCooperativeKernel((const void*)null_steps_kernel(p.per), dim3((unsigned)(ctas * nrep)), dim3(CT), args,
+                                    0, st);
+    if (e != cudaSuccess) return e;
+    k_null_clock<<<nrep, 256, 0, st>>>(d_descs, k0, steps, log, stride, theta, stats);
     return cudaGetLastError();
 }
 
