@@ -230,8 +230,8 @@ int kmc_set_barriers(kmc_batch* b, const kmc_barrier_table* tables, const double
 /* Turn the site-energy interactions on for every replica of the batch (e
  * NULL, or no shells, turns them off).  Plain form only: the event rates are
  * FP64 products of the table rate and the Boltzmann factor above, summed in
- * the canonical order.  Every replica then runs the colour-phase kernels
- * (the replica-resident kernel has no site energies).  The library keeps an
+ * the canonical order, in the resident kernels where the replica fits them
+ * and in the colour-phase kernels elsewhere.  The library keeps an
  * int32 energy field of every O site (4 bytes per site), rebuilt from the
  * vacancies and dopants at the next kmc_run after any state change, and
  * moved with each hop.
@@ -279,7 +279,7 @@ int kmc_read_site_field(kmc_batch* b, int32_t r, int32_t* host_field, size_t n);
  * replica, from three unit-charge solves).  The field is frozen between
  * refreshes: every `refresh_windows` windows kmc_run solves again from the
  * current vacancies (0: never; u stays as last solved or written).
- * Plain form only; the site-energy run pass of the colour-phase kernels. */
+ * Plain form only; the site-energy form of the window kernels. */
 typedef struct {
     double eps_r;             /* relative permittivity, > 0 */
     double q_vac;             /* vacancy charge in e (+2 for an O vacancy) */

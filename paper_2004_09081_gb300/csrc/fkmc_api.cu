@@ -195,6 +195,7 @@ struct kmc_batch {
     std::vector<int64_t> n_fe;
     std::vector<double> T;           // temperature of every replica (kmc_set_barriers)
     int n_vv = 0, n_bo = 0, e_self = 0;
+    int reach_vv = 0;                // largest cell offset of the V-V shells
     int64_t e_bound = 0;             // bound on |E_site|, 1e-4 eV units
     int64_t ncell_total = 0;
     uint8_t* fe = nullptr;           // one byte per cell, batch-wide cell index
@@ -422,7 +423,8 @@ int plan_residency(kmc_batch* b)
     b->rclass.clear();
     const int prec = b->opts.precision == FKMC_MIXED ? 1 : 0;
     const bool allowed = b->opts.schedule != 1 && (prec == 1 || b->opts.schedule == 0) &&
-                         b->cap <= RESIDENT_MAX_SLOTS && !site_path(b) && !b->grains_on;
+                         b->cap <= RESIDENT_MAX_SLOTS && !b->grains_on;
+    const int form = prec ? 1 : (site_path(b) ? 2 : 0);
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -447,11 +449,17 @@ int plan_residency(kmc_batch* b)
     b->run_ctas.assign(b->n, 0);
     for (int r = 0; r < b->n; ++r) {
         RepDesc& D = b->desc[r];
+        D.kslots = 8;
+        D.btab_smem = form == 2;
         int c = -1;
         size_t need = 0;
-        for (int k = 0; k < 4 && allowed && c < 0; ++k) {
-            need = resident_smem_bytes(D, b->cap, threads[k], 1, prec ? 2 : plain_ev, prec);
-            if (need <= bounds[k]) c = k;
+        for (int k = 0; k < 8 && allowed && c < 0; ++k) {
+            if (k == 4) {  // without the Boltzmann tables
+                if (!D.btab_smem) break;
+                D.btab_smem = 0;
+            }
+            need = resident_smem_bytes(D, b->cap, threads[k & 3], 1, prec ? 2 : plain_ev, prec);
+            if (need <= bounds[k & 3]) c = k & 3;
         }
         // the first draws of as many colour phases per batch as the class's shared
         // memory allows beside the state (8: one batch per window): four events per
@@ -474,18 +482,31 @@ int plan_residency(kmc_batch* b)
         const int force = b->opts.cluster_ctas;
         if (allowed && force >= 0 && (c < 0 || force >= 2)) {
             ClusterPlan pl{};
-            const int ev = prec ? 4 : plain_ev;
+            const int single_btab = D.btab_smem, single_ev = D.pre_ev;
             const int lo = force >= 2 ? force : 2, hi = force >= 2 ? force : CLUSTER_MAX_CTAS;
-            if (make_cluster_plan(D, b->cap, ev, prec, lo, hi, &pl) &&
-                cluster_fits(prec, pl.ncta, cluster_smem_bytes(D, pl, b->cap, ev, prec)) > 0) {
+            // (events drawn ahead, list entries), the next where the slabs do not fit
+            const int want[4][2] = {{prec ? 4 : plain_ev, 8}, {prec ? 4 : plain_ev, 4}, {4, 4}, {2, 4}};
+            bool found = false;
+            for (int q = 0; q < 8 && !found; ++q) {
+                const int k = q & 3;
+                D.btab_smem = form == 2 && q < 4;
+                if (form != 2 && q >= 4) break;
+                D.kslots = want[k][1];
+                found = make_cluster_plan(D, b->cap, want[k][0], prec, lo, hi, &pl) &&
+                        cluster_fits(form, pl.ncta, cluster_smem_bytes(D, pl, b->cap, want[k][0], prec)) > 0;
+                if (found) D.pre_ev = want[k][0];
+            }
+            if (found) {
                 pl.rep = r;
                 plans.push_back(pl);
                 D.resident = 1;
-                D.pre_ev = ev;
                 b->run_kernel[r] = 2;
                 b->run_ctas[r] = pl.ncta;
                 continue;
             }
+            D.kslots = 8;
+            D.btab_smem = single_btab;
+            D.pre_ev = single_ev;
         }
         D.resident = c >= 0 ? 1 : 0;
         if (c < 0) {
@@ -508,7 +529,7 @@ int plan_residency(kmc_batch* b)
         const int r = cls[3][k];
         ClusterPlan pl{};
         if (!make_cluster_plan(b->desc[r], b->cap, 4, prec, 2, 2, &pl) ||
-            cluster_fits(prec, 2, cluster_smem_bytes(b->desc[r], pl, b->cap, 4, prec)) <= 0) {
+            cluster_fits(form, 2, cluster_smem_bytes(b->desc[r], pl, b->cap, 4, prec)) <= 0) {
             ++k;
             continue;
         }
@@ -783,6 +804,7 @@ SiteArgs site_args(const kmc_batch* b)
     a.field = b->field;
     a.n_vv = b->n_vv;
     a.e_self = b->e_self;
+    a.reach = b->n_vv > 0 ? b->reach_vv + 1 : 0;
     a.gbound = b->grains_on ? b->gbound : nullptr;
     a.g_elec = b->elec_on ? b->d_elec_g : nullptr;
     return a;
@@ -838,7 +860,8 @@ int elec_cover(kmc_batch* b, int64_t um)
     rc = upload_desc(b);
     if (rc) return rc;
     if (b->btab != before) drop_window_graph(b);
-    return FKMC_OK;
+    rc = plan_residency(b);  // the tables' size enters the resident kernels' shared memory
+    return rc ? rc : upload_desc(b);
 }
 
 // V-cycles of the next automatic refresh
@@ -1226,6 +1249,8 @@ ResidentArgs resident_args(const kmc_batch* b)
     a.cap = b->cap;
     a.nbt = b->nbt;
     a.frag_tot = b->res_frags;
+    a.draw_ev = b->res_ev;
+    a.sa = site_args(b);
     a.stuck_wait_us = (uint32_t)b->opts.test_stuck_wait_us;
     a.rc = b->rcache;
     return a;
@@ -1233,7 +1258,7 @@ ResidentArgs resident_args(const kmc_batch* b)
 
 // one launch per class on the classes' streams, after `from` and before `to`
 // (largest classes first: their CTAs run longest and should take SMs first)
-cudaError_t launch_classes(kmc_batch* b, int prec, uint64_t w0, uint64_t windows, const Draw* draws, cudaEvent_t from,
+cudaError_t launch_classes(kmc_batch* b, int form, uint64_t w0, uint64_t windows, const Draw* draws, cudaEvent_t from,
                            cudaStream_t to)
 {
     const ResidentArgs args = resident_args(b);
@@ -1242,22 +1267,22 @@ cudaError_t launch_classes(kmc_batch* b, int prec, uint64_t w0, uint64_t windows
         auto& c = *it;
         le = cudaStreamWaitEvent(c.st, from, 0);
         if (le == cudaSuccess && c.slabs)
-            le = launch_cluster(prec, args, b->d_plans + c.start, c.count, c.cluster, c.smem, w0, windows, draws, c.st);
+            le = launch_cluster(form, args, b->d_plans + c.start, c.count, c.cluster, c.smem, w0, windows, draws, c.st);
         else if (le == cudaSuccess)
-            le = launch_resident(prec, args, b->d_reps + c.start, c.count, c.smem, c.threads, w0, windows, draws, c.st);
+            le = launch_resident(form, args, b->d_reps + c.start, c.count, c.smem, c.threads, w0, windows, draws, c.st);
         if (le == cudaSuccess) le = cudaEventRecord(c.done, c.st);
         if (le == cudaSuccess) le = cudaStreamWaitEvent(to, c.done, 0);
     }
     return le;
 }
 
-// The resident replicas' windows on a stream beside the caller's (res_st, after
+// The resident replicas' windows (the call's windows [w_first, w_first + windows)) on a stream beside the caller's (res_st, after
 // res_fork, ended by res_join).  Mixed form: the class launches captured once
 // per window count into a graph (fork, one launch per class, join).  Plain
 // form: the first draws of draw_windows windows at a time by k_draws on a
 // stream of their own, the next chunk's beside the current chunk's windows
 // (two buffers).
-int launch_resident_classes(kmc_batch* b, uint64_t windows, uint64_t* launches)
+int launch_resident_classes(kmc_batch* b, uint64_t w_first, uint64_t windows, uint64_t* launches)
 {
     if (!b->cap_st) CK(cudaStreamCreateWithFlags(&b->cap_st, cudaStreamNonBlocking), "stream");
     if (!b->res_st) {
@@ -1288,7 +1313,7 @@ int launch_resident_classes(kmc_batch* b, uint64_t windows, uint64_t* launches)
         CK(cudaStreamWaitEvent(b->res_st, b->res_fork, 0), "stream wait");
         CK(cudaGraphLaunch(b->res_exec, b->res_st), "graph launch");
         CK(cudaEventRecord(b->res_join, b->res_st), "event record");
-        *launches = b->rclass.size();
+        *launches += b->rclass.size();
         return FKMC_OK;
     }
     if (!b->draw_st) {
@@ -1303,9 +1328,10 @@ int launch_resident_classes(kmc_batch* b, uint64_t windows, uint64_t* launches)
     CK(cudaStreamWaitEvent(b->draw_st, b->res_fork, 0), "stream wait");
     const uint64_t step = (uint64_t)b->draw_windows;
     uint64_t done = 0;
-    for (uint64_t w0 = 0; w0 < windows; w0 += step, ++done) {
+    const int form = site_path(b) ? 2 : 0;
+    for (uint64_t w0 = w_first; w0 < w_first + windows; w0 += step, ++done) {
         const int k = (int)(done & 1);
-        const uint64_t nw = std::min(step, windows - w0);
+        const uint64_t nw = std::min(step, w_first + windows - w0);
         Draw* buf = b->draws + (size_t)k * b->res_frags * b->res_ev * step;
         if (done >= 2) CK(cudaStreamWaitEvent(b->draw_st, b->draw_free[k], 0), "stream wait");
         CK(launch_draws(b->d_desc, b->n, b->res_max_frag, w0, (int)nw, b->res_ev, b->res_frags, buf, b->draw_st),
@@ -1313,7 +1339,7 @@ int launch_resident_classes(kmc_batch* b, uint64_t windows, uint64_t* launches)
         CK(cudaEventRecord(b->draw_done[k], b->draw_st), "event record");
         CK(cudaStreamWaitEvent(b->res_st, b->draw_done[k], 0), "stream wait");
         CK(cudaEventRecord(b->draw_free[k], b->res_st), "event record");  // the windows before have ended
-        CK(launch_classes(b, 0, w0, nw, buf, b->draw_free[k], b->res_st), "resident launch");
+        CK(launch_classes(b, form, w0, nw, buf, b->draw_free[k], b->res_st), "resident launch");
         CK(cudaEventRecord(b->draw_free[k], b->res_st), "event record");
         *launches += 1 + b->rclass.size();
     }
@@ -1333,10 +1359,6 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
     std::vector<unsigned long long> before = b->stats_host;
     CK(cudaEventRecord(b->ev0, b->st), "event record");
     uint64_t res_launches = 0;
-    if (!b->rclass.empty() && windows > 0) {
-        int rc0 = launch_resident_classes(b, windows, &res_launches);
-        if (rc0) return rc0;
-    }
     uint64_t extra_launches = 0;
     if (site_path(b) && !b->field_valid) {
         int rc0 = rebuild_field(b);
@@ -1376,22 +1398,30 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
         }
         return FKMC_OK;
     };
-    if (b->any_global && windows > 0) {
-        CK(cudaMemsetAsync(b->wctl, 0, sizeof(unsigned long long) * 2, b->st), "memset");
-        const uint64_t every = b->elec_on ? (uint64_t)b->elec.refresh_windows : 0;
-        for (uint64_t wk = 0; wk < windows; ++wk) {
-            if (every > 0 && b->elec_age >= every) {  // the potential follows the vacancies
-                int rc1 = elec_refresh(b);
-                if (rc1) return rc1;
-                extra_launches += elec_launches(b);
-            }
+    if (b->any_global && windows > 0) CK(cudaMemsetAsync(b->wctl, 0, sizeof(unsigned long long) * 2, b->st), "memset");
+    const uint64_t every = b->elec_on ? (uint64_t)b->elec.refresh_windows : 0;
+    for (uint64_t wk = 0; wk < windows;) {
+        if (every > 0 && b->elec_age >= every) {  // the potential follows the vacancies
+            int rc1 = elec_refresh(b);
+            if (rc1) return rc1;
+            extra_launches += elec_launches(b);
+            rc1 = drop_resident_cache(b);  // the rates of every fragment changed
+            if (rc1) return rc1;
+        }
+        const uint64_t nw = every > 0 ? std::min(windows - wk, every - b->elec_age) : windows - wk;
+        if (!b->rclass.empty()) {
+            int rc2 = launch_resident_classes(b, wk, nw, &res_launches);
+            if (rc2) return rc2;
+        }
+        if (b->any_global) {
             int rc2 = ensure_graph();
             if (rc2) return rc2;
-            CK(cudaGraphLaunch(b->window_exec, b->st), "graph launch");
-            ++b->elec_age;
+            for (uint64_t k = 0; k < nw; ++k) CK(cudaGraphLaunch(b->window_exec, b->st), "graph launch");
         }
+        if (!b->rclass.empty()) CK(cudaStreamWaitEvent(b->st, b->res_join, 0), "stream wait");
+        wk += nw;
+        b->elec_age += nw;
     }
-    if (!b->rclass.empty() && windows > 0) CK(cudaStreamWaitEvent(b->st, b->res_join, 0), "stream wait");
     CK(cudaEventRecord(b->ev1, b->st), "event record");
     for (int r = 0; r < b->n; ++r) b->desc[r].window += windows;
     int rc = upload_desc(b);
@@ -1984,6 +2014,7 @@ int kmc_set_site_energy(kmc_batch* b, const kmc_site_energy* e)
     }
     if (!b->field || !b->d_vv || !b->d_bo || !b->fe) return fail(FKMC_ENOMEM, "device allocation failed");
     b->n_vv = sh.nvv;
+    b->reach_vv = reach_vv;
     b->n_bo = (int)bo.size();
     b->e_self = eself;
     b->e_bound = sh.bound;

@@ -70,7 +70,8 @@ struct RepDesc {
     uint64_t qg[6];
     uint64_t qng[6];
     int32_t pre_ev;        // resident kernels: events per fragment drawn ahead (2: block 0; 4: blocks 0, 1; 8: 0 .. 3)
-    int32_t pad_ev_;
+    int32_t btab_smem;     // resident kernels: 1: the Boltzmann tables lie in shared memory
+    int32_t kslots;        // resident kernels: entries of a fragment's vacancy list (4 or 8)
     // resident kernels
     int64_t vmap_off;      // first word of this replica's site -> record map
     int64_t tmp_off;       // first fragment of this replica in the record copies of the stage-out
@@ -111,6 +112,7 @@ struct SiteArgs {
     int32_t* field;       // E_site of every O site (batch-wide site index)
     int32_t n_vv;         // offsets per site type
     int32_t e_self;       // energy of the a/sqrt2 shell: a hop partner's share of its target
+    int32_t reach;        // cells around a hop whose vacancies' rates change with the shells (0: no shells)
     const uint8_t* gbound;  // grains: 1 per boundary cell (batch-wide cell index), or null
     const int32_t* g_elec;  // electrostatics: [replica][3][8] own-potential share of a hop, or null
 };

@@ -140,6 +140,8 @@ struct ResidentArgs {  // fixed for a batch and its plan
     int cap;
     NbTable nbt;
     int64_t frag_tot;  // fragments of all resident replicas (stride of the plain form's draws)
+    int draw_ev;       // events per fragment in the plain form's draws
+    SiteArgs sa;       // plain form with site energies
     uint32_t stuck_wait_us;
     ResCache rc;
 };
@@ -147,14 +149,15 @@ size_t resident_smem_bytes(const RepDesc& D, int cap, int threads, int pre_g, in
 size_t cluster_smem_bytes(const RepDesc& D, const ClusterPlan& p, int cap, int pre_ev, int prec);
 // the plan with the most CTAs in [min_ctas, max_ctas] whose slabs fit one SM's shared memory
 bool make_cluster_plan(const RepDesc& D, int cap, int pre_ev, int prec, int min_ctas, int max_ctas, ClusterPlan* out);
-int cluster_fits(int prec, int ncta, size_t smem);  // clusters of this shape the GPU can hold at once
+int cluster_fits(int form, int ncta, size_t smem);  // clusters of this shape the GPU can hold at once
 cudaError_t resident_prepare();
 // first draws of `windows` windows from w0 on, of every resident replica (plain form)
 cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uint64_t w0, int windows, int ev_per,
                          int64_t frag_tot, Draw* draws, cudaStream_t st);
-cudaError_t launch_resident(int prec, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
+// form: 0 plain, 1 mixed, 2 plain with site energies
+cudaError_t launch_resident(int form, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
                             uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st);
-cudaError_t launch_cluster(int prec, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,
+cudaError_t launch_cluster(int form, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,
                            size_t smem, uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st);
 
 }  // namespace fkmc

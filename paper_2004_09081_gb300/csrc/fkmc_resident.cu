@@ -47,6 +47,14 @@
 // mixed 22.8 -> 19.1, 128^3 mixed 55.2 -> 50.8; plain: five 32^3 replicas 155 ->
 // 29.8, 8^3 113 -> 28.5, 128^3 196 -> 75.5.
 //
+// With site energies (plain form) a visit's chain is some 8,000 cycles per event
+// instead of 3,500: the rates wait for the energy field's words in L2, after an
+// exchange behind the 116 atomics that move the vacancy's share.  Five doped 96^3
+// replicas 302 -> 190 us per window, 128^3 in its own potential 483 -> 420 with
+// the solves.  Holding a visit's moves back and correcting the rates by pair
+// energies instead was slower (190 -> 200): the pair energies cost as many
+// instructions as the wait.
+//
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -139,6 +147,7 @@ __device__ __forceinline__ uint32_t cluster_nctas()
 // every thread of every CTA of the cluster; release / acquire of shared memory
 __device__ __forceinline__ void cluster_sync()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -246,6 +255,7 @@ struct Layout {
     void* lim;             // Limit<PREC>::T by local fragment
     uint8_t* stale;        // 1: a vacancy came in since `slots` was written
     uint64_t* wlog;        // plain, per warp: E and R of events whose clock division is put off
+    double* btab;          // site energies: the Boltzmann tables lo[BOLTZ_LO], hi[bhi_len]
     uint32_t* slots;       // site keys of each local fragment's vacancies in site order (DEAD: none), or
                            // UNLISTED where it holds more than KSLOTS
     uint2* box;            // first cell and extent of each local fragment, 10 bits per dimension
@@ -263,7 +273,7 @@ struct Layout {
 };
 constexpr unsigned NO_ROW = 0xffffu;      // a fragment's row of first draws: none,
 constexpr unsigned ROW_FULL = 0x8000u;    // or row | ROW_FULL where every event of the row was drawn (else two)
-constexpr int KSLOTS = 8;
+constexpr int KSLOTS = 8;                  // entries of a fragment's list (or 4: RepDesc.kslots)
 constexpr int CLOCK_LOG = 8;  // events whose clock division the plain form puts off
 constexpr uint32_t UNLISTED = 0xfffffffeu;
 
@@ -271,10 +281,10 @@ constexpr uint32_t UNLISTED = 0xfffffffeu;
 // fragments of one colour at most.
 struct Sizes {
     int64_t words;
-    int nfl, maxc, cap, nwarps, ltot, lz, rows, pre_ev, prec;
+    int nfl, maxc, cap, nwarps, ltot, lz, rows, pre_ev, prec, kslots, btab;
 };
 
-constexpr int NARR = 17;
+constexpr int NARR = 18;
 
 __host__ __device__ inline size_t layout_bytes(const Sizes& z, size_t* off /* NARR offsets or null */)
 {
@@ -296,8 +306,9 @@ __host__ __device__ inline size_t layout_bytes(const Sizes& z, size_t* off /* NA
         (size_t)z.nwarps * z.cap * 4,    // 12 per-warp record indices
         (size_t)z.nwarps * z.cap * 8,    // 13 per-warp event types
         (size_t)z.nfl,                   // 14 stale flags
-        (size_t)z.nfl * KSLOTS * 4,      // 15 vacancies by fragment
+        (size_t)z.nfl * z.kslots * 4,    // 15 vacancies by fragment
         z.prec ? 0 : (size_t)z.nwarps * CLOCK_LOG * 16,  // 16 per-warp clock log (plain)
+        (size_t)z.btab * 8,              // 17 Boltzmann tables (site energies, where they fit)
     };
     size_t b = 0;
     for (int k = 0; k < NARR; ++k) {
@@ -323,6 +334,8 @@ __host__ __device__ inline Sizes sizes_single(const RepDesc& D, int cap, int nwa
     z.rows = rows;
     z.pre_ev = pre_ev;
     z.prec = prec;
+    z.kslots = D.kslots == 4 ? 4 : KSLOTS;
+    z.btab = D.btab_smem ? BOLTZ_LO + D.bhi_len : 0;
     return z;
 }
 
@@ -341,6 +354,8 @@ __host__ __device__ inline Sizes sizes_cluster(const RepDesc& D, const ClusterPl
     z.rows = 2;
     z.pre_ev = pre_ev;
     z.prec = prec;
+    z.kslots = D.kslots == 4 ? 4 : KSLOTS;
+    z.btab = D.btab_smem ? BOLTZ_LO + D.bhi_len : 0;
     return z;
 }
 
@@ -364,6 +379,7 @@ __device__ __forceinline__ Layout carve(unsigned char* dyn, const Sizes& z)
     L.wvac = reinterpret_cast<uint32_t*>(dyn + o[12]);
     L.wtype = reinterpret_cast<int8_t*>(dyn + o[13]);
     L.wlog = reinterpret_cast<uint64_t*>(dyn + o[16]);
+    L.btab = reinterpret_cast<double*>(dyn + o[17]);
     L.stale = dyn + o[14];
     L.slots = reinterpret_cast<uint32_t*>(dyn + o[15]);
     return L;
@@ -467,6 +483,28 @@ __device__ __forceinline__ void mark_owner(const Layout& S, const Geo& g, int x,
             if (came) st_peer8(peer_addr(S.stale + f, zm & 255u), 1);
         }
     }
+}
+
+// site index (within the replica) of a shell partner: packed SiteOff {t2, dc[3]} of a cell
+__device__ __forceinline__ int shell_lin(const Geo& g, int off, int x, int y, int z)
+{
+    const int t2 = (int)(int8_t)off;
+    const int px = wrapc(x + (int)(int8_t)(off >> 8), g.L0), py = wrapc(y + (int)(int8_t)(off >> 16), g.L1),
+              pz = wrapc(z + (int)(int8_t)(off >> 24), g.L2);
+    return ((t2 * g.L2 + pz) * g.L1 + py) * g.L0 + px;
+}
+
+// a cell of the interval [c - r, c + 1 + r] or [c - 1 - r, c + r] around the cells c and j of a
+// hop (j = c or a neighbour, periodic): its lower end (p = 0), c (1) or its upper end (2)
+__device__ __forceinline__ int box_cell(int c, int j, int p, int r, int L)
+{
+    if (p == 1) return c;
+    int d = j - c;
+    d = d > 1 ? -1 : (d < -1 ? 1 : d);
+    int v = p == 0 ? c + min(d, 0) - r : c + max(d, 0) + r;
+    while (v < 0) v += L;
+    while (v >= L) v -= L;
+    return v;
 }
 
 // index of a site in the site -> record map: sixteen entries per occupancy word
@@ -700,14 +738,15 @@ __global__ void __launch_bounds__(64) k_draws(const RepDesc* __restrict__ descs,
     }
 }
 
-template <int PREC, int NT, bool CL>
+template <int PREC, int NT, bool CL, bool SITE>
 __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     k_resident(const RepDesc* __restrict__ descs, const int32_t* __restrict__ reps,
                const ClusterPlan* __restrict__ plans, uint64_t w0, uint64_t windows, uint32_t* occ, VacRec* recs,
                VacRec* tmp, uint32_t* vmap, int32_t* counts, int32_t* tracer, unsigned long long* stats,
-               uint32_t* status, int cap, NbTable nbt, const Draw* __restrict__ draws, int64_t frag_tot,
-               uint32_t stuck_wait_us, ResCache rc)
+               uint32_t* status, int cap, NbTable nbt, const Draw* __restrict__ draws, int64_t frag_tot, int draw_ev,
+               uint32_t stuck_wait_us, ResCache rc, SiteArgs sa)
 {
+    static_assert(!SITE || PREC == 0, "site energies use the plain form");
     extern __shared__ __align__(128) unsigned char dyn[];
     __shared__ Shared sh;
     constexpr unsigned FULL = 0xffffffffu;
@@ -753,7 +792,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     const Layout S = carve(dyn, sz);
     using Lim = Limit<PREC>;
     typename Lim::T* const lim = reinterpret_cast<typename Lim::T*>(S.lim);
-    const int maxc = sz.maxc;
+    const int maxc = sz.maxc, ks = sz.kslots;
     const int fzb = P.fz0[me], fze = P.fz0[me + 1];
     const Geo geo{D.L[0], D.L[1], D.L[2], D.row_words, D.nf[0], D.nf[1], sh.zbeg[me], sh.zbeg[me + 1] - sh.zbeg[me],
                   fzb, me};
@@ -805,6 +844,9 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
         sh.coff[8] = s;
     }
     __syncthreads();
+    if constexpr (SITE) {
+        for (int k = tid; k < sz.btab; k += NT) S.btab[k] = sa.btab[D.btab_off + k];
+    }
     for (int c = 0; c < 8; ++c) {
         int cnt[2], lz0;
         const int n = colour_count(c, cnt, lz0);
@@ -829,21 +871,21 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
         const int64_t g = frag0 + f;
         const int c = counts[g];
         if (c > cap) atomicOr(status, STATUS_OVERFLOW);
-        uint32_t* const sl = S.slots + f * KSLOTS;
+        uint32_t* const sl = S.slots + f * ks;
         int have = 0;
         for (int k = 0; k < c && k < cap; ++k) {
             int t, x, y, z;
             split_key(recs[g * cap + k].key, t, x, y, z);
             vmap_s[map_index(geo, key32(t, x, y, z - geo.zb))] = (uint32_t)((g - D.frag_base) * cap + k);
-            if (c <= KSLOTS) {  // into the sorted list
+            if (c <= ks) {  // into the sorted list
                 const uint32_t key = key32(t, x, y, z);
                 int m = have++;
                 for (; m > 0 && sl[m - 1] > key; --m) sl[m] = sl[m - 1];
                 sl[m] = key;
             }
         }
-        for (int k = have; k < KSLOTS; ++k) sl[k] = DEAD;
-        if (c > KSLOTS) sl[0] = UNLISTED;
+        for (int k = have; k < ks; ++k) sl[k] = DEAD;
+        if (c > ks) sl[0] = UNLISTED;
         S.stale[f] = 0;
         // the limit the last launch left, where nothing changed the replica since
         lim[f] = sh.cached ? (typename Lim::T)rc.lim[g] : (c > 0 ? Lim::DIRTY : Lim::EMPTY);
@@ -908,7 +950,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
             S.pre_xs[o + 2 * k + 1] = b.x[3];
         } else {
             const int4 d = __ldg(
-                reinterpret_cast<const int4*>(draws + ((int64_t)wk * frag_tot + D.draw_off + fid) * pre_ev + k));
+                reinterpret_cast<const int4*>(draws + ((int64_t)wk * frag_tot + D.draw_off + fid) * draw_ev + k));
             reinterpret_cast<uint64_t*>(S.pre_E)[o + k] = (uint64_t)(uint32_t)d.x | (uint64_t)(uint32_t)d.y << 32;
             S.pre_xs[o + k] = (uint64_t)(uint32_t)d.z | (uint64_t)(uint32_t)d.w << 32;
         }
@@ -928,9 +970,49 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
         return dead ? NO_EVENT : ty;
     };
     auto rate_of = [&](int ty) -> uint64_t { return sh.rate[ty]; };
-    auto scan64 = [&](uint64_t v) -> uint64_t {  // inclusive prefix over the lanes, strides 1, 2, .. 16
+    // site energies: FP64 rate of the event of type ty from the site of key k to that of key nk in this
+    // lane's direction: the table rate times the two Boltzmann factors of the energy difference, in the
+    // order of the colour-phase kernel.  Field words come from L2: the exchanges update them by atomics.
+    const int32_t* const field_r = SITE ? sa.field + D.site_off : nullptr;
+    const double* const blo = SITE ? (sz.btab ? S.btab : sa.btab + D.btab_off) : nullptr;
+    auto site_rate = [&](int& ty, uint32_t k, uint32_t nk) -> uint64_t {
+        if (ty >= NO_EVENT) return 0ull;
+        int t, x, y, z, t2, jx, jy, jz;
+        split32(k, t, x, y, z);
+        split32(nk, t2, jx, jy, jz);
+        const int32_t Es = __ldcg(field_r + ((t * geo.L2 + z) * geo.L1 + y) * geo.L0 + x);
+        const int32_t Ej = __ldcg(field_r + ((t2 * geo.L2 + jz) * geo.L1 + jy) * geo.L0 + jx);
+        int32_t dm = Ej - sa.e_self - Es;
+        if (sa.g_elec) dm -= __ldg(sa.g_elec + 24 * D.replica + 8 * t + (lane & 7));
+        const int h = D.bhi_mid + (dm >> 9);
+        if (h < 0 || h >= D.bhi_len) {  // outside the bound the tables were built for: report, no event
+            atomicOr(status, STATUS_ENERGY_RANGE);
+            ty = NO_EVENT;
+            return 0ull;
+        }
+        return (uint64_t)__double_as_longlong(
+            __dmul_rn(__dmul_rn(__longlong_as_double((long long)sh.rate[ty]), blo[BOLTZ_LO + h]), blo[dm & 511]));
+    };
+    // moves a vacancy's share of the energy field from the site of key k to that of key nk (every lane a
+    // part); integer atomics: fragments of one colour may touch the same word
+    auto move_share = [&](uint32_t k, uint32_t nk) {
+        int t, x, y, z, t2, jx, jy, jz;
+        split32(k, t, x, y, z);
+        split32(nk, t2, jx, jy, jz);
+        int32_t* const fw = sa.field + D.site_off;
+        for (int o = lane; o < sa.n_vv; o += 32) {
+            const int2 a = __ldg(reinterpret_cast<const int2*>(sa.vv + t * SITE_MAX_VV + o));
+            const int2 c = __ldg(reinterpret_cast<const int2*>(sa.vv + t2 * SITE_MAX_VV + o));
+            atomicAdd(fw + shell_lin(geo, a.x, x, y, z), -a.y);
+            atomicAdd(fw + shell_lin(geo, c.x, jx, jy, jz), c.y);
+        }
+    };
+    // inclusive prefix over the lanes, strides 1, 2, .. 16; with values in the first `len` lanes only
+    // the strides below len (the others add zeros to those lanes)
+    auto scan64 = [&](uint64_t v, int len = 32) -> uint64_t {
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
+            if (o >= 8 && o >= len) break;
             const uint64_t u = __shfl_up_sync(FULL, (unsigned long long)v, o);
             if (lane >= o) {
                 if constexpr (PREC == 1) v += u;
@@ -997,7 +1079,15 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                 const int lf = S.flist[c0 + l];
                 const typename Lim::T m = lim[lf];
                 bool active = m == Lim::DIRTY;
-                if (!active && m != Lim::EMPTY) {
+                if (active && S.stale[lf] == 0) {  // marked, but without a vacancy?
+                    bool none = true;
+                    for (int q = 0; q < ks; ++q) none = none && S.slots[lf * ks + q] == DEAD;
+                    if (none) {
+                        lim[lf] = Lim::EMPTY;
+                        active = false;
+                    }
+                }
+                if (!active && m != Lim::EMPTY && m != Lim::DIRTY) {
                     const int o = (CL ? par * maxc + l : (int)(S.pre_row[lf] & (ROW_FULL - 1u))) * pre_ev;
                     if constexpr (PREC == 1) active = reinterpret_cast<const float*>(S.pre_E)[o] <= __uint_as_float(m);
                     else active = reinterpret_cast<const uint64_t*>(S.pre_E)[o] <= m;  // positive doubles
@@ -1024,8 +1114,8 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                 // the fragment's vacancies: its list, or, where it changed from outside or is too long
                 // for one, a scan of its rows.  Up to two chunks (8 vacancies) each lane keeps the site
                 // keys of its two events' slots, their rate types and their targets' keys in registers
-                uint32_t* const sl = S.slots + lf * KSLOTS;
-                uint32_t kc0 = sl[lane >> 3], kc1 = sl[4 + (lane >> 3)];
+                uint32_t* const sl = S.slots + lf * ks;
+                uint32_t kc0 = sl[lane >> 3], kc1 = ks > 4 ? sl[4 + (lane >> 3)] : DEAD;
                 const bool scan = S.stale[lf] != 0 || __shfl_sync(FULL, kc0, 0) == UNLISTED;
                 // key of slot lane & 7 (up to two chunks)
                 auto slot_key = [&]() -> uint32_t {
@@ -1072,10 +1162,15 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                 }
                 uint32_t nk0 = 0, nk1 = 0;
                 int ty0 = NO_EVENT, ty1 = NO_EVENT;
+                uint64_t sr0 = 0, sr1 = 0;  // site energies: the rates
                 auto compute_types = [&]() {
                     if (nch <= 2) {
                         ty0 = type_of(kc0, nk0);
                         if (nch == 2) ty1 = type_of(kc1, nk1);
+                        if constexpr (SITE) {
+                            sr0 = site_rate(ty0, kc0, nk0);
+                            if (nch == 2) sr1 = site_rate(ty1, kc1, nk1);
+                        }
                     } else {
                         for (int c = 0; c < nch; ++c) {
                             const int e = c * 32 + lane, m = e >> 3;
@@ -1085,6 +1180,18 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                             wtype[e] = (int8_t)ty;
                         }
                         __syncwarp();
+                    }
+                };
+                // rate of event c * 32 + lane beyond two chunks (site energies: computed again)
+                auto rate_at = [&](int c) -> uint64_t {
+                    int ty = wtype[c * 32 + lane];
+                    if constexpr (SITE) {
+                        const int m = (c * 32 + lane) >> 3;
+                        uint32_t nk = 0;
+                        if (ty < NO_EVENT) type_of(wkey[m], nk);
+                        return site_rate(ty, ty < NO_EVENT ? wkey[m] : key0, nk);
+                    } else {
+                        return rate_of(ty);
                     }
                 };
                 compute_types();
@@ -1124,13 +1231,14 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     // order, give the inclusive prefixes that the selection needs besides
                     uint64_t inc0 = 0, inc1 = 0;
                     if (nch <= 2) {
-                        inc0 = rate_of(ty0);
-                        inc1 = nch == 2 ? rate_of(ty1) : 0ull;
+                        inc0 = SITE ? sr0 : rate_of(ty0);
+                        inc1 = nch == 2 ? (SITE ? sr1 : rate_of(ty1)) : 0ull;
                         if constexpr (PREC == 1) {
                             tot = warp_total(inc0 + inc1);
                         } else {
-                            inc0 = scan64(inc0);
-                            tot = __shfl_sync(FULL, inc0, 31);
+                            const int len = n <= 2 ? 8 * max(n, 1) : 32;
+                            inc0 = scan64(inc0, len);
+                            tot = __shfl_sync(FULL, inc0, len - 1);
                             if (nch == 2) {
                                 inc1 = add(tot, scan64(inc1));
                                 tot = __shfl_sync(FULL, inc1, 31);
@@ -1138,12 +1246,12 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                         }
                     } else if constexpr (PREC == 1) {
                         unsigned long long part = 0;
-                        for (int c = 0; c < nch; ++c) part += rate_of(wtype[c * 32 + lane]);
+                        for (int c = 0; c < nch; ++c) part += rate_at(c);
                         tot = warp_total(part);
                     } else {
                         tot = 0;
                         for (int c = 0; c < nch; ++c)
-                            tot = __shfl_sync(FULL, add(tot, scan64(rate_of(wtype[c * 32 + lane]))), 31);
+                            tot = __shfl_sync(FULL, add(tot, scan64(rate_at(c))), 31);
                     }
                     if (tot == 0ull) break;
                     if (i >= MAX_EVENTS_PER_PHASE) {
@@ -1235,7 +1343,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     if (past) break;
                     if constexpr (PREC == 1) {  // the prefixes, only for an event that happens
                         if (nch <= 2) {
-                            inc0 = scan64(inc0);
+                            inc0 = scan64(inc0, n <= 2 ? 8 * n : 32);
                             if (nch == 2) inc1 = __shfl_sync(FULL, inc0, 31) + scan64(inc1);
                         }
                     }
@@ -1243,19 +1351,20 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     // nonzero rate, and the last of those where rounding left no prefix above it)
                     int e_sel = -1;
                     if (nch <= 2) {
-                        const bool h0 = inc0 > target && (PREC == 1 || ty0 < NO_EVENT);
-                        const bool h1 = nch == 2 && inc1 > target && (PREC == 1 || ty1 < NO_EVENT);
+                        const bool h0 = inc0 > target && (PREC == 1 || (SITE ? sr0 != 0ull : ty0 < NO_EVENT));
+                        const bool h1 =
+                            nch == 2 && inc1 > target && (PREC == 1 || (SITE ? sr1 != 0ull : ty1 < NO_EVENT));
                         const unsigned b0 = __ballot_sync(FULL, h0), b1 = __ballot_sync(FULL, h1);
                         e_sel = b0 ? __ffs(b0) - 1 : (b1 ? 32 + __ffs(b1) - 1 : -1);
                         if (PREC == 0 && e_sel < 0) {
-                            const unsigned l0 = __ballot_sync(FULL, rate_of(ty0) != 0ull),
-                                           l1 = __ballot_sync(FULL, nch == 2 && rate_of(ty1) != 0ull);
+                            const unsigned l0 = __ballot_sync(FULL, (SITE ? sr0 : rate_of(ty0)) != 0ull),
+                                           l1 = __ballot_sync(FULL, nch == 2 && (SITE ? sr1 : rate_of(ty1)) != 0ull);
                             e_sel = l1 ? 63 - __clz(l1) : 31 - __clz(l0);
                         }
                     } else {
                         uint64_t carry = 0;
                         for (int c = 0; c < nch && e_sel < 0; ++c) {
-                            const uint64_t v = rate_of(wtype[c * 32 + lane]);
+                            const uint64_t v = rate_at(c);
                             const uint64_t inc = add(carry, scan64(v));
                             const unsigned bal = __ballot_sync(FULL, inc > target && (PREC == 1 || v != 0ull));
                             if (bal) e_sel = c * 32 + __ffs(bal) - 1;
@@ -1263,7 +1372,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                         }
                         if (PREC == 0) {
                             for (int c = nch - 1; c >= 0 && e_sel < 0; --c) {
-                                const unsigned bal = __ballot_sync(FULL, rate_of(wtype[c * 32 + lane]) != 0ull);
+                                const unsigned bal = __ballot_sync(FULL, rate_at(c) != 0ull);
                                 if (bal) e_sel = c * 32 + 31 - __clz(bal);
                             }
                         }
@@ -1274,23 +1383,23 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     }
                     // the exchange: site s, its target j, the ion
                     const int m = e_sel >> 3;
-                    uint32_t ks, kj;
+                    uint32_t ks_, kj;
                     int ty;
                     if (nch <= 2) {
                         const bool c1 = e_sel >= 32;
-                        ks = __shfl_sync(FULL, c1 ? kc1 : kc0, e_sel & 31);
+                        ks_ = __shfl_sync(FULL, c1 ? kc1 : kc0, e_sel & 31);
                         kj = __shfl_sync(FULL, c1 ? nk1 : nk0, e_sel & 31);
                         ty = __shfl_sync(FULL, c1 ? ty1 : ty0, e_sel & 31);
                     } else {
-                        ks = wkey[m];
+                        ks_ = wkey[m];
                         uint32_t nk;
-                        type_of(ks, nk);
+                        type_of(ks_, nk);
                         kj = __shfl_sync(FULL, nk, e_sel & 7);
                         ty = wtype[e_sel];
                     }
                     // even lanes compute s's addresses, odd lanes j's
                     int tk, xk, yk, zk;
-                    split32((lane & 1) ? kj : ks, tk, xk, yk, zk);
+                    split32((lane & 1) ? kj : ks_, tk, xk, yk, zk);
                     const int wg = word_of(geo, tk, xk, yk, zk);  // word within the replica
                     if (lane < 2) {
                         const uint32_t flip = ((uint32_t)SP_V ^ (ty >= 3 ? (uint32_t)SP_H : (uint32_t)SP_O))
@@ -1310,7 +1419,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     flush();  // the exchange before
                     {
                         // displacement in units of a/2 along this lane's axis
-                        const int ts = (int)(ks >> 30), tj = (int)(kj >> 30);
+                        const int ts = (int)(ks_ >> 30), tj = (int)(kj >> 30);
                         const uint32_t e = __shfl_sync(FULL, dirs, e_sel & 7) >> (10 * ts);
                         const int ax = lane & 3;  // 0..2
                         pend_m = m;
@@ -1324,6 +1433,12 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                                 trs = 3 * (D.site_off + ls) + ax;
                                 trv = __ldcg(tracer + trj) - pend_d;
                             }
+                        }
+                    }
+                    if constexpr (SITE) {
+                        if (sa.n_vv > 0) {
+                            move_share(ks_, kj);
+                            __threadfence_block();  // before the rate reads
                         }
                     }
                     __syncwarp();  // the exchanged codes are in place
@@ -1342,10 +1457,10 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                         // without marking, so that no branch splits the warp)
                         // (with up to two vacancies lanes 16-31, which hold no event, do it beside the
                         // rate types of lanes 0-15)
-                        const uint32_t pk = (lane & 8) ? kj : ks;
+                        const uint32_t pk = (lane & 8) ? kj : ks_;
                         NbSite c;
                         int code;
-                        if (n <= 2) {
+                        if (!SITE && n <= 2) {
                             const bool dead = kc0 == DEAD;
                             const uint32_t k = lane < 16 ? (dead ? key0 : kc0) : pk;
                             c = nb_site(geo, dirs, k);
@@ -1361,6 +1476,20 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                         }
                         if (code == SP_V)
                             mark_owner<PREC, CL>(S, geo, c.x, c.y, c.z, lf, key32(c.t2, c.x, c.y, c.z) == kj);
+                        if constexpr (SITE) {
+                            // the energy field changed within the shells' reach of s and j, so every rate of
+                            // a vacancy one cell further did: the owners of the cells at -r, 0 and +r around
+                            // the two sites (fragment edges exceed r, so no fragment lies between those)
+                            if (sa.reach > 0 && lane < 27) {
+                                int t, x, y, z, t2, jx, jy, jz;
+                                split32(ks_, t, x, y, z);
+                                split32(kj, t2, jx, jy, jz);
+                                const int px = lane % 3, py = (lane / 3) % 3, pz = lane / 9;
+                                mark_owner<PREC, CL>(S, geo, box_cell(x, jx, px, sa.reach, geo.L0),
+                                                     box_cell(y, jy, py, sa.reach, geo.L1),
+                                                     box_cell(z, jz, pz, sa.reach, geo.L2), lf, false);
+                            }
+                        }
                     }
                     clock = nclock;
                     ++i;
@@ -1372,9 +1501,9 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     if (scan) S.stale[lf] = 0;
                 }
                 if (i > 0 || scan) {  // the fragment's list, in slot order
-                    if (nch <= 2) {
+                    if (n <= ks) {
                         const uint32_t k = slot_key();
-                        if (lane < KSLOTS) sl[lane] = k;
+                        if (lane < ks) sl[lane] = k;
                     } else if (lane == 0) {
                         sl[0] = UNLISTED;
                     }
@@ -1489,29 +1618,37 @@ bool make_cluster_plan(const RepDesc& D, int cap, int pre_ev, int prec, int min_
 
 using ResidentFn = void (*)(const RepDesc*, const int32_t*, const ClusterPlan*, uint64_t, uint64_t, uint32_t*, VacRec*,
                             VacRec*, uint32_t*, int32_t*, int32_t*, unsigned long long*, uint32_t*, int, NbTable,
-                            const Draw*, int64_t, uint32_t, ResCache);
+                            const Draw*, int64_t, int, uint32_t, ResCache, SiteArgs);
 
-static ResidentFn resident_kernel(int prec, int threads, bool cluster)
+template <int PREC, bool SITE>
+static ResidentFn resident_variant(int threads, bool cluster)
 {
-    if (cluster) return prec ? k_resident<1, CLUSTER_THREADS, true> : k_resident<0, CLUSTER_THREADS, true>;
-    if (threads == 128) return prec ? k_resident<1, 128, false> : k_resident<0, 128, false>;
-    if (threads == 256) return prec ? k_resident<1, 256, false> : k_resident<0, 256, false>;
-    return prec ? k_resident<1, 512, false> : k_resident<0, 512, false>;
+    if (cluster) return k_resident<PREC, CLUSTER_THREADS, true, SITE>;
+    if (threads == 128) return k_resident<PREC, 128, false, SITE>;
+    if (threads == 256) return k_resident<PREC, 256, false, SITE>;
+    return k_resident<PREC, 512, false, SITE>;
+}
+
+// form: 0 plain, 1 mixed, 2 plain with site energies
+static ResidentFn resident_kernel(int form, int threads, bool cluster)
+{
+    if (form == 1) return resident_variant<1, false>(threads, cluster);
+    return form == 2 ? resident_variant<0, true>(threads, cluster) : resident_variant<0, false>(threads, cluster);
 }
 
 cudaError_t resident_prepare()
 {
     cudaError_t e = cudaSuccess;
-    for (int prec = 0; prec < 2; ++prec) {
+    for (int form = 0; form < 3; ++form) {
         for (int threads : {128, 256, 512})
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(resident_kernel(prec, threads, false),
+                e = cudaFuncSetAttribute(resident_kernel(form, threads, false),
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_MAX_SMEM);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(resident_kernel(prec, 0, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(resident_kernel(form, 0, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)RESIDENT_MAX_SMEM);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(resident_kernel(prec, 0, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = cudaFuncSetAttribute(resident_kernel(form, 0, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     }
     return e;
 }
@@ -1533,12 +1670,12 @@ static cudaLaunchConfig_t cluster_config(int nclusters, int ncta, size_t smem, c
     return cfg;
 }
 
-int cluster_fits(int prec, int ncta, size_t smem)
+int cluster_fits(int form, int ncta, size_t smem)
 {
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = cluster_config(1, ncta, smem, nullptr, attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, resident_kernel(prec, 0, true), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, resident_kernel(form, 0, true), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1554,25 +1691,25 @@ cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uin
     return cudaGetLastError();
 }
 
-cudaError_t launch_resident(int prec, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
+cudaError_t launch_resident(int form, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
                             uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st)
 {
     if (nreps <= 0) return cudaSuccess;
-    resident_kernel(prec, threads, false)<<<nreps, threads, smem, st>>>(
+    resident_kernel(form, threads, false)<<<nreps, threads, smem, st>>>(
         a.descs, d_reps, nullptr, w0, windows, a.occ, a.recs, a.tmp, a.vmap, a.counts, a.tracer, a.stats, a.status,
-        a.cap, a.nbt, draws, a.frag_tot, a.stuck_wait_us, a.rc);
+        a.cap, a.nbt, draws, a.frag_tot, a.draw_ev, a.stuck_wait_us, a.rc, a.sa);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cluster(int prec, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,
+cudaError_t launch_cluster(int form, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,
                            size_t smem, uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st)
 {
     if (nplans <= 0) return cudaSuccess;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = cluster_config(nplans, ncta, smem, st, attr);
-    return cudaLaunchKernelEx(&cfg, resident_kernel(prec, 0, true), a.descs, (const int32_t*)nullptr, d_plans, w0,
+    return cudaLaunchKernelEx(&cfg, resident_kernel(form, 0, true), a.descs, (const int32_t*)nullptr, d_plans, w0,
                               windows, a.occ, a.recs, a.tmp, a.vmap, a.counts, a.tracer, a.stats, a.status, a.cap,
-                              a.nbt, draws, a.frag_tot, a.stuck_wait_us, a.rc);
+                              a.nbt, draws, a.frag_tot, a.draw_ev, a.stuck_wait_us, a.rc, a.sa);
 }
 
 }  // namespace fkmc

@@ -78,3 +78,25 @@ def test_many_windows_in_one_call(fk, orc, prec, ctas):
     """More than two chunks of the plain form's draws (64 windows each), and
     colour orders of more than two blocks of 64 windows."""
     check(*pair(fk, orc, (8, 8, 12), (2, 2, 4), 20, 90, 11, prec, ctas=ctas, n_tau=0.5), (150, 3, 200))
+
+
+VV = [(2, 0.343), (4, 0.235), (6, 0.200)]
+FE = [(1, -0.709), (5, -0.199), (9, -0.022)]
+
+
+# 16^3 cells fit one CTA; forced slabs; dense fragments (lists overflow, more than two chunks)
+@pytest.mark.parametrize("cells,nf,nv,ctas", [((16, 16, 16), (4, 4, 4), 30, 0), ((16, 16, 24), (4, 4, 6), 40, 4),
+                                              ((10, 11, 12), (2, 2, 2), 90, 0), ((10, 11, 16), (2, 2, 4), 140, 2)])
+def test_site_energies_in_the_resident_kernels(fk, orc, cells, nf, nv, ctas):
+    """Vacancy-vacancy and dopant shells: rates from the energy field, which every
+    exchange moves, and marks on all fragments within the shells' reach."""
+    b = fk.Batch([(*cells, 3.905)], [(nv, 60, 20)], 9, nfrag=nf, precision=0, tracer=True, cap_v=64,
+                 cluster_ctas=ctas)
+    b.set_site_energy(VV, FE)
+    b.set_barriers(0.6, 0.4, 900.0, field_z=1e7)
+    ref = orc.Lattice(cells, nf, nv, 60, seed=9, n_Fe=20, tracer=True)
+    ref.set_site_energy(vv=VV, fe=FE)
+    ref.set_rates(0.6, 0.4, 900.0, Ez=1e7, cap_v=64)
+    assert b.info().kernel == (2 if ctas else 1)
+    check(b, ref, (25, 1, 30))
+    assert np.array_equal(b.site_field(), [ref.site_energy(s) for s in range(ref.nsite)])
