@@ -143,6 +143,8 @@ struct kmc_batch {
     unsigned long long* scratch = nullptr;  // 7 moments
     unsigned long long* scratch_all = nullptr;  // 7 moments per replica
     unsigned long long* check_buf = nullptr;    // CHECK_WORDS sums of kmc_check_invariants
+    void* read_buf = nullptr;                   // read-outs: expanded codes or record rows (READ_BUF_MAX at most)
+    size_t read_bytes = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     std::vector<void*> owned;
     // replica-resident kernel: replicas grouped by shared-memory size class
@@ -1660,24 +1662,53 @@ int kmc_read_D(kmc_batch* b, int32_t r, int32_t species, double D_xyz[3], double
     return FKMC_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+constexpr size_t READ_BUF_MAX = (size_t)128 << 20;
+
+// the batch's read-out buffer with at least `bytes` (at most READ_BUF_MAX), or null
+void* read_buffer(kmc_batch* b, size_t bytes)
+{
+    if (bytes > b->read_bytes) {
+        b->dfree(b->read_buf);
+        b->read_buf = b->dalloc(bytes);
+        b->read_bytes = b->read_buf ? bytes : 0;
+    }
+    return b->read_buf;
+}
+
+// Writes one byte per page of a host buffer that a device copy is about to fill
+// whole: a page the process has not touched yet is mapped here in under a
+// microsecond, by the copy's own page fault in some fifty.
+void touch_pages(void* host, size_t bytes)
+{
+    volatile char* p = static_cast<volatile char*>(host);
+    for (size_t k = 0; k < bytes; k += 4096) p[k] = 0;
+}
+
+}  // namespace
+
+extern "C" {
+
 int kmc_read_state(kmc_batch* b, int32_t r, uint8_t* host_occ, size_t n)
 {
     if (!valid_replica(b, r) || !host_occ) return fail(FKMC_EINVAL, "bad replica or output");
     const RepDesc& D = b->desc[r];
     if ((int64_t)n != D.nsite) return fail(FKMC_EINVAL, "n must equal 3 nx ny nz");
-    const int64_t words = 3 * (int64_t)D.L[2] * D.L[1] * D.row_words;
-    std::vector<uint32_t> w(words);
-    CK(cudaMemcpyAsync(w.data(), b->occ + D.occ_word_off, sizeof(uint32_t) * words, cudaMemcpyDeviceToHost,
-                       b->st),
-       "state copy");
+    const int64_t rows = 3 * (int64_t)D.L[2] * D.L[1];
+    const int64_t chunk = std::min<int64_t>(rows, std::max<int64_t>(1, (int64_t)READ_BUF_MAX / D.L[0]));
+    uint8_t* buf = (uint8_t*)read_buffer(b, (size_t)(chunk * D.L[0]));
+    if (!buf) return fail(FKMC_ENOMEM, "device allocation failed (read-out)");
+    touch_pages(host_occ, n);
+    for (int64_t r0 = 0; r0 < rows; r0 += chunk) {
+        const int64_t nr = std::min(chunk, rows - r0);
+        CK(launch_unpack_state(D, b->occ, r0, nr, buf, b->st), "state kernel");
+        CK(cudaMemcpyAsync(host_occ + r0 * D.L[0], buf, (size_t)(nr * D.L[0]), cudaMemcpyDeviceToHost, b->st),
+           "state copy");
+    }
     CK(cudaStreamSynchronize(b->st), "synchronize");
-    int64_t s = 0;
-    for (int t = 0; t < 3; ++t)
-        for (int z = 0; z < D.L[2]; ++z)
-            for (int y = 0; y < D.L[1]; ++y) {
-                for (int x = 0; x < D.L[0]; ++x)
-                    host_occ[s++] = (uint8_t)((w[occ_index(D.row_words, D.L[1], t, x, y, z)] >> ((x & 15) * 2)) & 3u);
-            }
     return FKMC_OK;
 }
 
@@ -1751,6 +1782,31 @@ int kmc_read_records(kmc_batch* b, int32_t r, int64_t* rows, int64_t max_rows, i
     if (!valid_replica(b, r) || (!rows && max_rows > 0)) return fail(FKMC_EINVAL, "bad replica or output");
     const RepDesc& D = b->desc[r];
     const int64_t nfrag = (int64_t)D.nf[0] * D.nf[1] * D.nf[2];
+    // rows ordered on the device, as many as the replica has vacancies (a state that
+    // was uploaded with more records than that takes the host path below)
+    const int64_t want = std::min(std::max<int64_t>(max_rows, 0), b->n_vac[r]);
+    const size_t off_bytes = (sizeof(int64_t) * (size_t)(nfrag + 1) + 255) & ~(size_t)255;
+    const size_t need = off_bytes + sizeof(int64_t) * 6 * (size_t)want;
+    if (need <= READ_BUF_MAX) {
+        char* buf = (char*)read_buffer(b, need);
+        if (!buf) return fail(FKMC_ENOMEM, "device allocation failed (read-out)");
+        int64_t* off = (int64_t*)buf;
+        int64_t* d_rows = (int64_t*)(buf + off_bytes);
+        CK(launch_rows(D, b->recs, b->counts, b->cap, off, want, d_rows, b->st), "records kernel");
+        int64_t total = 0;
+        if (want > 0) {
+            touch_pages(rows, sizeof(int64_t) * 6 * (size_t)want);
+            CK(cudaMemcpyAsync(rows, d_rows, sizeof(int64_t) * 6 * (size_t)want, cudaMemcpyDeviceToHost, b->st),
+               "record copy");
+        }
+        CK(cudaMemcpyAsync(&total, off + nfrag, sizeof total, cudaMemcpyDeviceToHost, b->st), "record copy");
+        CK(cudaStreamSynchronize(b->st), "synchronize");
+        if (total <= want || want == max_rows || max_rows <= 0) {
+            for (int64_t k = 6 * total; k < 6 * want; ++k) rows[k] = 0;  // fewer records than vacancies
+            if (n_rows) *n_rows = total;
+            return FKMC_OK;
+        }
+    }
     std::vector<int32_t> cnt(nfrag);
     std::vector<VacRec> rec((size_t)nfrag * b->cap);
     CK(cudaMemcpyAsync(cnt.data(), b->counts + D.frag_base, sizeof(int32_t) * nfrag, cudaMemcpyDeviceToHost,
@@ -1794,6 +1850,7 @@ int kmc_read_tracer(kmc_batch* b, int32_t r, int32_t* host_disp, size_t n_sites)
     if (!b->tracer) return fail(FKMC_ESTATE, "tracer mode is off");
     const RepDesc& D = b->desc[r];
     if ((int64_t)n_sites != D.nsite) return fail(FKMC_EINVAL, "n_sites must equal 3 nx ny nz");
+    touch_pages(host_disp, sizeof(int32_t) * 3 * (size_t)D.nsite);
     CK(cudaMemcpyAsync(host_disp, b->tracer + 3 * D.site_off, sizeof(int32_t) * 3 * D.nsite,
                        cudaMemcpyDeviceToHost, b->st),
        "tracer copy");

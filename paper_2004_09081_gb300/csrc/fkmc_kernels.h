@@ -66,6 +66,12 @@ cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, in
                               VacRec* vac, uint32_t* types, uint32_t* occ, const uint8_t* gb,
                               unsigned long long* claims, int32_t* tracer, void* log_mem, double* theta,
                               unsigned long long* stats, uint32_t* status, cudaStream_t st);
+// read-outs: species codes of rows of the (t, z, y) order; record rows with their
+// offsets per fragment (offsets: fragments + 1 entries, the last the total)
+cudaError_t launch_unpack_state(const RepDesc& D, const uint32_t* occ, int64_t row0, int64_t rows, uint8_t* out,
+                                cudaStream_t st);
+cudaError_t launch_rows(const RepDesc& D, const VacRec* recs, const int32_t* counts, int cap, int64_t* offsets,
+                        int64_t max_rows, int64_t* rows, cudaStream_t st);
 cudaError_t launch_moments(const RepDesc& D, int species, const uint32_t* occ, const VacRec* recs,
                            const int32_t* counts, const int32_t* tracer, int cap,
                            unsigned long long* out, cudaStream_t st);

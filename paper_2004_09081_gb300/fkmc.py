@@ -245,10 +245,13 @@ def kmc_write_state(h, r: int, occ: np.ndarray):
 
 def kmc_read_records(h, r: int) -> np.ndarray:
     n = C.c_int64()
-    _check(load().kmc_read_records(h, r, None, 0, C.byref(n)))
-    out = np.zeros((max(n.value, 1), 6), np.int64)
-    _check(load().kmc_read_records(h, r, _ptr(out), n.value, C.byref(n)))
-    return out[: n.value]
+    room = max(kmc_get_replica_info(h, r).n_vac, 1)  # one record per vacancy
+    while True:
+        out = np.zeros((room, 6), np.int64)
+        _check(load().kmc_read_records(h, r, _ptr(out), room, C.byref(n)))
+        if n.value <= room:
+            return out[: n.value]
+        room = n.value
 
 
 def kmc_read_tracer(h, r: int, nsite: int) -> np.ndarray:
