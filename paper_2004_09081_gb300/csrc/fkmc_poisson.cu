@@ -58,10 +58,13 @@ __global__ void k_mg_rhs(const int32_t* cnt, int64_t n, double half_q, double ba
         f[i] = __dmul_rn(__dadd_rn(__dmul_rn(half_q, (double)cnt[i]), -background), scale);
 }
 
-// The level-by-level stencil kernels run on 3-D grids: blockIdx.y / blockIdx.z
-// are the row (y, z), threads walk x; all index arithmetic is 32-bit.  They are
-// templates over the number type: the V-cycle runs in FP32 (below, the FP64
-// defect correction around it), the final residual check in FP64.
+// The level-by-level stencil kernels run on 3-D grids of blocks of blockDim.x
+// columns and blockDim.y rows (256 threads, `tiles`), each thread NZ planes; all
+// index arithmetic is 32-bit.  They are templates over the number type: the
+// V-cycle runs in FP32 (below, the FP64 defect correction around it), the final
+// residual check in FP64.  A block per row of 128 threads, half of them without a
+// node in a red-black half-sweep, spent its time on starting 16,384 blocks: 10.8
+// us per half-sweep of 128^3, 10.9 per residual, 17 per prolongation.
 constexpr int XT = 128;
 constexpr double SIXTH = 1.0 / 6.0;
 
@@ -88,15 +91,20 @@ __device__ __forceinline__ T nb_sum(const T* v, int x, int y, int z, int nx, int
 
 // red-black Gauss-Seidel half-sweep over the nodes of one colour (all
 // dimensions even: the colouring is consistent across the periodic seams);
-// thread k of a row takes x = 2k + the row's colour offset
-template <typename T>
-__global__ void __launch_bounds__(XT) k_mg_rb(T* phi, const T* f, int nx, int ny, int nz, int colour)
+// column k of a row takes x = 2k + the row's colour offset
+template <typename T, int NZ>
+__global__ void __launch_bounds__(256) k_mg_rb(T* phi, const T* f, int nx, int ny, int nz, int colour)
 {
-    const int y = blockIdx.y, z = blockIdx.z;
-    const int x = 2 * (blockIdx.x * XT + threadIdx.x) + ((y + z + colour) & 1);
-    if (x >= nx) return;
-    const int i = (z * ny + y) * nx + x;
-    phi[i] = mul_rn(add_rn(f[i], nb_sum(phi, x, y, z, nx, ny, nz)), (T)SIXTH);
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (2 * k >= nx || y >= ny) return;
+#pragma unroll
+    for (int u = 0; u < NZ; ++u) {
+        const int z = blockIdx.z * NZ + u;
+        if (z >= nz) return;
+        const int x = 2 * k + ((y + z + colour) & 1);
+        const int i = (z * ny + y) * nx + x;
+        phi[i] = mul_rn(add_rn(f[i], nb_sum(phi, x, y, z, nx, ny, nz)), (T)SIXTH);
+    }
 }
 
 // damped Jacobi sweep, out = (1-w) in + w (f + sum nb) / 6
@@ -111,31 +119,65 @@ __global__ void __launch_bounds__(XT) k_mg_jacobi(const T* in, T* out, const T* 
 }
 
 // r = f - A phi
-template <typename T>
-__global__ void __launch_bounds__(XT) k_mg_residual(const T* phi, const T* f, T* r, int nx, int ny, int nz)
+template <typename T, int NZ>
+__global__ void __launch_bounds__(256) k_mg_residual(const T* phi, const T* f, T* r, int nx, int ny, int nz)
 {
-    const int y = blockIdx.y, z = blockIdx.z, x = blockIdx.x * XT + threadIdx.x;
-    if (x >= nx) return;
-    const int i = (z * ny + y) * nx + x;
-    r[i] = add_rn(f[i], -add_rn(mul_rn((T)6, phi[i]), -nb_sum(phi, x, y, z, nx, ny, nz)));
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= nx || y >= ny) return;
+#pragma unroll
+    for (int u = 0; u < NZ; ++u) {
+        const int z = blockIdx.z * NZ + u;
+        if (z >= nz) return;
+        const int i = (z * ny + y) * nx + x;
+        r[i] = add_rn(f[i], -add_rn(mul_rn((T)6, phi[i]), -nb_sum(phi, x, y, z, nx, ny, nz)));
+    }
+}
+
+// Conversions between FP32 and FP64 by integer instructions (an FP64-pipe
+// conversion costs as much as an FP64 add, and those bound the two kernels
+// below): the widening is exact, the narrowing rounds to nearest even; zeros,
+// denormals and overflows take the instruction.
+__device__ __forceinline__ double widen(float v)
+{
+    const uint32_t b = __float_as_uint(v);
+    const uint32_t e = (b >> 23) & 255u;
+    if (e == 0u || e == 255u) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t e = (hi >> 20) & 2047u;
+    if (e < 898u || e > 1149u) return __double2float_rn(v);
+    // 23 mantissa bits, the next one half a unit, the rest sticky
+    const uint32_t m = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+    const uint32_t half = (lo >> 28) & 1u, rest = (lo << 4) != 0u;
+    return __uint_as_float((hi & 0x80000000u) | (m + (half & (rest | (m & 1u)))));
 }
 
 // the defect of the FP64 potential, d = f - A phi in FP64, rounded to FP32: the
-// right-hand side of the FP32 correction cycle
-__global__ void __launch_bounds__(XT) k_mg_defect(const double* phi, const double* f, float* d, int nx, int ny,
-                                                   int nz)
+// right-hand side of the FP32 correction cycle.  Bound by the FP64 pipe: eight
+// instructions per node at 64 to 76 cycles per warp and SM quarter (33 us of 38
+// for 128^3).
+template <int NZ>
+__global__ void __launch_bounds__(256) k_mg_defect(const double* phi, const double* f, float* d, int nx, int ny, int nz)
 {
-    const int y = blockIdx.y, z = blockIdx.z, x = blockIdx.x * XT + threadIdx.x;
-    if (x >= nx) return;
-    const int i = (z * ny + y) * nx + x;
-    d[i] = __double2float_rn(__dadd_rn(f[i], -__dadd_rn(__dmul_rn(6.0, phi[i]), -nb_sum(phi, x, y, z, nx, ny, nz))));
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= nx || y >= ny) return;
+#pragma unroll
+    for (int u = 0; u < NZ; ++u) {
+        const int z = blockIdx.z * NZ + u;
+        if (z >= nz) return;
+        const int i = (z * ny + y) * nx + x;
+        d[i] = narrow(__dadd_rn(f[i], -__dadd_rn(__dmul_rn(6.0, phi[i]), -nb_sum(phi, x, y, z, nx, ny, nz))));
+    }
 }
 
 // phi += e (the FP32 correction, converted exactly)
 __global__ void k_mg_correct(double* phi, const float* e, int64_t n)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        phi[i] = __dadd_rn(phi[i], (double)e[i]);
+        phi[i] = __dadd_rn(phi[i], widen(e[i]));
 }
 
 // coarse f = 4 x full weighting of the fine residual (weights (1,2,1)^3 / 64);
@@ -160,21 +202,34 @@ __global__ void __launch_bounds__(XT) k_mg_restrict(const T* r, T* fc, int nx, i
     fc[(Z * cy + Y) * cx + X] = mul_rn(s, (T)(4.0 / 64.0));
 }
 
-// phi_fine += trilinear interpolation of the coarse correction
-template <typename T>
-__global__ void __launch_bounds__(XT) k_mg_prolong(const T* ec, T* phi, int nx, int ny, int nz)
+// phi_fine += trilinear interpolation of the coarse correction: a thread takes the
+// two fine nodes 2X and 2X + 1 of a row from the same coarse nodes
+template <typename T, int NZ>
+__global__ void __launch_bounds__(256) k_mg_prolong(const T* ec, T* phi, int nx, int ny, int nz)
 {
-    const int y = blockIdx.y, z = blockIdx.z, x = blockIdx.x * XT + threadIdx.x;
-    if (x >= nx) return;
+    const int X = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
     const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
-    const int X = x >> 1, Y = y >> 1, Z = z >> 1, ox = x & 1, oy = y & 1, oz = z & 1;
-    T s = 0;
-    for (int dz = 0; dz <= oz; ++dz)
-        for (int dy = 0; dy <= oy; ++dy)
-            for (int dx = 0; dx <= ox; ++dx)
-                s = add_rn(s, ec[(wrap_(Z + dz, cz) * cy + wrap_(Y + dy, cy)) * cx + wrap_(X + dx, cx)]);
-    const int i = (z * ny + y) * nx + x;
-    phi[i] = add_rn(phi[i], mul_rn(s, (T)(1.0 / (double)(1 << (ox + oy + oz)))));
+    if (X >= cx || y >= ny) return;
+    const int Y = y >> 1, oy = y & 1, X1 = X + 1 == cx ? 0 : X + 1;
+    const int Y1 = Y + 1 == cy ? 0 : Y + 1;
+#pragma unroll
+    for (int u = 0; u < NZ; ++u) {
+        const int z = blockIdx.z * NZ + u;
+        if (z >= nz) return;
+        const int Z = z >> 1, oz = z & 1, Z1 = Z + 1 == cz ? 0 : Z + 1;
+        T s0 = 0, s1 = 0;  // x = 2X, 2X + 1: coarse nodes in the order z, y, x
+        for (int dz = 0; dz <= oz; ++dz)
+            for (int dy = 0; dy <= oy; ++dy) {
+                const T* row = ec + ((dz ? Z1 : Z) * cy + (dy ? Y1 : Y)) * cx;
+                const T a = row[X], b = row[X1];
+                s0 = add_rn(s0, a);
+                s1 = add_rn(add_rn(s1, a), b);
+            }
+        const int i = (z * ny + y) * nx + 2 * X;
+        const T w0 = (T)(1.0 / (double)(1 << (oy + oz))), w1 = (T)(1.0 / (double)(2 << (oy + oz)));
+        phi[i] = add_rn(phi[i], mul_rn(s0, w0));
+        phi[i + 1] = add_rn(phi[i + 1], mul_rn(s1, w1));
+    }
 }
 
 // deterministic sum (or max |v|) in FP64: per-block partials (fixed grid), then
@@ -284,8 +339,11 @@ __device__ __forceinline__ T s_nb(const T* v, int x, int y, int z, int nx, int n
     return s;
 }
 
-template <typename T>
-__device__ void s_smooth(const SmallLevels& P, int l, T* phi, const T* f, T* tmp, int sweeps)
+// The steps of the levels in shared memory by NTH threads (tid 0 .. NTH - 1), `sync`
+// between them.
+template <int NTH, typename T, typename Sync>
+__device__ __forceinline__ void s_smooth(const SmallLevels& P, int l, T* phi, const T* f, T* tmp, int sweeps, int tid,
+                                         Sync sync)
 {
     const int nx = P.dim[l][0], ny = P.dim[l][1], nz = P.dim[l][2];
     const int n = nx * ny * nz;
@@ -295,18 +353,89 @@ __device__ void s_smooth(const SmallLevels& P, int l, T* phi, const T* f, T* tmp
         for (int half = 0; half < 2; ++half) {
             const T* in = even ? phi : (half == 0 ? phi : tmp);
             T* out = even ? phi : (half == 0 ? tmp : phi);
-            for (int i = threadIdx.x; i < n; i += ST) {
-                int x, y, z;
-                s_coords(P, l, i, x, y, z);
-                if (even && ((x + y + z) & 1) != half) continue;
-                const T gs = mul_rn(add_rn(f[i], s_nb(in, x, y, z, nx, ny, nz)), (T)SIXTH);
-                out[i] = even ? gs : add_rn(mul_rn((T)1 - w, in[i]), mul_rn(w, gs));
+            if (even) {  // node k of a half-sweep: x = 2 (k mod nx/2) + the row's offset
+                for (int i = tid; i < n / 2; i += NTH) {
+                    int x, y, z;
+                    s_coords(P, l, 2 * i, x, y, z);
+                    x += (y + z + half) & 1;
+                    const int at = (z * ny + y) * nx + x;
+                    out[at] = mul_rn(add_rn(f[at], s_nb(in, x, y, z, nx, ny, nz)), (T)SIXTH);
+                }
+            } else {
+                for (int i = tid; i < n; i += NTH) {
+                    int x, y, z;
+                    s_coords(P, l, i, x, y, z);
+                    const T gs = mul_rn(add_rn(f[i], s_nb(in, x, y, z, nx, ny, nz)), (T)SIXTH);
+                    out[i] = add_rn(mul_rn((T)1 - w, in[i]), mul_rn(w, gs));
+                }
             }
-            __syncthreads();
+            sync();
         }
     }
 }
 
+// down from level l: pre-smooth, residual, restrict
+template <int NTH, typename T, typename Sync>
+__device__ __forceinline__ void s_down(const SmallLevels& P, int l, T* phi_all, T* f_all, T* r_all, int tid, Sync sync)
+{
+    const int nx = P.dim[l][0], ny = P.dim[l][1], nz = P.dim[l][2];
+    const int n = nx * ny * nz;
+    T* phi = phi_all + P.offs[l];
+    const T* f = f_all + P.offs[l];
+    T* r = r_all + P.offs[l];
+    s_smooth<NTH>(P, l, phi, f, r, 2, tid, sync);
+    for (int i = tid; i < n; i += NTH) {
+        int x, y, z;
+        s_coords(P, l, i, x, y, z);
+        r[i] = add_rn(f[i], -add_rn(mul_rn((T)6, phi[i]), -s_nb(phi, x, y, z, nx, ny, nz)));
+    }
+    sync();
+    const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
+    T* fc = f_all + P.offs[l + 1];
+    T* pc = phi_all + P.offs[l + 1];
+    for (int i = tid; i < cx * cy * cz; i += NTH) {
+        int X, Y, Z;
+        s_coords(P, l + 1, i, X, Y, Z);
+        T s = 0;
+        for (int dz = -1; dz <= 1; ++dz)
+            for (int dy = -1; dy <= 1; ++dy)
+                for (int dx = -1; dx <= 1; ++dx) {
+                    const T w = (T)((2 - (dx != 0)) * (2 - (dy != 0)) * (2 - (dz != 0)));
+                    s = add_rn(s, mul_rn(w, r[nidx(wrap_(2 * X + dx, nx), wrap_(2 * Y + dy, ny), wrap_(2 * Z + dz, nz),
+                                                   nx, ny)]));
+                }
+        fc[i] = mul_rn(s, (T)(4.0 / 64.0));
+        pc[i] = 0;
+    }
+    sync();
+}
+
+// up to level l: prolong, post-smooth
+template <int NTH, typename T, typename Sync>
+__device__ __forceinline__ void s_up(const SmallLevels& P, int l, T* phi_all, const T* f_all, T* r_all, int tid,
+                                     Sync sync)
+{
+    const int nx = P.dim[l][0], ny = P.dim[l][1];
+    const int n = nx * ny * P.dim[l][2], cx = nx / 2, cy = ny / 2, cz = P.dim[l][2] / 2;
+    T* phi = phi_all + P.offs[l];
+    const T* ec = phi_all + P.offs[l + 1];
+    for (int i = tid; i < n; i += NTH) {
+        int x, y, z;
+        s_coords(P, l, i, x, y, z);
+        const int X = x >> 1, Y = y >> 1, Z = z >> 1, ox = x & 1, oy = y & 1, oz = z & 1;
+        T s = 0;
+        for (int dz = 0; dz <= oz; ++dz)
+            for (int dy = 0; dy <= oy; ++dy)
+                for (int dx = 0; dx <= ox; ++dx)
+                    s = add_rn(s, ec[nidx(wrap_(X + dx, cx), wrap_(Y + dy, cy), wrap_(Z + dz, cz), cx, cy)]);
+        phi[i] = add_rn(phi[i], mul_rn(s, (T)(1.0 / (double)(1 << (ox + oy + oz)))));
+    }
+    sync();
+    s_smooth<NTH>(P, l, phi, f_all + P.offs[l], r_all + P.offs[l], 2, tid, sync);
+}
+
+// The levels of at most 64 nodes run in the block's first warp: their steps are
+// too short to pay for a block barrier each.
 template <typename T>
 __global__ void __launch_bounds__(ST) k_mg_small(SmallLevels P, T* phi_g, const T* f_g)
 {
@@ -315,84 +444,56 @@ __global__ void __launch_bounds__(ST) k_mg_small(SmallLevels P, T* phi_g, const 
     T* f_all = phi_all + P.nodes;
     T* r_all = phi_all + 2 * P.nodes;
     __shared__ double red[ST];
+    const int tid = threadIdx.x;
     const int last = P.levels - 1;
+    auto nodes = [&](int l) { return P.dim[l][0] * P.dim[l][1] * P.dim[l][2]; };
+    auto block = [] { __syncthreads(); };
+    auto warp = [] { __syncwarp(); };
     {
-        const int n0 = P.dim[P.ls][0] * P.dim[P.ls][1] * P.dim[P.ls][2];
-        for (int i = threadIdx.x; i < n0; i += ST) {
+        const int n0 = nodes(P.ls);
+        for (int i = tid; i < n0; i += ST) {
             phi_all[i] = phi_g[P.off_ls + i];  // the iterate so far (zero below the finest level)
             f_all[i] = f_g[P.off_ls + i];
         }
         __syncthreads();
     }
-    for (int l = P.ls; l < last; ++l) {  // down: pre-smooth, residual, restrict
-        const int nx = P.dim[l][0], ny = P.dim[l][1], nz = P.dim[l][2];
-        const int n = nx * ny * nz;
-        T* phi = phi_all + P.offs[l];
-        const T* f = f_all + P.offs[l];
-        T* r = r_all + P.offs[l];
-        s_smooth(P, l, phi, f, r, 2);
-        for (int i = threadIdx.x; i < n; i += ST) {
-            int x, y, z;
-            s_coords(P, l, i, x, y, z);
-            r[i] = add_rn(f[i], -add_rn(mul_rn((T)6, phi[i]), -s_nb(phi, x, y, z, nx, ny, nz)));
+    int lw = P.ls;  // first level of the warp's
+    while (lw <= last && nodes(lw) > 64) ++lw;
+    for (int l = P.ls; l < min(lw, last); ++l) s_down<ST>(P, l, phi_all, f_all, r_all, tid, block);
+    // coarsest: zero-mean right-hand side (tree sum in FP64, fixed order), sweeps
+    T* f = f_all + P.offs[last];
+    const int n = nodes(last);
+    if (lw <= last) {
+        if (tid < 32) {
+            for (int l = lw; l < last; ++l) s_down<32>(P, l, phi_all, f_all, r_all, tid, warp);
+            double s = tid < n ? (double)f[tid] : 0.0;
+            if (n > 32) s = __dadd_rn(s, tid + 32 < n ? (double)f[tid + 32] : 0.0);
+            for (int w = 16; w; w >>= 1) s = __dadd_rn(s, __shfl_down_sync(0xffffffffu, s, w));
+            s = __shfl_sync(0xffffffffu, s, 0);
+            const T m = (T)__ddiv_rn(s, (double)n);
+            for (int i = tid; i < n; i += 32) f[i] = add_rn(f[i], -m);
+            __syncwarp();
+            s_smooth<32>(P, last, phi_all + P.offs[last], (const T*)f, r_all + P.offs[last], P.coarse_sweeps, tid, warp);
+            for (int l = last - 1; l >= lw; --l) s_up<32>(P, l, phi_all, (const T*)f_all, r_all, tid, warp);
         }
         __syncthreads();
-        const int cx = nx / 2, cy = ny / 2, cz = nz / 2;
-        T* fc = f_all + P.offs[l + 1];
-        T* pc = phi_all + P.offs[l + 1];
-        for (int i = threadIdx.x; i < cx * cy * cz; i += ST) {
-            int X, Y, Z;
-            s_coords(P, l + 1, i, X, Y, Z);
-            T s = 0;
-            for (int dz = -1; dz <= 1; ++dz)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        const T w = (T)((2 - (dx != 0)) * (2 - (dy != 0)) * (2 - (dz != 0)));
-                        s = add_rn(s, mul_rn(w, r[nidx(wrap_(2 * X + dx, nx), wrap_(2 * Y + dy, ny),
-                                                       wrap_(2 * Z + dz, nz), nx, ny)]));
-                    }
-            fc[i] = mul_rn(s, (T)(4.0 / 64.0));
-            pc[i] = 0;
-        }
-        __syncthreads();
-    }
-    {  // coarsest: zero-mean right-hand side (block tree sum in FP64, fixed order), sweeps
-        const int n = P.dim[last][0] * P.dim[last][1] * P.dim[last][2];
-        T* f = f_all + P.offs[last];
+    } else {
         double s = 0.0;
-        for (int i = threadIdx.x; i < n; i += ST) s = __dadd_rn(s, (double)f[i]);
-        red[threadIdx.x] = s;
+        for (int i = tid; i < n; i += ST) s = __dadd_rn(s, (double)f[i]);
+        red[tid] = s;
         __syncthreads();
         for (int w = ST / 2; w; w >>= 1) {
-            if (threadIdx.x < w) red[threadIdx.x] = __dadd_rn(red[threadIdx.x], red[threadIdx.x + w]);
+            if (tid < w) red[tid] = __dadd_rn(red[tid], red[tid + w]);
             __syncthreads();
         }
         const T m = (T)__ddiv_rn(red[0], (double)n);
-        for (int i = threadIdx.x; i < n; i += ST) f[i] = add_rn(f[i], -m);
+        for (int i = tid; i < n; i += ST) f[i] = add_rn(f[i], -m);
         __syncthreads();
-        s_smooth(P, last, phi_all + P.offs[last], (const T*)f, r_all + P.offs[last], P.coarse_sweeps);
+        s_smooth<ST>(P, last, phi_all + P.offs[last], (const T*)f, r_all + P.offs[last], P.coarse_sweeps, tid, block);
     }
-    for (int l = last - 1; l >= P.ls; --l) {  // up: prolong, post-smooth
-        const int nx = P.dim[l][0], ny = P.dim[l][1];
-        const int n = nx * ny * P.dim[l][2], cx = nx / 2, cy = ny / 2, cz = P.dim[l][2] / 2;
-        T* phi = phi_all + P.offs[l];
-        const T* ec = phi_all + P.offs[l + 1];
-        for (int i = threadIdx.x; i < n; i += ST) {
-            int x, y, z;
-            s_coords(P, l, i, x, y, z);
-            const int X = x >> 1, Y = y >> 1, Z = z >> 1, ox = x & 1, oy = y & 1, oz = z & 1;
-            T s = 0;
-            for (int dz = 0; dz <= oz; ++dz)
-                for (int dy = 0; dy <= oy; ++dy)
-                    for (int dx = 0; dx <= ox; ++dx)
-                        s = add_rn(s, ec[nidx(wrap_(X + dx, cx), wrap_(Y + dy, cy), wrap_(Z + dz, cz), cx, cy)]);
-            phi[i] = add_rn(phi[i], mul_rn(s, (T)(1.0 / (double)(1 << (ox + oy + oz)))));
-        }
-        __syncthreads();
-        s_smooth(P, l, phi, (const T*)(f_all + P.offs[l]), r_all + P.offs[l], 2);
-    }
-    const int n0 = P.dim[P.ls][0] * P.dim[P.ls][1] * P.dim[P.ls][2];
-    for (int i = threadIdx.x; i < n0; i += ST) phi_g[P.off_ls + i] = phi_all[i];
+    for (int l = min(lw, last) - 1; l >= P.ls; --l) s_up<ST>(P, l, phi_all, (const T*)f_all, r_all, tid, block);
+    const int n0 = nodes(P.ls);
+    for (int i = tid; i < n0; i += ST) phi_g[P.off_ls + i] = phi_all[i];
 }
 
 }  // namespace
@@ -422,6 +523,46 @@ static bool level_even(const MgPlan& p, int l)
     return p.dim[l][0] % 2 == 0 && p.dim[l][1] % 2 == 0 && p.dim[l][2] % 2 == 0;
 }
 
+// blocks of `columns` x rows, and the grid that covers columns x ny x nz with NZ planes per thread
+static dim3 tile_block(int columns)
+{
+    int bx = 8;
+    while (bx < 64 && bx < columns) bx *= 2;
+    return dim3((unsigned)bx, (unsigned)(256 / bx));
+}
+static dim3 tiles(int columns, int ny, int nz, int planes)
+{
+    const dim3 b = tile_block(columns);
+    return dim3((unsigned)((columns + b.x - 1) / b.x), (unsigned)((ny + b.y - 1) / b.y),
+                (unsigned)((nz + planes - 1) / planes));
+}
+// four planes per thread where that still leaves several blocks per SM (2^20 nodes), else one
+static bool deep(int nx, int ny, int nz) { return (int64_t)nx * ny * nz >= (1 << 20); }
+
+template <typename T>
+static void rb(T* u, const T* f, int nx, int ny, int nz, int colour, cudaStream_t st)
+{
+    if (deep(nx, ny, nz)) k_mg_rb<T, 4><<<tiles(nx / 2, ny, nz, 4), tile_block(nx / 2), 0, st>>>(u, f, nx, ny, nz, colour);
+    else k_mg_rb<T, 1><<<tiles(nx / 2, ny, nz, 1), tile_block(nx / 2), 0, st>>>(u, f, nx, ny, nz, colour);
+}
+template <typename T>
+static void residual(const T* u, const T* f, T* r, int nx, int ny, int nz, cudaStream_t st)
+{
+    if (deep(nx, ny, nz)) k_mg_residual<T, 4><<<tiles(nx, ny, nz, 4), tile_block(nx), 0, st>>>(u, f, r, nx, ny, nz);
+    else k_mg_residual<T, 1><<<tiles(nx, ny, nz, 1), tile_block(nx), 0, st>>>(u, f, r, nx, ny, nz);
+}
+template <typename T>
+static void prolong(const T* ec, T* u, int nx, int ny, int nz, cudaStream_t st)
+{
+    if (deep(nx, ny, nz)) k_mg_prolong<T, 4><<<tiles(nx / 2, ny, nz, 4), tile_block(nx / 2), 0, st>>>(ec, u, nx, ny, nz);
+    else k_mg_prolong<T, 1><<<tiles(nx / 2, ny, nz, 1), tile_block(nx / 2), 0, st>>>(ec, u, nx, ny, nz);
+}
+static void defect(const double* phi, const double* f, float* d, int nx, int ny, int nz, cudaStream_t st)
+{
+    if (deep(nx, ny, nz)) k_mg_defect<4><<<tiles(nx, ny, nz, 4), tile_block(nx), 0, st>>>(phi, f, d, nx, ny, nz);
+    else k_mg_defect<1><<<tiles(nx, ny, nz, 1), tile_block(nx), 0, st>>>(phi, f, d, nx, ny, nz);
+}
+
 static dim3 rows(int nx_threads, int ny, int nz) { return dim3((unsigned)((nx_threads + XT - 1) / XT), ny, nz); }
 
 // `sweeps` smoothing sweeps of level l on the level-stacked arrays u (iterate), f
@@ -435,8 +576,8 @@ static void smooth(const MgPlan& p, int l, T* u, const T* f, T* tmp, int sweeps,
     tmp += p.off[l];
     for (int k = 0; k < sweeps; ++k) {
         if (level_even(p, l)) {
-            k_mg_rb<T><<<rows(nx / 2, ny, nz), XT, 0, st>>>(u, f, nx, ny, nz, 0);
-            k_mg_rb<T><<<rows(nx / 2, ny, nz), XT, 0, st>>>(u, f, nx, ny, nz, 1);
+            rb(u, f, nx, ny, nz, 0, st);
+            rb(u, f, nx, ny, nz, 1, st);
         } else {  // two Jacobi half-steps through the scratch level buffer
             k_mg_jacobi<T><<<rows(nx, ny, nz), XT, 0, st>>>(u, tmp, f, nx, ny, nz, (T)(6.0 / 7.0));
             k_mg_jacobi<T><<<rows(nx, ny, nz), XT, 0, st>>>(tmp, u, f, nx, ny, nz, (T)(6.0 / 7.0));
@@ -515,12 +656,12 @@ static void vcycle(const MgPlan& p, int l, float* u, float* f, float* r, const M
         return;
     }
     smooth(p, l, u, f, r, 2, st);
-    k_mg_residual<float><<<rows(nx, ny, nz), XT, 0, st>>>(u + p.off[l], f + p.off[l], r + p.off[l], nx, ny, nz);
+    residual<float>(u + p.off[l], f + p.off[l], r + p.off[l], nx, ny, nz, st);
     const int64_t nc = (int64_t)p.dim[l + 1][0] * p.dim[l + 1][1] * p.dim[l + 1][2];
     k_mg_restrict<float><<<rows(nx / 2, ny / 2, nz / 2), XT, 0, st>>>(r + p.off[l], f + p.off[l + 1], nx, ny, nz);
     cudaMemsetAsync(u + p.off[l + 1], 0, sizeof(float) * nc, st);
     vcycle(p, l + 1, u, f, r, b, st);
-    k_mg_prolong<float><<<rows(nx, ny, nz), XT, 0, st>>>(u + p.off[l + 1], u + p.off[l], nx, ny, nz);
+    prolong<float>(u + p.off[l + 1], u + p.off[l], nx, ny, nz, st);
     smooth(p, l, u, f, r, 2, st);
 }
 
@@ -533,7 +674,7 @@ static void mixed_cycle(const MgPlan& p, const MgBuffers& b, cudaStream_t st)
 {
     const int nx = p.dim[0][0], ny = p.dim[0][1], nz = p.dim[0][2];
     const int64_t n = (int64_t)nx * ny * nz;
-    k_mg_defect<<<rows(nx, ny, nz), XT, 0, st>>>(b.phi, b.f, b.g, nx, ny, nz);
+    defect(b.phi, b.f, b.g, nx, ny, nz, st);
     cudaMemsetAsync(b.e, 0, sizeof(float) * n, st);
     vcycle(p, 0, b.e, b.g, b.s, b, st);
     k_mg_correct<<<grid_for(n), PT, 0, st>>>(b.phi, b.e, n);
@@ -569,8 +710,7 @@ cudaError_t elec_solve(const RepDesc& D, const VacRec* recs, const int32_t* coun
         if (e != cudaSuccess) return e;
     }
     if (resid_rel) {  // max |f - A phi| / max |f|, all in FP64
-        k_mg_residual<double><<<rows(p.dim[0][0], p.dim[0][1], p.dim[0][2]), XT, 0, st>>>(
-            b.phi, b.f, b.r, p.dim[0][0], p.dim[0][1], p.dim[0][2]);
+        residual<double>(b.phi, b.f, b.r, p.dim[0][0], p.dim[0][1], p.dim[0][2], st);
         k_mg_partial<double><<<MG_PARTIALS, PT, 0, st>>>(b.r, n, b.part, 1);
         k_mg_final<<<1, 32, 0, st>>>(b.part, MG_PARTIALS, b.scalar, 1);
         k_mg_partial<double><<<MG_PARTIALS, PT, 0, st>>>(b.f, n, b.part, 1);
