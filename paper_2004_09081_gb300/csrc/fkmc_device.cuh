@@ -262,7 +262,7 @@ __device__ __forceinline__ uint64_t window_bits(double theta, int F)
 }
 
 // FP64 bits of the clock after the event, from either form of the clock before it
-inline __device__ __noinline__ uint64_t mixed_clock_fp64(uint64_t clock, bool fp, float ratio, uint64_t th)
+__device__ __forceinline__ uint64_t mixed_clock_fp64(uint64_t clock, bool fp, float ratio, uint64_t th)
 {
     double c = __longlong_as_double((long long)clock);
     if (!fp && clock != 0)  // clock 2^(e-52), e + 1023 = th >> 52

@@ -166,25 +166,43 @@ template <bool GRAIN = false>
 __device__ __forceinline__ void compute_types(const RepDesc& D, const uint32_t* occ, const WarpSmem& S,
                                               int nslots, int nch, int lane, const uint8_t* gb = nullptr)
 {
-    for (int c = 0; c < nch; ++c) {
-        const int e = c * 32 + lane;
-        const int m = e >> 3, n = e & 7;
-        int ty = -1;
-        if (m < nslots && S.alive[m]) {
-            int t, x, y, z;
-            split_key(S.rec[S.order[m]].key, t, x, y, z);
-            const NbEntry nb = nb_entry(t, n);
-            const int jx = wrapc(x + nb.dc[0], D.L[0]);
-            const int jy = wrapc(y + nb.dc[1], D.L[1]);
-            const int jz = wrapc(z + nb.dc[2], D.L[2]);
-            const uint32_t w = __ldcg(occ + occ_word(D, nb.t2, jx, jy, jz));
-            const int code = (int)((w >> occ_shift(jx)) & 3u);
-            ty = code == SP_V ? -1 : code * 3 + nb.d[2] + 1;
-            if constexpr (GRAIN) {  // a hop touching a boundary cell takes the raised table
-                if (ty >= 0 && (gb[cell_index(D, x, y, z)] | gb[cell_index(D, jx, jy, jz)])) ty += 6;
+    // four chunks at a time, their reads issued before any is used: a dense
+    // fragment's visit is a chain of memory latencies, one per group instead of
+    // one per chunk
+    for (int c0 = 0; c0 < nch; c0 += 4) {
+        uint32_t w[4];
+        int sh[4], dz[4];
+        bool live[4], raised[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = (c0 + u) * 32 + lane;
+            const int m = e >> 3, n = e & 7;
+            live[u] = c0 + u < nch && m < nslots && S.alive[m];
+            w[u] = 0u;
+            sh[u] = dz[u] = 0;
+            raised[u] = false;
+            if (live[u]) {
+                int t, x, y, z;
+                split_key(S.rec[S.order[m]].key, t, x, y, z);
+                const NbEntry nb = nb_entry(t, n);
+                const int jx = wrapc(x + nb.dc[0], D.L[0]);
+                const int jy = wrapc(y + nb.dc[1], D.L[1]);
+                const int jz = wrapc(z + nb.dc[2], D.L[2]);
+                w[u] = __ldcg(occ + occ_word(D, nb.t2, jx, jy, jz));
+                sh[u] = occ_shift(jx);
+                dz[u] = nb.d[2];
+                if constexpr (GRAIN)  // a hop touching a boundary cell takes the raised table
+                    raised[u] = (gb[cell_index(D, x, y, z)] | gb[cell_index(D, jx, jy, jz)]) != 0;
             }
         }
-        S.types[e] = (int8_t)ty;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (c0 + u >= nch) break;
+            const int code = (int)((w[u] >> sh[u]) & 3u);
+            int ty = -1;
+            if (live[u] && code != SP_V) ty = code * 3 + dz[u] + 1 + (raised[u] ? 6 : 0);
+            S.types[(c0 + u) * 32 + lane] = (int8_t)ty;
+        }
     }
 }
 
@@ -895,6 +913,24 @@ __global__ void __launch_bounds__(128, 8) k_run_small(const RepDesc* __restrict_
 // (dc_z+1) << 6; z = 2 bits per neighbour: d_z + 1.
 __device__ __align__(16) uint4 g_lgeo[3];
 
+// what the one-thread-per-fragment passes keep in shared memory of a batch of one replica
+struct LaneTables {
+    RepDesc D;
+    uint4 geo[3];
+};
+
+template <bool ONE>
+__device__ __forceinline__ void load_tables(LaneTables& tab, const RepDesc* descs)
+{
+    if constexpr (ONE) {
+        static_assert(sizeof(RepDesc) % 8 == 0, "copied as 64-bit words");
+        for (int k = threadIdx.x; k < (int)(sizeof(RepDesc) / 8); k += blockDim.x)
+            reinterpret_cast<uint64_t*>(&tab.D)[k] = reinterpret_cast<const uint64_t*>(descs)[k];
+        if (threadIdx.x < 3) tab.geo[threadIdx.x] = g_lgeo[threadIdx.x];
+        __syncthreads();
+    }
+}
+
 // Rate types of the 8 events of the vacancy at `key` (mixed form), packed as
 // nibbles n = type + 1 (0: no event), and the sum of their fixed-point rates.
 // The 8 neighbour words are read from L2 (ld.global.cg: this thread's own
@@ -902,12 +938,12 @@ __device__ __align__(16) uint4 g_lgeo[3];
 // faces no coordinate wraps, and a neighbour's row is the vacancy's row plus
 // a 32-bit offset.
 template <bool GRAIN>
-__device__ __forceinline__ uint32_t lane_types(const RepDesc& D, const uint32_t* occ, const uint8_t* gb, uint64_t key,
-                                               unsigned long long& sum)
+__device__ __forceinline__ uint32_t lane_types(const RepDesc& D, const uint4* lgeo, const uint32_t* occ,
+                                               const uint8_t* gb, uint64_t key, unsigned long long& sum)
 {
     int t, x, y, z;
     split_key(key, t, x, y, z);
-    const uint4 geo = __ldg(g_lgeo + t);
+    const uint4 geo = lgeo[t];
     const uint64_t g8 = ((uint64_t)geo.y << 32) | geo.x;
     const int L0 = D.L[0], L1 = D.L[1], L2 = D.L[2];
     const uint32_t* occ_r = occ + D.occ_word_off;
@@ -1016,8 +1052,16 @@ __device__ __forceinline__ void order_pair(VacRec& a, VacRec& b)
 // the trajectory is the same.  After a hop only the moved vacancy and those
 // within a half-cell of its old or new site re-read their neighbour words;
 // every other rate is unchanged.
-template <bool GRAIN>
-__global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict__ descs, int nrep,
+// ONE: the batch holds one replica, whose descriptor and the neighbour table are
+// copied to shared memory: read through the L1 they compete with the lattice for
+// it, and a wait for them is a wait for memory (bias cube of 1300^3 cells, persistent
+// form: 346 -> 333 us per colour phase).
+// What bounds both forms is issue: 0.4 instructions per cycle and SM quarter for 3
+// to 4 warps at about 10 cycles each, 8 of 32 lanes active; DRAM is at 10-15%.
+// Choosing each turn the step most lanes are ready for was 5% slower, six blocks per
+// SM (80 registers) 23%: the shared memory they take is the L1's.
+template <bool GRAIN, bool ONE>
+__global__ void __launch_bounds__(128, 4) k_run_lane_reg(const RepDesc* __restrict__ descs_g, int nrep,
                                                       int64_t total_items, int phase, const unsigned long long* wctl,
                                                       const uint32_t* __restrict__ perms,
                                                       const uint8_t* __restrict__ cls, uint32_t* occ, VacRec* recs,
@@ -1026,6 +1070,10 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
 {
     constexpr int NL = LANE_REG_MAX_V;
     constexpr unsigned FULL = 0xffffffffu;
+    __shared__ LaneTables tab;
+    load_tables<ONE>(tab, descs_g);
+    const RepDesc* const descs = ONE ? &tab.D : descs_g;
+    const uint4* const lgeo = ONE ? tab.geo : g_lgeo;
     const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int rep = -1;
     int64_t fid = 0;
@@ -1074,7 +1122,7 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
 #pragma unroll
         for (int k = 0; k < NL; ++k) {
             sm[k] = 0ull;
-            ty[k] = k < nv ? lane_types<GRAIN>(D, occ, gb, r[k].key, sm[k]) : 0u;
+            ty[k] = k < nv ? lane_types<GRAIN>(D, lgeo, occ, gb, r[k].key, sm[k]) : 0u;
         }
         const uint64_t w = D.window + wctl[1];
         const uint64_t k1 = key_word(D.replica, PURPOSE_HOP);
@@ -1165,14 +1213,14 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
             cur.key = make_key(nb.t2, jx, jy, jz);
             const bool owned = jx >= lo_c[0] && jx < hi_c[0] && jy >= lo_c[1] && jy < hi_c[1] && jz >= lo_c[2] &&
                                jz < hi_c[2];
+            int64_t out_g = 0;
+            int out_slot = -1;
             if (!owned) {
                 const int gx = frag_of(jx, D.base[0], D.rem[0]);
                 const int gy = frag_of(jy, D.base[1], D.rem[1]);
                 const int gz = frag_of(jz, D.base[2], D.rem[2]);
-                const int64_t g2 = D.frag_base + ((int64_t)gz * D.nf[1] + gy) * D.nf[0] + gx;
-                const int slot = atomicAdd(counts + g2, 1);
-                if (slot < cap) recs[g2 * cap + slot] = cur;
-                else atomicOr(status, STATUS_OVERFLOW);
+                out_g = D.frag_base + ((int64_t)gz * D.nf[1] + gy) * D.nf[0] + gx;
+                out_slot = atomicAdd(counts + out_g, 1);  // used after the rates' reads below
                 alive &= ~(1u << m);
                 ++nhand;
             }
@@ -1202,13 +1250,17 @@ __global__ void __launch_bounds__(128) k_run_lane_reg(const RepDesc* __restrict_
                 for (int q = 1; q < NL; ++q)
                     if (q == k) kk = r[q].key;
                 unsigned long long sk = 0ull;
-                const uint32_t tk = lane_types<GRAIN>(D, occ, gb, kk, sk);
+                const uint32_t tk = lane_types<GRAIN>(D, lgeo, occ, gb, kk, sk);
 #pragma unroll
                 for (int q = 0; q < NL; ++q)
                     if (q == k) {
                         ty[q] = tk;
                         sm[q] = sk;
                     }
+            }
+            if (!owned) {
+                if (out_slot < cap) recs[out_g * cap + out_slot] = cur;
+                else atomicOr(status, STATUS_OVERFLOW);
             }
         }
         hops = (uint32_t)i;
@@ -1309,8 +1361,8 @@ __device__ __forceinline__ uint64_t shfl_u64(uint64_t v, int src)
 // i, 3 and 2 for odd i); the window test, selection and exchange are the same.
 // After a hop only the moved vacancy and those within a half-cell of its old
 // or new site re-read their neighbour words; every other rate is unchanged.
-template <bool GRAIN>
-__global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __restrict__ descs, int nrep,
+template <bool GRAIN, bool ONE>
+__global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __restrict__ descs_g, int nrep,
                                                            int64_t total_items, int phase, unsigned long long* wctl,
                                                            const uint32_t* __restrict__ perms, ActEntry* act,
                                                            int32_t* act_count, uint32_t* occ, VacRec* recs,
@@ -1322,6 +1374,10 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
     static_assert(NL <= 8, "slot order packs 8 slot indices of 4 bits");
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ LaneSlots S;
+    __shared__ LaneTables tab;
+    load_tables<ONE>(tab, descs_g);
+    const RepDesc* const descs = ONE ? &tab.D : descs_g;
+    const uint4* const lgeo = ONE ? tab.geo : g_lgeo;
     const int tid = threadIdx.x, lane = tid & 31;
     const unsigned below = (1u << lane) - 1u;
     const uint64_t wk = wctl[1];
@@ -1482,7 +1538,7 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
             const int k = __ffs(pending) - 1;
             pending &= pending - 1u;
             unsigned long long sk;
-            S.ty[k][tid] = lane_types<GRAIN>(D, occ, gb, S.key[k][tid], sk);
+            S.ty[k][tid] = lane_types<GRAIN>(D, lgeo, occ, gb, S.key[k][tid], sk);
             S.sum[k][tid] = sk;
         }
 
@@ -2107,7 +2163,17 @@ using LaneRegFn = void (*)(const RepDesc*, int, int64_t, int, const unsigned lon
                            const uint8_t*, uint32_t*, VacRec*, int32_t*, int32_t*, unsigned long long*, uint32_t*, int,
                            const uint8_t*);
 
-static LaneFn lane_kernel(bool grain) { return grain ? k_run_lane<true> : k_run_lane<false>; }
+static LaneFn lane_kernel(bool grain, bool one)
+{
+    if (one) return grain ? k_run_lane<true, true> : k_run_lane<false, true>;
+    return grain ? k_run_lane<true, false> : k_run_lane<false, false>;
+}
+
+static LaneRegFn lane_reg_kernel(bool grain, bool one)
+{
+    if (one) return grain ? k_run_lane_reg<true, true> : k_run_lane_reg<false, true>;
+    return grain ? k_run_lane_reg<true, false> : k_run_lane_reg<false, false>;
+}
 
 using SmallFn = void (*)(const RepDesc*, const ActEntry*, int64_t, const int32_t*, int, const unsigned long long*,
                         uint32_t*, VacRec*, int32_t*, int32_t*, unsigned long long*, uint32_t*, int, const uint8_t*);
@@ -2156,7 +2222,7 @@ cudaError_t small_pass_blocks(int prec, bool grain, int lane, int* blocks)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) {
         if (lane == LANE_PERSISTENT)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lane_kernel(grain), LANE_THREADS, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lane_kernel(grain, false), LANE_THREADS, 0);
         else
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, small_kernel(prec, grain), 128, 0);
     }
@@ -2185,8 +2251,8 @@ cudaError_t launch_window(int prec, const RepDesc* d_descs, int nrep, int64_t to
     const int lane = split_pass && !site && prec == 1 ? lane_form : LANE_NONE;
     const int split = !split_pass || site ? 0 : (lane == LANE_REGISTERS ? 2 : (lane == LANE_NONE ? 1 : 0));
     const SmallFn small = small_kernel(prec, grain);
-    const LaneFn lanek = lane_kernel(grain);
-    const LaneRegFn lanereg = grain ? k_run_lane_reg<true> : k_run_lane_reg<false>;
+    const LaneFn lanek = lane_kernel(grain, nrep == 1);
+    const LaneRegFn lanereg = lane_reg_kernel(grain, nrep == 1);
     for (int p = 0; p < 8; ++p) {
         if (lane == LANE_PERSISTENT) {  // every fragment of the colour; the dense ones listed for the warp pass after it
             lanek<<<small_blocks, LANE_THREADS, 0, st>>>(d_descs, nrep, total_items, p, wctl, perms, act, act_count,
