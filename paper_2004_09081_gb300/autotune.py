@@ -5,13 +5,13 @@ Knobs:
   edge         target fragment edge in cells, 4..8 (the partition gives each
                dimension an even fragment count nearest L/edge)
   n_tau        window length tau = n_tau / (8 k_fast), n_tau in {0.25, 0.5, 1, 2}
-  schedule     0: replica-resident kernel where the state fits one SM,
+  schedule     0: resident kernels where the state fits an SM or a cluster,
                1: colour-phase kernels for every replica
   cluster_top  how many of the largest replicas run as 2-CTA clusters
                (-1: SMs/8, 0: none)
 
 Warps per CTA follow from the replica's shared-memory class in the resident
-kernel (128, 256 or 1024 threads) and are not searched.
+kernel (128, 256 or 512 threads) and are not searched.
 
 Accuracy: the synchronous-sublattice windows approximate the serial kMC of
 Sec. II.A; a vacancy that crosses into a fragment whose colour already ran

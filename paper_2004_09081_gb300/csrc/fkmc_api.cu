@@ -6,6 +6,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -449,19 +450,54 @@ int plan_residency(kmc_batch* b)
     b->any_global = false;
     b->run_kernel.assign(b->n, 0);
     b->run_ctas.assign(b->n, 0);
+    const int force = b->opts.cluster_ctas;
+    // puts replica r on a cluster of lo..hi CTAs, if one fits beside room others; its CTAs, or 0
+    auto on_cluster = [&](int r, int lo, int hi, int room) -> int {
+        RepDesc& D = b->desc[r];
+        const RepDesc before = D;
+        ClusterPlan pl{};
+        // (events drawn ahead, list entries), the next where the slabs do not fit
+        const int want[4][2] = {{prec ? 4 : plain_ev, 8}, {prec ? 4 : plain_ev, 4}, {4, 4}, {2, 4}};
+        for (int q = 0; q < (form == 2 ? 8 : 4); ++q) {
+            const int k = q & 3;
+            D.btab_smem = form == 2 && q < 4;
+            D.kslots = want[k][1];
+            if (!make_cluster_plan(D, b->cap, want[k][0], prec, lo, hi, &pl) || pl.ncta > room ||
+                cluster_fits(form, pl.ncta, cluster_smem_bytes(D, pl, b->cap, want[k][0], prec)) <= 0)
+                continue;
+            D.pre_ev = want[k][0];
+            pl.rep = r;
+            plans.push_back(pl);
+            D.resident = 1;
+            b->run_kernel[r] = 2;
+            b->run_ctas[r] = pl.ncta;
+            return pl.ncta;
+        }
+        D = before;
+        return 0;
+    };
+    // fragments and vacancies per colour phase
+    auto phase_frags = [&](int r) {
+        const int32_t* nf = b->desc[r].nf;
+        return (int64_t)((nf[0] + 1) / 2) * ((nf[1] + 1) / 2) * ((nf[2] + 1) / 2);
+    };
+    auto phase_vacs = [&](int r) {
+        const int32_t* nf = b->desc[r].nf;
+        return (double)b->n_vac[r] / ((nf[0] > 1 ? 2 : 1) * (nf[1] > 1 ? 2 : 1) * (nf[2] > 1 ? 2 : 1));
+    };
     for (int r = 0; r < b->n; ++r) {
         RepDesc& D = b->desc[r];
-        D.kslots = 8;
-        D.btab_smem = form == 2;
         int c = -1;
         size_t need = 0;
-        for (int k = 0; k < 8 && allowed && c < 0; ++k) {
-            if (k == 4) {  // without the Boltzmann tables
-                if (!D.btab_smem) break;
-                D.btab_smem = 0;
+        // (Boltzmann tables in shared memory, list entries), the next where the state does not fit
+        const int lay[4][2] = {{form == 2, 8}, {0, 8}, {form == 2, 4}, {0, 4}};
+        for (int q = 0; q < 4 && allowed && c < 0; ++q) {
+            D.btab_smem = lay[q][0];
+            D.kslots = lay[q][1];
+            for (int k = 0; k < 4 && c < 0; ++k) {
+                need = resident_smem_bytes(D, b->cap, threads[k], 1, prec ? 2 : plain_ev, prec);
+                if (need <= bounds[k]) c = k;
             }
-            need = resident_smem_bytes(D, b->cap, threads[k & 3], 1, prec ? 2 : plain_ev, prec);
-            if (need <= bounds[k & 3]) c = k & 3;
         }
         // the first draws of as many colour phases per batch as the class's shared
         // memory allows beside the state (8: one batch per window): four events per
@@ -481,35 +517,9 @@ int plan_residency(kmc_batch* b)
         }
         // a cluster: a replica too large for one SM (or every replica, with
         // cluster_ctas forced), on the most CTAs that fit
-        const int force = b->opts.cluster_ctas;
-        if (allowed && force >= 0 && (c < 0 || force >= 2)) {
-            ClusterPlan pl{};
-            const int single_btab = D.btab_smem, single_ev = D.pre_ev;
-            const int lo = force >= 2 ? force : 2, hi = force >= 2 ? force : CLUSTER_MAX_CTAS;
-            // (events drawn ahead, list entries), the next where the slabs do not fit
-            const int want[4][2] = {{prec ? 4 : plain_ev, 8}, {prec ? 4 : plain_ev, 4}, {4, 4}, {2, 4}};
-            bool found = false;
-            for (int q = 0; q < 8 && !found; ++q) {
-                const int k = q & 3;
-                D.btab_smem = form == 2 && q < 4;
-                if (form != 2 && q >= 4) break;
-                D.kslots = want[k][1];
-                found = make_cluster_plan(D, b->cap, want[k][0], prec, lo, hi, &pl) &&
-                        cluster_fits(form, pl.ncta, cluster_smem_bytes(D, pl, b->cap, want[k][0], prec)) > 0;
-                if (found) D.pre_ev = want[k][0];
-            }
-            if (found) {
-                pl.rep = r;
-                plans.push_back(pl);
-                D.resident = 1;
-                b->run_kernel[r] = 2;
-                b->run_ctas[r] = pl.ncta;
-                continue;
-            }
-            D.kslots = 8;
-            D.btab_smem = single_btab;
-            D.pre_ev = single_ev;
-        }
+        if (allowed && force >= 0 && (c < 0 || force >= 2) &&
+            on_cluster(r, force >= 2 ? force : 2, force >= 2 ? force : CLUSTER_MAX_CTAS, INT_MAX) > 0)
+            continue;
         D.resident = c >= 0 ? 1 : 0;
         if (c < 0) {
             b->any_global = true;
@@ -519,6 +529,69 @@ int plan_residency(kmc_batch* b)
         need_of[r] = need;
         b->run_kernel[r] = 1;
         b->run_ctas[r] = 1;
+    }
+    // how many SMs the classes take (a class's CTAs per SM, by registers: 4, 4, 2, 1)
+    const double share[4] = {0.25, 0.25, 0.5, 1.0};
+    auto sms_used = [&]() {
+        double used = 0.0;
+        for (int c = 0; c < 4; ++c) used += share[c] * (double)cls[c].size();
+        for (const ClusterPlan& pl : plans) used += pl.ncta;
+        return used;
+    };
+    // a replica with four visits or more per warp and phase, or 128 fragments or more
+    // to look at, on a cluster instead of one CTA while SMs are free: of 48^3 cells in
+    // 12^3 fragments, 0.02 vacancies per site, plain 289 -> 117 us per window (mixed
+    // 137 -> 85), in 8^3 fragments 510 -> 277 (mixed 197 -> 158). Fewer visits are not
+    // worth the cluster's barriers: 32^3 cells in 8^3 fragments at 0.001 take 26 us
+    // on one CTA, 31 on four (mixed 23 and 29), and at 0.005 44 and 45 (36 and 40).
+    // Half as many CTAs as layers of fragments: a phase takes every other layer (48^3
+    // cells at 0.02 take the same on four CTAs as on eight); four at least (64 x 64 x 16
+    // cells in 16 x 16 x 4 fragments at 0.001: 38 us on two, 35 on four). A quarter of the SMs stays
+    // free, as clusters need neighbouring SMs.
+    if (force >= 0 && allowed && b->opts.test_stuck_wait_us == 0) {
+        std::vector<int> dense;
+        for (int c = 0; c < 4; ++c)
+            for (int r : cls[c]) {
+                const int64_t F = phase_frags(r);
+                const int nz = b->desc[r].nf[2];
+                if (nz >= 4 && (F >= 128 || (F >= 64 && phase_vacs(r) >= 64.0))) dense.push_back(r);
+            }
+        std::sort(dense.begin(), dense.end(), [&](int a, int q) {
+            return b->n_vac[a] != b->n_vac[q] ? b->n_vac[a] > b->n_vac[q] : a < q;
+        });
+        for (int r : dense) {
+            const int room = (int)(0.75 * sms - sms_used());
+            if (room < 2) break;
+            const int most = std::min<int>(std::max(4, b->desc[r].nf[2] / 2), CLUSTER_MAX_CTAS);
+            if (on_cluster(r, 2, most, room) <= 0) continue;
+            for (int c = 0; c < 4; ++c) {
+                auto it = std::find(cls[c].begin(), cls[c].end(), r);
+                if (it != cls[c].end()) cls[c].erase(it);
+            }
+        }
+    }
+    // a dense replica alone on the colour-phase passes, which spread over every SM:
+    // 128^3 cells in 32^3 fragments at 0.02 (61 vacancies per warp and phase) take 498 us
+    // per window on 16 CTAs and 344 in passes (mixed 350 and 191), 96^3 cells in 24^3
+    // fragments at 0.02 (35) 265 and 296 (mixed 203 and 168), 128^3 cells in 32^3 at 0.005
+    // (15) 175 and 233 (mixed 113 and 127). With several replicas the clusters fill the
+    // SMs that one leaves idle, so the line holds up to a quarter of them.
+    if (force == 0 && b->opts.schedule == 0 && sms_used() <= 0.25 * sms) {
+        const double line = prec ? 24.0 : 40.0;
+        auto to_passes = [&](int r, int ncta) {
+            const int busy = std::min(ncta, std::max(1, b->desc[r].nf[2] / 2));
+            if (phase_vacs(r) <= line * busy * (CLUSTER_THREADS / 32)) return false;
+            b->desc[r].resident = 0;
+            b->run_kernel[r] = b->run_ctas[r] = 0;
+            b->any_global = true;
+            return true;
+        };
+        for (int c = 0; c < 4; ++c)
+            cls[c].erase(std::remove_if(cls[c].begin(), cls[c].end(), [&](int r) { return to_passes(r, 1); }),
+                         cls[c].end());
+        plans.erase(std::remove_if(plans.begin(), plans.end(),
+                                   [&](const ClusterPlan& pl) { return to_passes(pl.rep, pl.ncta); }),
+                    plans.end());
     }
     // largest replicas (by vacancies, the work per phase) first in every class: the
     // longest-running CTAs start earliest, which shortens the tail of the launch
@@ -545,23 +618,18 @@ int plan_residency(kmc_batch* b)
     }
     for (int r : pairs) cls[3].erase(std::find(cls[3].begin(), cls[3].end(), r));
     // more warps for the replicas with the most vacancies while every CTA still has
-    // its share of an SM (a class's CTAs per SM: by registers 4, 4, 2, 1): a phase
-    // takes as long as its slowest visit, so a visit should not wait for a warp
+    // its share of an SM: a phase takes as long as its slowest visit, so a visit
+    // should not wait for a warp
     {
-        const double share[4] = {0.25, 0.25, 0.5, 1.0};
-        double used = 0.0;
+        double used = sms_used();
         std::vector<std::pair<int64_t, int>> order;
         for (int c = 0; c < 4; ++c)
-            for (int r : cls[c]) {
-                used += share[c];
-                order.push_back({b->n_vac[r], r});
-            }
-        for (const ClusterPlan& pl : plans) used += pl.ncta;
+            for (int r : cls[c]) order.push_back({b->n_vac[r], r});
         std::sort(order.rbegin(), order.rend());
         for (auto& o : order) {
             const int r = o.second;
             const RepDesc& D = b->desc[r];
-            const int maxc = ((D.nf[0] + 1) / 2) * ((D.nf[1] + 1) / 2) * ((D.nf[2] + 1) / 2);
+            const int64_t maxc = phase_frags(r);
             for (int c = 0; c < 3; ++c) {
                 auto it = std::find(cls[c].begin(), cls[c].end(), r);
                 if (it == cls[c].end()) continue;

@@ -43,14 +43,14 @@
 // few in the plain one, records and tracer written an exchange late.
 // Measured (one GB300, whole calls with read-out, against linked per-fragment
 // lists for the mixed form and per-phase launches for the plain form): 256
-// uneven replicas mixed 61.4 -> 55.7 us per window, 24 traced 32^3 replicas
-// mixed 22.8 -> 19.1, 128^3 mixed 55.2 -> 50.8; plain: five 32^3 replicas 155 ->
-// 29.8, 8^3 113 -> 28.5, 128^3 196 -> 75.5.
+// uneven replicas mixed 60.5 -> 51.8 us per window, 24 traced 32^3 replicas
+// mixed 22.7 -> 18.7, 128^3 mixed 54.9 -> 48.0; plain: five 32^3 replicas 154 ->
+// 27.6, 8^3 112 -> 27.6, 128^3 195 -> 68.9.
 //
 // With site energies (plain form) a visit's chain is some 8,000 cycles per event
 // instead of 3,500: the rates wait for the energy field's words in L2, after an
 // exchange behind the 116 atomics that move the vacancy's share.  Five doped 96^3
-// replicas 302 -> 190 us per window, 128^3 in its own potential 483 -> 420 with
+// replicas 302 -> 167 us per window, 128^3 in its own potential 482 -> 332 with
 // the solves.  Holding a visit's moves back and correcting the rates by pair
 // energies instead was slower (190 -> 200): the pair energies cost as many
 // instructions as the wait.

@@ -19,13 +19,13 @@ def fk():
     return fkmc
 
 
-def pair(fk, orc, cells, nf, nv, nh, seed, prec, T=900.0, Ez=2e7, cap=64, n_tau=1.0, ctas=0, tracer=True):
+def pair(fk, orc, cells, nf, nv, nh, seed, prec, T=900.0, Ez=2e7, cap=64, n_tau=1.0, ctas=0, tracer=True, kernel=None):
     b = fk.Batch([(*cells, 4.01)], [(nv, nh)], seed, nfrag=nf, precision=prec, tracer=tracer, cap_v=cap, n_tau=n_tau,
                  cluster_ctas=ctas)
     b.set_barriers(0.6, 0.4, T, field_z=Ez)
     ref = orc.Lattice(cells, nf, nv, nh, seed=seed, tracer=tracer)
     ref.set_rates(0.6, 0.4, T, Ez=Ez, a_ang=4.01, cap_v=cap, n_tau=n_tau, precision=prec)
-    assert b.info().kernel == (2 if ctas else 1)
+    assert b.info().kernel == (kernel if kernel is not None else 2 if ctas else 1)
     return b, ref
 
 
@@ -100,3 +100,21 @@ def test_site_energies_in_the_resident_kernels(fk, orc, cells, nf, nv, ctas):
     assert b.info().kernel == (2 if ctas else 1)
     check(b, ref, (25, 1, 30))
     assert np.array_equal(b.site_field(), [ref.site_energy(s) for s in range(ref.nsite)])
+
+
+def test_many_small_fragments_with_short_lists(fk, orc):
+    """4,096 fragments of 2 x 2 x 2 cells in one layer: too many for lists of eight
+    entries in one CTA's shared memory, and one layer cannot be cut into slabs."""
+    cells, nf = (128, 128, 2), (64, 64, 1)
+    check(*pair(fk, orc, cells, nf, 900, 4000, 3, 1, cap=16), (12, 1))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("cells,nf,nv,kernel", [
+    ((32, 32, 32), (8, 8, 8), 511, 1),    # below 64 vacancies per phase: one CTA
+    ((32, 32, 32), (8, 8, 8), 512, 2),    # four visits per warp and phase: a cluster
+    ((24, 24, 24), (12, 12, 12), 40, 2),  # 216 fragments per phase
+    ((64, 64, 2), (32, 32, 1), 2600, 0),  # over the line of both forms: the phase passes
+])
+def test_dense_replicas_change_kernels(fk, orc, prec, cells, nf, nv, kernel):
+    check(*pair(fk, orc, cells, nf, nv, 500, 5, prec, kernel=kernel), (8, 1, 40))
