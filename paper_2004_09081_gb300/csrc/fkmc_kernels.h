@@ -158,6 +158,7 @@ bool make_cluster_plan(const RepDesc& D, int cap, int pre_ev, int prec, int min_
 int cluster_fits(int form, int ncta, size_t smem);  // clusters of this shape the GPU can hold at once
 cudaError_t resident_prepare();
 // first draws of `windows` windows from w0 on, of every resident replica (plain form)
+cudaError_t launch_gate(cudaStream_t st);  // an empty kernel
 cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uint64_t w0, int windows, int ev_per,
                          int64_t frag_tot, Draw* draws, cudaStream_t st);
 // form: 0 plain, 1 mixed, 2 plain with site energies

@@ -710,6 +710,9 @@ size_t cluster_smem_bytes(const RepDesc& D, const ClusterPlan& p, int cap, int p
     return layout_bytes(sizes_cluster(D, p, cap, CLUSTER_THREADS / 32, pre_ev, prec), nullptr);
 }
 
+// Put before a launch to let another one take its SMs first.
+__global__ void k_gate() {}
+
 // First draws of the plain form, one window after the other: event ev of
 // fragment f of window w0 + z at ((z frag_tot + draw_off + f) ev_per + ev).
 // The FP64 logarithm (some 45 FP64 instructions at 64 cycles of an SM quarter's
@@ -1680,6 +1683,12 @@ int cluster_fits(int form, int ncta, size_t smem)
         return 0;
     }
     return n;
+}
+
+cudaError_t launch_gate(cudaStream_t st)
+{
+    k_gate<<<1, 32, 0, st>>>();
+    return cudaGetLastError();
 }
 
 cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uint64_t w0, int windows, int ev_per,
