@@ -497,11 +497,11 @@ def main():
     value = hops_all / t_max
 
     peak, peak_kind = load_peaks()
-    all_resident = (not null) and n_launch <= args.steps * 5  # class launches only, no per-phase launches
     kinds = [b.info(r).kernel for r in range(nrep)]
+    all_resident = (not null) and all(k > 0 for k in kinds)  # class launches only, no per-phase launches
     on_cluster = all_resident and all(k == 2 for k in kinds)
     if null:
-        # one unit = one null-event step (rates, propose, apply + clock: three launches)
+        # one unit = one null-event step (rates, propose, apply + clock)
         units = args.steps * W
         tag, kname = "k_null_step_" + args.workload, "k_null_* (null-event step: rates, propose, apply + clock)"
         note = ("algorithmic bytes per step, 4-byte words: every vacancy's record and 8 neighbour words "
@@ -513,7 +513,7 @@ def main():
         units = args.steps
         if on_cluster:
             tag = "k_cluster_" + args.workload
-            kname = "k_cluster (cluster-resident window kernel, %d CTAs per replica)" % b.info(0).ctas
+            kname = "k_resident (cluster-resident window kernel, %d CTAs per replica)" % b.info(0).ctas
         else:
             tag, kname = "k_resident_" + args.workload, "k_resident (replica-resident window kernel)"
         note = ("lattice state lives in shared memory for the whole launch: DRAM traffic is the stage-in/out "
