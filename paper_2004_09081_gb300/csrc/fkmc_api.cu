@@ -413,18 +413,70 @@ int rate_table_impl(const kmc_barrier_table* t, double T_K, double Ez, double a_
 
 bool valid_replica(const kmc_batch* b, int32_t r) { return b && r >= 0 && r < b->n; }
 
-// Decide which replicas run in the replica-resident kernel and group them
-// into shared-memory size classes (one launch per class, on forked streams).
-int plan_residency(kmc_batch* b)
+// Forgets the launch classes and the captured launches that hold them.
+void drop_classes(kmc_batch* b)
 {
-    if (int rc0 = drop_resident_cache(b)) return rc0;
-    if (b->res_exec) cudaGraphExecDestroy(b->res_exec);  // it holds the old classes' launches
+    if (b->res_exec) cudaGraphExecDestroy(b->res_exec);
     b->res_exec = nullptr;
     for (auto& c : b->rclass) {
         if (c.st) cudaStreamDestroy(c.st);
         if (c.done) cudaEventDestroy(c.done);
     }
     b->rclass.clear();
+}
+
+// Every replica on the colour-phase passes, which need no memory of their own.
+void plan_passes(kmc_batch* b)
+{
+    drop_classes(b);
+    for (RepDesc& D : b->desc) D.resident = 0;
+    b->run_kernel.assign(b->n, 0);
+    b->run_ctas.assign(b->n, 0);
+    b->any_global = true;
+    b->res_frags = b->res_max_frag = 0;
+}
+
+// Device buffers of the resident replicas: site -> record maps, stage-out copies,
+// first draws (plain form).  False where the allocator has no room.
+bool resident_buffers(kmc_batch* b, int prec, int plain_ev)
+{
+    int64_t sites = 0, frags = 0;
+    b->res_max_frag = 0;
+    for (RepDesc& D : b->desc) {
+        D.vmap_off = sites;
+        D.tmp_off = D.draw_off = frags;
+        if (!D.resident) continue;
+        const int64_t nf = (int64_t)D.nf[0] * D.nf[1] * D.nf[2];
+        sites += 48 * (int64_t)D.L[2] * D.L[1] * D.row_words;  // sixteen sites per occupancy word
+        frags += nf;
+        b->res_max_frag = std::max(b->res_max_frag, nf);
+    }
+    b->res_frags = frags;
+    b->res_ev = plain_ev;
+    auto grow = [&](void** p, size_t* have, size_t want) -> bool {
+        if (want <= *have) return true;
+        b->dfree(*p);
+        *p = b->dalloc(want);
+        *have = *p ? want : 0;
+        return *p != nullptr;
+    };
+    b->draw_windows = 0;
+    if (frags == 0) return true;
+    if (prec == 0) {  // two buffers of up to 64 windows, 64 MB together where one window fits
+        const int64_t per = frags * plain_ev * (int64_t)sizeof(Draw);
+        b->draw_windows = (int)std::max<int64_t>(1, std::min<int64_t>(64, ((int64_t)32 << 20) / per));
+        if (!grow((void**)&b->draws, &b->draws_bytes, 2 * (size_t)per * b->draw_windows)) return false;
+    }
+    return grow((void**)&b->vmap, &b->vmap_bytes, sizeof(uint32_t) * (size_t)sites) &&
+           grow((void**)&b->rec_tmp, &b->tmp_bytes, sizeof(VacRec) * (size_t)frags * b->cap);
+}
+
+// Decide which replicas run in the replica-resident kernel and group them
+// into shared-memory size classes (one launch per class, on forked streams).
+int plan_residency(kmc_batch* b)
+{
+    if (int rc0 = drop_resident_cache(b)) return rc0;
+    drop_classes(b);
     const int prec = b->opts.precision == FKMC_MIXED ? 1 : 0;
     const bool allowed = b->opts.schedule != 1 && (prec == 1 || b->opts.schedule == 0) &&
                          b->cap <= RESIDENT_MAX_SLOTS && !b->grains_on;
@@ -688,37 +740,10 @@ int plan_residency(kmc_batch* b)
         CK(cudaMemcpyAsync(b->d_plans, plans.data(), sizeof(ClusterPlan) * plans.size(), cudaMemcpyHostToDevice,
                            b->st),
            "cluster plan upload");
-    // the resident replicas' buffers: site -> record maps, stage-out copies, first draws (plain form)
-    int64_t sites = 0, frags = 0;
-    b->res_max_frag = 0;
-    for (RepDesc& D : b->desc) {
-        D.vmap_off = sites;
-        D.tmp_off = D.draw_off = frags;
-        if (!D.resident) continue;
-        const int64_t nf = (int64_t)D.nf[0] * D.nf[1] * D.nf[2];
-        sites += 48 * (int64_t)D.L[2] * D.L[1] * D.row_words;  // sixteen sites per occupancy word
-        frags += nf;
-        b->res_max_frag = std::max(b->res_max_frag, nf);
+    if (!resident_buffers(b, prec, plain_ev)) {
+        if (b->opts.schedule == 2) return fail(FKMC_ENOMEM, "device allocation failed (resident replicas)");
+        plan_passes(b);
     }
-    b->res_frags = frags;
-    b->res_ev = plain_ev;
-    auto grow = [&](void** p, size_t* have, size_t want) -> bool {
-        if (want <= *have) return true;
-        b->dfree(*p);
-        *p = b->dalloc(want);
-        *have = *p ? want : 0;
-        return *p != nullptr;
-    };
-    b->draw_windows = 0;
-    if (frags > 0 && prec == 0) {  // two buffers of up to 64 windows, 64 MB together where one window fits
-        const int64_t per = frags * plain_ev * (int64_t)sizeof(Draw);
-        b->draw_windows = (int)std::max<int64_t>(1, std::min<int64_t>(64, ((int64_t)32 << 20) / per));
-        if (!grow((void**)&b->draws, &b->draws_bytes, 2 * (size_t)per * b->draw_windows))
-            return fail(FKMC_ENOMEM, "device allocation failed (first draws)");
-    }
-    if (frags > 0 && (!grow((void**)&b->vmap, &b->vmap_bytes, sizeof(uint32_t) * (size_t)sites) ||
-                      !grow((void**)&b->rec_tmp, &b->tmp_bytes, sizeof(VacRec) * (size_t)frags * b->cap)))
-        return fail(FKMC_ENOMEM, "device allocation failed (resident replicas)");
     return FKMC_OK;
 }
 
@@ -919,20 +944,33 @@ int rebuild_field(kmc_batch* b)
 
 void drop_window_graph(kmc_batch* b);
 
+// What a change of rates, options or composition needs before the next run: the
+// Boltzmann tables (`tables`, where site energies are on), the plan that their size
+// enters, and the descriptors.  On an error nothing runs until kmc_set_barriers
+// succeeds: the plan, the buffers and the device's descriptors need not agree.
+int apply_rates(kmc_batch* b, bool tables)
+{
+    b->rates_set = false;
+    const double* before = b->btab;
+    int rc = tables && site_path(b) ? build_btab(b) : FKMC_OK;
+    if (b->btab != before) drop_window_graph(b);  // it holds the old tables
+    if (!rc) rc = plan_residency(b);
+    if (!rc) rc = upload_desc(b);
+    if (rc) {
+        drop_classes(b);
+        return rc;
+    }
+    b->rates_set = true;
+    return FKMC_OK;
+}
+
 // the Boltzmann tables must cover electrostatic energies up to |u| = um
 int elec_cover(kmc_batch* b, int64_t um)
 {
     if (um <= b->elec_umax) return FKMC_OK;
     b->elec_umax = 2 * um + 1024;
     if (!b->rates_set) return FKMC_OK;  // kmc_set_barriers builds the tables
-    const double* before = b->btab;
-    int rc = build_btab(b);
-    if (rc) return rc;
-    rc = upload_desc(b);
-    if (rc) return rc;
-    if (b->btab != before) drop_window_graph(b);
-    rc = plan_residency(b);  // the tables' size enters the resident kernels' shared memory
-    return rc ? rc : upload_desc(b);
+    return apply_rates(b, true);
 }
 
 // V-cycles of the next automatic refresh
@@ -1288,17 +1326,7 @@ int kmc_set_barriers(kmc_batch* b, const kmc_barrier_table* tables, const double
     int rc = FKMC_OK;
     for (int r = 0; r < b->n && rc == FKMC_OK; ++r) rc = grain_tables(b, r);
     if (rc) return rc;
-    if (site_path(b)) {
-        rc = build_btab(b);
-        if (rc) return rc;
-    }
-    b->rates_set = false;  // a failed plan leaves nothing to run
-    rc = plan_residency(b);
-    if (rc) return rc;
-    rc = upload_desc(b);
-    if (rc) return rc;
-    b->rates_set = true;
-    return FKMC_OK;
+    return apply_rates(b, true);
 }
 
 }  // extern "C"
@@ -1848,13 +1876,7 @@ int kmc_write_state(kmc_batch* b, int32_t r, const uint8_t* host_occ, size_t n)
     b->elec_age = UINT64_MAX / 2;  // the potential is solved again at the next refresh point
     b->phi_prev_valid = false;  // and from zero: the vacancies may have moved anywhere
     drop_window_graph(b);       // the captured solves hold the vacancy count
-    if (b->rates_set) {
-        int rc = plan_residency(b);
-        if (rc) return rc;
-        rc = upload_desc(b);
-        if (rc) return rc;
-    }
-    return FKMC_OK;
+    return b->rates_set ? apply_rates(b, false) : FKMC_OK;
 }
 
 int kmc_read_records(kmc_batch* b, int32_t r, int64_t* rows, int64_t max_rows, int64_t* n_rows)
@@ -2092,11 +2114,7 @@ int kmc_upload_state(kmc_batch* b, const void* host, size_t bytes)
         b->phi_prev_valid = false;
     }
     drop_window_graph(b);  // the captured solves hold the vacancy counts
-    if (b->rates_set) {
-        rc = plan_residency(b);
-        if (rc) return rc;
-    }
-    return upload_desc(b);
+    return b->rates_set ? apply_rates(b, false) : upload_desc(b);
 }
 
 int kmc_set_site_energy(kmc_batch* b, const kmc_site_energy* e)
@@ -2116,12 +2134,7 @@ int kmc_set_site_energy(kmc_batch* b, const kmc_site_energy* e)
             CK(run_pass_blocks(site_path(b) ? FKMC_PLAIN : b->opts.precision, b->cap, site_path(b), b->grains_on,
                                &b->run_blocks),
                "occupancy query");
-            if (b->rates_set) {
-                int rc = plan_residency(b);
-                if (rc) return rc;
-                rc = upload_desc(b);
-                if (rc) return rc;
-            }
+            if (b->rates_set) return apply_rates(b, false);
         }
         return FKMC_OK;
     }
@@ -2168,14 +2181,8 @@ int kmc_set_site_energy(kmc_batch* b, const kmc_site_energy* e)
     }
     drop_window_graph(b);
     CK(run_pass_blocks(FKMC_PLAIN, b->cap, true, b->grains_on, &b->run_blocks), "occupancy query");
-    if (b->rates_set) {
-        int rc = build_btab(b);
-        if (rc) return rc;
-        rc = plan_residency(b);
-        if (rc) return rc;
-        rc = upload_desc(b);
-        if (rc) return rc;
-    }
+    if (b->rates_set)
+        if (int rc = apply_rates(b, true)) return rc;
     CK(cudaStreamSynchronize(b->st), "synchronize");
     return FKMC_OK;
 }
@@ -2219,13 +2226,7 @@ int kmc_set_electrostatics(kmc_batch* b, const kmc_electrostatics* e)
         CK(run_pass_blocks(site_path(b) ? FKMC_PLAIN : b->opts.precision, b->cap, site_path(b), b->grains_on,
                            &b->run_blocks),
            "occupancy query");
-        if (b->rates_set) {
-            int rc = site_path(b) ? build_btab(b) : FKMC_OK;
-            if (!rc) rc = plan_residency(b);
-            if (!rc) rc = upload_desc(b);
-            if (rc) return rc;
-        }
-        return FKMC_OK;
+        return b->rates_set ? apply_rates(b, true) : FKMC_OK;
     }
     if (b->opts.precision != FKMC_PLAIN) return fail(FKMC_EINVAL, "electrostatics need the plain form");
     if (!(e->eps_r > 0.0) || !(e->eps_r <= 1e6) || !std::isfinite(e->q_vac) || std::fabs(e->q_vac) > 8.0 ||
@@ -2314,9 +2315,7 @@ int kmc_set_electrostatics(kmc_batch* b, const kmc_electrostatics* e)
     drop_window_graph(b);
     CK(run_pass_blocks(FKMC_PLAIN, b->cap, true, b->grains_on, &b->run_blocks), "occupancy query");
     if (b->rates_set) {
-        rc = build_btab(b);
-        if (!rc) rc = plan_residency(b);
-        if (!rc) rc = upload_desc(b);
+        rc = apply_rates(b, true);
         if (rc) return rc;
     }
     CK(cudaStreamSynchronize(b->st), "synchronize");
@@ -2427,10 +2426,7 @@ int kmc_set_grains(kmc_batch* b, const kmc_grains* g)
             int rc = grain_tables(b, r);
             if (rc) return rc;
         }
-        int rc = plan_residency(b);
-        if (rc) return rc;
-        rc = upload_desc(b);
-        if (rc) return rc;
+        if (int rc = apply_rates(b, false)) return rc;
     }
     CK(cudaStreamSynchronize(b->st), "synchronize");
     return FKMC_OK;

@@ -1,0 +1,129 @@
+"""Calls that meet an allocator without room: a batch either goes on without the
+memory (the colour-phase passes need none of their own) or refuses to run until
+its rates are set again; nothing is launched on a buffer that is not there."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+CELLS, NV, NH = (12, 12, 12), 20, 40
+VV = [(2, 0.343), (4, 0.235), (6, 0.200)]
+
+
+@pytest.fixture(scope="module")
+def fk():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2004_09081_gb300 import fkmc
+    fkmc.load()
+    return fkmc
+
+
+class Limited:
+    """Torch memory through the ABI's callback: records the sizes asked for, and
+    from `limit` on gives nothing after `fail_from` requests."""
+
+    def __init__(self, fk):
+        self.inner = fk.TorchAllocator()
+        self.sizes, self.fail_from = [], None
+        self.c_alloc = fk.kmc_alloc_fn(self._alloc)
+        self.c_free = self.inner.c_free
+
+    def limit(self, fail_from):
+        self.sizes, self.fail_from = [], fail_from
+
+    def _alloc(self, ctx, n):
+        self.sizes.append(n)
+        if self.fail_from is not None and len(self.sizes) > self.fail_from:
+            return None
+        return self.inner._alloc(ctx, n)
+
+
+def lattice(fk, prec, al, **kw):
+    b = fk.Batch([(*CELLS, 4.01)], [(NV, NH)], 8, edge=4, precision=prec, cap_v=32, alloc=al, **kw)
+    return b
+
+
+def reference(orc, prec, windows, site=False):
+    ref = orc.Lattice(CELLS, None, NV, NH, seed=8, edge=4)
+    if site:
+        ref.set_site_energy(vv=VV)
+    ref.set_rates(0.7, 0.35, 800.0, a_ang=4.01, cap_v=32, precision=prec)
+    ref.run(windows)
+    return ref
+
+
+def same(b, ref):
+    assert np.array_equal(b.state(), ref.occupancy())
+    assert np.array_equal(b.records(), ref.records())
+    assert b.info().hops == ref.counters()["hops"] > 0
+
+
+# the first request (first draws or site map), and each later one
+@pytest.mark.parametrize("fail_from", [0, 1, 2])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_without_the_resident_buffers_the_passes_run(fk, orc, prec, fail_from):
+    al = Limited(fk)
+    b = lattice(fk, prec, al)
+    b.set_grains(4, 1, 0.2)
+    b.set_barriers(0.7, 0.35, 800.0)  # grains: no resident replica, no buffers
+    al.limit(fail_from)
+    b.set_grains(0)
+    need = 3 - prec  # draws (plain form), site map, records
+    assert b.info().kernel == (0 if fail_from < need else 1)
+    b.run(15)
+    al.limit(None)
+    same(b, reference(orc, prec, 15))
+    b.set_barriers(0.7, 0.35, 800.0)
+    assert b.info().kernel == 1
+    b.run(10)
+    same(b, reference(orc, prec, 25))
+
+
+@pytest.mark.parametrize("fail_from", [0, 1])
+def test_resident_only_batch_is_refused_without_its_buffers(fk, orc, fail_from):
+    al = Limited(fk)
+    b = lattice(fk, 1, al, schedule=2)
+    al.limit(fail_from)
+    with pytest.raises(fk.KmcError) as e:
+        b.set_barriers(0.7, 0.35, 800.0)
+    assert e.value.code == fk.FKMC_ENOMEM
+    with pytest.raises(fk.KmcError) as e:
+        b.run(1)
+    assert e.value.code == fk.FKMC_ESTATE
+    al.limit(None)
+    b.set_barriers(0.7, 0.35, 800.0)
+    b.run(15)
+    same(b, reference(orc, 1, 15))
+
+
+def test_failed_energy_tables_stop_the_batch(fk, orc):
+    """kmc_set_site_energy with an allocator that fails from each request on: where
+    the call fails before the interactions are on, the batch runs on without them;
+    where the Boltzmann tables fail, it is refused until the rates are set."""
+    seen = set()
+    for k in range(8):
+        al = Limited(fk)
+        b = lattice(fk, 0, al)
+        b.set_barriers(0.7, 0.35, 800.0)
+        al.limit(k)
+        try:
+            b.set_site_energy(VV)
+            seen.add("set")
+        except fk.KmcError as e:
+            assert e.code == fk.FKMC_ENOMEM
+            try:
+                b.run(40)
+                seen.add("runs without")
+                al.limit(None)
+                same(b, reference(orc, 0, 40))
+                continue
+            except fk.KmcError as e2:
+                assert e2.code == fk.FKMC_ESTATE
+                seen.add("refused")
+        al.limit(None)
+        b.set_barriers(0.7, 0.35, 800.0)
+        b.run(40)
+        same(b, reference(orc, 0, 40, site=True))
+    assert seen == {"set", "runs without", "refused"}
