@@ -2374,17 +2374,11 @@ int kmc_write_potential_energy(kmc_batch* b, int32_t r, const int32_t* u, size_t
         if (rc_) return rc_;
     }
     b->elec_age = 0;
-    b->elec_umax = 0;  // re-derive the tables' range from what was written
-    const int64_t keep = um;
-    int rc = elec_cover(b, keep);
-    if (rc) return rc;
-    if (b->rates_set) {
-        rc = build_btab(b);  // g may have grown the bound too
-        if (!rc) rc = upload_desc(b);
-        if (rc) return rc;
-        drop_window_graph(b);
-    }
-    return FKMC_OK;
+    // the tables' range follows what was written, u and g both (g enters energy_bound
+    // by itself, so that an all-zero u can need larger tables too)
+    b->elec_umax = um > 0 ? 2 * um + 1024 : 0;
+    drop_window_graph(b);
+    return b->rates_set ? apply_rates(b, true) : FKMC_OK;
 }
 
 int kmc_set_grains(kmc_batch* b, const kmc_grains* g)

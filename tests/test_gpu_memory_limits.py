@@ -127,3 +127,34 @@ def test_failed_energy_tables_stop_the_batch(fk, orc):
         b.run(40)
         same(b, reference(orc, 0, 40, site=True))
     assert seen == {"set", "runs without", "refused"}
+
+
+def plan(b):
+    i = b.info()
+    return i.kernel, i.ctas, i.draw_phases, i.draw_events
+
+
+def test_own_potential_alone_outgrows_the_planned_tables(fk, orc):
+    """An all-zero potential written with a larger own-potential table needs larger
+    Boltzmann tables, and with them a new plan: the shared memory that was planned
+    for the smaller ones does not hold them."""
+    cells, nf, nv = (32, 32, 32), (8, 8, 8), 200
+    b = fk.Batch([(*cells, 4.01)], [(nv, 0)], 5, nfrag=nf, precision=0, cap_v=32)
+    b.set_electrostatics(eps_r=100.0, refresh_windows=0)
+    u = np.zeros(3 * 32 ** 3, np.int32)
+    g = np.full((3, 8), -100, np.int32)
+    b.write_potential_energy(u, g)
+    b.set_barriers(0.6, 0.6, 900.0)
+    small = plan(b)
+    g[0, 0] = -400000  # one direction closed by 20 eV
+    b.write_potential_energy(u, g)
+    grown = plan(b)
+    b.set_barriers(0.6, 0.6, 900.0)
+    assert grown == plan(b) != small
+    b.write_potential_energy(u, g)
+    b.run(60)
+    ref = orc.Lattice(cells, nf, nv, 0, seed=5)
+    ref.set_elec(u, g)
+    ref.set_rates(0.6, 0.6, 900.0, a_ang=4.01, cap_v=32)
+    ref.run(60)
+    same(b, ref)
