@@ -1796,6 +1796,22 @@ void touch_pages(void* host, size_t bytes)
     for (size_t k = 0; k < bytes; k += 4096) p[k] = 0;
 }
 
+// The state without a device buffer: the packed words, expanded here.
+int unpack_on_host(kmc_batch* b, const RepDesc& D, uint8_t* host_occ)
+{
+    std::vector<uint32_t> w((size_t)3 * D.L[2] * D.L[1] * D.row_words);
+    CK(cudaMemcpyAsync(w.data(), b->occ + D.occ_word_off, sizeof(uint32_t) * w.size(), cudaMemcpyDeviceToHost, b->st),
+       "state copy");
+    CK(cudaStreamSynchronize(b->st), "synchronize");
+    int64_t s = 0;
+    for (int t = 0; t < 3; ++t)
+        for (int z = 0; z < D.L[2]; ++z)
+            for (int y = 0; y < D.L[1]; ++y)
+                for (int x = 0; x < D.L[0]; ++x)
+                    host_occ[s++] = (uint8_t)((w[occ_index(D.row_words, D.L[1], t, x, y, z)] >> ((x & 15) * 2)) & 3u);
+    return FKMC_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1808,7 +1824,7 @@ int kmc_read_state(kmc_batch* b, int32_t r, uint8_t* host_occ, size_t n)
     const int64_t rows = 3 * (int64_t)D.L[2] * D.L[1];
     const int64_t chunk = std::min<int64_t>(rows, std::max<int64_t>(1, (int64_t)READ_BUF_MAX / D.L[0]));
     uint8_t* buf = (uint8_t*)read_buffer(b, (size_t)(chunk * D.L[0]));
-    if (!buf) return fail(FKMC_ENOMEM, "device allocation failed (read-out)");
+    if (!buf) return unpack_on_host(b, D, host_occ);
     touch_pages(host_occ, n);
     for (int64_t r0 = 0; r0 < rows; r0 += chunk) {
         const int64_t nr = std::min(chunk, rows - r0);
@@ -1885,13 +1901,13 @@ int kmc_read_records(kmc_batch* b, int32_t r, int64_t* rows, int64_t max_rows, i
     const RepDesc& D = b->desc[r];
     const int64_t nfrag = (int64_t)D.nf[0] * D.nf[1] * D.nf[2];
     // rows ordered on the device, as many as the replica has vacancies (a state that
-    // was uploaded with more records than that takes the host path below)
+    // was uploaded with more records than that takes the host path below, as does a
+    // read-out that finds no room for the buffer)
     const int64_t want = std::min(std::max<int64_t>(max_rows, 0), b->n_vac[r]);
     const size_t off_bytes = (sizeof(int64_t) * (size_t)(nfrag + 1) + 255) & ~(size_t)255;
     const size_t need = off_bytes + sizeof(int64_t) * 6 * (size_t)want;
-    if (need <= READ_BUF_MAX) {
-        char* buf = (char*)read_buffer(b, need);
-        if (!buf) return fail(FKMC_ENOMEM, "device allocation failed (read-out)");
+    char* const buf = need <= READ_BUF_MAX ? (char*)read_buffer(b, need) : nullptr;
+    if (buf) {
         int64_t* off = (int64_t*)buf;
         int64_t* d_rows = (int64_t*)(buf + off_bytes);
         CK(launch_rows(D, b->recs, b->counts, b->cap, off, want, d_rows, b->st), "records kernel");

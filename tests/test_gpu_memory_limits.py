@@ -129,6 +129,19 @@ def test_failed_energy_tables_stop_the_batch(fk, orc):
     assert seen == {"set", "runs without", "refused"}
 
 
+def test_read_outs_without_a_device_buffer(fk, orc):
+    al = Limited(fk)
+    b = lattice(fk, 1, al)
+    b.set_barriers(0.7, 0.35, 800.0)
+    b.run(15)
+    ref = reference(orc, 1, 15)
+    al.limit(0)
+    same(b, ref)
+    assert al.sizes  # the buffer was asked for
+    al.limit(None)
+    same(b, ref)
+
+
 def plan(b):
     i = b.info()
     return i.kernel, i.ctas, i.draw_phases, i.draw_events
