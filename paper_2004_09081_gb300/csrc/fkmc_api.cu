@@ -12,6 +12,7 @@
 #include <cstring>
 #include <iterator>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "fkmc.h"
@@ -250,7 +251,7 @@ struct kmc_batch {
     std::vector<double> theta_host;
     uint32_t* null_types = nullptr;        // one launch for many steps: packed event types per vacancy
     void* null_log = nullptr;              // and each replica's barrier and sums per step
-    size_t null_types_bytes = 0;
+    size_t null_types_bytes = 0, null_log_size = 0;
     cudaGraphExec_t null_exec = nullptr;
     int64_t null_exec_picks = -1, null_exec_vac = -1;
     bool null_exec_grains = false;
@@ -1597,24 +1598,37 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
         if (b->null_exec) cudaGraphExecDestroy(b->null_exec);
         b->null_exec = nullptr;
     }
-    if (!b->claims) {
-        b->claims = (unsigned long long*)b->dalloc(sizeof(unsigned long long) * b->nsite_total);
-        b->nacc = (unsigned long long*)b->dalloc(sizeof(unsigned long long) * 3 * b->n);
-        b->theta = (double*)b->dalloc(sizeof(double) * b->n);
-        b->nE = (double*)b->dalloc(sizeof(double) * b->n);
-        b->nctl = (unsigned long long*)b->dalloc(sizeof(unsigned long long) * 3);
-        if (!b->claims || !b->nacc || !b->theta || !b->nE || !b->nctl)
+    if (!b->theta) {  // the last of the five: all of them are there once it is
+        auto have = [&](auto*& p, size_t bytes) {
+            if (!p) p = static_cast<std::remove_reference_t<decltype(p)>>(b->dalloc(bytes));
+            return p != nullptr;
+        };
+        if (!have(b->claims, sizeof(unsigned long long) * b->nsite_total) ||
+            !have(b->nacc, sizeof(unsigned long long) * 3 * b->n) || !have(b->nE, sizeof(double) * b->n) ||
+            !have(b->nctl, sizeof(unsigned long long) * 3) || !have(b->theta, sizeof(double) * b->n))
             return fail(FKMC_ENOMEM, "device allocation failed (null-event buffers)");
         CK(cudaMemcpyAsync(b->theta, b->theta_host.data(), sizeof(double) * b->n, cudaMemcpyHostToDevice, b->st),
            "clock upload");
     }
-    if (sizeof(uint32_t) * (size_t)total_vac > b->null_types_bytes || !b->null_log) {
-        b->dfree(b->null_types);
-        b->null_types = (uint32_t*)b->dalloc(sizeof(uint32_t) * (size_t)total_vac);
-        b->null_types_bytes = b->null_types ? sizeof(uint32_t) * (size_t)total_vac : 0;
-        if (!b->null_log) b->null_log = b->dalloc(null_log_bytes(b->n));
-        if (!b->null_types || !b->null_log) return fail(FKMC_ENOMEM, "device allocation failed (null-event buffers)");
+    // one launch for many steps: where its grid holds the vacancies and its two buffers
+    // can be had, else the launches of each step
+    NullStepsPlan plan;
+    int64_t max_vac = 0, max_sites = 0;
+    for (int r = 0; r < b->n; ++r) {
+        max_vac = std::max(max_vac, b->n_vac[r]);
+        max_sites = std::max(max_sites, b->desc[r].nsite);
     }
+    auto grow = [&](void** p, size_t* have, size_t want) -> bool {
+        if (want <= *have) return true;
+        b->dfree(*p);
+        *p = b->dalloc(want);
+        *have = *p ? want : 0;
+        return *p != nullptr;
+    };
+    const int log_steps = (int)std::min<uint64_t>(NULL_LOG_STEPS, steps);
+    const bool one_launch = steps > 0 && null_steps_plan(b->n, max_vac, max_sites, &plan) &&
+                            grow((void**)&b->null_types, &b->null_types_bytes, sizeof(uint32_t) * (size_t)total_vac) &&
+                            grow(&b->null_log, &b->null_log_size, null_log_bytes(b->n, log_steps));
     if (total_picks > b->props_cap) {
         if (b->null_exec) cudaGraphExecDestroy(b->null_exec);
         b->null_exec = nullptr;
@@ -1637,13 +1651,7 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
     CK(launch_null_gather(b->d_desc, b->n, b->recs, b->counts, b->nfrag_total, b->cap, b->vac, b->status, b->st),
        "null gather");
     ++launches;
-    NullStepsPlan plan;
-    int64_t max_vac = 0, max_sites = 0;
-    for (int r = 0; r < b->n; ++r) {
-        max_vac = std::max(max_vac, b->n_vac[r]);
-        max_sites = std::max(max_sites, b->desc[r].nsite);
-    }
-    if (steps > 0 && null_steps_plan(b->n, max_vac, max_sites, &plan)) {
+    if (one_launch) {
         for (uint64_t k = 0; k < steps; k += NULL_LOG_STEPS) {
             CK(launch_null_steps(plan, b->d_desc, b->n, k, (int)std::min<uint64_t>(NULL_LOG_STEPS, steps - k), b->vac,
                                  b->null_types, b->occ, b->grains_on ? b->gbound : nullptr, b->claims, b->tracer,

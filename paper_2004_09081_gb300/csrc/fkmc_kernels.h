@@ -60,7 +60,7 @@ constexpr int NULL_LOG_STEPS = 4096;
 struct NullStepsPlan {
     int ctas, per;  // CTAs per replica, vacancies and picks per thread
 };
-size_t null_log_bytes(int nrep);
+size_t null_log_bytes(int nrep, int steps);  // their log, `steps` of them at most per launch
 bool null_steps_plan(int nrep, int64_t max_vac, int64_t max_sites, NullStepsPlan* out);
 cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, int nrep, uint64_t k0, int steps,
                               VacRec* vac, uint32_t* types, uint32_t* occ, const uint8_t* gb,

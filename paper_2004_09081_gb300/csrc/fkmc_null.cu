@@ -702,7 +702,10 @@ static NullStepsFn null_steps_kernel(int per)
     return per == 1 ? k_null_steps<1> : (per == 2 ? k_null_steps<2> : k_null_steps<4>);
 }
 
-size_t null_log_bytes(int nrep) { return (sizeof(NullStep) * NULL_LOG_STEPS + sizeof(NullBarrier)) * (size_t)nrep + 32; }
+size_t null_log_bytes(int nrep, int steps)
+{
+    return (sizeof(NullStep) * steps + sizeof(NullBarrier)) * (size_t)nrep + 32;
+}
 
 // One launch for many steps: the CTAs that hold the largest replica at the
 // fewest vacancies and picks per thread (1, 2 or 4), all replicas' CTAs resident

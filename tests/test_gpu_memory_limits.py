@@ -171,3 +171,74 @@ def test_own_potential_alone_outgrows_the_planned_tables(fk, orc):
     ref.set_rates(0.6, 0.6, 900.0, a_ang=4.01, cap_v=32)
     ref.run(60)
     same(b, ref)
+
+
+def null_reference(orc, steps, cells=CELLS, nv=NV, nh=NH, replica=0):
+    ref = orc.Lattice(cells, None, nv, nh, seed=8, edge=4, replica=replica)
+    ref.set_rates(0.7, 0.35, 800.0, a_ang=4.01, cap_v=32, precision=1)
+    ref.null_run(steps, 8)
+    return ref
+
+
+def test_null_event_form_asks_for_what_its_steps_need(fk, orc):
+    """Claims, vacancies and picks, and a word per vacancy and 32 bytes per step where
+    one launch makes the steps."""
+    al = Limited(fk)
+    b = lattice(fk, 1, al)
+    b.set_barriers(0.7, 0.35, 800.0)
+    al.limit(None)
+    b.run_null(3, 8)
+    assert sum(al.sizes) < 8 * b.nsite() + 100 * NV + 4096
+    al.limit(None)
+    b.run_null(50, 8)
+    assert sum(al.sizes) < 50 * 32 + 4096
+    same(b, null_reference(orc, 53))
+
+
+def test_null_event_form_beyond_one_launch(fk, orc):
+    """More replicas than the GPU holds CTAs for: launches per step, no step log."""
+    n, cells, nv, nh = 5000, (4, 4, 4), 3, 20
+    al = Limited(fk)
+    b = fk.Batch([(*cells, 4.01)] * n, [(nv, nh)] * n, 8, edge=4, precision=1, cap_v=32, alloc=al)
+    b.set_barriers(0.7, 0.35, 800.0)
+    al.limit(None)
+    b.run_null(20, 8)
+    assert sum(al.sizes) < n * (8 * b.nsite() + 100 * nv + 100)
+    for r in (0, 1, n - 1):
+        ref = null_reference(orc, 20, cells, nv, nh, r)
+        assert np.array_equal(b.state(r), ref.occupancy()) and np.array_equal(b.records(r), ref.records())
+
+
+def test_null_event_form_at_every_failing_request(fk, orc):
+    done = 0
+    for k in range(12):
+        al = Limited(fk)
+        b = lattice(fk, 1, al)
+        b.set_barriers(0.7, 0.35, 800.0)
+        al.limit(k)
+        try:
+            b.run_null(20, 8)
+        except fk.KmcError as e:
+            assert e.code == fk.FKMC_ENOMEM
+            continue
+        al.limit(None)
+        same(b, null_reference(orc, 20))
+        done += 1
+    assert done >= 3  # without both buffers of the one launch, without its log, with everything
+
+
+def test_null_event_form_after_failed_calls(fk, orc):
+    """One request more granted by each call: what the earlier ones left is used, and
+    nothing that is missing."""
+    al = Limited(fk)
+    b = lattice(fk, 1, al)
+    b.set_barriers(0.7, 0.35, 800.0)
+    for k in range(10):
+        al.limit(1)
+        try:
+            b.run_null(20, 8)
+        except fk.KmcError as e:
+            assert e.code == fk.FKMC_ENOMEM
+    al.limit(None)
+    assert b.info().null_steps >= 40
+    same(b, null_reference(orc, b.info().null_steps))
