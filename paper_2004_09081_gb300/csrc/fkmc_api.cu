@@ -148,6 +148,7 @@ struct kmc_batch {
     unsigned long long* check_buf = nullptr;    // CHECK_WORDS sums of kmc_check_invariants
     void* read_buf = nullptr;                   // read-outs: expanded codes or record rows (READ_BUF_MAX at most)
     size_t read_bytes = 0;
+    bool records_match = true;                  // every replica holds one record per vacancy, as far as the host knows
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     std::vector<void*> owned;
     // replica-resident kernel: replicas grouped by shared-memory size class
@@ -363,6 +364,7 @@ int check_status(kmc_batch* b)
     uint32_t s = 0;
     CK(cudaMemcpyAsync(&s, b->status, sizeof s, cudaMemcpyDeviceToHost, b->st), "status copy");
     CK(cudaStreamSynchronize(b->st), "synchronize");
+    if (s) b->records_match = false;
     if (s & STATUS_OVERFLOW)
         return fail(FKMC_EOVERFLOW, "a fragment received more vacancies than cap_v slots");
     if (s & STATUS_TIMEOUT) return fail(FKMC_ETIMEOUT, "a device-side wait ran out of time");
@@ -1919,16 +1921,24 @@ int kmc_read_records(kmc_batch* b, int32_t r, int64_t* rows, int64_t max_rows, i
         int64_t* off = (int64_t*)buf;
         int64_t* d_rows = (int64_t*)(buf + off_bytes);
         CK(launch_rows(D, b->recs, b->counts, b->cap, off, want, d_rows, b->st), "records kernel");
-        int64_t total = 0;
-        if (want > 0) {
-            touch_pages(rows, sizeof(int64_t) * 6 * (size_t)want);
-            CK(cudaMemcpyAsync(rows, d_rows, sizeof(int64_t) * 6 * (size_t)want, cudaMemcpyDeviceToHost, b->st),
+        int64_t total = want;
+        auto read_total = [&]() -> int {
+            CK(cudaMemcpyAsync(&total, off + nfrag, sizeof total, cudaMemcpyDeviceToHost, b->st), "record copy");
+            CK(cudaStreamSynchronize(b->st), "synchronize");
+            return FKMC_OK;
+        };
+        // a state that may hold fewer records than the replica has vacancies: rows beyond
+        // the last are not the call's to write, so the total comes first
+        if (!b->records_match)
+            if (int rc = read_total()) return rc;
+        const int64_t n = std::min(total, want);
+        if (n > 0) {
+            touch_pages(rows, sizeof(int64_t) * 6 * (size_t)n);
+            CK(cudaMemcpyAsync(rows, d_rows, sizeof(int64_t) * 6 * (size_t)n, cudaMemcpyDeviceToHost, b->st),
                "record copy");
         }
-        CK(cudaMemcpyAsync(&total, off + nfrag, sizeof total, cudaMemcpyDeviceToHost, b->st), "record copy");
-        CK(cudaStreamSynchronize(b->st), "synchronize");
+        if (int rc = read_total()) return rc;
         if (total <= want || want == max_rows || max_rows <= 0) {
-            for (int64_t k = 6 * total; k < 6 * want; ++k) rows[k] = 0;  // fewer records than vacancies
             if (n_rows) *n_rows = total;
             return FKMC_OK;
         }
@@ -2102,6 +2112,7 @@ int kmc_upload_state(kmc_batch* b, const void* host, size_t bytes)
         if (rows[r].n_vac < 0 || rows[r].n_H < 0 || rows[r].n_vac + rows[r].n_H > b->desc[r].nsite)
             return fail(FKMC_EINVAL, "state blob: bad composition");
     }
+    b->records_match = false;  // the blob's counts are the caller's
     std::vector<BlobPart> parts;
     size_t off = blob_parts(b, &parts);
     for (const BlobPart& p : parts) {
