@@ -135,10 +135,11 @@ typedef struct {
                            fragments holding one or two vacancies, 4 or 2 per warp in lock-step.
                            0 (default) = where a phase holds 32768 fragments or more,
                            1 = always, 2 = always and in the grouped form, -1 = never */
-    int32_t test_stuck_wait_us; /* test of the device-side bounded wait (0 = off): the one-CTA
-                                   resident kernel, after staging its state, waits on a barrier that nothing
-                                   completes, gives up after this many microseconds (<= 2e6) and
-                                   kmc_run returns FKMC_ETIMEOUT with the state untouched */
+    int32_t test_stuck_wait_us; /* test of the device-side bounded waits (0 = off): the one-CTA
+                                   resident kernel, after staging its state, and the null-event form's
+                                   one launch for many steps, before the first, wait on a barrier that
+                                   nothing completes and give up after this many microseconds (<= 2e6);
+                                   kmc_run or kmc_run_null returns FKMC_ETIMEOUT with the state untouched */
     int32_t lane_form;  /* mixed form, one-thread-per-fragment pass: 0 (default) = by phase size,
                            1 = registers (up to 4 vacancies, beside the general pass),
                            2 = persistent (up to 8 vacancies in shared memory, a grid that
@@ -160,7 +161,8 @@ typedef struct {
     uint64_t handoffs; /* exchanges that moved a vacancy into another fragment */
     uint64_t windows;  /* windows run by this call */
     double gpu_ms;     /* device time of the call's kernels (CUDA events) */
-    uint64_t launches; /* kernel launches made by the call */
+    uint64_t launches; /* kernel launches made by the call, without the empty kernels that order
+                          the launches of resident replicas of several sizes */
 } kmc_run_stats;
 
 typedef struct {
@@ -378,12 +380,17 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats);
  * The state is shared with kmc_run (records are regathered by id before and
  * returned to their fragments after); kmc_read_msd's t adds this clock.
  * Vacancy ids must be 0 .. N_V-1 (true after creation and kmc_write_state).
- * Needs 8 bytes per site (claims) and 24 bytes per vacancy of extra device
- * memory, allocated at the first call.
+ * Needs 8 bytes per site (claims), 24 bytes per vacancy and 16 per pick of extra
+ * device memory, allocated at the first call.  Where the GPU holds threads for every
+ * vacancy at once, one launch makes up to 4096 steps and takes 4 bytes more per
+ * vacancy and 32 per step and replica; without room for those the launches of
+ * each step run.
  * Errors: FKMC_ESTATE before kmc_set_barriers; FKMC_EINVAL for n_frg < 1,
  * more than 2^32 - 16 steps, or with site energies on; FKMC_ENOMEM;
  * FKMC_EOVERFLOW if a fragment cannot take its vacancies back (cap_v);
- * FKMC_ECUDA. */
+ * FKMC_ETIMEOUT if a device-side wait (2 s) gave up: null_steps does not count
+ * the call, part of whose steps may have been made, so that the state and the
+ * clocks are then invalid; FKMC_ECUDA. */
 int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* stats);
 
 /* Exact integer moments of the displacements of one species of replica r:

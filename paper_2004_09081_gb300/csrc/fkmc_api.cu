@@ -359,11 +359,12 @@ uint64_t window_launches(const kmc_batch* b)
                : 17;
 }
 
-int check_status(kmc_batch* b)
+int check_status(kmc_batch* b, uint32_t* word = nullptr)
 {
     uint32_t s = 0;
     CK(cudaMemcpyAsync(&s, b->status, sizeof s, cudaMemcpyDeviceToHost, b->st), "status copy");
     CK(cudaStreamSynchronize(b->st), "synchronize");
+    if (word) *word = s;
     if (s) b->records_match = false;
     if (s & STATUS_OVERFLOW)
         return fail(FKMC_EOVERFLOW, "a fragment received more vacancies than cap_v slots");
@@ -1657,7 +1658,8 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
         for (uint64_t k = 0; k < steps; k += NULL_LOG_STEPS) {
             CK(launch_null_steps(plan, b->d_desc, b->n, k, (int)std::min<uint64_t>(NULL_LOG_STEPS, steps - k), b->vac,
                                  b->null_types, b->occ, b->grains_on ? b->gbound : nullptr, b->claims, b->tracer,
-                                 b->null_log, b->theta, b->stats, b->status, b->st),
+                                 b->null_log, b->theta, b->stats, b->status, (uint32_t)b->opts.test_stuck_wait_us,
+                                 b->st),
                "null-event steps");
             launches += 2;
         }
@@ -1693,15 +1695,17 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
        "null scatter");
     ++launches;
     CK(cudaEventRecord(b->ev1, b->st), "event record");
-    for (int r = 0; r < b->n; ++r) b->desc[r].null_step += steps;
-    rc = upload_desc(b);
-    if (rc) return rc;
     CK(cudaMemcpyAsync(b->stats_host.data(), b->stats, sizeof(unsigned long long) * 2 * b->n, cudaMemcpyDeviceToHost,
                        b->st),
        "stats copy");
     CK(cudaMemcpyAsync(b->theta_host.data(), b->theta, sizeof(double) * b->n, cudaMemcpyDeviceToHost, b->st),
        "clock copy");
-    rc = check_status(b);
+    uint32_t word = 0;
+    rc = check_status(b, &word);
+    // after a wait that ran out the steps are incomplete and do not count
+    if (!(word & STATUS_TIMEOUT))
+        for (int r = 0; r < b->n; ++r) b->desc[r].null_step += steps;
+    if (const int rc_ = upload_desc(b)) return rc_;
     b->field_valid = false;
     {
         const int rc_ = drop_resident_cache(b);

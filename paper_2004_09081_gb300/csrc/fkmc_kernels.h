@@ -65,7 +65,7 @@ bool null_steps_plan(int nrep, int64_t max_vac, int64_t max_sites, NullStepsPlan
 cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, int nrep, uint64_t k0, int steps,
                               VacRec* vac, uint32_t* types, uint32_t* occ, const uint8_t* gb,
                               unsigned long long* claims, int32_t* tracer, void* log_mem, double* theta,
-                              unsigned long long* stats, uint32_t* status, cudaStream_t st);
+                              unsigned long long* stats, uint32_t* status, uint32_t stuck_wait_us, cudaStream_t st);
 // read-outs: species codes of rows of the (t, z, y) order; record rows with their
 // offsets per fragment (offsets: fragments + 1 entries, the last the total)
 cudaError_t launch_unpack_state(const RepDesc& D, const uint32_t* occ, int64_t row0, int64_t rows, uint8_t* out,

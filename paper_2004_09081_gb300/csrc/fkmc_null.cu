@@ -373,9 +373,10 @@ struct NullBarrier {
 
 constexpr unsigned long long NULL_WAIT_NS = 2000000000ull;  // bound on one barrier wait
 
-// Barrier number `target / ctas` of the replica's CTAs; false when a wait ran
-// out (here or elsewhere), after which every CTA leaves.
-__device__ __forceinline__ bool null_barrier(NullBarrier* bar, unsigned target)
+// Barrier number `target / ctas` of the replica's CTAs; false when a wait of
+// `limit` ns ran out (here or elsewhere), after which every CTA leaves.
+__device__ __forceinline__ bool null_barrier(NullBarrier* bar, unsigned target,
+                                             unsigned long long limit = NULL_WAIT_NS)
 {
     __shared__ int stop;
     __threadfence();  // this thread's writes before the arrival
@@ -390,7 +391,7 @@ __device__ __forceinline__ bool null_barrier(NullBarrier* bar, unsigned target)
         while ((int)(c - target) < 0) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&bar->count) : "memory");
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            if (t - t0 > NULL_WAIT_NS) {
+            if (t - t0 > limit) {
                 atomicExch(&bar->stop, 1u);
                 out = 1;
                 break;
@@ -418,11 +419,14 @@ __device__ __forceinline__ void warp_sum_max(unsigned long long v, unsigned long
 // Steps k0 .. k0 + steps - 1 of every replica (CTAs [r ctas, (r + 1) ctas): replica
 // r).  types: one word per vacancy, nibble n = rate type of event n + 1 (0: no
 // event).  log: per replica and step, cleared by the caller, as are the barriers.
+// stuck_ns > 0: a test of the barrier's bounded wait, which first waits that long for
+// one arrival more than there are CTAs, and makes no step.  A launch behind one whose
+// wait ran out makes none either.
 template <int PER>
 __global__ void __launch_bounds__(CT)
     k_null_steps(const RepDesc* __restrict__ descs, int ctas, uint64_t k0, int steps, VacRec* vac, uint32_t* types,
                  uint32_t* occ, const uint8_t* __restrict__ gb, unsigned long long* claims, int32_t* tracer,
-                 NullStep* log, int log_stride, NullBarrier* bars, uint32_t* status)
+                 NullStep* log, int log_stride, NullBarrier* bars, uint32_t* status, unsigned long long stuck_ns)
 {
     __shared__ RepDesc D;
     __shared__ PickKeys pk[2];           // by step parity
@@ -434,8 +438,17 @@ __global__ void __launch_bounds__(CT)
     const int rep = (int)(blockIdx.x / ctas), me = (int)(blockIdx.x - rep * ctas);
     NullBarrier* const bar = bars + rep;
     unsigned target = 0;
-    if (tid == 0) D = descs[rep];
+    __shared__ bool late;
+    if (tid == 0) {
+        D = descs[rep];
+        late = (*reinterpret_cast<volatile uint32_t*>(status) & STATUS_TIMEOUT) != 0u;
+    }
     __syncthreads();
+    if (late) return;
+    if (stuck_ns && !null_barrier(bar, (unsigned)ctas + 1u, stuck_ns)) {
+        if (tid == 0) atomicOr(status, STATUS_TIMEOUT);
+        return;
+    }
     if (tid < 16) q[tid] = tid == 0 || tid > 12 ? 0ull : (tid <= 6 ? D.qn[tid - 1] : D.qng[tid - 7]);
     const int nv = (int)D.null_nv, np = (int)D.null_nfrg;
     VacRec* const vr = vac + D.vac_off;
@@ -695,7 +708,7 @@ cudaError_t launch_null_step(const RepDesc* d_descs, int nrep, int64_t total_vac
 }
 
 using NullStepsFn = void (*)(const RepDesc*, int, uint64_t, int, VacRec*, uint32_t*, uint32_t*, const uint8_t*,
-                             unsigned long long*, int32_t*, NullStep*, int, NullBarrier*, uint32_t*);
+                             unsigned long long*, int32_t*, NullStep*, int, NullBarrier*, uint32_t*, unsigned long long);
 
 static NullStepsFn null_steps_kernel(int per)
 {
@@ -739,8 +752,9 @@ bool null_steps_plan(int nrep, int64_t max_vac, int64_t max_sites, NullStepsPlan
 cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, int nrep, uint64_t k0, int steps,
                               VacRec* vac, uint32_t* types, uint32_t* occ, const uint8_t* gb,
                               unsigned long long* claims, int32_t* tracer, void* log_mem, double* theta,
-                              unsigned long long* stats, uint32_t* status, cudaStream_t st)
+                              unsigned long long* stats, uint32_t* status, uint32_t stuck_wait_us, cudaStream_t st)
 {
+    unsigned long long stuck_ns = 1000ull * stuck_wait_us;
     NullBarrier* bars = reinterpret_cast<NullBarrier*>(log_mem);
     NullStep* log = reinterpret_cast<NullStep*>(reinterpret_cast<char*>(log_mem) + ((sizeof(NullBarrier) * nrep + 31) & ~(size_t)31));
     int stride = steps;
@@ -749,7 +763,7 @@ cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, in
     if (e != cudaSuccess) return e;
     int ctas = p.ctas;
     void* args[] = {(void*)&d_descs, &ctas, &k0, &steps, &vac, &types, &occ, (void*)&gb, &claims, &tracer, &log,
-                    &stride, &bars, &status};
+                    &stride, &bars, &status, &stuck_ns};
     e = cudaLaunchCooperativeKernel((const void*)null_steps_kernel(p.per), dim3((unsigned)(ctas * nrep)), dim3(CT), args,
                                     0, st);
     if (e != cudaSuccess) return e;

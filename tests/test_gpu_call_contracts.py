@@ -37,3 +37,29 @@ def test_rows_beyond_the_records_are_left_alone(fk):
     fk._check(fk.load().kmc_read_records(b.h, 0, fk._ptr(rows), nv + more, ctypes.byref(total)))
     assert total.value == nv
     assert np.array_equal(rows[:nv], rec) and (rows[nv:] == -7).all()
+
+
+@pytest.mark.parametrize("steps", [5, 9000])
+def test_null_event_barrier_gives_up(fk, orc, steps):
+    """The barrier between a step's parts waits for an arrival that never comes, gives
+    up after 2 ms and reports it; no step is made or counted, later launches of the
+    call make none, and the context stays usable."""
+    cells, nv, nh = (12, 12, 12), 20, 60
+    kw = dict(edge=4, precision=1, cap_v=32)
+    b = fk.Batch([(*cells, 4.01)] * 3, [(nv, nh)] * 3, 3, test_stuck_wait_us=2000, **kw)
+    b.set_barriers(0.7, 0.35, 800.0)
+    before = [(b.state(r), b.records(r)) for r in range(3)]
+    with pytest.raises(fk.KmcError) as e:
+        b.run_null(steps, nv)
+    assert e.value.code == fk.FKMC_ETIMEOUT
+    for r in range(3):
+        assert np.array_equal(b.state(r), before[r][0]) and np.array_equal(b.records(r), before[r][1])
+        assert (b.info(r).null_steps, b.info(r).null_theta, b.info(r).hops) == (0, 0.0, 0)
+    ok = fk.Batch([(*cells, 4.01)], [(nv, nh)], 3, **kw)
+    ok.set_barriers(0.7, 0.35, 800.0)
+    ok.run_null(30, nv)
+    ref = orc.Lattice(cells, None, nv, nh, seed=3, edge=4)
+    ref.set_rates(0.7, 0.35, 800.0, a_ang=4.01, cap_v=32, precision=1)
+    ref.null_run(30, nv)
+    assert np.array_equal(ok.records(), ref.records())
+    assert ok.info().null_theta == ref.null_clock()["theta"]
