@@ -1233,12 +1233,15 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     // the total of the fragment's events; the plain form's scans, in the canonical
                     // order, give the inclusive prefixes that the selection needs besides
                     uint64_t inc0 = 0, inc1 = 0;
+                    bool nz0 = false, nz1 = false;  // plain: this lane's events have a rate
                     if (nch <= 2) {
                         inc0 = SITE ? sr0 : rate_of(ty0);
                         inc1 = nch == 2 ? (SITE ? sr1 : rate_of(ty1)) : 0ull;
                         if constexpr (PREC == 1) {
                             tot = warp_total(inc0 + inc1);
                         } else {
+                            nz0 = inc0 != 0ull;
+                            nz1 = inc1 != 0ull;
                             const int len = n <= 2 ? 8 * max(n, 1) : 32;
                             inc0 = scan64(inc0, len);
                             tot = __shfl_sync(FULL, inc0, len - 1);
@@ -1354,14 +1357,12 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     // nonzero rate, and the last of those where rounding left no prefix above it)
                     int e_sel = -1;
                     if (nch <= 2) {
-                        const bool h0 = inc0 > target && (PREC == 1 || (SITE ? sr0 != 0ull : ty0 < NO_EVENT));
-                        const bool h1 =
-                            nch == 2 && inc1 > target && (PREC == 1 || (SITE ? sr1 != 0ull : ty1 < NO_EVENT));
+                        const bool h0 = inc0 > target && (PREC == 1 || nz0);
+                        const bool h1 = nch == 2 && inc1 > target && (PREC == 1 || nz1);
                         const unsigned b0 = __ballot_sync(FULL, h0), b1 = __ballot_sync(FULL, h1);
                         e_sel = b0 ? __ffs(b0) - 1 : (b1 ? 32 + __ffs(b1) - 1 : -1);
                         if (PREC == 0 && e_sel < 0) {
-                            const unsigned l0 = __ballot_sync(FULL, (SITE ? sr0 : rate_of(ty0)) != 0ull),
-                                           l1 = __ballot_sync(FULL, nch == 2 && (SITE ? sr1 : rate_of(ty1)) != 0ull);
+                            const unsigned l0 = __ballot_sync(FULL, nz0), l1 = __ballot_sync(FULL, nz1);
                             e_sel = l1 ? 63 - __clz(l1) : 31 - __clz(l0);
                         }
                     } else {

@@ -1,7 +1,7 @@
 """Paths that no other comparison with the oracle takes: the colour-phase passes in
 the plain form where the replica would fit the resident kernels, with and without
 site energies; the two-CTA slabs of kmc_opts.cluster_top; the mixed clock beyond
-its integer form; the multigrid's four-plane kernels
+its integer form; rates that underflow to zero; the multigrid's four-plane kernels
 where the planes do not divide by four; tables that grow within a call."""
 import numpy as np
 import pytest
@@ -139,6 +139,20 @@ def test_mixed_clock_beyond_its_integer_form(fk, orc, nv, seed, window, event, s
     check(b, ref, (1,))
     assert ref.counters()["hops"] - before > event  # the event happened
     check(b, ref, (3,))
+
+
+@pytest.mark.parametrize("sched", [0, 1])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_rates_that_underflow_to_zero(fk, orc, prec, sched):
+    """O hops at 30 K and 2 eV have the rate 0 in FP64: such an event is never taken,
+    also where rounding puts its prefix above those before it."""
+    cells, nf, nv, nh = (10, 12, 9), (2, 4, 2), 40, 1500
+    b = fk.Batch([(*cells, 4.01)], [(nv, nh)], 4, nfrag=nf, precision=prec, tracer=True, cap_v=64, schedule=sched)
+    b.set_barriers(2.0, 0.2, 30.0)
+    assert b.info().k64[0] == 0.0 < b.info().k64[3]
+    ref = orc.Lattice(cells, nf, nv, nh, seed=4, tracer=True)
+    ref.set_rates(2.0, 0.2, 30.0, a_ang=4.01, cap_v=64, precision=prec)
+    check(b, ref, (60, 60))
 
 
 def test_multigrid_with_planes_that_do_not_divide_by_four(fk, orc):
