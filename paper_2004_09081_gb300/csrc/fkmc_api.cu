@@ -504,34 +504,47 @@ int plan_residency(kmc_batch* b)
     std::vector<size_t> cmax(4, 0), need_of(b->n, 0);
     std::vector<ClusterPlan> plans;
     std::vector<int> pairs;  // replicas that may run on two CTAs (kmc_opts.cluster_top)
-    b->any_global = false;
     b->run_kernel.assign(b->n, 0);
     b->run_ctas.assign(b->n, 0);
     const int force = b->opts.cluster_ctas;
-    // puts replica r on a cluster of lo..hi CTAs, if one fits beside room others; its CTAs, or 0
-    auto on_cluster = [&](int r, int lo, int hi, int room) -> int {
-        RepDesc& D = b->desc[r];
-        const RepDesc before = D;
-        ClusterPlan pl{};
+    // clusters of nc CTAs that the GPU holds at once (one CTA of these kernels fills an
+    // SM's registers, whatever its shared memory)
+    int fit_count[CLUSTER_MAX_CTAS + 1];
+    std::fill(fit_count, fit_count + CLUSTER_MAX_CTAS + 1, -1);
+    auto fits = [&](int nc) -> int {
+        if (fit_count[nc] < 0) fit_count[nc] = cluster_fits(form, nc, RESIDENT_MAX_SMEM);
+        return fit_count[nc];
+    };
+    // replica r on the most of lo..hi CTAs that hold it and that the GPU can place
+    struct Placed {
+        RepDesc D;
+        ClusterPlan pl;
+    };
+    auto slabs_of = [&](int r, int lo, int hi, Placed* out) -> bool {
         // (events drawn ahead, list entries), the next where the slabs do not fit
         const int want[4][2] = {{prec ? 4 : plain_ev, 8}, {prec ? 4 : plain_ev, 4}, {4, 4}, {2, 4}};
-        for (int q = 0; q < (form == 2 ? 8 : 4); ++q) {
-            const int k = q & 3;
-            D.btab_smem = form == 2 && q < 4;
-            D.kslots = want[k][1];
-            if (!make_cluster_plan(D, b->cap, want[k][0], prec, lo, hi, &pl) || pl.ncta > room ||
-                cluster_fits(form, pl.ncta, cluster_smem_bytes(D, pl, b->cap, want[k][0], prec)) <= 0)
-                continue;
-            D.pre_ev = want[k][0];
-            pl.rep = r;
-            plans.push_back(pl);
-            D.resident = 1;
-            b->run_kernel[r] = 2;
-            b->run_ctas[r] = pl.ncta;
-            return pl.ncta;
+        for (int nc = std::min(hi, (int)b->desc[r].nf[2]); nc >= lo; --nc) {
+            if (fits(nc) <= 0) continue;
+            for (int q = 0; q < (form == 2 ? 8 : 4); ++q) {
+                out->D = b->desc[r];
+                out->D.btab_smem = form == 2 && q < 4;
+                out->D.kslots = want[q & 3][1];
+                out->D.pre_ev = want[q & 3][0];
+                out->pl = ClusterPlan{};
+                if (!make_cluster_plan(out->D, b->cap, out->D.pre_ev, prec, nc, nc, &out->pl)) continue;
+                out->pl.rep = r;
+                out->D.resident = 1;
+                return true;
+            }
         }
-        D = before;
-        return 0;
+        return false;
+    };
+    auto put_on_cluster = [&](const Placed& c) {
+        const int r = c.pl.rep;
+        b->desc[r] = c.D;
+        plans.push_back(c.pl);
+        b->run_kernel[r] = 2;
+        b->run_ctas[r] = c.pl.ncta;
     };
     // fragments and vacancies per colour phase
     auto phase_frags = [&](int r) {
@@ -542,6 +555,7 @@ int plan_residency(kmc_batch* b)
         const int32_t* nf = b->desc[r].nf;
         return (double)b->n_vac[r] / ((nf[0] > 1 ? 2 : 1) * (nf[1] > 1 ? 2 : 1) * (nf[2] > 1 ? 2 : 1));
     };
+    std::vector<int> wide;  // replicas that only a cluster can hold
     for (int r = 0; r < b->n; ++r) {
         RepDesc& D = b->desc[r];
         int c = -1;
@@ -572,16 +586,16 @@ int plan_residency(kmc_batch* b)
                 break;
             }
         }
-        // a cluster: a replica too large for one SM (or every replica, with
-        // cluster_ctas forced), on the most CTAs that fit
-        if (allowed && force >= 0 && (c < 0 || force >= 2) &&
-            on_cluster(r, force >= 2 ? force : 2, force >= 2 ? force : CLUSTER_MAX_CTAS, INT_MAX) > 0)
-            continue;
-        D.resident = c >= 0 ? 1 : 0;
-        if (c < 0) {
-            b->any_global = true;
+        // a cluster: a replica too large for one SM, below, or, with cluster_ctas
+        // forced, every replica with exactly so many CTAs
+        Placed forced;
+        if (allowed && force >= 2 && slabs_of(r, force, force, &forced)) {
+            put_on_cluster(forced);
             continue;
         }
+        if (c < 0 && allowed && force == 0) wide.push_back(r);
+        D.resident = c >= 0 ? 1 : 0;
+        if (c < 0) continue;
         cls[c].push_back(r);
         need_of[r] = need;
         b->run_kernel[r] = 1;
@@ -589,41 +603,158 @@ int plan_residency(kmc_batch* b)
     }
     // how many SMs the classes take (a class's CTAs per SM, by registers: 4, 4, 2, 1)
     const double share[4] = {0.25, 0.25, 0.5, 1.0};
-    auto sms_used = [&]() {
+    auto singles_sms = [&]() {
         double used = 0.0;
         for (int c = 0; c < 4; ++c) used += share[c] * (double)cls[c].size();
+        return used;
+    };
+    auto sms_used = [&]() {
+        double used = singles_sms();
         for (const ClusterPlan& pl : plans) used += pl.ncta;
         return used;
     };
-    // a replica with four visits or more per warp and phase, or 128 fragments or more
-    // to look at, on a cluster instead of one CTA while SMs are free: of 48^3 cells in
-    // 12^3 fragments, 0.02 vacancies per site, plain 289 -> 117 us per window (mixed
-    // 137 -> 85), in 8^3 fragments 510 -> 277 (mixed 197 -> 158). Fewer visits are not
-    // worth the cluster's barriers: 32^3 cells in 8^3 fragments at 0.001 take 26 us
-    // on one CTA, 31 on four (mixed 23 and 29), and at 0.005 44 and 45 (36 and 40).
-    // Half as many CTAs as layers of fragments: a phase takes every other layer (48^3
+    // Estimate of a resident replica's window, us: the cost of a phase's chain with one
+    // visit, of each further visit per warp, of each vacancy beyond the first in a visit,
+    // and of the screen and draws per fragment and CTA.  Fitted to 60 timings on one GB300
+    // of 32^3 .. 128^3 cells at 0.001 to 0.01 vacancies per site, on one CTA and on 2 to 16
+    // (within 30%); the lines below need no better.
+    auto window_us = [&](int r, int nc, double warps) {
+        static const double c1[3] = {24.0, 20.0, 40.0}, cn[3] = {41.0, 36.0, 63.0}, per_visit[3] = {4.6, 3.7, 8.0},
+                            per_vac[3] = {7.0, 4.0, 7.0}, per_frag[3] = {0.04, 0.04, 0.08};
+        const int32_t* nf = b->desc[r].nf;
+        const int busy = nc > 1 ? std::min(nc, std::max(1, nf[2] / 2)) : 1;  // a phase takes every other layer
+        return (nc > 1 ? cn : c1)[form] + per_visit[form] * phase_vacs(r) / (warps * busy) +
+               per_vac[form] * (double)b->n_vac[r] / ((double)nf[0] * nf[1] * nf[2]) +
+               per_frag[form] * (double)phase_frags(r) / busy;
+    };
+    // a set of replicas on clusters of at most hi CTAs: their share of the GPU (1: it is
+    // full, as the GPU can place no more of them at once) and the longest window
+    struct Group {
+        std::vector<Placed> on;
+        double load = 0.0, us = 0.0;
+        int most = 0;  // CTAs of the largest
+    };
+    auto group = [&](const std::vector<int>& list, int lo, int hi, auto limit) {
+        Group g;
+        Placed p;
+        for (int r : list)
+            if (slabs_of(r, lo, std::min(hi, limit(r)), &p)) {
+                g.load += 1.0 / fits(p.pl.ncta);
+                g.us = std::max(g.us, window_us(r, p.pl.ncta, CLUSTER_THREADS / 32));
+                g.most = std::max(g.most, p.pl.ncta);
+                g.on.push_back(p);
+            }
+        return g;
+    };
+    // Replicas that only a cluster can hold: the most CTAs at which all run at once, and
+    // where no size does, the one with the shortest estimate (waves times window).  64^3
+    // cells in 16^3 fragments at 0.001 vacancies per site, mixed: 39 us per window on 16
+    // CTAs, 49 on 3, but the GPU holds 7 clusters of 16 and 46 of 3, so that 32 replicas
+    // take 190 us on 16 CTAs and 45 on 4.
+    double load = singles_sms() / sms, cluster_load = 0.0, slowest = 0.0;
+    if (!wide.empty()) {
+        Group best;
+        double best_us = 0.0;
+        for (int hi = CLUSTER_MAX_CTAS; hi >= 2;) {
+            Group g = group(wide, 2, hi, [](int) { return CLUSTER_MAX_CTAS; });
+            if (g.on.size() < best.on.size() || g.most == 0) break;  // too few CTAs for some
+            const double us = std::ceil(load + g.load - 1e-9) * g.us;
+            hi = g.most - 1;
+            if (best.on.empty() || us < best_us) {
+                best = std::move(g);
+                best_us = us;
+                if (load + best.load <= 1.0) break;
+            }
+        }
+        for (const Placed& p : best.on) put_on_cluster(p);
+        load += best.load;
+        cluster_load = best.load;
+        slowest = best.us;
+    }
+    // Replicas with four visits or more per warp and phase, or 128 fragments or more to
+    // look at, on clusters instead of one CTA each where the GPU can place all of them at
+    // once: of 48^3 cells in 12^3 fragments, 0.02 vacancies per site, plain 289 -> 117 us
+    // per window (mixed 137 -> 85), in 8^3 fragments 510 -> 277 (mixed 197 -> 158). Fewer
+    // visits are not worth the cluster's barriers: 32^3 cells in 8^3 fragments at 0.001
+    // take 26 us on one CTA, 31 on four (mixed 23 and 29), and at 0.005 44 and 45 (36 and
+    // 40). Half as many CTAs as layers of fragments: a phase takes every other layer (48^3
     // cells at 0.02 take the same on four CTAs as on eight); four at least (64 x 64 x 16
-    // cells in 16 x 16 x 4 fragments at 0.001: 38 us on two, 35 on four). A quarter of the SMs stays
-    // free, as clusters need neighbouring SMs.
-    if (force >= 0 && allowed && b->opts.test_stuck_wait_us == 0) {
+    // cells in 16 x 16 x 4 fragments at 0.001: 38 us on two, 35 on four). All or none: a
+    // batch waits for its slowest replica, and with some on clusters the rest have fewer
+    // SMs (152 replicas of 32^3 cells at 0.01, 19 on clusters: mixed 52 -> 83, plain 142 ->
+    // 203 us).
+    if (force == 0 && allowed && b->opts.test_stuck_wait_us == 0) {
         std::vector<int> dense;
+        double freed = 0.0;
         for (int c = 0; c < 4; ++c)
             for (int r : cls[c]) {
                 const int64_t F = phase_frags(r);
-                const int nz = b->desc[r].nf[2];
-                if (nz >= 4 && (F >= 128 || (F >= 64 && phase_vacs(r) >= 64.0))) dense.push_back(r);
+                if (b->desc[r].nf[2] >= 4 && (F >= 128 || (F >= 64 && phase_vacs(r) >= 64.0))) {
+                    dense.push_back(r);
+                    freed += share[c];
+                }
             }
         std::sort(dense.begin(), dense.end(), [&](int a, int q) {
             return b->n_vac[a] != b->n_vac[q] ? b->n_vac[a] > b->n_vac[q] : a < q;
         });
-        for (int r : dense) {
-            const int room = (int)(0.75 * sms - sms_used());
-            if (room < 2) break;
-            const int most = std::min<int>(std::max(4, b->desc[r].nf[2] / 2), CLUSTER_MAX_CTAS);
-            if (on_cluster(r, 2, most, room) <= 0) continue;
-            for (int c = 0; c < 4; ++c) {
-                auto it = std::find(cls[c].begin(), cls[c].end(), r);
-                if (it != cls[c].end()) cls[c].erase(it);
+        for (int hi = CLUSTER_MAX_CTAS; hi >= 4 && !dense.empty();) {
+            Group g = group(dense, 4, hi, [&](int r) { return std::max(4, b->desc[r].nf[2] / 2); });
+            if (g.on.size() < dense.size()) break;
+            if (load - freed / sms + g.load > 0.9) {
+                hi = g.most - 1;
+                continue;
+            }
+            for (const Placed& p : g.on) put_on_cluster(p);
+            for (int c = 0; c < 4; ++c)
+                cls[c].erase(std::remove_if(cls[c].begin(), cls[c].end(), [&](int r) { return b->run_kernel[r] == 2; }),
+                             cls[c].end());
+            load += g.load - freed / sms;
+            cluster_load += g.load;
+            slowest = std::max(slowest, g.us);
+            break;
+        }
+    }
+    // Many replicas on the colour-phase passes, which take the batch as one: where the
+    // resident kernels need several waves, or the plain form's first draws (0.25 ns each
+    // over the whole GPU, for empty fragments too) longer than the windows they are for.
+    // Both sides are estimates; T_pass is fitted to 8 to 1216 replicas of the shapes above.
+    // 64 replicas of 96^3 cells in 24^3 fragments at 0.001: plain 1778 us per window on
+    // clusters, 450 in passes (mixed 507 and 227); 1216 of 48^3: plain 2078 and 805 (mixed
+    // 372 and 538).
+    if (force == 0 && allowed && b->opts.schedule == 0) {
+        int64_t frags = 0, res_vac = 0;
+        double mean_vac = 0.0;
+        for (int r = 0; r < b->n; ++r) {
+            if (!b->desc[r].resident) continue;
+            const int64_t nf = (int64_t)b->desc[r].nf[0] * b->desc[r].nf[1] * b->desc[r].nf[2];
+            frags += nf;
+            res_vac += b->n_vac[r];
+            mean_vac = std::max(mean_vac, (double)b->n_vac[r] / (double)nf);
+        }
+        // one CTA each: a replica takes its share of an SM for its window's time
+        double work = std::ceil(cluster_load - 1e-9) * slowest;
+        for (int c = 0; c < 4; ++c)
+            for (int r : cls[c]) {
+                const double us = window_us(r, 1, threads[c] / 32);
+                work += us * share[c] / sms;
+                slowest = std::max(slowest, us);
+            }
+        const double draws_us = prec ? 0.0 : 0.25e-3 * (double)frags * plain_ev;
+        if (load > 1.0 || draws_us > slowest) {
+            static const double base[3] = {175.0, 98.0, 205.0}, per_vac[3] = {20.0, 12.0, 20.0},
+                                per_frag[3] = {1.6e-4, 0.7e-4, 1.8e-4}, per_v[3] = {7.5e-4, 3.6e-4, 16e-4};
+            const double waves_us = std::max(work, slowest);
+            const double resident_us = std::max(waves_us, draws_us) + 0.4 * std::min(waves_us, draws_us);
+            const double passes_us = base[form] + per_vac[form] * mean_vac + per_frag[form] * (double)frags +
+                                     per_v[form] * (double)res_vac;
+            // (waves disturb each other more than the estimate has it, with site energies most)
+            static const double bias[3] = {1.0, 0.95, 0.9};
+            if (passes_us * (load > 1.0 ? bias[form] : 1.12) < resident_us) {
+                for (RepDesc& D : b->desc) D.resident = 0;
+                b->run_kernel.assign(b->n, 0);
+                b->run_ctas.assign(b->n, 0);
+                plans.clear();
+                for (int c = 0; c < 4; ++c) cls[c].clear();
             }
         }
     }
@@ -640,7 +771,6 @@ int plan_residency(kmc_batch* b)
             if (phase_vacs(r) <= line * busy * (CLUSTER_THREADS / 32)) return false;
             b->desc[r].resident = 0;
             b->run_kernel[r] = b->run_ctas[r] = 0;
-            b->any_global = true;
             return true;
         };
         for (int c = 0; c < 4; ++c)
@@ -709,6 +839,7 @@ int plan_residency(kmc_batch* b)
         });
     for (int c = 0; c < 4; ++c)
         for (int r : cls[c]) cmax[c] = std::max(cmax[c], need_of[r]);
+    b->any_global = std::any_of(b->desc.begin(), b->desc.end(), [](const RepDesc& D) { return !D.resident; });
     if (b->opts.schedule == 2 && b->any_global)
         return fail(FKMC_EINVAL, "schedule 2 needs every replica to fit the resident kernel (mixed form)");
     std::vector<int32_t> order;
@@ -1512,7 +1643,7 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
         }
         return FKMC_OK;
     };
-    if (b->any_global && windows > 0) CK(cudaMemsetAsync(b->wctl, 0, sizeof(unsigned long long) * 2, b->st), "memset");
+    uint64_t passes_at = UINT64_MAX, pass_windows = 0;  // the passes' window counter; windows they ran
     const uint64_t every = b->elec_on ? (uint64_t)b->elec.refresh_windows : 0;
     for (uint64_t wk = 0; wk < windows;) {
         if (every > 0 && b->elec_age >= every) {  // the potential follows the vacancies
@@ -1530,7 +1661,15 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
         if (b->any_global) {
             int rc2 = ensure_graph();
             if (rc2) return rc2;
+            if (passes_at != wk) {  // the first, or the first after a refresh that changed the plan
+                const unsigned long long at[2] = {wk, 0};
+                CK(wk == 0 ? cudaMemsetAsync(b->wctl, 0, sizeof at, b->st)
+                           : cudaMemcpyAsync(b->wctl, at, sizeof at, cudaMemcpyHostToDevice, b->st),
+                   "window counter");
+            }
             for (uint64_t k = 0; k < nw; ++k) CK(cudaGraphLaunch(b->window_exec, b->st), "graph launch");
+            passes_at = wk + nw;
+            pass_windows += nw;
         }
         if (!b->rclass.empty()) CK(cudaStreamWaitEvent(b->st, b->res_join, 0), "stream wait");
         wk += nw;
@@ -1553,7 +1692,7 @@ int kmc_run(kmc_batch* b, uint64_t windows, kmc_run_stats* stats)
         stats->windows = windows;
         stats->launches =
             res_launches +
-            (b->any_global ? window_launches(b) * windows : 0) +
+            window_launches(b) * pass_windows +
             extra_launches;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, b->ev0, b->ev1);
