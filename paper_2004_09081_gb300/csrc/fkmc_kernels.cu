@@ -162,10 +162,32 @@ __host__ __device__ inline size_t warp_smem_bytes(int cap, bool site)
 
 // Rate types of every event of the fragment, read from the occupancy words
 // in L2 (ld.global.cg, so that this warp's own exchanges are seen).
-template <bool GRAIN = false>
+template <bool GRAIN, int PREC>
 __device__ __forceinline__ void compute_types(const RepDesc& D, const uint32_t* occ, const WarpSmem& S,
                                               int nslots, int nch, int lane, const uint8_t* gb = nullptr)
 {
+    // one chunk by itself (plain form: 78 -> 77 us per window of 128 x 128 x 2 cells in
+    // 2 x 2 x 2 fragments; the mixed form's dense fragments lose 4% to the second path)
+    if (PREC == 0 && nch <= 1) {
+        const int m = lane >> 3, n = lane & 7;
+        int ty = -1;
+        if (m < nslots && S.alive[m]) {
+            int t, x, y, z;
+            split_key(S.rec[S.order[m]].key, t, x, y, z);
+            const NbEntry nb = nb_entry(t, n);
+            const int jx = wrapc(x + nb.dc[0], D.L[0]);
+            const int jy = wrapc(y + nb.dc[1], D.L[1]);
+            const int jz = wrapc(z + nb.dc[2], D.L[2]);
+            const uint32_t w = __ldcg(occ + occ_word(D, nb.t2, jx, jy, jz));
+            const int code = (int)((w >> occ_shift(jx)) & 3u);
+            ty = code == SP_V ? -1 : code * 3 + nb.d[2] + 1;
+            if constexpr (GRAIN) {  // a hop touching a boundary cell takes the raised table
+                if (ty >= 0 && (gb[cell_index(D, x, y, z)] | gb[cell_index(D, jx, jy, jz)])) ty += 6;
+            }
+        }
+        S.types[lane] = (int8_t)ty;
+        return;
+    }
     // four chunks at a time, their reads issued before any is used: a dense
     // fragment's visit is a chain of memory latencies, one per group instead of
     // one per chunk
@@ -469,7 +491,7 @@ __global__ void __launch_bounds__(128, 8) k_run(const RepDesc* __restrict__ desc
     const int nslots = nv;
     const int nch = (nslots + 3) >> 2;  // 32 events per chunk
     if constexpr (SITE) compute_rates_site<GRAIN>(D, occ, sa, S, nslots, nch, lane, status);
-    else compute_types<GRAIN>(D, occ, S, nslots, nch, lane, sa.gbound);
+    else compute_types<GRAIN, PREC>(D, occ, S, nslots, nch, lane, sa.gbound);
     __syncwarp();
     // rate of event index e (lane-local chunk element)
     auto rate_of = [&](int e) -> V {
@@ -648,7 +670,7 @@ __global__ void __launch_bounds__(128, 8) k_run(const RepDesc* __restrict__ desc
         else mclock = nclock;
         ++i;
         if constexpr (SITE) compute_rates_site<GRAIN>(D, occ, sa, S, nslots, nch, lane, status);
-        else compute_types<GRAIN>(D, occ, S, nslots, nch, lane, sa.gbound);
+        else compute_types<GRAIN, PREC>(D, occ, S, nslots, nch, lane, sa.gbound);
         __syncwarp();
     }
 
@@ -937,13 +959,15 @@ __device__ __forceinline__ void load_tables(LaneTables& tab, const RepDesc* desc
 // exchanges are atomics there) before any is used.  Away from the lattice's
 // faces no coordinate wraps, and a neighbour's row is the vacancy's row plus
 // a 32-bit offset.
-template <bool GRAIN>
+template <bool GRAIN, bool ONE>
 __device__ __forceinline__ uint32_t lane_types(const RepDesc& D, const uint4* lgeo, const uint32_t* occ,
                                                const uint8_t* gb, uint64_t key, unsigned long long& sum)
 {
     int t, x, y, z;
     split_key(key, t, x, y, z);
-    const uint4 geo = lgeo[t];
+    uint4 geo;
+    if constexpr (ONE) geo = lgeo[t];
+    else geo = __ldg(lgeo + t);
     const uint64_t g8 = ((uint64_t)geo.y << 32) | geo.x;
     const int L0 = D.L[0], L1 = D.L[1], L2 = D.L[2];
     const uint32_t* occ_r = occ + D.occ_word_off;
@@ -1122,14 +1146,13 @@ __global__ void __launch_bounds__(128, 4) k_run_lane_reg(const RepDesc* __restri
 #pragma unroll
         for (int k = 0; k < NL; ++k) {
             sm[k] = 0ull;
-            ty[k] = k < nv ? lane_types<GRAIN>(D, lgeo, occ, gb, r[k].key, sm[k]) : 0u;
+            ty[k] = k < nv ? lane_types<GRAIN, ONE>(D, lgeo, occ, gb, r[k].key, sm[k]) : 0u;
         }
         const uint64_t w = D.window + wctl[1];
         const uint64_t k1 = key_word(D.replica, PURPOSE_HOP);
         U64x4 blk{};
         uint64_t clock = 0;
         bool fp = false;  // the clock's form (mixed_clock)
-        const uint64_t th = window_bits(D.theta_tau, D.F);
         uint64_t i = 0;
         for (;;) {
             unsigned long long total = 0ull;
@@ -1145,7 +1168,7 @@ __global__ void __launch_bounds__(128, 4) k_run_lane_reg(const RepDesc* __restri
             const uint64_t xs = odd ? blk.x[3] : blk.x[1];
             const float Ef = neglog32(odd ? blk.x[2] : blk.x[0]);
             uint64_t nclock = 0;
-            if (mixed_clock(clock, fp, __fdiv_rn(Ef, u64_to_float_rn(total)), th, nclock)) break;
+            if (mixed_clock(clock, fp, __fdiv_rn(Ef, u64_to_float_rn(total)), window_bits(D.theta_tau, D.F), nclock)) break;
             const unsigned long long target = __umul64hi(xs, total);
             // slot m and neighbour n of the first event whose prefix exceeds the target
             int m = NL - 1;
@@ -1220,7 +1243,11 @@ __global__ void __launch_bounds__(128, 4) k_run_lane_reg(const RepDesc* __restri
                 const int gy = frag_of(jy, D.base[1], D.rem[1]);
                 const int gz = frag_of(jz, D.base[2], D.rem[2]);
                 out_g = D.frag_base + ((int64_t)gz * D.nf[1] + gy) * D.nf[0] + gx;
-                out_slot = atomicAdd(counts + out_g, 1);  // used after the rates' reads below
+                out_slot = atomicAdd(counts + out_g, 1);  // ONE: used after the rates' reads below
+                if constexpr (!ONE) {  // here, holding it costs registers that the descriptor's reads need
+                    if (out_slot < cap) recs[out_g * cap + out_slot] = cur;
+                    else atomicOr(status, STATUS_OVERFLOW);
+                }
                 alive &= ~(1u << m);
                 ++nhand;
             }
@@ -1250,7 +1277,7 @@ __global__ void __launch_bounds__(128, 4) k_run_lane_reg(const RepDesc* __restri
                 for (int q = 1; q < NL; ++q)
                     if (q == k) kk = r[q].key;
                 unsigned long long sk = 0ull;
-                const uint32_t tk = lane_types<GRAIN>(D, lgeo, occ, gb, kk, sk);
+                const uint32_t tk = lane_types<GRAIN, ONE>(D, lgeo, occ, gb, kk, sk);
 #pragma unroll
                 for (int q = 0; q < NL; ++q)
                     if (q == k) {
@@ -1258,7 +1285,7 @@ __global__ void __launch_bounds__(128, 4) k_run_lane_reg(const RepDesc* __restri
                         sm[q] = sk;
                     }
             }
-            if (!owned) {
+            if (ONE && !owned) {
                 if (out_slot < cap) recs[out_g * cap + out_slot] = cur;
                 else atomicOr(status, STATUS_OVERFLOW);
             }
@@ -1538,7 +1565,7 @@ __global__ void __launch_bounds__(LANE_THREADS) k_run_lane(const RepDesc* __rest
             const int k = __ffs(pending) - 1;
             pending &= pending - 1u;
             unsigned long long sk;
-            S.ty[k][tid] = lane_types<GRAIN>(D, lgeo, occ, gb, S.key[k][tid], sk);
+            S.ty[k][tid] = lane_types<GRAIN, ONE>(D, lgeo, occ, gb, S.key[k][tid], sk);
             S.sum[k][tid] = sk;
         }
 
