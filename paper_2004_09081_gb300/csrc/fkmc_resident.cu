@@ -59,6 +59,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 
 #include "fkmc_device.cuh"
 #include "fkmc_kernels.h"
@@ -850,44 +851,47 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     if constexpr (SITE) {
         for (int k = tid; k < sz.btab; k += NT) S.btab[k] = sa.btab[D.btab_off + k];
     }
-    for (int c = 0; c < 8; ++c) {
-        int cnt[2], lz0;
-        const int n = colour_count(c, cnt, lz0);
-        for (int l = tid; l < n; l += NT) {
-            const int i0 = l % cnt[0], i1 = (l / cnt[0]) % cnt[1], i2 = l / (cnt[0] * cnt[1]);
-            const int f0 = D.nf[0] == 1 ? 0 : 2 * i0 + (c & 1), f1 = D.nf[1] == 1 ? 0 : 2 * i1 + ((c >> 1) & 1);
-            const int f2 = lz0 + 2 * i2, lf = ((f2 - fzb) * D.nf[1] + f1) * D.nf[0] + f0;
-            S.flist[sh.coff[c] + l] = (uint16_t)lf;
-            const int o0 = frag_start(f0, D.base[0], D.rem[0]), e0 = frag_start(f0 + 1, D.base[0], D.rem[0]) - o0;
-            const int o1 = frag_start(f1, D.base[1], D.rem[1]), e1 = frag_start(f1 + 1, D.base[1], D.rem[1]) - o1;
-            const int o2 = frag_start(f2, D.base[2], D.rem[2]), e2 = frag_start(f2 + 1, D.base[2], D.rem[2]) - o2;
-            S.box[lf] = make_uint2((uint32_t)o0 | (uint32_t)o1 << 10 | (uint32_t)o2 << 20,
-                                   (uint32_t)(e0 - 1) | (uint32_t)(e1 - 1) << 10 | (uint32_t)(e2 - 1) << 20);
-        }
+    for (int lf = tid; lf < nfl; lf += NT) {
+        const int q = lf / D.nf[0], f0 = lf - q * D.nf[0], lz = q / D.nf[1], f1 = q - lz * D.nf[1], f2 = fzb + lz;
+        const int c = (f0 & 1) | (f1 & 1) << 1 | (f2 & 1) << 2;
+        // its place in its colour: this CTA's first layer of the colour is fzb or the next one
+        const int l = ((f2 - fzb) / 2 * half_up(D.nf[1] - (c >> 1 & 1)) + f1 / 2) * half_up(D.nf[0] - (c & 1)) + f0 / 2;
+        S.flist[sh.coff[c] + l] = (uint16_t)lf;
+        const int o0 = frag_start(f0, D.base[0], D.rem[0]), e0 = frag_start(f0 + 1, D.base[0], D.rem[0]) - o0;
+        const int o1 = frag_start(f1, D.base[1], D.rem[1]), e1 = frag_start(f1 + 1, D.base[1], D.rem[1]) - o1;
+        const int o2 = frag_start(f2, D.base[2], D.rem[2]), e2 = frag_start(f2 + 1, D.base[2], D.rem[2]) - o2;
+        S.box[lf] = make_uint2((uint32_t)o0 | (uint32_t)o1 << 10 | (uint32_t)o2 << 20,
+                               (uint32_t)(e0 - 1) | (uint32_t)(e1 - 1) << 10 | (uint32_t)(e2 - 1) << 20);
     }
     // sites of this slab count from vmap_s, sites of the replica from vmap_r
     uint32_t* const vmap_r = vmap + D.vmap_off;
     uint32_t* const vmap_s = vmap_r + (int64_t)geo.zb * D.L[1] * D.row_words * 48;
     VacRec* const recs_r = recs + D.frag_base * cap;  // record indices count from here
     const uint32_t rec_lim = (uint32_t)(D.nf[0] * D.nf[1] * D.nf[2] * cap);
+    // one thread per fragment, its next count on the way while it is staged and four records at a time
+    int c_next = tid < nfl ? counts[frag0 + tid] : 0;
     for (int f = tid; f < nfl; f += NT) {
         const int64_t g = frag0 + f;
-        const int c = counts[g];
+        const int c = c_next;
+        if (f + NT < nfl) c_next = counts[g + NT];
         if (c > cap) atomicOr(status, STATUS_OVERFLOW);
         uint32_t* const sl = S.slots + f * ks;
-        int have = 0;
-        for (int k = 0; k < c && k < cap; ++k) {
-            int t, x, y, z;
-            split_key(recs[g * cap + k].key, t, x, y, z);
-            vmap_s[map_index(geo, key32(t, x, y, z - geo.zb))] = (uint32_t)((g - D.frag_base) * cap + k);
-            if (c <= ks) {  // into the sorted list
-                const uint32_t key = key32(t, x, y, z);
-                int m = have++;
-                for (; m > 0 && sl[m - 1] > key; --m) sl[m] = sl[m - 1];
-                sl[m] = key;
-            }
+        for (int k = 0; k < ks; ++k) sl[k] = DEAD;
+        const uint32_t at = (uint32_t)((g - D.frag_base) * cap);
+        for (int k0 = 0; k0 < c && k0 < cap; k0 += 4) {
+            uint64_t k64[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < c) k64[u] = recs[g * cap + k0 + u].key;  // (cap is a multiple of 8)
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < c) {
+                    int t, x, y, z;
+                    split_key(k64[u], t, x, y, z);
+                    vmap_s[map_index(geo, key32(t, x, y, z - geo.zb))] = at + k0 + u;
+                    if (k0 + u < ks) sl[k0 + u] = key32(t, x, y, z);  // the first visit sorts them
+                }
         }
-        for (int k = have; k < ks; ++k) sl[k] = DEAD;
         if (c > ks) sl[0] = UNLISTED;
         S.stale[f] = 0;
         // the limit the last launch left, where nothing changed the replica since
@@ -1544,41 +1548,103 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     }
     VacRec* const tmp_r = tmp + (D.tmp_off + (int64_t)fzb * D.nf[1] * D.nf[0]) * cap;
-    for (int f = warp; f < nfl; f += NW) {
-        const uint2 bx = S.box[f];
-        int n = gather(S, geo, wkey, cap, lane, (int)(bx.x & 1023u), (int)((bx.x >> 10) & 1023u), (int)(bx.x >> 20),
-                       (int)(bx.y & 1023u) + 1, (int)((bx.y >> 10) & 1023u) + 1, (int)(bx.y >> 20) + 1);
-        if (n > cap) {
-            if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
-            n = cap;
+    // a record: key and id | displacement, as three words
+    auto index_of = [&](uint32_t key) -> uint32_t { return min(__ldcg(vmap_r + map_index(geo, key)), rec_lim - 1); };
+    auto put_copy = [&](int f, int slot, uint32_t key, int2 d01, int2 d2id) {
+        int t, x, y, z;
+        split32(key, t, x, y, z);
+        VacRec& o = tmp_r[(int64_t)f * cap + slot];
+        o.key = make_key(t, x, y, z);
+        *reinterpret_cast<int2*>(&o.d[0]) = d01;
+        *reinterpret_cast<int2*>(&o.d[2]) = d2id;
+    };
+    static_assert(sizeof(VacRec) == 24 && offsetof(VacRec, d) == 8 && offsetof(VacRec, id) == 20, "copied as words");
+    // A valid list gives a fragment's vacancies; a fragment without one is scanned for it
+    // first, or, where a list cannot hold them, copied at once.  (A scan of every fragment,
+    // and the chain vmap - record - copy for one fragment of a warp after the other, made a
+    // call of one window take 166 us on 64^3 cells in 2^3-cell fragments and 68 on 32^3 in
+    // 4^3-cell ones, now 65 and 41 at 0.001 vacancies per site.)
+    for (int f0 = warp; f0 < nfl; f0 += 32 * NW) {
+        const int f = f0 + NW * lane;
+        for (unsigned td = __ballot_sync(FULL, f < nfl && (S.stale[f] != 0 || S.slots[f * ks] == UNLISTED)); td;
+             td &= td - 1) {
+            const int fs = f0 + NW * (__ffs(td) - 1);
+            const uint2 bx = S.box[fs];
+            int n = gather(S, geo, wkey, cap, lane, (int)(bx.x & 1023u), (int)((bx.x >> 10) & 1023u), (int)(bx.x >> 20),
+                           (int)(bx.y & 1023u) + 1, (int)((bx.y >> 10) & 1023u) + 1, (int)(bx.y >> 20) + 1);
+            if (n > cap) {
+                if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
+                n = cap;
+            }
+            if (n <= ks) {
+                if (lane < ks) S.slots[fs * ks + lane] = lane < n ? wkey[lane] : DEAD;
+            } else {
+                for (int m = lane; m < n; m += 32) {
+                    const VacRec* src = recs_r + index_of(wkey[m]);
+                    put_copy(fs, m, wkey[m], __ldcg(reinterpret_cast<const int2*>(&src->d[0])),
+                             __ldcg(reinterpret_cast<const int2*>(&src->d[2])));
+                }
+                if (lane == 0) S.stale[fs] = (uint8_t)n;  // more than a list holds: copied
+            }
+            __syncwarp();
+            if (n <= ks && lane == 0) S.stale[fs] = 0;
+            __syncwarp();
         }
-        for (int k = lane; k < n; k += 32) {
-            const uint32_t key = wkey[k];
-            const VacRec* src = recs_r + min(__ldcg(vmap_r + map_index(geo, key)), rec_lim - 1);
-            int t, x, y, z;
-            split32(key, t, x, y, z);
-            VacRec rr;
-            rr.key = make_key(t, x, y, z);
-            rr.d[0] = __ldcg(&src->d[0]);
-            rr.d[1] = __ldcg(&src->d[1]);
-            rr.d[2] = __ldcg(&src->d[2]);
-            rr.id = __ldcg(&src->id);
-            tmp_r[(int64_t)f * cap + k] = rr;
+    }
+    __syncthreads();
+    for (int f = tid; f < nfl; f += NT) {  // one thread per fragment, the reads of four records in flight
+        int n = S.stale[f];
+        if (n == 0) {
+            uint32_t key[KSLOTS];
+#pragma unroll
+            for (int q = 0; q < KSLOTS; ++q) {
+                key[q] = q < ks ? S.slots[f * ks + q] : DEAD;
+                n += key[q] != DEAD ? 1 : 0;
+            }
+            if (n > 0) {
+#pragma unroll
+                for (int q0 = 0; q0 < KSLOTS; q0 += 4) {
+                    uint32_t at[4];
+                    int2 d01[4], d2id[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) at[u] = key[q0 + u] != DEAD ? index_of(key[q0 + u]) : 0u;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (key[q0 + u] != DEAD) {
+                            d01[u] = __ldcg(reinterpret_cast<const int2*>(&recs_r[at[u]].d[0]));
+                            d2id[u] = __ldcg(reinterpret_cast<const int2*>(&recs_r[at[u]].d[2]));
+                        }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (key[q0 + u] != DEAD) {
+                            int r = 0;  // its place in site order
+#pragma unroll
+                            for (int q = 0; q < KSLOTS; ++q) r += key[q] < key[q0 + u] ? 1 : 0;
+                            put_copy(f, r, key[q0 + u], d01[u], d2id[u]);
+                        }
+                }
+            }
         }
-        __syncwarp();
-        if (lane == 0) {
-            counts[frag0 + f] = n;
-            rc.lim[frag0 + f] = (uint64_t)lim[f];
-        }
+        counts[frag0 + f] = n;
+        S.stale[f] = (uint8_t)n;  // for the move back
+        rc.lim[frag0 + f] = (uint64_t)lim[f];
     }
     if (my_hand && lane == 0) atomicAdd(&sh.hand, my_hand);
     if (my_hops) atomicAdd(&sh.hops, my_hops);
     if constexpr (CL) cluster_sync();
     else __syncthreads();
-    for (int f = warp; f < nfl; f += NW) {
-        const int n = __ldcg(counts + frag0 + f);
-        for (int k = lane; k < n; k += 32) {  // the thread that wrote the copy
-            recs[(frag0 + f) * cap + k] = tmp_r[(int64_t)f * cap + k];
+    for (int f = tid; f < nfl; f += NT) {
+        const int n = S.stale[f];
+        const VacRec* const from = tmp_r + (int64_t)f * cap;
+        VacRec* const to = recs + (frag0 + f) * cap;
+        for (int k0 = 0; k0 < n; k0 += 4) {  // (cap is a multiple of 8)
+            VacRec r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < n) r[u] = from[k0 + u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (k0 + u < n) to[k0 + u] = r[u];
         }
     }
     if (tid == 0) {
