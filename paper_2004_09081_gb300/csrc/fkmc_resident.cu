@@ -614,44 +614,70 @@ __device__ __forceinline__ int gather(const Layout& S, const Geo& g, uint32_t* w
     if (rpl * ex <= 16) return gather_rows<uint32_t>(S, g, wkey, cap, lane, lo0, lo1, lo2, ex, ey, rows, rpl);
     if (rpl * ex <= 31 && ex <= 16)
         return gather_rows<uint64_t>(S, g, wkey, cap, lane, lo0, lo1, lo2, ex, ey, rows, rpl);
-    const int hi0 = lo0 + ex;
-    // larger boxes: 16-cell pieces of rows, one site type after the other
+    // larger boxes: a lane takes 16-cell pieces of rows, all three site types at once; the
+    // keys go to wkey as they are found and are put into site order by rank.  (One type
+    // after the other, in order: 96^3 cells in 12^3-cell fragments at 0.001 vacancies per
+    // site, most of whose visits scan, 102 us per window, now 86.)
     const int pieces = (ex + 15) >> 4, items = rows * pieces;
     int n = 0;
-    for (int t = 0; t < 3; ++t) {
-        for (int base = 0; base < items; base += 32) {
-            const int it = base + lane;
-            uint32_t m = 0;
-            int x0 = 0, y = 0, z = 0;
-            if (it < items) {
-                const int r = it / pieces, p = it - r * pieces;
-                z = r / ey;
-                y = lo1 + r - z * ey;
-                z += lo2;
-                x0 = lo0 + 16 * p;
-                const int len = min(16, hi0 - x0), off = (x0 & 15) * 2;
-                const uint32_t* w = S.occ + word_of(g, t, x0, y, z - g.zb);
-                const uint32_t v = __funnelshift_r(w[0], off + 2 * len > 32 ? w[3] : 0u, off);
-                m = (v >> 1) & ~v & 0x55555555u & (uint32_t)((1ull << (2 * len)) - 1ull);
+    for (int base = 0; base < items; base += 32) {
+        const int it = base + lane;
+        uint32_t m[3] = {0, 0, 0};
+        int x0 = 0, y = 0, z = 0;
+        if (it < items) {
+            const int r = pieces == 1 ? it : it / pieces, p = it - r * pieces;
+            z = (int)(((float)r + 0.5f) * __fdividef(1.0f, (float)ey));  // r / ey, exact for r < 2^19
+            y = lo1 + r - z * ey;
+            z += lo2;
+            x0 = lo0 + 16 * p;
+            const int len = min(16, lo0 + ex - x0), off = (x0 & 15) * 2;
+            const uint32_t* w = S.occ + word_of(g, 0, x0, y, z - g.zb);
+            const bool two = off + 2 * len > 32;
+            const uint32_t mask = 0x55555555u & (uint32_t)((1ull << (2 * len)) - 1ull);
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                const uint32_t v = __funnelshift_r(w[t], two ? w[3 + t] : 0u, off);
+                m[t] = (v >> 1) & ~v & mask;
             }
-            const int c = __popc(m);
-            if (!__any_sync(FULL, c != 0)) continue;
+        }
+        const int c = __popc(m[0]) + __popc(m[1]) + __popc(m[2]);
+        const unsigned some = __ballot_sync(FULL, c != 0);
+        if (!some) continue;
+        int slot;
+        if (!__any_sync(FULL, c > 1)) {
+            slot = n + __popc(some & ((1u << lane) - 1u));
+            n += __popc(some);
+        } else {
             int s = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int u = __shfl_up_sync(FULL, s, o);
                 if (lane >= o) s += u;
             }
-            int slot = n + s - c;
+            slot = n + s - c;
             n += __shfl_sync(FULL, s, 31);
-            while (m) {
-                const int b = (__ffs(m) - 1) >> 1;
-                m &= m - 1;
+        }
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+            while (m[t]) {
+                const int b = (__ffs(m[t]) - 1) >> 1;
+                m[t] &= m[t] - 1;
                 if (slot < cap) wkey[slot] = key32(t, x0 + b, y, z);
                 ++slot;
             }
-        }
     }
+    __syncwarp();
+    const int have = min(n, cap);  // at most RESIDENT_MAX_SLOTS = 64: two keys per lane
+    const uint32_t k0 = lane < have ? wkey[lane] : DEAD, k1 = lane + 32 < have ? wkey[lane + 32] : DEAD;
+    int r0 = 0, r1 = 0;
+    for (int q = 0; q < have; ++q) {
+        const uint32_t v = wkey[q];
+        r0 += v < k0 ? 1 : 0;
+        r1 += v < k1 ? 1 : 0;
+    }
+    __syncwarp();
+    if (k0 != DEAD) wkey[r0] = k0;
+    if (k1 != DEAD) wkey[r1] = k1;
     __syncwarp();
     return n;
 }
