@@ -1753,7 +1753,9 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
            "clock upload");
     }
     // one launch for many steps: where its grid holds the vacancies and its two buffers
-    // can be had, else the launches of each step
+    // can be had, else the launches of each step.  (One step alone is cheaper in its own
+    // launches: a call on 64^3 cells 92 us, 97 with the barriers and the clock's launch;
+    // two steps 115 and 106.)
     NullStepsPlan plan;
     int64_t max_vac = 0, max_sites = 0;
     for (int r = 0; r < b->n; ++r) {
@@ -1768,7 +1770,7 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
         return *p != nullptr;
     };
     const int log_steps = (int)std::min<uint64_t>(NULL_LOG_STEPS, steps);
-    const bool one_launch = steps > 0 && null_steps_plan(b->n, max_vac, max_sites, &plan) &&
+    const bool one_launch = steps > 1 && null_steps_plan(b->n, max_vac, max_sites, &plan) &&
                             grow((void**)&b->null_types, &b->null_types_bytes, sizeof(uint32_t) * (size_t)total_vac) &&
                             grow(&b->null_log, &b->null_log_size, null_log_bytes(b->n, log_steps));
     if (total_picks > b->props_cap) {
@@ -1794,7 +1796,8 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
        "null gather");
     ++launches;
     if (one_launch) {
-        for (uint64_t k = 0; k < steps; k += NULL_LOG_STEPS) {
+        const uint64_t run = b->opts.test_stuck_wait_us ? std::min<uint64_t>(steps, NULL_LOG_STEPS) : steps;
+        for (uint64_t k = 0; k < run; k += NULL_LOG_STEPS) {
             CK(launch_null_steps(plan, b->d_desc, b->n, k, (int)std::min<uint64_t>(NULL_LOG_STEPS, steps - k), b->vac,
                                  b->null_types, b->occ, b->grains_on ? b->gbound : nullptr, b->claims, b->tracer,
                                  b->null_log, b->theta, b->stats, b->status, (uint32_t)b->opts.test_stuck_wait_us,
@@ -1834,6 +1837,9 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
        "null scatter");
     ++launches;
     CK(cudaEventRecord(b->ev1, b->st), "event record");
+    for (int r = 0; r < b->n; ++r) b->desc[r].null_step += steps;
+    rc = upload_desc(b);  // ahead of the copies: its wait is for the kernels anyway
+    if (rc) return rc;
     CK(cudaMemcpyAsync(b->stats_host.data(), b->stats, sizeof(unsigned long long) * 2 * b->n, cudaMemcpyDeviceToHost,
                        b->st),
        "stats copy");
@@ -1841,10 +1847,10 @@ int kmc_run_null(kmc_batch* b, uint64_t steps, int64_t n_frg, kmc_run_stats* sta
        "clock copy");
     uint32_t word = 0;
     rc = check_status(b, &word);
-    // after a wait that ran out the steps are incomplete and do not count
-    if (!(word & STATUS_TIMEOUT))
-        for (int r = 0; r < b->n; ++r) b->desc[r].null_step += steps;
-    if (const int rc_ = upload_desc(b)) return rc_;
+    if (word & STATUS_TIMEOUT) {  // a wait ran out: the steps are incomplete and do not count
+        for (int r = 0; r < b->n; ++r) b->desc[r].null_step -= steps;
+        if (const int rc_ = upload_desc(b)) return rc_;
+    }
     b->field_valid = false;
     {
         const int rc_ = drop_resident_cache(b);

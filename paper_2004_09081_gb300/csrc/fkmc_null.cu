@@ -375,8 +375,7 @@ constexpr unsigned long long NULL_WAIT_NS = 2000000000ull;  // bound on one barr
 
 // Barrier number `target / ctas` of the replica's CTAs; false when a wait of
 // `limit` ns ran out (here or elsewhere), after which every CTA leaves.
-__device__ __forceinline__ bool null_barrier(NullBarrier* bar, unsigned target,
-                                             unsigned long long limit = NULL_WAIT_NS)
+__device__ __forceinline__ bool null_barrier(NullBarrier* bar, unsigned target, unsigned long long limit)
 {
     __shared__ int stop;
     __threadfence();  // this thread's writes before the arrival
@@ -419,14 +418,12 @@ __device__ __forceinline__ void warp_sum_max(unsigned long long v, unsigned long
 // Steps k0 .. k0 + steps - 1 of every replica (CTAs [r ctas, (r + 1) ctas): replica
 // r).  types: one word per vacancy, nibble n = rate type of event n + 1 (0: no
 // event).  log: per replica and step, cleared by the caller, as are the barriers.
-// stuck_ns > 0: a test of the barrier's bounded wait, which first waits that long for
-// one arrival more than there are CTAs, and makes no step.  A launch behind one whose
-// wait ran out makes none either.
+// A launch behind one whose wait ran out makes no step.
 template <int PER>
 __global__ void __launch_bounds__(CT)
     k_null_steps(const RepDesc* __restrict__ descs, int ctas, uint64_t k0, int steps, VacRec* vac, uint32_t* types,
                  uint32_t* occ, const uint8_t* __restrict__ gb, unsigned long long* claims, int32_t* tracer,
-                 NullStep* log, int log_stride, NullBarrier* bars, uint32_t* status, unsigned long long stuck_ns)
+                 NullStep* log, int log_stride, NullBarrier* bars, uint32_t* status)
 {
     __shared__ RepDesc D;
     __shared__ PickKeys pk[2];           // by step parity
@@ -445,10 +442,6 @@ __global__ void __launch_bounds__(CT)
     }
     __syncthreads();
     if (late) return;
-    if (stuck_ns && !null_barrier(bar, (unsigned)ctas + 1u, stuck_ns)) {
-        if (tid == 0) atomicOr(status, STATUS_TIMEOUT);
-        return;
-    }
     if (tid < 16) q[tid] = tid == 0 || tid > 12 ? 0ull : (tid <= 6 ? D.qn[tid - 1] : D.qng[tid - 7]);
     const int nv = (int)D.null_nv, np = (int)D.null_nfrg;
     VacRec* const vr = vac + D.vac_off;
@@ -535,7 +528,7 @@ __global__ void __launch_bounds__(CT)
             atomicMax(&st->max, m2);
         }
         keys_of(step + 1);
-        if (!null_barrier(bar, target += ctas)) break;
+        if (!null_barrier(bar, target += ctas, NULL_WAIT_NS)) break;
         // ---- picks: event or null event, claims
         if (tid == 0) rmax = __ldcg(&st->max);
         uint64_t key[PER];
@@ -575,7 +568,7 @@ __global__ void __launch_bounds__(CT)
             atomicMin(cl + ls[u], mine);
             atomicMin(cl + lj[u], mine);
         }
-        if (!null_barrier(bar, target += ctas)) break;
+        if (!null_barrier(bar, target += ctas, NULL_WAIT_NS)) break;
         // ---- exchanges of the picks that hold both their claims
         unsigned done = 0;
 #pragma unroll
@@ -615,9 +608,18 @@ __global__ void __launch_bounds__(CT)
             done += __popc(__ballot_sync(FULL, did));
         }
         if (lane == 0 && done) atomicAdd(&st->updated, (unsigned long long)done);
-        if (!null_barrier(bar, target += ctas)) break;
+        if (!null_barrier(bar, target += ctas, NULL_WAIT_NS)) break;
     }
     if (tid == 0 && *reinterpret_cast<volatile unsigned*>(&bar->stop) != 0u) atomicOr(status, STATUS_TIMEOUT);
+}
+
+// The test of the barrier's bounded wait: the replica's CTAs wait for one arrival more
+// than there are of them.
+__global__ void __launch_bounds__(CT) k_null_stuck(int ctas, NullBarrier* bars, uint32_t* status,
+                                                   unsigned long long limit)
+{
+    if (!null_barrier(bars + blockIdx.x / ctas, (unsigned)ctas + 1u, limit) && threadIdx.x == 0)
+        atomicOr(status, STATUS_TIMEOUT);
 }
 
 // The clocks and hop counters of `steps` steps from their log, one block per
@@ -708,7 +710,7 @@ cudaError_t launch_null_step(const RepDesc* d_descs, int nrep, int64_t total_vac
 }
 
 using NullStepsFn = void (*)(const RepDesc*, int, uint64_t, int, VacRec*, uint32_t*, uint32_t*, const uint8_t*,
-                             unsigned long long*, int32_t*, NullStep*, int, NullBarrier*, uint32_t*, unsigned long long);
+                             unsigned long long*, int32_t*, NullStep*, int, NullBarrier*, uint32_t*);
 
 static NullStepsFn null_steps_kernel(int per)
 {
@@ -754,7 +756,6 @@ cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, in
                               unsigned long long* claims, int32_t* tracer, void* log_mem, double* theta,
                               unsigned long long* stats, uint32_t* status, uint32_t stuck_wait_us, cudaStream_t st)
 {
-    unsigned long long stuck_ns = 1000ull * stuck_wait_us;
     NullBarrier* bars = reinterpret_cast<NullBarrier*>(log_mem);
     NullStep* log = reinterpret_cast<NullStep*>(reinterpret_cast<char*>(log_mem) + ((sizeof(NullBarrier) * nrep + 31) & ~(size_t)31));
     int stride = steps;
@@ -762,8 +763,14 @@ cudaError_t launch_null_steps(const NullStepsPlan& p, const RepDesc* d_descs, in
                                                  sizeof(NullStep) * (size_t)nrep * stride), st);
     if (e != cudaSuccess) return e;
     int ctas = p.ctas;
+    if (stuck_wait_us) {  // the steps' launch then finds the status set
+        unsigned long long limit = 1000ull * stuck_wait_us;
+        void* stuck[] = {&ctas, &bars, &status, &limit};
+        e = cudaLaunchCooperativeKernel((const void*)k_null_stuck, dim3((unsigned)(ctas * nrep)), dim3(CT), stuck, 0, st);
+        if (e != cudaSuccess) return e;
+    }
     void* args[] = {(void*)&d_descs, &ctas, &k0, &steps, &vac, &types, &occ, (void*)&gb, &claims, &tracer, &log,
-                    &stride, &bars, &status, &stuck_ns};
+                    &stride, &bars, &status};
     e = cudaLaunchCooperativeKernel((const void*)null_steps_kernel(p.per), dim3((unsigned)(ctas * nrep)), dim3(CT), args,
                                     0, st);
     if (e != cudaSuccess) return e;
