@@ -613,17 +613,17 @@ int plan_residency(kmc_batch* b)
         for (const ClusterPlan& pl : plans) used += pl.ncta;
         return used;
     };
-    // Estimate of a resident replica's window, us: the cost of a phase's chain with one
-    // visit, of each further visit per warp, of each vacancy beyond the first in a visit,
-    // and of the screen and draws per fragment and CTA.  Fitted to 60 timings on one GB300
-    // of 32^3 .. 128^3 cells at 0.001 to 0.01 vacancies per site, on one CTA and on 2 to 16
-    // (within 30%); the lines below need no better.
+    // Estimate of a resident replica's window, us: the longest of a phase's visits (on one
+    // CTA it grows with their number), each visit per warp, each vacancy of a fragment, and
+    // the screen and draws per fragment and CTA.  Fitted to 70 timings on one GB300 of 8^3
+    // .. 128^3 cells at 0.001 to 0.02 vacancies per site, on one CTA and on 2 to 16 (within
+    // 30%); the lines below need no better.
     auto window_us = [&](int r, int nc, double warps) {
-        static const double c1[3] = {24.0, 20.0, 40.0}, cn[3] = {41.0, 36.0, 63.0}, per_visit[3] = {4.6, 3.7, 8.0},
+        static const double c1[3] = {6.5, 5.5, 11.0}, cn[3] = {41.0, 36.0, 63.0}, per_visit[3] = {4.6, 3.7, 8.0},
                             per_vac[3] = {7.0, 4.0, 7.0}, per_frag[3] = {0.04, 0.04, 0.08};
         const int32_t* nf = b->desc[r].nf;
         const int busy = nc > 1 ? std::min(nc, std::max(1, nf[2] / 2)) : 1;  // a phase takes every other layer
-        return (nc > 1 ? cn : c1)[form] + per_visit[form] * phase_vacs(r) / (warps * busy) +
+        return (nc > 1 ? cn[form] : c1[form] * std::log(1.0 + phase_vacs(r))) + per_visit[form] * phase_vacs(r) / (warps * busy) +
                per_vac[form] * (double)b->n_vac[r] / ((double)nf[0] * nf[1] * nf[2]) +
                per_frag[form] * (double)phase_frags(r) / busy;
     };
@@ -715,12 +715,13 @@ int plan_residency(kmc_batch* b)
         }
     }
     // Many replicas on the colour-phase passes, which take the batch as one: where the
-    // resident kernels need several waves, or the plain form's first draws (0.25 ns each
-    // over the whole GPU, for empty fragments too) longer than the windows they are for.
+    // resident kernels need several waves, or the plain form's first draws (for empty
+    // fragments too; 0.125 ns each beside CTAs of one replica, 0.25 ns beside clusters,
+    // which leave fewer SMs) longer than the windows they are for.
     // Both sides are estimates; T_pass is fitted to 8 to 1216 replicas of the shapes above.
     // 64 replicas of 96^3 cells in 24^3 fragments at 0.001: plain 1778 us per window on
-    // clusters, 450 in passes (mixed 507 and 227); 1216 of 48^3: plain 2078 and 805 (mixed
-    // 372 and 538).
+    // clusters, 450 in passes (mixed 507 and 227); 608 of 48^3: plain 617 and 533 (mixed
+    // 156 and 272), 304 of them 307 and 367.
     if (force == 0 && allowed && b->opts.schedule == 0) {
         int64_t frags = 0, res_vac = 0;
         double mean_vac = 0.0;
@@ -739,17 +740,20 @@ int plan_residency(kmc_batch* b)
                 work += us * share[c] / sms;
                 slowest = std::max(slowest, us);
             }
-        const double draws_us = prec ? 0.0 : 0.25e-3 * (double)frags * plain_ev;
-        if (load > 1.0 || draws_us > slowest) {
+        const bool beside = cluster_load > 0.0;
+        const double draws_us = prec ? 0.0 : (beside ? 0.25e-3 : 0.125e-3) * (double)frags * plain_ev;
+        // (mixed replicas on one CTA each are faster there in any number)
+        if ((prec ? cluster_load : load) > 1.0 || draws_us > slowest) {
             static const double base[3] = {175.0, 98.0, 205.0}, per_vac[3] = {20.0, 12.0, 20.0},
                                 per_frag[3] = {1.6e-4, 0.7e-4, 1.8e-4}, per_v[3] = {7.5e-4, 3.6e-4, 16e-4};
             const double waves_us = std::max(work, slowest);
-            const double resident_us = std::max(waves_us, draws_us) + 0.4 * std::min(waves_us, draws_us);
+            const double resident_us = std::max(waves_us, draws_us) + (beside ? 0.4 : 0.7) * std::min(waves_us, draws_us);
             const double passes_us = base[form] + per_vac[form] * mean_vac + per_frag[form] * (double)frags +
                                      per_v[form] * (double)res_vac;
-            // (waves disturb each other more than the estimate has it, with site energies most)
+            // (waves of clusters disturb each other more than the estimate has it, with site
+            // energies most; a batch that runs at once is the safer choice)
             static const double bias[3] = {1.0, 0.95, 0.9};
-            if (passes_us * (load > 1.0 ? bias[form] : 1.12) < resident_us) {
+            if (passes_us * (load <= 1.0 ? 1.12 : (cluster_load > 1.0 ? bias[form] : 1.02)) < resident_us) {
                 for (RepDesc& D : b->desc) D.resident = 0;
                 b->run_kernel.assign(b->n, 0);
                 b->run_ctas.assign(b->n, 0);
@@ -806,31 +810,44 @@ int plan_residency(kmc_batch* b)
     for (int r : pairs) cls[3].erase(std::find(cls[3].begin(), cls[3].end(), r));
     // more warps for the replicas with the most vacancies while every CTA still has
     // its share of an SM: a phase takes as long as its slowest visit, so a visit
-    // should not wait for a warp
-    {
-        double used = sms_used();
-        std::vector<std::pair<int64_t, int>> order;
-        for (int c = 0; c < 4; ++c)
-            for (int r : cls[c]) order.push_back({b->n_vac[r], r});
-        std::sort(order.rbegin(), order.rend());
-        for (auto& o : order) {
-            const int r = o.second;
-            const RepDesc& D = b->desc[r];
-            const int64_t maxc = phase_frags(r);
-            for (int c = 0; c < 3; ++c) {
-                auto it = std::find(cls[c].begin(), cls[c].end(), r);
-                if (it == cls[c].end()) continue;
-                const int to = c < 2 ? 2 : 3;
-                const int warps = threads[c] / 32;  // one visit per warp, at most maxc of them
-                const size_t nd = resident_smem_bytes(D, b->cap, threads[to], D.pre_g, D.pre_ev, prec);
-                if (maxc <= warps || o.first <= 4 * warps || used + share[to] - share[c] > (double)sms ||
-                    nd > RESIDENT_MAX_SMEM)
-                    break;
-                used += share[to] - share[c];
-                cls[c].erase(it);
-                cls[to].push_back(r);
-                need_of[r] = nd;
+    // should not wait for a warp.  First to 256 threads, then to 512, and where not all
+    // can have them, only those with a quarter more vacancies than the largest left
+    // behind, for which the batch would wait all the same: 300 replicas of 24^3 cells
+    // took 40 us per window (mixed) with 100 of them on 512 threads, and 22 with none.
+    // The plain form leaves half the SMs to k_draws (100 of 32^3: 73 -> 60 us).
+    const double most_sms = (prec ? 1.0 : 0.5) * sms;
+    for (int to = 2; to <= 3; ++to) {
+        std::vector<std::pair<int64_t, int>> want;  // (vacancies, replica)
+        for (int c = to - 2; c < to; ++c)
+            for (int r : cls[c]) {
+                const int warps = threads[c] / 32;  // one visit per warp, at most phase_frags of them
+                if ((to == 2 || c == 2) && phase_frags(r) > warps && b->n_vac[r] > 4 * warps) want.push_back({b->n_vac[r], r});
             }
+        std::sort(want.rbegin(), want.rend());
+        auto class_of = [&](int r) {
+            int c = 0;
+            while (c < 3 && std::find(cls[c].begin(), cls[c].end(), r) == cls[c].end()) ++c;
+            return c;
+        };
+        double used = sms_used();
+        size_t k = 0;
+        for (; k < want.size(); ++k) {
+            const double more = share[to] - share[class_of(want[k].second)];
+            if (used + more > most_sms) break;
+            used += more;
+        }
+        if (k < want.size()) {
+            const double left = 1.25 * (double)want[k].first;
+            while (k > 0 && (double)want[k - 1].first < left) --k;
+        }
+        for (size_t i = 0; i < k; ++i) {
+            const int r = want[i].second, c = class_of(r);
+            const RepDesc& D = b->desc[r];
+            const size_t nd = resident_smem_bytes(D, b->cap, threads[to], D.pre_g, D.pre_ev, prec);
+            if (nd > bounds[to]) continue;
+            cls[c].erase(std::find(cls[c].begin(), cls[c].end(), r));
+            cls[to].push_back(r);
+            need_of[r] = nd;
         }
     }
     for (int c = 0; c < 4; ++c)
