@@ -777,7 +777,8 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": "u64+f32+f64" if precision else "f64",
             "data": "synthetic",
             "config": {"workload": wl.name, "replicas": nrep, "windows_per_step": W,
-                       "precision": ("mixed (fp32 rates -> u64 fixed point, fp32 variate, fp64 clock)"
+                       "precision": ("mixed (fp32 rates -> u64 fixed point, fp32 variate, integer clock with the "
+                                      "outcome of an fp64 one)"
                                      if precision else "plain fp64"),
                        "n_tau": wl.n_tau, "edge": edge, "launch_opts": tuned_opts, "autotune": tuned,
                        "window_deficit": deficit,

@@ -62,7 +62,8 @@ extern "C" {
 
 /* arithmetic forms */
 #define FKMC_PLAIN 0 /* FP64 rates, FP64 prefix sums, FP64 clock */
-#define FKMC_MIXED 1 /* FP32 rates quantised to u64 fixed point, exact integer sums, FP32 variate + FP64 clock */
+#define FKMC_MIXED 1 /* FP32 rates quantised to u64 fixed point, exact integer sums, FP32 variate,
+                        the window test of an FP64 clock (in integers wherever those are exact) */
 
 typedef struct {
     int32_t nx, ny, nz; /* cells per dimension, each >= 1 and <= 65535 */

@@ -1464,7 +1464,6 @@ int kmc_set_barriers(kmc_batch* b, const kmc_barrier_table* tables, const double
             kmax32 = std::max(kmax32, k32[i]);
         }
         D.F = F;
-        D.two_pow_F = std::ldexp(1.0, F);
         D.tau = b->opts.n_tau / (8.0 * kmax);
         D.theta_tau = D.tau * (double)kmax32;
     }
