@@ -124,9 +124,11 @@ typedef struct {
     void* alloc_ctx;
     int32_t schedule;   /* 0 = auto: replicas whose state fits the shared memory of one SM, or of a
                            thread-block cluster (cluster_ctas), run in the resident kernels,
-                           the rest, and a dense replica that leaves most SMs idle there,
-                           one launch per colour phase; 1 = colour-phase launches
-                           only; 2 = resident kernels only (mixed form) */
+                           the rest, a dense replica that leaves most SMs idle there, and
+                           batches of so many replicas that the resident kernels would take
+                           longer (or whose buffers the device has no room for), one launch
+                           per colour phase; 1 = colour-phase launches only; 2 = resident
+                           kernels only (mixed form) */
     int32_t cluster_top; /* mixed form: how many of the largest replicas of the largest
                             shared-memory class run as 2-CTA thread-block clusters, a z-slab
                             each.  -1 (default) = SMs / 8, 0 = none */
@@ -149,9 +151,10 @@ typedef struct {
                              cluster-resident kernel (a thread-block cluster of up to 16 CTAs,
                              each holding a z-slab of fragment layers in shared memory, peers'
                              slabs reached through distributed shared memory) where its slabs
-                             fit.  0 (default) = so, with the most CTAs that fit, and also for
-                             a smaller replica whose phases hold many visits, on half as many
-                             CTAs as fragment layers (four at least), while SMs are free; -1 = never
+                             fit.  0 (default) = so, with the most CTAs at which all of the
+                             batch's clusters run at once, and also for smaller replicas whose
+                             phases hold many visits, on half as many CTAs as fragment layers
+                             (four at least), where all of those run at once; -1 = never
                              (the colour-phase kernels); 2..16 = every replica with that many
                              fragment layers or more, with exactly this many CTAs */
     int32_t reserved[2];

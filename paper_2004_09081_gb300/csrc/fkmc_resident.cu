@@ -34,26 +34,28 @@
 //           changed sites -- exactly the fragments whose total changed.
 //           Fragments of one colour never touch each other's sites (edges >= 2).
 //
-// What bounds it: dependent instructions.  A running warp issues one every 5 to
-// 6 cycles (2.2 of them fixed latency, 0.8 shared memory, 0.4 each branches and
-// instruction fetch), a phase lasts as long as its slowest visit (one to three
-// events, some 900 instructions), and no pipe is near its rate.  So a visit does
+// What bounds it: dependent instructions.  A running warp issues one every 6 to
+// 8 cycles (2.2 to 2.6 of them fixed latency, 1.0 to 1.1 shared memory, 0.3 to
+// 1.0 L2, 0.5 to 1.3 instruction fetch; 256 uneven replicas and one of 128^3
+// cells, calls of 8 and 16 windows), a phase lasts as long as its slowest visit
+// (one to three events, some 900 instructions), and no pipe is near its rate: a
+// quarter SM issues in 7 to 23% of its cycles.  So a visit does
 // as little as it can in sequence: totals by warp reductions with the prefix
 // scan only for events that happen, no FP64 instruction in the mixed form and
 // few in the plain one, records and tracer written an exchange late.
 // Measured (one GB300, whole calls with read-out, against linked per-fragment
 // lists for the mixed form and per-phase launches for the plain form): 256
-// uneven replicas mixed 60.5 -> 51.8 us per window, 24 traced 32^3 replicas
-// mixed 22.7 -> 18.7, 128^3 mixed 54.9 -> 48.0; plain: five 32^3 replicas 154 ->
-// 27.6, 8^3 112 -> 27.6, 128^3 195 -> 68.9.
+// uneven replicas mixed 60.5 -> 52.2 us per window, 24 traced 32^3 replicas
+// mixed 22.7 -> 18.4, 128^3 mixed 54.9 -> 47.7; plain: five 32^3 replicas 154 ->
+// 27.4, 8^3 112 -> 28.0, 128^3 195 -> 69.2.
 //
 // With site energies (plain form) a visit's chain is some 8,000 cycles per event
 // instead of 3,500: the rates wait for the energy field's words in L2, after an
 // exchange behind the 116 atomics that move the vacancy's share.  Five doped 96^3
-// replicas 302 -> 167 us per window, 128^3 in its own potential 482 -> 332 with
-// the solves.  Holding a visit's moves back and correcting the rates by pair
-// energies instead was slower (190 -> 200): the pair energies cost as many
-// instructions as the wait.
+// replicas 302 -> 156 us per window (182 in the first pass on a new state), 128^3
+// in its own potential 482 -> 313 with the solves.  Holding a visit's moves back
+// and correcting the rates by pair energies instead was slower (190 -> 200): the
+// pair energies cost as many instructions as the wait.
 //
 #include <cuda_runtime.h>
 
