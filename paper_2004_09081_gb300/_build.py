@@ -17,7 +17,7 @@ NVCC_FLAGS = [
     "-gencode", "arch=compute_103a,code=sm_103a",
     # no fused multiply-add anywhere: the plain form is bit-reproducible
     "--fmad=false", "-Xcompiler", "-fPIC,-ffp-contract=off",
-    "-shared",
+    "-shared", "-t", "0",  # the sources side by side
 ]
 
 

@@ -174,6 +174,7 @@ struct kmc_batch {
         cudaStream_t st;
         cudaEvent_t done;
         bool slabs;
+        bool long_lists;  // a replica of the class has lists of sixteen vacancies
     };
     std::vector<RClass> rclass;
     cudaEvent_t fork = nullptr;
@@ -515,6 +516,17 @@ int plan_residency(kmc_batch* b)
         if (fit_count[nc] < 0) fit_count[nc] = cluster_fits(form, nc, RESIDENT_MAX_SMEM);
         return fit_count[nc];
     };
+    // lists of sixteen vacancies where a fragment often holds more than eight and is so
+    // large that scanning it is slow (more than 31 cells per lane), mixed form: 96^3 cells
+    // in 12^3-cell fragments at 0.001 vacancies per site (5.2 a fragment) 85.7 -> 76.3 us
+    // per window; fragments of 8^3 cells gain less than the longer code costs the rest
+    auto long_lists = [&](int r) {
+        const RepDesc& D = b->desc[r];
+        int e[3];
+        for (int d = 0; d < 3; ++d) e[d] = D.base[d] + (D.rem[d] > 0 ? 1 : 0);
+        return prec == 1 && (double)b->n_vac[r] > 4.0 * D.nf[0] * D.nf[1] * D.nf[2] &&
+               (int64_t)((e[1] * e[2] + 31) / 32) * e[0] > 31;
+    };
     // replica r on the most of lo..hi CTAs that hold it and that the GPU can place
     struct Placed {
         RepDesc D;
@@ -522,14 +534,16 @@ int plan_residency(kmc_batch* b)
     };
     auto slabs_of = [&](int r, int lo, int hi, Placed* out) -> bool {
         // (events drawn ahead, list entries), the next where the slabs do not fit
-        const int want[4][2] = {{prec ? 4 : plain_ev, 8}, {prec ? 4 : plain_ev, 4}, {4, 4}, {2, 4}};
+        const int ev = prec ? 4 : plain_ev;
+        const int want[5][2] = {{ev, 16}, {ev, 8}, {ev, 4}, {4, 4}, {2, 4}};
         for (int nc = std::min(hi, (int)b->desc[r].nf[2]); nc >= lo; --nc) {
             if (fits(nc) <= 0) continue;
-            for (int q = 0; q < (form == 2 ? 8 : 4); ++q) {
+            for (int q = long_lists(r) ? 0 : 1; q < (form == 2 ? 10 : 5); ++q) {
+                if (q == 5 && !long_lists(r)) continue;
                 out->D = b->desc[r];
-                out->D.btab_smem = form == 2 && q < 4;
-                out->D.kslots = want[q & 3][1];
-                out->D.pre_ev = want[q & 3][0];
+                out->D.btab_smem = form == 2 && q < 5;
+                out->D.kslots = want[q % 5][1];
+                out->D.pre_ev = want[q % 5][0];
                 out->pl = ClusterPlan{};
                 if (!make_cluster_plan(out->D, b->cap, out->D.pre_ev, prec, nc, nc, &out->pl)) continue;
                 out->pl.rep = r;
@@ -561,8 +575,8 @@ int plan_residency(kmc_batch* b)
         int c = -1;
         size_t need = 0;
         // (Boltzmann tables in shared memory, list entries), the next where the state does not fit
-        const int lay[4][2] = {{form == 2, 8}, {0, 8}, {form == 2, 4}, {0, 4}};
-        for (int q = 0; q < 4 && allowed && c < 0; ++q) {
+        const int lay[6][2] = {{form == 2, 16}, {0, 16}, {form == 2, 8}, {0, 8}, {form == 2, 4}, {0, 4}};
+        for (int q = long_lists(r) ? 0 : 2; q < 6 && allowed && c < 0; ++q) {
             D.btab_smem = lay[q][0];
             D.kslots = lay[q][1];
             for (int k = 0; k < 4 && c < 0; ++k) {
@@ -862,8 +876,11 @@ int plan_residency(kmc_batch* b)
     std::vector<int32_t> order;
     for (int c = 0; c < 4; ++c) {
         if (cls[c].empty()) continue;
-        kmc_batch::RClass rc{(int)order.size(), (int)cls[c].size(), cmax[c], threads[c], 1, nullptr, nullptr, false};
-        for (int r : cls[c]) order.push_back(r);
+        kmc_batch::RClass rc{(int)order.size(), (int)cls[c].size(), cmax[c], threads[c], 1, nullptr, nullptr, false, false};
+        for (int r : cls[c]) {
+            order.push_back(r);
+            rc.long_lists = rc.long_lists || b->desc[r].kslots == 16;
+        }
         CK(cudaStreamCreateWithFlags(&rc.st, cudaStreamNonBlocking), "stream");
         CK(cudaEventCreateWithFlags(&rc.done, cudaEventDisableTiming), "event");
         b->rclass.push_back(rc);
@@ -882,7 +899,8 @@ int plan_residency(kmc_batch* b)
             smem = std::max(smem, cluster_smem_bytes(D, plans[e], b->cap, D.pre_ev, prec));
             ++e;
         }
-        kmc_batch::RClass rc{(int)k, (int)(e - k), smem, CLUSTER_THREADS, plans[k].ncta, nullptr, nullptr, true};
+        kmc_batch::RClass rc{(int)k, (int)(e - k), smem, CLUSTER_THREADS, plans[k].ncta, nullptr, nullptr, true, false};
+        for (size_t i = k; i < e; ++i) rc.long_lists = rc.long_lists || b->desc[plans[i].rep].kslots == 16;
         CK(cudaStreamCreateWithFlags(&rc.st, cudaStreamNonBlocking), "stream");
         CK(cudaEventCreateWithFlags(&rc.done, cudaEventDisableTiming), "event");
         b->rclass.push_back(rc);  // launched last-first: a cluster takes its SMs before single CTAs spread out
@@ -1527,10 +1545,11 @@ cudaError_t launch_classes(kmc_batch* b, int form, uint64_t w0, uint64_t windows
             if (!first) le = cudaEventRecord(c.done, c.st);
             if (le == cudaSuccess) le = cudaStreamWaitEvent(std::next(it)->st, first ? from : c.done, 0);
         }
+        const int f = c.long_lists ? 3 : form;
         if (le == cudaSuccess && c.slabs)
-            le = launch_cluster(form, args, b->d_plans + c.start, c.count, c.cluster, c.smem, w0, windows, draws, c.st);
+            le = launch_cluster(f, args, b->d_plans + c.start, c.count, c.cluster, c.smem, w0, windows, draws, c.st);
         else if (le == cudaSuccess)
-            le = launch_resident(form, args, b->d_reps + c.start, c.count, c.smem, c.threads, w0, windows, draws, c.st);
+            le = launch_resident(f, args, b->d_reps + c.start, c.count, c.smem, c.threads, w0, windows, draws, c.st);
         if (le == cudaSuccess) le = cudaEventRecord(c.done, c.st);
         if (le == cudaSuccess) le = cudaStreamWaitEvent(to, c.done, 0);
     }

@@ -71,7 +71,7 @@ struct __align__(16) RepDesc {
     uint64_t qng[6];
     int32_t pre_ev;        // resident kernels: events per fragment drawn ahead (2: block 0; 4: blocks 0, 1; 8: 0 .. 3)
     int32_t btab_smem;     // resident kernels: 1: the Boltzmann tables lie in shared memory
-    int32_t kslots;        // resident kernels: entries of a fragment's vacancy list (4 or 8)
+    int32_t kslots;        // resident kernels: entries of a fragment's vacancy list (4, 8 or 16)
     // resident kernels
     int64_t vmap_off;      // first word of this replica's site -> record map
     int64_t tmp_off;       // first fragment of this replica in the record copies of the stage-out

@@ -161,7 +161,7 @@ cudaError_t resident_prepare();
 cudaError_t launch_gate(cudaStream_t st);  // an empty kernel
 cudaError_t launch_draws(const RepDesc* d_descs, int nrep, int64_t max_frag, uint64_t w0, int windows, int ev_per,
                          int64_t frag_tot, Draw* draws, cudaStream_t st);
-// form: 0 plain, 1 mixed, 2 plain with site energies
+// form: 0 plain, 1 mixed, 2 plain with site energies, 3 mixed with lists of sixteen vacancies
 cudaError_t launch_resident(int form, const ResidentArgs& a, const int32_t* d_reps, int nreps, size_t smem, int threads,
                             uint64_t w0, uint64_t windows, const Draw* draws, cudaStream_t st);
 cudaError_t launch_cluster(int form, const ResidentArgs& a, const ClusterPlan* d_plans, int nplans, int ncta,

@@ -276,7 +276,8 @@ struct Layout {
 };
 constexpr unsigned NO_ROW = 0xffffu;      // a fragment's row of first draws: none,
 constexpr unsigned ROW_FULL = 0x8000u;    // or row | ROW_FULL where every event of the row was drawn (else two)
-constexpr int KSLOTS = 8;                  // entries of a fragment's list (or 4: RepDesc.kslots)
+constexpr int KSLOTS = 8;                  // entries of a fragment's list (or 4 or 16: RepDesc.kslots)
+constexpr int LONG_SLOTS = 16;
 constexpr int CLOCK_LOG = 8;  // events whose clock division the plain form puts off
 constexpr uint32_t UNLISTED = 0xfffffffeu;
 
@@ -337,7 +338,7 @@ __host__ __device__ inline Sizes sizes_single(const RepDesc& D, int cap, int nwa
     z.rows = rows;
     z.pre_ev = pre_ev;
     z.prec = prec;
-    z.kslots = D.kslots == 4 ? 4 : KSLOTS;
+    z.kslots = D.kslots == 4 ? 4 : (D.kslots == LONG_SLOTS ? LONG_SLOTS : KSLOTS);
     z.btab = D.btab_smem ? BOLTZ_LO + D.bhi_len : 0;
     return z;
 }
@@ -357,7 +358,7 @@ __host__ __device__ inline Sizes sizes_cluster(const RepDesc& D, const ClusterPl
     z.rows = 2;
     z.pre_ev = pre_ev;
     z.prec = prec;
-    z.kslots = D.kslots == 4 ? 4 : KSLOTS;
+    z.kslots = D.kslots == 4 ? 4 : (D.kslots == LONG_SLOTS ? LONG_SLOTS : KSLOTS);
     z.btab = D.btab_smem ? BOLTZ_LO + D.bhi_len : 0;
     return z;
 }
@@ -770,7 +771,9 @@ __global__ void __launch_bounds__(64) k_draws(const RepDesc* __restrict__ descs,
     }
 }
 
-template <int PREC, int NT, bool CL, bool SITE>
+// LONG: replicas of the launch may have lists of LONG_SLOTS (kept out of the others' code:
+// the branch alone costs them 2%)
+template <int PREC, int NT, bool CL, bool SITE, bool LONG>
 __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     k_resident(const RepDesc* __restrict__ descs, const int32_t* __restrict__ reps,
                const ClusterPlan* __restrict__ plans, uint64_t w0, uint64_t windows, uint32_t* occ, VacRec* recs,
@@ -1157,8 +1160,22 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     const uint32_t u = __shfl_sync(FULL, kc0, (lane & 3) * 8), v = __shfl_sync(FULL, kc1, (lane & 3) * 8);
                     return lane & 4 ? v : u;
                 };
-                int n;
-                if (!scan) {
+                int n = 0;
+                bool sorted = false;
+                if (LONG && !scan && ks == LONG_SLOTS) {  // with more than eight entries: by rank to wkey
+                    const uint32_t k = lane < LONG_SLOTS ? sl[lane] : DEAD;
+                    const unsigned held = __ballot_sync(FULL, k != DEAD);
+                    if (held >> KSLOTS) {
+                        int r = 0;
+#pragma unroll
+                        for (int q = 0; q < LONG_SLOTS; ++q) r += __shfl_sync(FULL, k, q) < k ? 1 : 0;
+                        if (k != DEAD) wkey[r] = k;
+                        __syncwarp();
+                        n = __popc(held);
+                        sorted = true;
+                    }
+                }
+                if (!scan && !sorted) {
                     n = __popc(__ballot_sync(FULL, kc0 != DEAD) & 0x01010101u) +
                         __popc(__ballot_sync(FULL, kc1 != DEAD) & 0x01010101u);
                     // the last visit left its slots' order: into site order where its exchanges changed it
@@ -1175,7 +1192,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                         kc1 = m + 4 < n ? wkey[m + 4] : DEAD;
                     }
                 } else {
-                    n = gather(S, geo, wkey, cap, lane, lo0, lo1, lo2, ex, ey, ez);
+                    if (scan) n = gather(S, geo, wkey, cap, lane, lo0, lo1, lo2, ex, ey, ez);
                     if (n > cap) {
                         if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
                         n = cap;
@@ -1537,9 +1554,11 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                     if (scan) S.stale[lf] = 0;
                 }
                 if (i > 0 || scan) {  // the fragment's list, in slot order
-                    if (n <= ks) {
+                    if (LONG && n > KSLOTS && n <= ks) {
+                        if (lane < ks) sl[lane] = lane < n ? wkey[lane] : DEAD;
+                    } else if (n <= ks) {
                         const uint32_t k = slot_key();
-                        if (lane < ks) sl[lane] = k;
+                        if (lane < ks) sl[lane] = !LONG || lane < KSLOTS ? k : DEAD;
                     } else if (lane == 0) {
                         sl[0] = UNLISTED;
                     }
@@ -1594,8 +1613,10 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
     // 4^3-cell ones, now 65 and 41 at 0.001 vacancies per site.)
     for (int f0 = warp; f0 < nfl; f0 += 32 * NW) {
         const int f = f0 + NW * lane;
-        for (unsigned td = __ballot_sync(FULL, f < nfl && (S.stale[f] != 0 || S.slots[f * ks] == UNLISTED)); td;
-             td &= td - 1) {
+        bool todo = f < nfl && (S.stale[f] != 0 || S.slots[f * ks] == UNLISTED);
+        if (LONG && f < nfl)
+            for (int q = KSLOTS; q < ks; ++q) todo = todo || S.slots[f * ks + q] != DEAD;  // more than the copies below take
+        for (unsigned td = __ballot_sync(FULL, todo); td; td &= td - 1) {
             const int fs = f0 + NW * (__ffs(td) - 1);
             const uint2 bx = S.box[fs];
             int n = gather(S, geo, wkey, cap, lane, (int)(bx.x & 1023u), (int)((bx.x >> 10) & 1023u), (int)(bx.x >> 20),
@@ -1604,7 +1625,8 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                 if (lane == 0) atomicOr(status, STATUS_OVERFLOW);
                 n = cap;
             }
-            if (n <= ks) {
+            const bool listed = n <= KSLOTS && n <= ks;
+            if (listed) {
                 if (lane < ks) S.slots[fs * ks + lane] = lane < n ? wkey[lane] : DEAD;
             } else {
                 for (int m = lane; m < n; m += 32) {
@@ -1615,7 +1637,7 @@ __global__ void __launch_bounds__(NT, (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1)))
                 if (lane == 0) S.stale[fs] = (uint8_t)n;  // more than a list holds: copied
             }
             __syncwarp();
-            if (n <= ks && lane == 0) S.stale[fs] = 0;
+            if (listed && lane == 0) S.stale[fs] = 0;
             __syncwarp();
         }
     }
@@ -1718,26 +1740,27 @@ using ResidentFn = void (*)(const RepDesc*, const int32_t*, const ClusterPlan*, 
                             VacRec*, uint32_t*, int32_t*, int32_t*, unsigned long long*, uint32_t*, int, NbTable,
                             const Draw*, int64_t, int, uint32_t, ResCache, SiteArgs);
 
-template <int PREC, bool SITE>
+template <int PREC, bool SITE, bool LONG = false>
 static ResidentFn resident_variant(int threads, bool cluster)
 {
-    if (cluster) return k_resident<PREC, CLUSTER_THREADS, true, SITE>;
-    if (threads == 128) return k_resident<PREC, 128, false, SITE>;
-    if (threads == 256) return k_resident<PREC, 256, false, SITE>;
-    return k_resident<PREC, 512, false, SITE>;
+    if (cluster) return k_resident<PREC, CLUSTER_THREADS, true, SITE, LONG>;
+    if (threads == 128) return k_resident<PREC, 128, false, SITE, LONG>;
+    if (threads == 256) return k_resident<PREC, 256, false, SITE, LONG>;
+    return k_resident<PREC, 512, false, SITE, LONG>;
 }
 
-// form: 0 plain, 1 mixed, 2 plain with site energies
+// form: 0 plain, 1 mixed, 2 plain with site energies, 3 mixed with long lists
 static ResidentFn resident_kernel(int form, int threads, bool cluster)
 {
     if (form == 1) return resident_variant<1, false>(threads, cluster);
+    if (form == 3) return resident_variant<1, false, true>(threads, cluster);
     return form == 2 ? resident_variant<0, true>(threads, cluster) : resident_variant<0, false>(threads, cluster);
 }
 
 cudaError_t resident_prepare()
 {
     cudaError_t e = cudaSuccess;
-    for (int form = 0; form < 3; ++form) {
+    for (int form = 0; form < 4; ++form) {
         for (int threads : {128, 256, 512})
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(resident_kernel(form, threads, false),

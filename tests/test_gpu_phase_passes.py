@@ -1,8 +1,9 @@
 """Paths that no other comparison with the oracle takes: the colour-phase passes in
 the plain form where the replica would fit the resident kernels, with and without
 site energies; the two-CTA slabs of kmc_opts.cluster_top; the mixed clock beyond
-its integer form; rates that underflow to zero; the multigrid's four-plane kernels
-where the planes do not divide by four; tables that grow within a call."""
+its integer form; rates that underflow to zero; long vacancy lists; the multigrid's
+four-plane kernels where the planes do not divide by four; tables that grow within
+a call."""
 import numpy as np
 import pytest
 
@@ -153,6 +154,20 @@ def test_rates_that_underflow_to_zero(fk, orc, prec, sched):
     ref = orc.Lattice(cells, nf, nv, nh, seed=4, tracer=True)
     ref.set_rates(2.0, 0.2, 30.0, a_ang=4.01, cap_v=64, precision=prec)
     check(b, ref, (60, 60))
+
+
+# 4.5 to 20 vacancies per fragment of 12^3 (and 10 x 11 x 13) cells: lists of sixteen fill
+# past eight, overflow and refill; one CTA and two slabs
+@pytest.mark.parametrize("ctas", [0, 2])
+@pytest.mark.parametrize("cells,nf,nv", [((24, 24, 24), (2, 2, 2), 36), ((24, 24, 24), (2, 2, 2), 70),
+                                         ((20, 22, 26), (2, 2, 2), 120), ((24, 24, 24), (2, 2, 2), 160)])
+def test_lists_of_sixteen(fk, orc, cells, nf, nv, ctas):
+    b = fk.Batch([(*cells, 4.01)], [(nv, 2500)], 6, nfrag=nf, precision=1, tracer=True, cap_v=64, cluster_ctas=ctas)
+    b.set_barriers(0.6, 0.4, 900.0, field_z=2e7)
+    ref = orc.Lattice(cells, nf, nv, 2500, seed=6, tracer=True)
+    ref.set_rates(0.6, 0.4, 900.0, Ez=2e7, a_ang=4.01, cap_v=64, precision=1)
+    assert b.info().kernel == (2 if ctas else 1)
+    check(b, ref, (30, 1, 30, 1))
 
 
 def test_multigrid_with_planes_that_do_not_divide_by_four(fk, orc):
